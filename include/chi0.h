@@ -50,7 +50,8 @@ typedef enum {
 } chi0_status;
 
 typedef enum {
-  CHI0_FP64 = 0,        /* FP64 end to end (CUDA-core DFMA contraction) */
+  CHI0_FP64 = 0,        /* FP64 accuracy end to end (contraction by exact modular products on the tensor
+                           cores, or FP64 multiply-adds where that is faster) */
   CHI0_SPLIT_BF16 = 1,  /* FP32 pair stage; contraction on tcgen05 with hi+lo BF16 operands */
   CHI0_SPLIT_FP16 = 2   /* FP32 pair stage; contraction on tcgen05 with hi+lo FP16 operands */
 } chi0_precision;
@@ -116,7 +117,8 @@ chi0_status chi0_plan_hermitian(chi0_plan plan, int* on);
  * on the plan), or of the last failed plan creation when plan is NULL. */
 const char* chi0_last_error(chi0_plan plan);
 
-/* Bytes of device workspace held by the plan. */
+/* Bytes of device workspace held by the plan.  It grows on the first use of some calls (the
+ * contraction of FP64 plans, the pipelined build, the dielectric inverse). */
 size_t chi0_workspace_bytes(chi0_plan plan);
 
 /* Synchronise `stream` and report device-side failures recorded since the
@@ -146,7 +148,10 @@ chi0_status chi0_pairs(chi0_plan plan, int iq, const void* psi_v, const int32_t*
  * For the explicit bands E_col = E_c and w_col = 1; for an energy-grid state
  * of Eq. 4, E_col = E_i and w_col = g(E_i) dE_i.
  * M: (device) [n_v*n_c][n_G[iq]] complex; E_v (device) [n_v]; E_col, w_col (device) [n_c];
- * chi0: (device) [n_freq][n_G[iq]][n_G[iq]] complex128, accumulated in place (caller zeroes it). */
+ * chi0: (device) [n_freq][n_G[iq]][n_G[iq]] complex128, accumulated in place (caller zeroes it).
+ * FP64 plans allocate the workspace of the tensor-core contraction on the first call that gains from
+ * it (at most about 16 GB); inside a stream capture before such a call, or when it cannot be had, the
+ * sums run as FP64 multiply-adds. */
 chi0_status chi0_accumulate(chi0_plan plan, int iq, const void* M, int n_v, int n_c,
                             const double* E_v, const double* E_col, const double* w_col,
                             void* chi0, void* stream);

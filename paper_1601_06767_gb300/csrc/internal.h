@@ -85,6 +85,9 @@ struct chi0_plan_s {
   void* wfn_ws = nullptr;    // scratch of the three-pass wavefunction transform (FP32 plans on 96^3)
   size_t wfn_ws_bytes = 0;
   void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
+  void* d_mod = nullptr;     // workspace of the FP64 contraction on the tensor cores (first use)
+  size_t mod_bytes = 0;
+  int mod_state = 0;         // -1: could not be allocated (the CUDA-core contraction runs)
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)
@@ -143,6 +146,24 @@ cudaError_t launch_weights(const chi0_plan_s* p, int64_t p0, int64_t K, int n_c,
                            const double* E_col, const double* w_col, double2* f, cudaStream_t s);
 cudaError_t launch_contract_f64(const chi0_plan_s* p, int nG, const double2* M, int64_t K,
                                 const double2* f, double2* chi, cudaStream_t s);
+// FP64 contraction by exact modular products on the tensor cores (kern_mod.cu)
+struct ModSizes {
+  int Kc, nw, rows, ldR, n_part;   // pairs, frequencies and chi0 rows at a time; row stride of the residues
+  size_t off_a, off_r, off_part, off_scale, off_exp, bytes;
+};
+ModSizes mod_sizes(const chi0_plan_s* p, int nG);
+int mod_launches(const chi0_plan_s* p, int nG);   // kernels per block of pairs
+bool mod_gemm_usable();
+cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_t K, const double2* f, double2* chi,
+                                void* ws, cudaStream_t s);
+// residue products R[plane][rows][cols] = A[plane mod a_planes] B[plane mod b_planes]^T
+struct ModGemm {
+  const uint16_t* A;               // [a_planes][rows_a][Kp]
+  const uint16_t* B;               // [b_planes][cols][Kp]
+  int16_t* R;                      // [planes][rows][ldR]
+  int rows_a, row0, rows, cols, ldR, Kp, planes, a_planes, b_planes;
+};
+cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s);
 // one q-point's share of a batched tensor-core contraction
 struct TcJob {
   int nG;

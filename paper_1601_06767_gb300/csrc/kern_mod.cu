@@ -1,0 +1,638 @@
+// FP64 contraction of Eq. 1 on the tensor cores (CHI0_FP64 plans):
+//   chi0[w][G][H] += sum_p f_p(w) M_p(G) conj(M_p(H))
+// as exact modular products (modgemm.cuh): FP64 accuracy from 26 FP16 products.
+//
+// Steps of a block of K pairs: row norms and scales (k_mod_fmax, k_mod_rowmax,
+// k_mod_norms, k_mod_scales), residue planes of conj(M) and of W_w = f(w) M
+// (k_mod_pack), 26 products per frequency with their sums reduced modulo m
+// (k_mod_gemm), reconstruction and addition into chi0 (k_mod_add).
+//
+// The CUDA-core contraction ran at the FP64 pipe's rate (two multiply-adds per clock
+// and SM): 790 ms for 2048 pairs, N_G 2500, nine frequencies.  This form takes
+// 6.4 ms: 4.0 ms of products (the 16-bit tensor pipe 67 % busy at 1.9 GHz, 1.6
+// PFLOP/s executed), 1.3 ms reconstruction, 0.75 ms planes, 0.2 ms norms.  The
+// static 8-atom contraction (3840 pairs, N_G 350): 15.97 ms -> 0.20 ms.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
+#include <algorithm>
+#include <string>
+
+#include "cplx.cuh"
+#include "internal.h"
+#include "modgemm.cuh"
+#include "tc_ptx.cuh"
+
+namespace chi0 {
+namespace {
+
+using mod::NM;
+using mod::NPL;
+
+// ---------------------------------------------------------------------------
+// scales
+// ---------------------------------------------------------------------------
+// ef[w] = largest magnitude word of the factors f[w][0..K)
+__global__ void __launch_bounds__(256) k_mod_fmax(const double2* __restrict__ f, int64_t K, uint32_t* __restrict__ ef) {
+  __shared__ uint32_t red[8];
+  uint32_t m = 0;
+  for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
+    const double2 v = f[(int64_t)blockIdx.x * K + k];
+    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) m = max(m, red[i]);
+    ef[blockIdx.x] = m;
+  }
+}
+
+constexpr int ST_COLS = 64, ST_ROWS = 128;   // a statistics block: 64 sphere points x 128 pairs
+
+// eg[G] = largest magnitude word of M[0..K)[G] (eg cleared by the caller)
+__global__ void __launch_bounds__(256) k_mod_rowmax(const double2* __restrict__ M, int nG, int64_t K,
+                                                    uint32_t* __restrict__ eg) {
+  const int G = blockIdx.x * ST_COLS + (threadIdx.x & 63);
+  if (G >= nG) return;
+  const int64_t k1 = min(K, (int64_t)(blockIdx.y + 1) * ST_ROWS);
+  uint32_t m = 0;
+  for (int64_t k = (int64_t)blockIdx.y * ST_ROWS + (threadIdx.x >> 6); k < k1; k += 4) {
+    const double2 v = M[k * nG + G];
+    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  atomicMax(eg + G, m);
+}
+
+// part[block of pairs][slot][G] = sum over the block of |M|^2 4^-eg (slot 0) and of
+// |f(w)|^2 |M|^2 4^-(eg + ef) (slot 1 + w): FP64 sums in a fixed order (a scale that
+// depended on the order could move a result by its rounding from run to run)
+__global__ void __launch_bounds__(256) k_mod_norms(const double2* __restrict__ M, int nG, int64_t K,
+                                                   const double2* __restrict__ f, int n_freq,
+                                                   const uint32_t* __restrict__ eg, const uint32_t* __restrict__ ef,
+                                                   double* __restrict__ part) {
+  __shared__ double f2[ST_ROWS];
+  __shared__ double red[4][ST_COLS];
+  const int g = threadIdx.x & 63, r = threadIdx.x >> 6, G = blockIdx.x * ST_COLS + g;
+  const int64_t k0 = (int64_t)blockIdx.y * ST_ROWS;
+  double m2[ST_ROWS / 4];
+  const uint32_t wg = G < nG ? eg[G] : 0;
+  const bool use = wg >= 0x00100000u && wg < 0x7ff00000u;
+  // 2^-eg in two steps: its exponent may leave the normal range
+  const int e = mod::word_exp(wg);
+  const double s1 = use ? mod::pow2d(-(e / 2)) : 0.0, s2 = use ? mod::pow2d(-(e - e / 2)) : 0.0;
+#pragma unroll
+  for (int j = 0; j < ST_ROWS / 4; ++j) {
+    const int64_t k = k0 + r + 4 * j;
+    m2[j] = 0.0;
+    if (use && k < K) {
+      const double2 v = M[k * nG + G];
+      const double x = v.x * s1 * s2, y = v.y * s1 * s2;
+      m2[j] = fma(x, x, y * y);
+    }
+  }
+  for (int slot = 0; slot <= n_freq; ++slot) {
+    __syncthreads();
+    if (slot > 0 && threadIdx.x < ST_ROWS) {
+      const int64_t k = k0 + threadIdx.x;
+      double v = 0.0;
+      const uint32_t wf = ef[slot - 1];
+      if (k < K && wf >= 0x00100000u && wf < 0x7ff00000u) {
+        const double2 d = f[(int64_t)(slot - 1) * K + k];
+        const int q = mod::word_exp(wf);
+        const double t1 = mod::pow2d(-(q / 2)), t2 = mod::pow2d(-(q - q / 2));
+        const double x = d.x * t1 * t2, y = d.y * t1 * t2;
+        v = fma(x, x, y * y);
+      }
+      f2[threadIdx.x] = v;
+    }
+    __syncthreads();
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < ST_ROWS / 4; ++j) s = slot ? fma(m2[j], f2[r + 4 * j], s) : s + m2[j];
+    red[r][g] = s;
+    __syncthreads();
+    if (r == 0 && G < nG)
+      part[((size_t)blockIdx.y * (n_freq + 1) + slot) * nG + G] = (red[0][g] + red[1][g]) + (red[2][g] + red[3][g]);
+  }
+}
+
+// scale exponents: slot 0 (conj(M), operand B) and 1 + w (W_w, operand A)
+__global__ void __launch_bounds__(256) k_mod_scales(const double* __restrict__ part, int n_part, int nG, int n_freq,
+                                                    const uint32_t* __restrict__ eg, const uint32_t* __restrict__ ef,
+                                                    int* __restrict__ scale) {
+  const int G = blockIdx.x * blockDim.x + threadIdx.x, slot = blockIdx.y;
+  if (G >= nG) return;
+  double s = 0.0;
+  for (int b = 0; b < n_part; ++b) s += part[((size_t)b * (n_freq + 1) + slot) * nG + G];
+  const uint32_t wg = eg[G], wf = slot ? ef[slot - 1] : 0x3ff00000u;
+  int r;
+  if (wg >= 0x7ff00000u || wf >= 0x7ff00000u) r = mod::NO_SCALE;   // the result row is NaN
+  else r = mod::scale_exp(s, mod::word_exp(wg) + (slot ? mod::word_exp(wf) : 0), slot ? mod::BETA_A : mod::BETA_B);
+  scale[(size_t)slot * nG + G] = r;
+}
+
+// ---------------------------------------------------------------------------
+// residue planes
+// ---------------------------------------------------------------------------
+constexpr int PK_G = 16, PK_K = 64;   // tile: 16 sphere points x 64 pairs, transposed through shared memory
+
+// Planes [26][nG][Kp] (FP16) of conj(M) into Bp (when not NULL) and of W_w = f(w) M,
+// w = w0 .. w0 + nw, into Ap (26 planes per frequency).  A warp holds one sphere
+// point, a lane two neighbouring pairs: 128-byte stores per plane.
+__global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M, int nG, int64_t K, int Kp,
+                                                  const double2* __restrict__ f, int w0, int nw,
+                                                  const int* __restrict__ scale, uint32_t* __restrict__ Bp,
+                                                  uint32_t* __restrict__ Ap) {
+  __shared__ double2 tile[PK_K][PK_G + 1];
+  __shared__ double2 fs[PK_K];
+  const int G0 = blockIdx.x * PK_G;
+  const int64_t p0 = (int64_t)blockIdx.y * PK_K;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int e = threadIdx.x; e < PK_K * PK_G; e += blockDim.x) {
+    const int pp = e / PK_G, g = e - pp * PK_G;
+    double2 v = make_double2(0.0, 0.0);
+    if (p0 + pp < K && G0 + g < nG) v = M[(p0 + pp) * nG + G0 + g];
+    tile[pp][g] = v;
+  }
+  const size_t plane = (size_t)nG * (Kp / 2);
+  for (int slot = Bp ? -1 : 0; slot < nw; ++slot) {
+    __syncthreads();
+    if (slot >= 0 && threadIdx.x < PK_K) {
+      const int64_t p = p0 + threadIdx.x;
+      fs[threadIdx.x] = p < K ? f[(int64_t)(w0 + slot) * K + p] : make_double2(0.0, 0.0);
+    }
+    __syncthreads();
+    const int* sc = scale + (size_t)(slot < 0 ? 0 : 1 + w0 + slot) * nG;
+    uint32_t* dst = slot < 0 ? Bp : Ap + (size_t)slot * NPL * plane;
+    for (int g = warp; g < PK_G; g += 8) {
+      const int G = G0 + g;
+      if (G >= nG) break;
+      const int s = sc[G];
+      double2 a = tile[2 * lane][g], b = tile[2 * lane + 1][g];
+      if (slot >= 0) {
+        a = cmul(fs[2 * lane], a);
+        b = cmul(fs[2 * lane + 1], b);
+      }
+      mod::store_residues(mod::limbs(mod::quantise(a.x, s)), mod::limbs(mod::quantise(a.y, s)),
+                          mod::limbs(mod::quantise(b.x, s)), mod::limbs(mod::quantise(b.y, s)), slot < 0,
+                          dst + (size_t)G * (Kp / 2) + p0 / 2 + lane, plane);
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// modular products
+// ---------------------------------------------------------------------------
+// R[b][i][j] = sum_k A[b][i][k] B[b][j][k] (mod m of plane b), |R| <= 257.
+// A CTA pair computes a 256 x 256 tile with tcgen05.mma.cta_group::2 (each CTA
+// holds 128 rows of A and 128 of B: 32 KB per 512 MMA cycles, half the operand
+// traffic per flop of two single-CTA 128 x 128 tiles).  Warp 0 issues the TMA
+// loads (128-byte rows of 64 k) into a ring, warp 1 of the first CTA the MMAs into
+// two 256-column accumulators, warps 4..11 drain them: a chain is 256 k (the
+// longest whose sums are exact), 2048 MMA cycles, against 128 elements per thread
+// of four FP32 operations each (in packed pairs), so the reductions hide behind
+// the MMAs.  The register split is the contraction kernels' (kern_tc.cu).
+constexpr int GM = 256, GN = 256, GK = 64;
+constexpr int CHAIN = 256 / GK;                    // stages per accumulation chain
+constexpr int A_BYTES = (GM / 2) * GK * 2, B_BYTES = (GN / 2) * GK * 2;
+constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int STAGES = 6;
+constexpr int EPI_WARP0 = 4, EPI_WARPS = 8, THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
+constexpr int REG_LAUNCH = 168, REG_LOW = 72, REG_HIGH = 216;
+static_assert(EPI_WARP0 * 32 * REG_LOW + EPI_WARPS * 32 * REG_HIGH <= THREADS * REG_LAUNCH,
+              "register split exceeds the launch's registers");
+constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 1024 + 256;
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory above the per-block limit");
+constexpr uint64_t WAIT_BUDGET_NS = 2000000000ull;
+
+struct GemmArgs {
+  CUtensorMap tmA, tmB;
+  int16_t* R;
+  int rows, cols, ldR;         // output of one plane: rows x cols, ldR = cols rounded up to 8
+  int row0;                    // first row of A
+  int tiles_m, tiles_n, n_b;   // tiles and planes
+  int a_planes, b_planes;      // planes of A and B (a plane index is taken modulo these)
+  int nK;                      // stages of GK
+};
+
+// Residues are kept in blocks of 32 rows x 8 columns (512 bytes): a warp, whose lanes
+// hold 32 rows of the accumulator, writes whole blocks.  Index of (plane b, row, column).
+__host__ __device__ __forceinline__ size_t res_plane(int rows, int ldR) { return (size_t)((rows + 31) / 32) * 32 * ldR; }
+__device__ __forceinline__ size_t res_index(int rows, int ldR, int b, int row, int col) {
+  return b * res_plane(rows, ldR) + ((size_t)(row >> 5) * (ldR >> 3) + (col >> 3)) * 256 + (row & 31) * 8 + (col & 7);
+}
+
+struct GemmBars {
+  uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2], done;
+  uint32_t tmem_base;
+};
+static_assert(sizeof(GemmBars) <= 256, "barriers");
+
+// K-major tile of 128-byte rows written by TMA with 128-byte swizzling; 8-row groups 1024 bytes apart
+__device__ __forceinline__ uint64_t sdesc_sw128(const void* tile) {
+  const uint64_t addr = tc::smem_u32(tile);
+  return ((addr >> 4) & 0x3FFFull) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
+}
+
+// item -> (plane, tile row, tile column): planes outermost (both operand planes stay in L2), inside
+// a plane groups of 8 tile rows, column by column
+__device__ __forceinline__ void gemm_item(const GemmArgs& P, int item, int& b, int& tm, int& tn) {
+  const int tiles = P.tiles_m * P.tiles_n;
+  b = item / tiles;
+  const int t = item - b * tiles;
+  const int grp = t / (8 * P.tiles_n), first = grp * 8, rows = min(8, P.tiles_m - first);
+  const int within = t - grp * 8 * P.tiles_n;
+  tm = first + within % rows;
+  tn = within / rows;
+}
+
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+__constant__ float c_mod[NM] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f, 433.f, 421.f, 409.f, 401.f, 397.f, 389.f};
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
+  extern __shared__ __align__(1024) unsigned char smem_mod[];
+  unsigned char* tiles = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_mod) + 1023) & ~uintptr_t(1023));
+  GemmBars* bar = reinterpret_cast<GemmBars*>(tiles + STAGES * STAGE_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = tc::cluster_rank();
+  const bool leader = rank == 0;
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int nK = P.nK, n_items = P.tiles_m * P.tiles_n * P.n_b;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&bar->tfull[b], 1);
+      tc::mbar_init(&bar->tempty[b], 2 * EPI_WARPS);
+    }
+    tc::mbar_init(&bar->done, 1);
+    tc::fence_mbar_init();
+    tc::prefetch_tmap(&P.tmA);
+    tc::prefetch_tmap(&P.tmB);
+  }
+  if (warp == 1) {
+    tc::tmem_alloc_pair(&bar->tmem_base, 512);
+    tc::tmem_relinquish_pair();
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();      // barriers of both CTAs initialised before any remote use
+  tc::fence_after();
+  const uint32_t tbase = bar->tmem_base;
+
+  if (warp < EPI_WARP0) {
+    tc::setmaxnreg_dec<REG_LOW>();
+    if (warp == 0) {
+      if (lane == 0) {
+        // ---------------- TMA producer (both CTAs) ----------------
+        int64_t gs = 0;
+        int slot = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int item = pair; item < n_items && ok; item += npairs) {
+          int b, tm, tn;
+          gemm_item(P, item, b, tm, tn);
+          const int arow = P.row0 + tm * GM + (int)rank * (GM / 2), brow = tn * GN + (int)rank * (GN / 2);
+          const int pa = b % P.a_planes, pb = b % P.b_planes;
+          for (int kc = 0; kc < nK; ++kc, ++gs) {
+            const int s = slot;
+            if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, status, 1, WAIT_BUDGET_NS)) { ok = false; break; }
+            if (++slot == STAGES) {
+              slot = 0;
+              ph ^= 1u;
+            }
+            // the first CTA's barrier counts the loads of both CTAs
+            if (leader) tc::mbar_arrive_expect_tx(&bar->full[s], 2 * STAGE_BYTES);
+            const uint32_t fb = tc::mapa(&bar->full[s], 0);
+            unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+            tc::tma_load_3d_pair(st, &P.tmA, fb, kc * GK, arow, pa);
+            tc::tma_load_3d_pair(st + A_BYTES, &P.tmB, fb, kc * GK, brow, pb);
+          }
+        }
+        // copies of this CTA still in flight land before it may exit
+        for (int64_t g = max((int64_t)0, gs - STAGES); g < gs; ++g)
+          tc::mbar_wait(&bar->empty[g % STAGES], (uint32_t)((g / STAGES) & 1), status, 1, WAIT_BUDGET_NS);
+      }
+    } else if (warp == 1) {
+      if (lane == 0 && leader) {
+        // ---------------- MMA issuer (first CTA of the pair) ----------------
+        int64_t gc = 0;
+        int slot = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        constexpr uint32_t idesc = tc::idesc_f16(false, false, GM, GN);
+        for (int item = pair; item < n_items && ok; item += npairs) {
+          for (int kc = 0, pos = 0; kc < nK; ++kc) {
+            const int buf = (int)(gc & 1);
+            if (pos == 0) {
+              if (!tc::mbar_wait(&bar->tempty[buf], (uint32_t)(((gc >> 1) & 1) ^ 1), status, 1, WAIT_BUDGET_NS)) {
+                ok = false;
+                break;
+              }
+              tc::fence_after();
+            }
+            const int s = slot;
+            if (!tc::mbar_wait(&bar->full[s], ph, status, 1, WAIT_BUDGET_NS)) {
+              ok = false;
+              break;
+            }
+            if (++slot == STAGES) {
+              slot = 0;
+              ph ^= 1u;
+            }
+            tc::fence_after();
+            const unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+            const uint64_t da = sdesc_sw128(st), db = sdesc_sw128(st + A_BYTES);
+            const uint32_t d = tbase + buf * GN;
+#pragma unroll
+            for (int ks = 0; ks < GK / 16; ++ks)   // a K step of 16 is 32 bytes of the row
+              tc::mma_f16_pair(d, da + ks * 2, db + ks * 2, idesc, (pos > 0 || ks > 0) ? 1u : 0u);
+            tc::mma_commit_pair(&bar->empty[s], 0x3);
+            if (++pos == CHAIN || kc == nK - 1) {
+              tc::mma_commit_pair(&bar->tfull[buf], 0x3);
+              ++gc;
+              pos = 0;
+            }
+          }
+        }
+        tc::mma_commit_pair(&bar->done, 0x1);
+        tc::mbar_wait(&bar->done, 0, status, 1, WAIT_BUDGET_NS);
+      }
+    }
+  } else {
+    tc::setmaxnreg_inc<REG_HIGH>();
+    // ---------------- epilogue (both CTAs, own 128 rows) ----------------
+    const int ew = warp - EPI_WARP0, quad = warp & 3, half = ew >> 2;
+    const int nch = (nK + CHAIN - 1) / CHAIN;
+    int64_t gc = 0;
+    bool ok = true;
+    for (int item = pair; item < n_items && ok; item += npairs) {
+      int b, tm, tn;
+      gemm_item(P, item, b, tm, tn);
+      const float m = c_mod[(b % NPL) >> 1], im = 1.0f / m;
+      const uint64_t inv2 = pack2(im, im), neg2 = pack2(-m, -m);
+      const uint64_t magic = pack2(12582912.f, 12582912.f), nmagic = pack2(-12582912.f, -12582912.f);
+      uint64_t acc[64];
+#pragma unroll
+      for (int i = 0; i < 64; ++i) acc[i] = 0ull;
+      for (int c = 0; c < nch; ++c, ++gc) {
+        const int buf = (int)(gc & 1);
+        if (!tc::mbar_wait(&bar->tfull[buf], (uint32_t)((gc >> 1) & 1), status, 1, WAIT_BUDGET_NS)) { ok = false; break; }
+        tc::fence_after();
+        const uint32_t ta = tbase + ((uint32_t)(quad * 32) << 16) + buf * GN + half * 128;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float v[32];
+          tc::tmem_ld32(ta + 32 * j, v);
+          tc::tmem_ld_wait();
+          tc::reg_after_wait(v);
+          if (j == 3) {
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive_cluster(tc::mapa(&bar->tempty[buf], 0));
+          }
+          // acc = (acc + x) - m round((acc + x) / m): |acc + x| <= 254^2 256 + 257 < 2^24, every step exact
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const uint64_t y = add2(acc[16 * j + i], pack2(v[2 * i], v[2 * i + 1]));
+            const uint64_t t = add2(fma2(y, inv2, magic), nmagic);
+            acc[16 * j + i] = fma2(t, neg2, y);
+          }
+        }
+      }
+      if (!ok) break;
+      const int row = tm * GM + (int)rank * (GM / 2) + quad * 32 + lane, col = tn * GN + half * 128;
+      if (row < (P.rows + 31) / 32 * 32) {
+        int16_t* o = P.R + res_index(P.rows, P.ldR, b, row, col);
+        // the low 16 bits of 1.5 2^23 + r are r in two's complement
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          if (col + 8 * i < P.ldR) {
+            uint32_t w[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              float x, y;
+              unpack2(add2(acc[4 * i + k], magic), x, y);
+              w[k] = __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x5410);
+            }
+            *reinterpret_cast<uint4*>(o + 256 * i) = make_uint4(w[0], w[1], w[2], w[3]);
+          }
+        }
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();      // neither CTA leaves while the pair's MMAs may still read its operands
+  tc::fence_after();
+  if (warp == 1) tc::tmem_dealloc_pair(tbase, 512);
+}
+
+// ---------------------------------------------------------------------------
+// reconstruction
+// ---------------------------------------------------------------------------
+// Fractions of the real and imaginary parts of four elements: r points at eight columns of one row,
+// the lane takes the even ones (sh = 16) or the odd ones (sh = 0)
+template <int I = 0>
+__device__ __forceinline__ void gather_fractions(const int16_t* __restrict__ r, size_t plane, int sh,
+                                                 mod::Frac (&re)[4], mod::Frac (&im)[4]) {
+  const uint4 u = __ldcs(reinterpret_cast<const uint4*>(r + (2 * I) * plane));
+  const uint4 v = __ldcs(reinterpret_cast<const uint4*>(r + (2 * I + 1) * plane));
+  const uint32_t uw[4] = {u.x, u.y, u.z, u.w}, vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    mod::frac_add_uv<I>(re[c], im[c], (int)(uw[c] << sh) >> 16, (int)(vw[c] << sh) >> 16);
+  if constexpr (I + 1 < NM) gather_fractions<I + 1>(r, plane, sh, re, im);
+}
+
+// chi[w][row0 + i][j] += the value of R's planes (w, i, j).  A warp takes 16 rows x 8
+// columns (half a residue block); two neighbouring lanes share a row and take its
+// even and odd columns, so that each access to chi covers whole 32-byte sectors.
+// Grid (column blocks / 4, half row blocks, frequencies).
+__global__ void __launch_bounds__(128) k_mod_add(const int16_t* __restrict__ R, int rows, int row0, int nG, int ldR,
+                                                 const int* __restrict__ scale, int w0, double2* __restrict__ chi) {
+  const int lane = threadIdx.x & 31, w = blockIdx.z;
+  const int j0 = 8 * (blockIdx.x * 4 + (threadIdx.x >> 5)), i = blockIdx.y * 16 + (lane >> 1);
+  if (j0 >= nG || i >= rows) return;
+  mod::Frac re[4] = {}, im[4] = {};
+  gather_fractions(R + res_index(rows, ldR, w * NPL, i, j0), res_plane(rows, ldR), lane & 1 ? 0 : 16, re, im);
+  const int G = row0 + i, sa = scale[(size_t)(1 + w0 + w) * nG + G];
+  double2* o = chi + ((size_t)(w0 + w) * nG + G) * nG + j0 + (lane & 1);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int j = j0 + 2 * c + (lane & 1);
+    if (j >= nG) break;
+    const int sb = scale[j];
+    double2 d;
+    if (sa == mod::NO_SCALE || sb == mod::NO_SCALE) d = make_double2(nan(""), nan(""));
+    else d = make_double2(mod::frac_value(re[c], -sa - sb), mod::frac_value(im[c], -sa - sb));
+    double2 v = o[2 * c];
+    v.x += d.x;
+    v.y += d.y;
+    o[2 * c] = v;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// host
+// ---------------------------------------------------------------------------
+PFN_cuTensorMapEncodeTiled_v12000 encoder() {
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(f);
+  }();
+  return fn;
+}
+
+bool encode(CUtensorMap* tm, const void* base, int Kp, int rows, int planes) {
+  cuuint64_t dims[3] = {(cuuint64_t)Kp, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)Kp * 2, (cuuint64_t)Kp * 2 * rows};
+  cuuint32_t box[3] = {GK, 128, 1}, estr[3] = {1, 1, 1};
+  return encoder()(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int round64(int64_t x) { return (int)((x + 63) / 64 * 64); }
+size_t al256(size_t x) { return (x + 255) / 256 * 256; }
+
+}  // namespace
+
+// The register split of the kernel adds up to REG_LAUNCH per thread (see kern_tc.cu): a build with
+// another count is never launched.
+bool mod_gemm_usable() {
+  static const bool ok = [] {
+    cudaFuncAttributes a;
+    if (!encoder() || cudaFuncGetAttributes(&a, k_mod_gemm) != cudaSuccess || a.numRegs != REG_LAUNCH ||
+        cudaFuncSetAttribute(k_mod_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return true;
+  }();
+  return ok;
+}
+
+cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s) {
+  GemmArgs P{};
+  if (!encode(&P.tmA, g.A, g.Kp, g.rows_a, g.a_planes) || !encode(&P.tmB, g.B, g.Kp, g.cols, g.b_planes))
+    return cudaErrorInvalidValue;
+  P.R = g.R;
+  P.rows = g.rows;
+  P.cols = g.cols;
+  P.ldR = g.ldR;
+  P.row0 = g.row0;
+  P.tiles_m = (g.rows + GM - 1) / GM;
+  P.tiles_n = (g.cols + GN - 1) / GN;
+  P.n_b = g.planes;
+  P.a_planes = g.a_planes;
+  P.b_planes = g.b_planes;
+  P.nK = g.Kp / GK;
+  int dev = 0, nsm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  const int pairs = (int)std::min<int64_t>((int64_t)P.tiles_m * P.tiles_n * P.n_b, std::max(1, nsm / 2));
+  k_mod_gemm<<<2 * pairs, THREADS, SMEM_BYTES, s>>>(P, p->d_status);
+  return cudaGetLastError();
+}
+
+// Workspace of the contraction: pairs and frequencies held at a time, rows of chi0 per product
+ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
+  constexpr int64_t kPlanes = (int64_t)4 << 30, kRes = (int64_t)4 << 30;   // operand planes, residues
+  ModSizes z;
+  z.ldR = (nG + 7) / 8 * 8;
+  const int64_t per_pair = (int64_t)NPL * 2 * nG;
+  z.Kc = (int)std::min<int64_t>(round64(p->max_pairs), std::max<int64_t>(64, kPlanes / per_pair / 64 * 64));
+  // enough frequencies per launch for 40 waves of CTA pairs, within the same memory
+  const int64_t tiles = (int64_t)((nG + GM - 1) / GM) * ((nG + GN - 1) / GN) * NPL;
+  int64_t nw = std::min<int64_t>(p->n_freq, std::max<int64_t>(1, (40 * 76 + tiles - 1) / tiles));
+  nw = std::max<int64_t>(1, std::min(nw, kPlanes / (per_pair * z.Kc)));
+  nw = std::max<int64_t>(1, std::min(nw, kRes / ((int64_t)NPL * 2 * nG * z.ldR)));
+  z.nw = (int)nw;
+  z.rows = (int)std::min<int64_t>(nG, std::max<int64_t>(GM, kRes / ((int64_t)NPL * 2 * z.ldR * nw) / GM * GM));
+  z.n_part = (z.Kc + ST_ROWS - 1) / ST_ROWS;
+  const size_t nf1 = (size_t)p->n_freq + 1;
+  z.off_a = al256((size_t)per_pair * z.Kc);
+  z.off_r = z.off_a + al256((size_t)per_pair * z.Kc * nw);
+  z.off_part = z.off_r + al256((size_t)NPL * 2 * nw * res_plane(z.rows, z.ldR));
+  z.off_scale = z.off_part + al256(nf1 * z.n_part * nG * sizeof(double));
+  z.off_exp = z.off_scale + al256(nf1 * nG * sizeof(int));
+  z.bytes = z.off_exp + al256((nG + nf1) * sizeof(uint32_t));
+  return z;
+}
+
+int mod_launches(const chi0_plan_s* p, int nG) {
+  const ModSizes z = mod_sizes(p, nG);
+  const int groups = (p->n_freq + z.nw - 1) / z.nw, panels = (nG + z.rows - 1) / z.rows;
+  return 4 + groups * (1 + 2 * panels);
+}
+
+// K <= mod_sizes().Kc pairs of M with factors f [n_freq][K]
+cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_t K, const double2* f, double2* chi,
+                                void* ws, cudaStream_t s) {
+  const ModSizes z = mod_sizes(p, nG);
+  unsigned char* b = reinterpret_cast<unsigned char*>(ws);
+  uint16_t* Bp = reinterpret_cast<uint16_t*>(b);
+  uint16_t* Ap = reinterpret_cast<uint16_t*>(b + z.off_a);
+  int16_t* R = reinterpret_cast<int16_t*>(b + z.off_r);
+  double* part = reinterpret_cast<double*>(b + z.off_part);
+  int* scale = reinterpret_cast<int*>(b + z.off_scale);
+  uint32_t* eg = reinterpret_cast<uint32_t*>(b + z.off_exp);
+  uint32_t* ef = eg + nG;
+  const int nf = p->n_freq, Kp = round64(K);
+  cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * nG, s);
+  if (e != cudaSuccess) return e;
+  const int n_part = (int)((K + ST_ROWS - 1) / ST_ROWS);
+  const dim3 gst((nG + ST_COLS - 1) / ST_COLS, n_part);
+  k_mod_fmax<<<nf, 256, 0, s>>>(f, K, ef);
+  k_mod_rowmax<<<gst, 256, 0, s>>>(M, nG, K, eg);
+  k_mod_norms<<<gst, 256, 0, s>>>(M, nG, K, f, nf, eg, ef, part);
+  k_mod_scales<<<dim3((nG + 255) / 256, nf + 1), 256, 0, s>>>(part, n_part, nG, nf, eg, ef, scale);
+  for (int w0 = 0; w0 < nf; w0 += z.nw) {
+    const int nw = std::min(z.nw, nf - w0);
+    k_mod_pack<<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(M, nG, K, Kp, f, w0, nw, scale,
+                                                                     w0 == 0 ? (uint32_t*)Bp : nullptr, (uint32_t*)Ap);
+    for (int r0 = 0; r0 < nG; r0 += z.rows) {
+      const int rows = std::min(z.rows, nG - r0);
+      ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, NPL * nw, NPL * nw, NPL};
+      e = launch_mod_gemm(p, g, s);
+      if (e != cudaSuccess) return e;
+      k_mod_add<<<dim3((z.ldR / 8 + 3) / 4, (rows + 15) / 16, nw), 128, 0, s>>>(R, rows, r0, nG, z.ldR, scale, w0, chi);
+    }
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace chi0

@@ -103,6 +103,7 @@ void free_plan(chi0_plan_s* p) {
   cudaFree(w.T3d); cudaFree(w.T3f);
   cudaFree(p->d_omega); cudaFree(p->d_D); cudaFree(p->d_M); cudaFree(p->d_f);
   cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->d_inv); cudaFree(p->wfn_ws);
+  cudaFree(p->d_mod);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
     cudaFree(p->bq_M[i]);
     cudaFree(p->bq_f[i]);
@@ -738,12 +739,50 @@ chi0_status chi0_pairs(chi0_plan p, int iq, const void* psi_v, const int32_t* v_
   return pairs_impl(p, iq, psi_v, v_idx, n_v, psi_c, c_idx, 0, n_c, M, n_c, (cudaStream_t)stream);
 }
 
+// Where the tensor-core form of the FP64 contraction pays: estimates in microseconds from a sweep of
+// N_G 1-2500, 1-9 frequencies and 8-4096 pairs.  The CUDA-core kernel takes 4.1 us per pair while its
+// 64 x 64 tiles do not fill the GPU and runs at 1.1 TFLOP/s beyond; the modular products take some
+// ten short launches, an output cost (reconstruction, one chain of products) per element of chi0 and a
+// slope 25 to 100 times smaller (N_G 350, one frequency: 32 pairs 146 against 77, 8 pairs 80 against
+// 76; 4096 pairs 16931 against 220).
+static bool mod_pays(int nG, int n_freq, int64_t K) {
+  const double n2 = (double)nG * nG * n_freq;
+  const double direct = std::max(4.1 * K, 8.0 * n2 * K / 1.1e6);
+  const double modular = 60.0 + 10.0 * (n_freq - 1) + n2 * (3e-5 + 4.5e-8 * K);
+  return modular < direct;
+}
+
+// Workspace of the FP64 contraction on the tensor cores for the plan's largest sphere, allocated on
+// first use: not inside a stream capture (the CUDA-core kernel runs there unless an earlier call has
+// allocated it) and given up for good when the memory cannot be had.
+static bool mod_ready(chi0_plan p, cudaStream_t s) {
+  if (p->d_mod) return true;
+  if (p->mod_state < 0 || !chi0::mod_gemm_usable()) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  size_t need = 0;
+  for (auto& q : p->q) need = std::max(need, chi0::mod_sizes(p, q.nG).bytes);
+  if (cudaMalloc(&p->d_mod, need) != cudaSuccess) {
+    cudaGetLastError();
+    p->d_mod = nullptr;
+    p->mod_state = -1;
+    return false;
+  }
+  p->mod_bytes = need;
+  p->ws_bytes += need;
+  return true;
+}
+
 static chi0_status accumulate_impl(chi0_plan p, int iq, const void* M, int n_v, int n_c,
                                    const double* E_v, const double* E_col, const double* w_col,
                                    void* chi, cudaStream_t s) {
   const int nG = p->q[iq].nG;
   const int64_t np = (int64_t)n_v * n_c;
-  const int64_t blk = p->block_pairs > 0 ? std::min(p->block_pairs, p->max_pairs) : p->max_pairs;
+  int64_t blk = p->block_pairs > 0 ? std::min(p->block_pairs, p->max_pairs) : p->max_pairs;
+  if (!chi0::is_split(p)) blk = std::min<int64_t>(blk, chi0::mod_sizes(p, nG).Kc);
   for (int64_t p0 = 0; p0 < np; p0 += blk) {
     int64_t K = std::min<int64_t>(blk, np - p0);
     {
@@ -757,8 +796,13 @@ static chi0_status accumulate_impl(chi0_plan p, int iq, const void* M, int n_v, 
       if (e != cudaSuccess)
         return fail(p, CHI0_ERR_CUDA, "tensor-core contraction: " + why + " " + cudaGetErrorString(e));
     } else {
-      chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, 1);
-      CK(p, chi0::launch_contract_f64(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, s));
+      if (mod_pays(nG, p->n_freq, K) && mod_ready(p, s)) {
+        chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, chi0::mod_launches(p, nG));
+        CK(p, chi0::launch_contract_mod(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, p->d_mod, s));
+      } else {
+        chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, 1);
+        CK(p, chi0::launch_contract_f64(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, s));
+      }
     }
   }
   return CHI0_OK;
@@ -1041,6 +1085,7 @@ chi0_status chi0_build_batched(chi0_plan p, const void* const* psi_v, int n_v, c
   key.push_back(psi_c); key.push_back(c_idx); key.push_back(E_col); key.push_back(w_col);
   key.push_back((const void*)(intptr_t)n_v); key.push_back((const void*)(intptr_t)n_c);
   if (!p->graph_exec || key != p->graph_key) {
+    if (!chi0::is_split(p)) mod_ready(p, s);   // its workspace cannot be allocated inside the capture
     if (p->graph_exec) { cudaGraphExecDestroy(p->graph_exec); p->graph_exec = nullptr; }
     if (!p->cap_stream) CK(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     const bool timing = p->prof_timing;

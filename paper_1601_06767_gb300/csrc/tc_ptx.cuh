@@ -129,8 +129,11 @@ __device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
 }
+// Arrive on a barrier of either CTA of the pair.  It orders tensor-memory reads (tcgen05 fences
+// around it) and no global memory, so it takes the default scope: with a cluster-scope release the
+// arrival waits for the thread's global stores or reductions to be performed.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
 // TMA tile into this CTA's shared memory; completion counted on a barrier that
 // may belong to the peer CTA (cluster address)
