@@ -194,7 +194,8 @@ chi0_status chi0_build_batched(chi0_plan plan, const void* const* psi_v, int n_v
  *   f'_p(w)      = -(w_p/2) [(dE_p - w + i d)^-2 + (dE_p + w + i d)^-2],
  *   grad_Ev[iv]  = sum_ic grad dE_p,   grad_Ecol[ic] = -sum_iv grad dE_p.
  * Complex gradients use the dL/dRe + i dL/dIm convention.  Give exactly one of
- *   grad_chi0 (device) [n_freq][n_G][n_G] complex128: dense Gamma (FP64 CUDA-core products), or
+ *   grad_chi0 (device) [n_freq][n_G][n_G] complex128: dense Gamma (FP64 products: exact modular
+ *             products on the tensor cores in a workspace as for chi0_accumulate, or multiply-adds), or
  *   diag_g    (device) [n_freq][n_G] double: Gamma_w = diag(diag_g[w]) (one fused pass; n_freq <= 64).
  * M, E_v, E_col, w_col as for chi0_accumulate.  Outputs (written, not accumulated):
  * grad_M (device) [n_v*n_c][n_G] complex (the plan's complex type), grad_Ev (device) [n_v],

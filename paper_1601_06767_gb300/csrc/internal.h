@@ -85,9 +85,9 @@ struct chi0_plan_s {
   void* wfn_ws = nullptr;    // scratch of the three-pass wavefunction transform (FP32 plans on 96^3)
   size_t wfn_ws_bytes = 0;
   void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
-  void* d_mod = nullptr;     // workspace of the FP64 contraction on the tensor cores (first use)
+  void* d_mod = nullptr;     // workspace of the modular products (first use)
   size_t mod_bytes = 0;
-  int mod_state = 0;         // -1: could not be allocated (the CUDA-core contraction runs)
+  size_t mod_limit = SIZE_MAX;   // smallest size that could not be allocated (the CUDA-core kernels run instead)
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)
@@ -164,6 +164,15 @@ struct ModGemm {
   int rows_a, row0, rows, cols, ldR, Kp, planes, a_planes, b_planes;
 };
 cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s);
+// scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B
+cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+                                 uint16_t* planes, cudaStream_t s);
+cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+                                 uint16_t* planes, cudaStream_t s);
+// the same of the conjugate transpose of X [n][rows] (operand B; ws: mod_cols_ws_bytes)
+size_t mod_cols_ws_bytes(int n, int rows);
+cudaError_t launch_mod_pack_cols_conj(const double2* X, int n, int rows, int Kp, int* scale, uint16_t* planes,
+                                      void* ws, cudaStream_t s);
 // one q-point's share of a batched tensor-core contraction
 struct TcJob {
   int nG;
@@ -185,6 +194,12 @@ cudaError_t launch_backward(chi0_plan_s* p, int nG, const void* M, int64_t p0, i
                             const double* E_v, const double* E_col, const double* w_col, const double2* gamma,
                             const double* diag, void* gM, double* gEv, double* gEc, double* work, cudaStream_t s);
 int bwd_max_freq();
+// dense adjoint of all pairs on the tensor cores (kern_bwd.cu): workspace, where it pays, the launches
+size_t bwd_mod_ws_bytes(const chi0_plan_s* p, int nG, int64_t n_pairs);
+bool bwd_mod_pays(const chi0_plan_s* p, int nG, int64_t n_pairs);
+cudaError_t launch_backward_mod(chi0_plan_s* p, int nG, const void* M, int64_t n_pairs, int n_c, const double* E_v,
+                                const double* E_col, const double* w_col, const double2* gamma, void* gM, double* gEv,
+                                double* gEc, double* work, void* ws, cudaStream_t s);
 // first-order energy-substitution estimate of Eq. 3/4 (one block; writes the grid energy of every
 // band to E_sub when it is not NULL and the sum to *out, both device pointers)
 cudaError_t launch_energy_substitution(const double* E_c, const double* sens, int n_c, int N0, double dE, double E_max,

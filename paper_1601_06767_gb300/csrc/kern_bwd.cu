@@ -8,9 +8,13 @@
 // Diagonal upstream (Gamma_w = diag(g_w), g real): one fused bandwidth-bound pass
 //   grad M_p(G) = sum_w 2 Re f_p(w) g_w(G) M_p(G),  grad dE_p = sum_w Re f'_p(w) sum_G g_w(G) |M_p(G)|^2.
 // Dense upstream: two FP64 complex products per frequency, Y = M Gamma^T and
-// Z = M conj(Gamma), combined in the epilogue.
+// Z = M conj(Gamma), as modular products on the tensor cores (modgemm.cuh) combined
+// by k_bwd_mod, or as FP64 multiply-adds combined in the epilogue (k_bwd_dense).
+#include <algorithm>
+
 #include "cplx.cuh"
 #include "internal.h"
+#include "modgemm.cuh"
 
 namespace chi0 {
 namespace {
@@ -189,6 +193,85 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
   }
 }
 
+// Dense upstream from the residues of Y and Z (modgemm.cuh), frequencies w0 .. w0 + nw: plane set
+// 2 w holds Y, 2 w + 1 holds Z of the block's pairs.
+//   gM[k][G] (+)= sum_w conj(f) Y + f Z;  part[k][tile] (+)= Re( f' conj(sum_{G in tile} conj(M) Y) )
+// A CTA takes 16 pairs x 64 sphere points, a warp 16 x 8 of them (half a residue block): two
+// neighbouring lanes share a pair and take its even and odd points.  Bound by the integer pipe
+// (reconstruction of two values from 52 residues), the FP64 pipe a third of it: 356 us for 4096
+// pairs, N_G 1200, one frequency (530 us with one CTA per SM, before its registers were bounded).
+// The whole adjoint of that size: 77.0 -> 1.02 ms.
+template <typename C>
+__global__ void __launch_bounds__(256, 2)
+k_bwd_mod(const int16_t* __restrict__ R, int rows, int ldR, const int* __restrict__ sA, const int* __restrict__ sB,
+          const C* __restrict__ M, int nG, int64_t p0, int n_c, const double* __restrict__ E_v,
+          const double* __restrict__ E_col, const double* __restrict__ w_col, const double2* __restrict__ omega, int w0,
+          int nw, double delta, C* __restrict__ gM, double* __restrict__ part, int ntile) {
+  __shared__ double2 sf[16], sfp[16];
+  __shared__ double red[8][16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, odd = lane & 1, r = lane >> 1;
+  const int i = blockIdx.y * 16 + r, j0 = blockIdx.x * 64 + warp * 8;     // pair of the block, first point
+  const int64_t k = i;
+  const bool in = i < rows && j0 < nG;
+  const size_t plane = mod::res_plane(rows, ldR);
+  double2 g[4], m[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const int G = j0 + 2 * c + odd;
+    g[c] = m[c] = make_double2(0.0, 0.0);
+    if (in && G < nG) {
+      m[c] = ld_d(M, k * nG + G);
+      if (w0 > 0) g[c] = ld_d(gM, k * nG + G);
+    }
+  }
+  double t = 0.0;
+  for (int w = 0; w < nw; ++w) {
+    __syncthreads();
+    if (threadIdx.x < 16 && blockIdx.y * 16 + threadIdx.x < rows) {
+      const int64_t p = p0 + blockIdx.y * 16 + threadIdx.x, iv = p / n_c, ic = p - iv * n_c;
+      factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, omega[w0 + w], delta, &sf[threadIdx.x], &sfp[threadIdx.x]);
+    }
+    __syncthreads();
+    if (!in) continue;
+    double2 y[4], z[4];
+#pragma unroll
+    for (int part2 = 0; part2 < 2; ++part2) {
+      mod::Frac re[4] = {}, im[4] = {};
+      mod::gather_fractions(R + mod::res_index(rows, ldR, (2 * w + part2) * mod::NPL, i, j0), plane, odd ? mod::ODD : mod::EVEN, re, im);
+      const int sa = sA[k];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int G = min(j0 + 2 * c + odd, nG - 1), sb = sB[(size_t)(2 * w + part2) * nG + G];
+        double2 v;
+        if (sa == mod::NO_SCALE || sb == mod::NO_SCALE) v = make_double2(nan(""), nan(""));
+        else v = make_double2(mod::frac_value(re[c], -sa - sb), mod::frac_value(im[c], -sa - sb));
+        if (part2) z[c] = v; else y[c] = v;
+      }
+    }
+    const double2 f = sf[r], fc = make_double2(f.x, -f.y), fp = sfp[r];
+    double2 q = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      cfma(g[c], fc, y[c]);
+      cfma(g[c], f, z[c]);
+      if (j0 + 2 * c + odd < nG) cfma(q, make_double2(m[c].x, -m[c].y), y[c]);
+    }
+    t += fp.x * q.x + fp.y * q.y;     // Re(f' conj(q))
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (in && j0 + 2 * c + odd < nG) st_c(gM, k * nG + j0 + 2 * c + odd, g[c]);
+  t += __shfl_xor_sync(0xffffffffu, t, 1);
+  if (!odd) red[warp][r] = t;
+  __syncthreads();
+  if (threadIdx.x < 16 && blockIdx.y * 16 + threadIdx.x < rows) {
+    double s = 0.0;
+    for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
+    double* o = part + (int64_t)(blockIdx.y * 16 + threadIdx.x) * ntile + blockIdx.x;
+    *o = w0 > 0 ? *o + s : s;
+  }
+}
+
 // gdE[k] = sum_t part[k][t]
 __global__ void k_rowsum(const double* __restrict__ part, int64_t K, int ntile, double* __restrict__ gdE) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -299,6 +382,100 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
   k_reduce_rows<<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEv);
   k_reduce_cols<<<(unsigned)((n_c + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEc);
   return cudaGetLastError();
+}
+
+// Where the tensor-core form of the dense adjoint pays: estimates in microseconds.  A tile of
+// k_bwd_dense takes 4.1 us per sphere point of the contraction (FP64 pipe), so even one pair costs that
+// times N_G per frequency; the modular form costs its launches, the planes of Gamma and the products.
+bool bwd_mod_pays(const chi0_plan_s* p, int nG, int64_t n_pairs) {
+  const double n2 = (double)nG * nG, K = (double)n_pairs;
+  const double direct = p->n_freq * std::max(4.1 * nG, 16.0 * n2 * K / 1.1e6);
+  const double modular = 80.0 + p->n_freq * (20.0 + 6e-5 * n2 + 7e-5 * K * nG + 9e-8 * n2 * K);
+  return modular < direct;
+}
+
+// Memory of a pass over the pairs: planes of Gamma and Gamma^H for nw frequencies, planes of M and
+// residues of Y and Z for kc pairs, scales
+struct BwdMod {
+  int Kp, ldR, nw, kc;
+  size_t off_a, off_r, off_sa, off_sb, off_ws, bytes;
+};
+static BwdMod bwd_mod_sizes(const chi0_plan_s* p, int nG, int64_t n_pairs) {
+  constexpr int64_t kMem = (int64_t)4 << 30;
+  auto al = [](size_t x) { return (x + 255) / 256 * 256; };
+  BwdMod z;
+  z.Kp = (nG + 63) / 64 * 64;
+  z.ldR = (nG + 7) / 8 * 8;
+  const int64_t gam = (int64_t)2 * mod::NPL * 2 * nG * z.Kp;                  // one frequency's planes
+  z.nw = (int)std::max<int64_t>(1, std::min<int64_t>(p->n_freq, kMem / gam));
+  const int64_t per_pair = (int64_t)2 * z.nw * mod::NPL * 2 * z.ldR;           // residues of one pair
+  z.kc = (int)std::min<int64_t>({n_pairs, p->max_pairs, std::max<int64_t>(256, kMem / per_pair / 256 * 256)});
+  z.off_a = al((size_t)gam * z.nw);
+  z.off_r = z.off_a + al((size_t)mod::NPL * 2 * z.kc * z.Kp);
+  z.off_sa = z.off_r + al((size_t)2 * z.nw * mod::NPL * 2 * mod::res_plane(z.kc, z.ldR));
+  z.off_sb = z.off_sa + al(sizeof(int) * (size_t)z.kc);
+  z.off_ws = z.off_sb + al(sizeof(int) * (size_t)2 * z.nw * nG);
+  z.bytes = z.off_ws + al(mod_cols_ws_bytes(nG, nG));
+  return z;
+}
+size_t bwd_mod_ws_bytes(const chi0_plan_s* p, int nG, int64_t n_pairs) { return bwd_mod_sizes(p, nG, n_pairs).bytes; }
+
+template <typename C>
+static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pairs, int n_c, const double* E_v,
+                                const double* E_col, const double* w_col, const double2* gamma, C* gM, double* gEv,
+                                double* gEc, double* work, void* ws, cudaStream_t s) {
+  const BwdMod z = bwd_mod_sizes(p, nG, n_pairs);
+  unsigned char* b = reinterpret_cast<unsigned char*>(ws);
+  uint16_t* Bp = reinterpret_cast<uint16_t*>(b);
+  uint16_t* Ap = reinterpret_cast<uint16_t*>(b + z.off_a);
+  int16_t* R = reinterpret_cast<int16_t*>(b + z.off_r);
+  int* sA = reinterpret_cast<int*>(b + z.off_sa);
+  int* sB = reinterpret_cast<int*>(b + z.off_sb);
+  const size_t set = (size_t)mod::NPL * nG * z.Kp;       // 16-bit words of one operand's planes
+  const int ntile = (nG + 63) / 64;
+  cudaError_t e;
+  // every pair block keeps its sums over the frequencies in gM and part: with several groups of
+  // frequencies the groups run inside the block and the planes of Gamma are made again for each
+  for (int64_t p0 = 0; p0 < n_pairs; p0 += z.kc) {
+    const int K = (int)std::min<int64_t>(z.kc, n_pairs - p0);
+    double* gdE = work;
+    double* part = work + K;
+    e = launch_mod_pack_rows(M + p0 * nG, K, nG, nG, z.Kp, true, sA, Ap, s);
+    if (e != cudaSuccess) return e;
+    for (int w0 = 0; w0 < p->n_freq; w0 += z.nw) {
+      const int nw = std::min(z.nw, p->n_freq - w0);
+      if (p0 == 0 || z.nw < p->n_freq)
+        for (int w = 0; w < nw; ++w) {
+          const double2* G = gamma + (size_t)(w0 + w) * nG * nG;
+          e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG, Bp + 2 * w * set, s);
+          if (e == cudaSuccess)
+            e = launch_mod_pack_cols_conj(G, nG, nG, z.Kp, sB + (size_t)(2 * w + 1) * nG, Bp + (2 * w + 1) * set,
+                                          b + z.off_ws, s);
+          if (e != cudaSuccess) return e;
+        }
+      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL};
+      e = launch_mod_gemm(p, g, s);
+      if (e != cudaSuccess) return e;
+      k_bwd_mod<C><<<dim3(ntile, (K + 15) / 16), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,
+                                                              w_col, p->d_omega, w0, nw, p->delta, gM + p0 * nG, part,
+                                                              ntile);
+    }
+    k_rowsum<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(part, K, ntile, gdE);
+    const int64_t rows = (p0 + K - 1) / n_c - p0 / n_c + 1;
+    k_reduce_rows<<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEv);
+    k_reduce_cols<<<(unsigned)((n_c + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEc);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_backward_mod(chi0_plan_s* p, int nG, const void* M, int64_t n_pairs, int n_c, const double* E_v,
+                                const double* E_col, const double* w_col, const double2* gamma, void* gM, double* gEv,
+                                double* gEc, double* work, void* ws, cudaStream_t s) {
+  if (is_split(p))
+    return bwd_mod_impl<float2>(p, nG, (const float2*)M, n_pairs, n_c, E_v, E_col, w_col, gamma, (float2*)gM, gEv, gEc,
+                                work, ws, s);
+  return bwd_mod_impl<double2>(p, nG, (const double2*)M, n_pairs, n_c, E_v, E_col, w_col, gamma, (double2*)gM, gEv, gEc,
+                               work, ws, s);
 }
 
 cudaError_t launch_backward(chi0_plan_s* p, int nG, const void* M, int64_t p0, int64_t K, int n_c, const double* E_v,

@@ -28,6 +28,13 @@ namespace {
 
 using mod::NM;
 using mod::NPL;
+using mod::gather_fractions;
+using mod::res_index;
+using mod::res_plane;
+using mod::add2;
+using mod::fma2;
+using mod::pack2;
+using mod::unpack2;
 
 // ---------------------------------------------------------------------------
 // scales
@@ -175,11 +182,66 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
         a = cmul(fs[2 * lane], a);
         b = cmul(fs[2 * lane + 1], b);
       }
-      mod::store_residues(mod::limbs(mod::quantise(a.x, s)), mod::limbs(mod::quantise(a.y, s)),
-                          mod::limbs(mod::quantise(b.x, s)), mod::limbs(mod::quantise(b.y, s)), slot < 0,
+      mod::store_residues(mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s)),
+                          mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), slot < 0,
                           dst + (size_t)G * (Kp / 2) + p0 / 2 + lane, plane);
     }
   }
+}
+
+// Rows whose contraction index is contiguous: X [rows][n] with row stride ld.
+__device__ __forceinline__ double2 ld_wide(const float2* p, size_t i) { return make_double2(p[i].x, p[i].y); }
+__device__ __forceinline__ double2 ld_wide(const double2* p, size_t i) { return p[i]; }
+
+// scale[row]: a CTA per row, the largest magnitude and then the norm (FP32, relative to the
+// largest: what underflows there does not count), summed in a fixed order
+template <typename C>
+__global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X, int n, size_t ld, int beta,
+                                                        int* __restrict__ scale) {
+  __shared__ uint32_t mx[4];
+  __shared__ float sm[4];
+  const C* x = X + blockIdx.x * ld;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t m = 0;
+  for (int i = threadIdx.x; i < n; i += 128) {
+    const double2 v = ld_wide(x, i);
+    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if (lane == 0) mx[warp] = m;
+  __syncthreads();
+  m = max(max(mx[0], mx[1]), max(mx[2], mx[3]));
+  const int e = mod::word_exp(m);
+  float s = 0.f;
+  if (m >= 0x00100000u && m < 0x7ff00000u)
+    for (int i = threadIdx.x; i < n; i += 128) {
+      const double2 v = ld_wide(x, i);
+      const float a = mod::scaled_abs(v.x, e), b = mod::scaled_abs(v.y, e);
+      s = fmaf(a, a, fmaf(b, b, s));
+    }
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) sm[warp] = s;
+  __syncthreads();
+  if (threadIdx.x == 0)
+    scale[blockIdx.x] = m >= 0x7ff00000u ? mod::NO_SCALE
+                                         : mod::scale_exp((double)((sm[0] + sm[1]) + (sm[2] + sm[3])), e, beta);
+}
+
+// planes [26][rows][Kp] of X; a warp takes 64 elements of a row
+template <typename C>
+__global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, int rows, int n, size_t ld, int Kp,
+                                                       const int* __restrict__ scale, uint32_t* __restrict__ dst) {
+  const int lane = threadIdx.x & 31, segs = Kp / 64;
+  const int64_t unit = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (unit >= (int64_t)rows * segs) return;
+  const int r = (int)(unit / segs), k = (int)(unit - (int64_t)r * segs) * 64 + 2 * lane;
+  const C* x = X + r * ld;
+  const int s = scale[r];
+  const double2 a = k < n ? ld_wide(x, k) : make_double2(0.0, 0.0);
+  const double2 b = k + 1 < n ? ld_wide(x, k + 1) : make_double2(0.0, 0.0);
+  mod::store_residues(mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s)),
+                      mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), false,
+                      dst + (size_t)r * (Kp / 2) + k / 2, (size_t)rows * (Kp / 2));
 }
 
 // ---------------------------------------------------------------------------
@@ -217,13 +279,6 @@ struct GemmArgs {
   int nK;                      // stages of GK
 };
 
-// Residues are kept in blocks of 32 rows x 8 columns (512 bytes): a warp, whose lanes
-// hold 32 rows of the accumulator, writes whole blocks.  Index of (plane b, row, column).
-__host__ __device__ __forceinline__ size_t res_plane(int rows, int ldR) { return (size_t)((rows + 31) / 32) * 32 * ldR; }
-__device__ __forceinline__ size_t res_index(int rows, int ldR, int b, int row, int col) {
-  return b * res_plane(rows, ldR) + ((size_t)(row >> 5) * (ldR >> 3) + (col >> 3)) * 256 + (row & 31) * 8 + (col & 7);
-}
-
 struct GemmBars {
   uint64_t full[STAGES], empty[STAGES], tfull[2], tempty[2], done;
   uint32_t tmem_base;
@@ -247,25 +302,6 @@ __device__ __forceinline__ void gemm_item(const GemmArgs& P, int item, int& b, i
   const int within = t - grp * 8 * P.tiles_n;
   tm = first + within % rows;
   tn = within / rows;
-}
-
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 
 __constant__ float c_mod[NM] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f, 433.f, 421.f, 409.f, 401.f, 397.f, 389.f};
@@ -417,7 +453,7 @@ k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
             __syncwarp();
             if (lane == 0) tc::mbar_arrive_cluster(tc::mapa(&bar->tempty[buf], 0));
           }
-          // acc = (acc + x) - m round((acc + x) / m): |acc + x| <= 254^2 256 + 257 < 2^24, every step exact
+          // acc = (acc + x) - m round((acc + x) / m): |acc + x| <= 255^2 256 + 257 < 2^24, every step exact
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint64_t y = add2(acc[16 * j + i], pack2(v[2 * i], v[2 * i + 1]));
@@ -457,20 +493,6 @@ k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
 // ---------------------------------------------------------------------------
 // reconstruction
 // ---------------------------------------------------------------------------
-// Fractions of the real and imaginary parts of four elements: r points at eight columns of one row,
-// the lane takes the even ones (sh = 16) or the odd ones (sh = 0)
-template <int I = 0>
-__device__ __forceinline__ void gather_fractions(const int16_t* __restrict__ r, size_t plane, int sh,
-                                                 mod::Frac (&re)[4], mod::Frac (&im)[4]) {
-  const uint4 u = __ldcs(reinterpret_cast<const uint4*>(r + (2 * I) * plane));
-  const uint4 v = __ldcs(reinterpret_cast<const uint4*>(r + (2 * I + 1) * plane));
-  const uint32_t uw[4] = {u.x, u.y, u.z, u.w}, vw[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int c = 0; c < 4; ++c)
-    mod::frac_add_uv<I>(re[c], im[c], (int)(uw[c] << sh) >> 16, (int)(vw[c] << sh) >> 16);
-  if constexpr (I + 1 < NM) gather_fractions<I + 1>(r, plane, sh, re, im);
-}
-
 // chi[w][row0 + i][j] += the value of R's planes (w, i, j).  A warp takes 16 rows x 8
 // columns (half a residue block); two neighbouring lanes share a row and take its
 // even and odd columns, so that each access to chi covers whole 32-byte sectors.
@@ -480,22 +502,23 @@ __global__ void __launch_bounds__(128) k_mod_add(const int16_t* __restrict__ R, 
   const int lane = threadIdx.x & 31, w = blockIdx.z;
   const int j0 = 8 * (blockIdx.x * 4 + (threadIdx.x >> 5)), i = blockIdx.y * 16 + (lane >> 1);
   if (j0 >= nG || i >= rows) return;
-  mod::Frac re[4] = {}, im[4] = {};
-  gather_fractions(R + res_index(rows, ldR, w * NPL, i, j0), res_plane(rows, ldR), lane & 1 ? 0 : 16, re, im);
   const int G = row0 + i, sa = scale[(size_t)(1 + w0 + w) * nG + G];
   double2* o = chi + ((size_t)(w0 + w) * nG + G) * nG + j0 + (lane & 1);
+  double2 v[4];                                  // read early: the loads run beside those of the residues
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    if (j0 + 2 * c + (lane & 1) < nG) v[c] = o[2 * c];
+  mod::Frac re[4] = {}, im[4] = {};
+  gather_fractions(R + res_index(rows, ldR, w * NPL, i, j0), res_plane(rows, ldR), lane & 1 ? mod::ODD : mod::EVEN, re, im);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int j = j0 + 2 * c + (lane & 1);
     if (j >= nG) break;
     const int sb = scale[j];
-    double2 d;
-    if (sa == mod::NO_SCALE || sb == mod::NO_SCALE) d = make_double2(nan(""), nan(""));
-    else d = make_double2(mod::frac_value(re[c], -sa - sb), mod::frac_value(im[c], -sa - sb));
-    double2 v = o[2 * c];
-    v.x += d.x;
-    v.y += d.y;
-    o[2 * c] = v;
+    const bool bad = sa == mod::NO_SCALE || sb == mod::NO_SCALE;
+    v[c].x += bad ? nan("") : mod::frac_value(re[c], -sa - sb);
+    v[c].y += bad ? nan("") : mod::frac_value(im[c], -sa - sb);
+    o[2 * c] = v[c];
   }
 }
 
@@ -591,6 +614,41 @@ ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
   z.off_exp = z.off_scale + al256(nf1 * nG * sizeof(int));
   z.bytes = z.off_exp + al256((nG + nf1) * sizeof(uint32_t));
   return z;
+}
+
+template <typename C>
+static cudaError_t pack_rows(const C* X, int rows, int n, size_t ld, int Kp, int beta, int* scale, uint16_t* planes,
+                             cudaStream_t s) {
+  k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale);
+  const int64_t units = (int64_t)rows * (Kp / 64);
+  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, (uint32_t*)planes);
+  return cudaGetLastError();
+}
+cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+                                 uint16_t* planes, cudaStream_t s) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, s);
+}
+cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+                                 uint16_t* planes, cudaStream_t s) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, s);
+}
+size_t mod_cols_ws_bytes(int n, int rows) {
+  return al256(sizeof(uint32_t) * rows) + sizeof(double) * ((n + ST_ROWS - 1) / ST_ROWS) * (size_t)rows;
+}
+cudaError_t launch_mod_pack_cols_conj(const double2* X, int n, int rows, int Kp, int* scale, uint16_t* planes,
+                                      void* ws, cudaStream_t s) {
+  uint32_t* eg = reinterpret_cast<uint32_t*>(ws);
+  double* part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(ws) + al256(sizeof(uint32_t) * rows));
+  cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * rows, s);
+  if (e != cudaSuccess) return e;
+  const int n_part = (n + ST_ROWS - 1) / ST_ROWS;
+  const dim3 gst((rows + ST_COLS - 1) / ST_COLS, n_part);
+  k_mod_rowmax<<<gst, 256, 0, s>>>(X, rows, n, eg);
+  k_mod_norms<<<gst, 256, 0, s>>>(X, rows, n, nullptr, 0, eg, nullptr, part);
+  k_mod_scales<<<dim3((rows + 255) / 256, 1), 256, 0, s>>>(part, n_part, rows, 0, eg, nullptr, scale);
+  k_mod_pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale,
+                                                                     (uint32_t*)planes, nullptr);
+  return cudaGetLastError();
 }
 
 int mod_launches(const chi0_plan_s* p, int nG) {

@@ -12,8 +12,8 @@
 //   x + i y  ->  (u, v) = (x + I y, x - I y)  (mod m_i)
 // turns one complex product into two independent real ones: 26 real products for
 // 13 moduli, where a digit split of 54 bits into six 9-bit terms needs 84.
-// Residues are centred (|r| <= 254), exact in FP16, and a sum of 256 products is
-// at most 254^2 256 < 2^24: exact in the tensor cores' FP32 accumulators, in any
+// Residues are centred (|r| <= 255), exact in FP16, and a sum of 256 products is
+// at most 255^2 256 < 2^24: exact in the tensor cores' FP32 accumulators, in any
 // order and rounding.  The only error is the rounding to integers, about 0.08 x
 // 2^-53 of |A_m| |B_n| (0.3 x 2^-53 for the same sum by FP64 fused multiply-adds
 // over Gaussian rows).
@@ -31,24 +31,18 @@ constexpr int NO_SCALE = -(1 << 28);      // scale exponent of a row holding an 
 
 typedef unsigned __int128 u128;
 
+constexpr int NL = 5, LB = 12;        // limbs of a scaled integer: 12 bits each, the last one signed
+
 struct Tables {
   int m[NM] = {509, 505, 493, 481, 461, 457, 449, 433, 421, 409, 401, 397, 389};
-  int c1[NM] = {}, c2[NM] = {};                   // 2^20, 2^40 (mod m), centred
-  int i0[NM] = {}, i1[NM] = {}, i2[NM] = {};      // I, I 2^20, I 2^40 (mod m), centred
-  uint32_t bias[NM] = {};                         // multiple of m above 2^30, plus (m - 1) / 2
-  uint32_t mag[NM] = {};                          // ceil(2^40 / m): floor(t / m) = t mag >> 40 for t < 2^31
+  int c[NM][NL] = {}, ic[NM][NL] = {};            // 2^(12 j) and I 2^(12 j) (mod m), centred
   // C = sum_i s_i a_i (mod 1) in units of P, s = u + v for the real part and u - v for the
-  // imaginary part: a 96-bit fraction (hi, mid, lo)
-  uint32_t re[NM][3] = {}, im[NM][3] = {};
+  // imaginary part: a 96-bit fraction in three words, the lower two balanced (signed)
+  int re[NM][3] = {}, im[NM][3] = {};
   uint64_t p_top = 0;                             // P = p_top 2^p_exp, top bit set
   int p_exp = 0;
 };
 
-constexpr int cpow_mod(int b, int e, int m) {
-  int64_t r = 1, x = ((b % m) + m) % m;
-  for (; e > 0; --e) r = r * x % m;
-  return (int)r;
-}
 constexpr int cinv_mod(int a, int m) {            // by search: the moduli are small
   for (int x = 1; x < m; ++x)
     if ((int64_t)a * x % m == 1) return x;
@@ -65,14 +59,10 @@ constexpr Tables make_tables() {
     int I = 0;
     for (int x = 2; x < m && !I; ++x)
       if (x * x % m == m - 1) I = x;
-    const int p20 = (1 << 20) % m, p40 = (int)((int64_t)p20 * p20 % m);
-    t.c1[i] = centred(p20, m);
-    t.c2[i] = centred(p40, m);
-    t.i0[i] = centred(I, m);
-    t.i1[i] = centred(I * p20 % m, m);
-    t.i2[i] = centred(I * p40 % m, m);
-    t.bias[i] = (uint32_t)(((1 << 30) / m + 1) * m + (m - 1) / 2);
-    t.mag[i] = (uint32_t)(((uint64_t)1 << 40) / (unsigned)m + 1);
+    for (int j = 0, pw = 1; j < NL; ++j, pw = pw * ((1 << LB) % m) % m) {
+      t.c[i][j] = centred(pw, m);
+      t.ic[i][j] = centred(I * pw % m, m);
+    }
     int q = 1;                                    // P / m (mod m)
     for (int j = 0; j < NM; ++j)
       if (j != i) q = q * (t.m[j] % m) % m;
@@ -80,10 +70,11 @@ constexpr Tables make_tables() {
     const int ar = w * half % m, ai = ar * cinv_mod(I, m) % m;
     for (int c = 0; c < 2; ++c) {
       const u128 f = (((u128)(unsigned)(c ? ai : ar) << 97) / (unsigned)m + 1) >> 1;   // rounded, below 2^96
-      uint32_t* o = c ? t.im[i] : t.re[i];
-      o[0] = (uint32_t)(f >> 64);
-      o[1] = (uint32_t)(f >> 32);
-      o[2] = (uint32_t)f;
+      int* o = c ? t.im[i] : t.re[i];
+      o[2] = (int)(uint32_t)f;
+      const u128 f1 = (f >> 32) + (o[2] < 0 ? 1 : 0);
+      o[1] = (int)(uint32_t)f1;
+      o[0] = (int)(uint32_t)((f1 >> 32) + (o[1] < 0 ? 1 : 0));
     }
   }
   int top = 127;
@@ -99,11 +90,11 @@ static_assert((T.p_top >> 60) >= 10, "P / 2 covers the largest component");
 
 // the constants of modulus I as compile-time scalars (device code takes them as immediates)
 template <int I> struct Mod {
-  static constexpr int m = T.m[I], c1 = T.c1[I], c2 = T.c2[I], i0 = T.i0[I], i1 = T.i1[I], i2 = T.i2[I];
-  static constexpr int bias = (int)T.bias[I];
-  static constexpr uint32_t mag = T.mag[I];
-  static constexpr uint32_t re0 = T.re[I][0], re1 = T.re[I][1], re2 = T.re[I][2];
-  static constexpr uint32_t im0 = T.im[I][0], im1 = T.im[I][1], im2 = T.im[I][2];
+  static constexpr float m = (float)T.m[I], inv = 1.0f / (float)T.m[I];
+  static constexpr float c1 = T.c[I][1], c2 = T.c[I][2], c3 = T.c[I][3], c4 = T.c[I][4];   // c[0] = 1
+  static constexpr float i0 = T.ic[I][0], i1 = T.ic[I][1], i2 = T.ic[I][2], i3 = T.ic[I][3], i4 = T.ic[I][4];
+  static constexpr int re0 = T.re[I][0], re1 = T.re[I][1], re2 = T.re[I][2];
+  static constexpr int im0 = T.im[I][0], im1 = T.im[I][1], im2 = T.im[I][2];
 };
 constexpr uint64_t P_TOP = T.p_top;
 constexpr int P_EXP = T.p_exp;
@@ -120,12 +111,19 @@ __device__ __forceinline__ double pow2d(int k) { return __hiloint2double((k + 10
 // exponent e with x < 2^(e + 1) for the largest magnitude word of a set (0 for zeros and subnormals)
 __device__ __forceinline__ int word_exp(uint32_t w) { return (int)(w >> 20) - 1023; }
 
-// scale exponent s with norm 2^s <= 2^beta, from norm^2 = n2 4^e (n2 > 0 an FP64 sum)
+// scale exponent s with norm 2^s <= 2^beta, from norm^2 = n2 4^e (n2 > 0, to a relative 1e-5)
 __device__ __forceinline__ int scale_exp(double n2, int e, int beta) {
   if (!(n2 > 0.0)) return 0;                      // a row of zeros
   int k;
-  frexp(n2 * (1.0 + 1e-9), &k);                   // n2 < 2^k
+  frexp(n2 * (1.0 + 2e-5), &k);                   // n2 < 2^k
   return beta - e - ((k + 1) >> 1);               // norm < 2^(e + k / 2)
+}
+
+// |x| 2^-e truncated to FP32, for |x| < 2^(e + 1) (integer operations; zero below 2^(e - 126))
+__device__ __forceinline__ float scaled_abs(double x, int e) {
+  const uint32_t hi = mag_word(x), lo = (uint32_t)__double2loint(x);
+  const int ef = (int)(hi >> 20) - 1023 - e + 127;
+  return ef > 0 ? __uint_as_float(((uint32_t)ef << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29)) : 0.f;
 }
 
 // round(x 2^s) for |x 2^s| < 2^58 (integer operations only: the FP64 pipe is narrow)
@@ -141,64 +139,102 @@ __device__ __forceinline__ int64_t quantise(double x, int s) {
   return b < 0 ? -(int64_t)q : (int64_t)q;
 }
 
-// limbs of a signed integer below 2^58: a = l0 + l1 2^20 + l2 2^40
-struct Limbs {
-  int l0, l1, l2;
-};
-__device__ __forceinline__ Limbs limbs(int64_t a) {
-  return Limbs{(int)(a & 0xfffff), (int)((a >> 20) & 0xfffff), (int)(a >> 40)};
+// packed FP32 pairs
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
 }
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t both(float x) { return pack2(x, x); }
 
-// t >= 0 (below 2^31), returns the FP16 bits of 1536 + (t mod m) - (m - 1) / 2
-template <int I>
-__device__ __forceinline__ uint32_t residue_bits(uint32_t t) {
-  const uint32_t q = __umulhi(t, Mod<I>::mag) >> 8;
-  return t - q * (uint32_t)Mod<I>::m + (0x6600u - (uint32_t)((Mod<I>::m - 1) / 2));
-}
-// two biased residues to two FP16 numbers
-__device__ __forceinline__ uint32_t unbias(uint32_t lo, uint32_t hi) {
-  uint32_t r;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(lo | (hi << 16)), "r"(0x66006600u));
+// limbs of two signed integers below 2^58 as packed FP32 numbers: a = sum_j l_j 2^(12 j)
+struct Limbs {
+  uint64_t l[NL];
+};
+__device__ __forceinline__ Limbs limbs(int64_t a, int64_t b) {
+  const int al = (int)a, ah = (int)(a >> 32), bl = (int)b, bh = (int)(b >> 32);
+  const int x[NL] = {al & 0xfff, (al >> 12) & 0xfff, (int)__funnelshift_r(al, ah, 24) & 0xfff, (ah >> 4) & 0xfff, ah >> 16};
+  const int y[NL] = {bl & 0xfff, (bl >> 12) & 0xfff, (int)__funnelshift_r(bl, bh, 24) & 0xfff, (bh >> 4) & 0xfff, bh >> 16};
+  Limbs r;
+#pragma unroll
+  for (int j = 0; j < NL; ++j)    // integers below 2^22 in magnitude
+    r.l[j] = add2(pack2(__int_as_float(x[j] + 0x4b400000), __int_as_float(y[j] + 0x4b400000)), both(-12582912.f));
   return r;
 }
 
-// residues (u, v) modulo m_I of two complex integers (k and k + 1): a packed FP16
-// pair of each
+// x - m round(x / m) for integers |x| < 2^24: |result| <= 255 (the quotient is within 2^-9 of exact)
 template <int I>
-__device__ __forceinline__ void residues2(const Limbs& xr, const Limbs& xi, const Limbs& yr, const Limbs& yi,
-                                          uint32_t& u, uint32_t& v) {
-  const int ax = xr.l0 + Mod<I>::c1 * xr.l1 + Mod<I>::c2 * xr.l2 + Mod<I>::bias;
-  const int bx = Mod<I>::i0 * xi.l0 + Mod<I>::i1 * xi.l1 + Mod<I>::i2 * xi.l2;
-  const int ay = yr.l0 + Mod<I>::c1 * yr.l1 + Mod<I>::c2 * yr.l2 + Mod<I>::bias;
-  const int by = Mod<I>::i0 * yi.l0 + Mod<I>::i1 * yi.l1 + Mod<I>::i2 * yi.l2;
-  u = unbias(residue_bits<I>((uint32_t)(ax + bx)), residue_bits<I>((uint32_t)(ay + by)));
-  v = unbias(residue_bits<I>((uint32_t)(ax - bx)), residue_bits<I>((uint32_t)(ay - by)));
+__device__ __forceinline__ uint32_t residue2(uint64_t x) {
+  const uint64_t q = add2(fma2(x, both(Mod<I>::inv), both(12582912.f)), both(-12582912.f));
+  float lo, hi;
+  unpack2(fma2(q, both(-Mod<I>::m), x), lo, hi);
+  uint32_t r;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+  return r;
+}
+
+// residues (u, v) modulo m_I of two complex integers (k and k + 1; limbs of the real and imaginary
+// parts): a packed FP16 pair of each.  Packed FP32 multiply-adds on 12-bit limbs: every sum is an
+// integer below 2 x 254 x (4 x 4095 + 512) < 2^23.04, exact.
+template <int I>
+__device__ __forceinline__ void residues2(const Limbs& x, const Limbs& y, uint32_t& u, uint32_t& v) {
+  using C = Mod<I>;
+  uint64_t a = fma2(both(C::c1), x.l[1], x.l[0]);
+  a = fma2(both(C::c2), x.l[2], a);
+  a = fma2(both(C::c3), x.l[3], a);
+  a = fma2(both(C::c4), x.l[4], a);
+  uint64_t b = mul2(both(C::i0), y.l[0]);
+  b = fma2(both(C::i1), y.l[1], b);
+  b = fma2(both(C::i2), y.l[2], b);
+  b = fma2(both(C::i3), y.l[3], b);
+  b = fma2(both(C::i4), y.l[4], b);
+  u = residue2<I>(add2(a, b));
+  v = residue2<I>(fma2(b, both(-1.f), a));
 }
 
 // all residues of two complex integers into planes of `plane` words each: u of modulus i at
 // plane 2 i, v at 2 i + 1 (conj: of the conjugates, u and v exchanged)
 template <int I = 0>
-__device__ __forceinline__ void store_residues(const Limbs& xr, const Limbs& xi, const Limbs& yr, const Limbs& yi,
-                                               bool conj, uint32_t* __restrict__ dst, size_t plane) {
+__device__ __forceinline__ void store_residues(const Limbs& x, const Limbs& y, bool conj, uint32_t* __restrict__ dst,
+                                               size_t plane) {
   uint32_t u, v;
-  residues2<I>(xr, xi, yr, yi, u, v);
+  residues2<I>(x, y, u, v);
   dst[(2 * I) * plane] = conj ? v : u;
   dst[(2 * I + 1) * plane] = conj ? u : v;
-  if constexpr (I + 1 < NM) store_residues<I + 1>(xr, xi, yr, yi, conj, dst, plane);
+  if constexpr (I + 1 < NM) store_residues<I + 1>(x, y, conj, dst, plane);
 }
 
 // ---------------------------------------------------------------------------
 // reconstruction
 // ---------------------------------------------------------------------------
-// f += s a with a 96-bit fraction a (mod 1); hi holds the top 64 bits, lo a carry-save sum of
-// the products with the low word
+// f += s a with a 96-bit fraction a (mod 1): three multiply-adds, the sums of the products with
+// the three words kept apart (fraction = top 2^-32 + mid 2^-64 + lo 2^-96)
 struct Frac {
-  uint64_t hi;
-  int64_t lo;
+  uint32_t top;
+  int64_t mid, lo;
 };
-__device__ __forceinline__ void frac_add(Frac& f, int s, uint32_t a0, uint32_t a1, uint32_t a2) {
-  f.lo += (int64_t)s * (int64_t)a2;
-  f.hi += (uint64_t)((int64_t)s * (int64_t)a1) + ((uint64_t)((uint32_t)s * a0) << 32);
+__device__ __forceinline__ void frac_add(Frac& f, int s, int a0, int a1, int a2) {
+  f.lo += (int64_t)s * a2;
+  f.mid += (int64_t)s * a1;
+  f.top += (uint32_t)s * (uint32_t)a0;
 }
 // the residues (u, v) modulo m_I of a complex element
 template <int I>
@@ -210,7 +246,7 @@ __device__ __forceinline__ void frac_add_uv(Frac& re, Frac& im, int u, int v) {
 // the signed fraction f in [-1/2, 1/2) times P 2^k as a double (one rounding, to nearest).
 // The fraction carries an error of 2^-84: what is below 2^-82 is zero.
 __device__ __forceinline__ double frac_value(const Frac& f, int k) {
-  uint64_t h = f.hi + (uint64_t)(f.lo >> 32);
+  uint64_t h = ((uint64_t)f.top << 32) + (uint64_t)f.mid + (uint64_t)(f.lo >> 32);
   uint32_t l = (uint32_t)f.lo;
   const bool neg = (int64_t)h < 0;
   if (neg) {
@@ -228,7 +264,10 @@ __device__ __forceinline__ double frac_value(const Frac& f, int k) {
     z = 64 + __clz((int)l);
     t = (uint64_t)l << (z - 32);
   }
-  uint64_t q = __umul64hi(t, P_TOP);            // in [2^62, 2^64)
+  // t P_TOP / 2^64 without the product of the low words (2^-62): in [2^62 - 1, 2^64)
+  const uint32_t th = (uint32_t)(t >> 32), tl = (uint32_t)t;
+  constexpr uint32_t ph = (uint32_t)(P_TOP >> 32), pl = (uint32_t)P_TOP;
+  uint64_t q = (uint64_t)th * ph + __umulhi(th, pl) + __umulhi(tl, ph);
   const int n = (int)(~q >> 63);                  // 1 when the top bit is clear
   q <<= n;
   uint64_t man = (q >> 11) + ((q >> 10) & 1u);    // 53 bits, rounded to nearest (a tie upwards)
@@ -244,6 +283,38 @@ __device__ __forceinline__ double frac_value(const Frac& f, int k) {
   // beyond the normal numbers
   const double x = __longlong_as_double((long long)(sgn | (1023ull << 52) | (man & 0xfffffffffffffull)));
   return scalbn(x, e - 1023);
+}
+
+// Residues are kept in blocks of 32 rows x 8 columns (512 bytes): a warp, whose lanes
+// hold 32 rows of the accumulator, writes whole blocks.  Index of (plane b, row, column).
+__host__ __device__ __forceinline__ size_t res_plane(int rows, int ldR) { return (size_t)((rows + 31) / 32) * 32 * ldR; }
+__device__ __forceinline__ size_t res_index(int rows, int ldR, int b, int row, int col) {
+  return b * res_plane(rows, ldR) + ((size_t)(row >> 5) * (ldR >> 3) + (col >> 3)) * 256 + (row & 31) * 8 + (col & 7);
+}
+
+// Fractions of the real and imaginary parts of four elements: r points at eight columns of one row,
+// the lane takes the even ones (sh = EVEN: sign-extended low halves) or the odd ones (sh = ODD)
+constexpr uint32_t EVEN = 0x9910, ODD = 0xbb32;   // byte selectors, the sign byte replicated
+template <int I0, int I, int N>
+__device__ __forceinline__ void add_words(const uint4 (&w)[2 * N], uint32_t sh, Frac (&re)[4], Frac (&im)[4]) {
+  const uint4 u = w[2 * (I - I0)], v = w[2 * (I - I0) + 1];
+  const uint32_t uw[4] = {u.x, u.y, u.z, u.w}, vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+    frac_add_uv<I>(re[c], im[c], (int)__byte_perm(uw[c], 0, sh), (int)__byte_perm(vw[c], 0, sh));
+  if constexpr (I + 1 < I0 + N) add_words<I0, I + 1, N>(w, sh, re, im);
+}
+// loads of N moduli first, then their sums: the loads of a thread are in flight together
+template <int I0 = 0, int N = 7>
+__device__ __forceinline__ void gather_fractions(const int16_t* __restrict__ r, size_t plane, uint32_t sh,
+                                                 Frac (&re)[4], Frac (&im)[4]) {
+  uint4 w[2 * N];
+#pragma unroll
+  for (int i = 0; i < 2 * N; ++i)    // volatile: kept together, ahead of the sums
+    asm volatile("ld.global.cs.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w[i].x), "=r"(w[i].y), "=r"(w[i].z), "=r"(w[i].w) : "l"(r + (2 * I0 + i) * plane));
+  add_words<I0, I0, N>(w, sh, re, im);
+  if constexpr (I0 + N < NM) gather_fractions<I0 + N, NM - N>(r, plane, sh, re, im);
 }
 
 }  // namespace mod

@@ -752,28 +752,42 @@ static bool mod_pays(int nG, int n_freq, int64_t K) {
   return modular < direct;
 }
 
-// Workspace of the FP64 contraction on the tensor cores for the plan's largest sphere, allocated on
-// first use: not inside a stream capture (the CUDA-core kernel runs there unless an earlier call has
-// allocated it) and given up for good when the memory cannot be had.
-static bool mod_ready(chi0_plan p, cudaStream_t s) {
-  if (p->d_mod) return true;
-  if (p->mod_state < 0 || !chi0::mod_gemm_usable()) return false;
+// Workspace of the modular products (FP64 contraction, dense adjoint), at least `need` bytes,
+// allocated on first use and grown when a later call needs more: not inside a stream capture (the
+// CUDA-core kernels run there unless an earlier call has allocated enough).  A size that could not be
+// had is not asked for again.
+static bool mod_ready(chi0_plan p, size_t need, cudaStream_t s) {
+  if (need >= p->mod_limit || !chi0::mod_gemm_usable()) return false;
+  if (need <= p->mod_bytes) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
-  size_t need = 0;
-  for (auto& q : p->q) need = std::max(need, chi0::mod_sizes(p, q.nG).bytes);
+  // graphs of batched builds hold the old address
+  if (p->graph_exec) {
+    cudaGraphExecDestroy(p->graph_exec);
+    p->graph_exec = nullptr;
+  }
+  if (p->d_mod) cudaFree(p->d_mod);   // waits for the work that uses it
+  p->d_mod = nullptr;
+  p->ws_bytes -= p->mod_bytes;
+  p->mod_bytes = 0;
   if (cudaMalloc(&p->d_mod, need) != cudaSuccess) {
     cudaGetLastError();
     p->d_mod = nullptr;
-    p->mod_state = -1;
+    p->mod_limit = need;
     return false;
   }
   p->mod_bytes = need;
   p->ws_bytes += need;
   return true;
+}
+// bytes the contraction takes at most over the plan's spheres
+static size_t mod_contract_bytes(chi0_plan p) {
+  size_t need = 0;
+  for (auto& q : p->q) need = std::max(need, chi0::mod_sizes(p, q.nG).bytes);
+  return need;
 }
 
 static chi0_status accumulate_impl(chi0_plan p, int iq, const void* M, int n_v, int n_c,
@@ -796,7 +810,7 @@ static chi0_status accumulate_impl(chi0_plan p, int iq, const void* M, int n_v, 
       if (e != cudaSuccess)
         return fail(p, CHI0_ERR_CUDA, "tensor-core contraction: " + why + " " + cudaGetErrorString(e));
     } else {
-      if (mod_pays(nG, p->n_freq, K) && mod_ready(p, s)) {
+      if (mod_pays(nG, p->n_freq, K) && mod_ready(p, mod_contract_bytes(p), s)) {
         chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, chi0::mod_launches(p, nG));
         CK(p, chi0::launch_contract_mod(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, p->d_mod, s));
       } else {
@@ -957,6 +971,11 @@ chi0_status chi0_backward(chi0_plan p, int iq, const void* M, int n_v, int n_c, 
   CK(p, cudaMemsetAsync(grad_Ev, 0, sizeof(double) * n_v, s));
   CK(p, cudaMemsetAsync(grad_Ecol, 0, sizeof(double) * n_c, s));
   const int64_t np = (int64_t)n_v * n_c;
+  if (grad_chi0 && chi0::bwd_mod_pays(p, nG, np) && mod_ready(p, chi0::bwd_mod_ws_bytes(p, nG, np), s)) {
+    CK(p, chi0::launch_backward_mod(p, nG, M, np, n_c, E_v, E_col, w_col, (const double2*)grad_chi0, grad_M, grad_Ev,
+                                    grad_Ecol, p->d_bwd, p->d_mod, s));
+    return CHI0_OK;
+  }
   for (int64_t p0 = 0; p0 < np; p0 += p->max_pairs) {
     const int64_t K = std::min<int64_t>(p->max_pairs, np - p0);
     CK(p, chi0::launch_backward(p, nG, M, p0, K, n_c, E_v, E_col, w_col, (const double2*)grad_chi0, diag_g,
@@ -1085,7 +1104,7 @@ chi0_status chi0_build_batched(chi0_plan p, const void* const* psi_v, int n_v, c
   key.push_back(psi_c); key.push_back(c_idx); key.push_back(E_col); key.push_back(w_col);
   key.push_back((const void*)(intptr_t)n_v); key.push_back((const void*)(intptr_t)n_c);
   if (!p->graph_exec || key != p->graph_key) {
-    if (!chi0::is_split(p)) mod_ready(p, s);   // its workspace cannot be allocated inside the capture
+    if (!chi0::is_split(p)) mod_ready(p, mod_contract_bytes(p), s);   // its workspace cannot be allocated inside the capture
     if (p->graph_exec) { cudaGraphExecDestroy(p->graph_exec); p->graph_exec = nullptr; }
     if (!p->cap_stream) CK(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     const bool timing = p->prof_timing;

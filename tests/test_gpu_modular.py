@@ -1,5 +1,5 @@
-"""The FP64 contraction as modular products on the tensor cores, at the edges of
-its tiles (256 x 256 outputs, 64-pair stages, 256-pair chains, pair blocks).
+"""The FP64 contraction and the dense adjoint as modular products on the tensor
+cores, at the edges of the tiles (256 x 256 outputs, 64-pair stages, 256-pair chains, pair blocks).
 
 Integer pair elements and factors f = -w (omega = 0, delta = 0, dE = -1) make
 every chi0 element an integer that FP64 matrix products give exactly.  The
@@ -64,3 +64,33 @@ def test_scales_zeros_and_nonfinite_rows():
     got = _accumulate(Ms, np.ones(K), n=24)[0]
     fin = np.isfinite(got.real) & np.isfinite(got.imag)
     assert np.all(fin[~bad][:, ~bad]) and not fin[bad].any() and not fin[:, bad].any()
+
+
+@pytest.mark.parametrize("nG,n_v,n_c,n_freq,max_pairs,precision", [
+    (63, 1, 1, 1, 0, "fp64"), (64, 3, 11, 2, 0, "fp64"), (129, 5, 51, 1, 0, "bf16"), (257, 7, 43, 3, 64, "fp64"),
+    (300, 2, 128, 1, 0, "fp64"), (300, 9, 29, 2, 128, "fp16"),
+])
+def test_dense_adjoint_edges(nG, n_v, n_c, n_freq, max_pairs, precision):
+    """Against FP64 matrix products.  Both sides carry a few sqrt(N_G) 2^-53 of the sums' magnitudes
+    (5e-15 at N_G 300), so 1e-13; complex64 gradients one rounding of 2^-24 per frequency group."""
+    import torch
+    from oracle import chi0_grad
+    from paper_1601_06767_gb300 import Chi0Plan
+    from synth.mgo import g_sphere
+    rng = np.random.default_rng(nG + n_v)
+    K = n_v * n_c
+    cdt = np.complex128 if precision == "fp64" else np.complex64
+    M = (rng.standard_normal((K, nG)) + 1j * rng.standard_normal((K, nG))).astype(cdt)
+    Ev, Ec, w = -rng.uniform(0, 0.25, n_v), rng.uniform(0.2, 2.0, n_c), rng.uniform(0.5, 2.0, n_c)
+    omega = np.concatenate([[0.0], 1j * np.arange(1, n_freq)])
+    Gamma = rng.standard_normal((n_freq, nG, nG)) + 1j * rng.standard_normal((n_freq, nG, nG))
+    dE = (Ev[:, None] - Ec[None]).reshape(-1)
+    rM, rd = chi0_grad(M.astype(complex), dE, np.tile(w, n_v), omega, 1e-3, Gamma)
+    rd = rd.reshape(n_v, n_c)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    with Chi0Plan(24, [g_sphere(nG, (0.0, 0.0, 0.0))], omega, 1e-3, precision=precision, max_pairs=max_pairs) as plan:
+        gM, gEv, gEc = plan.backward(0, dev(M), n_v, n_c, dev(Ev), dev(Ec), dev(w), grad_chi=dev(Gamma))
+        plan.sync_status()
+    rel = lambda a, b: np.linalg.norm(a.cpu().numpy() - b) / np.linalg.norm(b)
+    assert rel(gM, rM) < (1e-13 if precision == "fp64" else 2.0 ** -24)
+    assert rel(gEv, rd.sum(1)) < 1e-13 and rel(gEc, -rd.sum(0)) < 1e-13
