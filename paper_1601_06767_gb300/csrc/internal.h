@@ -11,6 +11,13 @@
 
 namespace chi0 {
 
+// Frequency pairs +-k of one axis for the fixed-point transforms (kern_fx.cu)
+struct FxAxis {
+  int n = 0, units = 0, items = 0;    // points, folded terms per table row, frequency pairs
+  const int4* item = nullptr;         // [items] (k odd on an even axis, output of +k or -1, output of -k or -1, 0)
+  const int4* coef = nullptr;         // [items][units] cos and sin in two limbs each
+};
+
 // Pruned-transform structure of one dielectric sphere (one q-point).
 // Stage 1 runs along i3 and keeps k3 in [k3min, k3min+nk3); stage 2 along i2
 // keeps k2 in [k2min, k2min+nk2); the kept (k2,k3) box of every plane i1 is
@@ -30,6 +37,8 @@ struct SphereQ {
   int ncol = 0;                       // distinct (k2, k3) columns holding sphere points
   int* col_off = nullptr;             // [ncol] (k2-k2min)*nk3 + (k3-k3min) of each column
   int* col_start = nullptr;           // [ncol + 1] first entry of each column (entries in column order)
+  FxAxis fx[3];                       // FP64 plans: axes 1, 2, 3 of the fixed-point pair stage
+  int* fx_map = nullptr;              // [ncol][nk1] sphere point of (column, k1 - k1min), or -1
   double2* T1d = nullptr; float2* T1f = nullptr;   // [n1][nk1]   exp(+2 pi i k1 i1/n1)
   double2* T2d = nullptr; float2* T2f = nullptr;   // [n2][nk2p]  exp(+2 pi i k2 i2/n2)
   double2* T3d = nullptr; float2* T3f = nullptr;   // [n3][nk3p]  exp(+2 pi i k3 i3/n3)
@@ -48,6 +57,13 @@ struct WfnSphere {
 };
 
 }  // namespace chi0
+
+// device memory allocated on first use and grown when a later call needs more
+struct LazyWs {
+  void* p = nullptr;
+  size_t bytes = 0;
+  size_t limit = SIZE_MAX;            // smallest size that could not be had (not asked for again)
+};
 
 struct chi0_plan_s {
   int device = 0;
@@ -85,9 +101,9 @@ struct chi0_plan_s {
   void* wfn_ws = nullptr;    // scratch of the three-pass wavefunction transform (FP32 plans on 96^3)
   size_t wfn_ws_bytes = 0;
   void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
-  void* d_mod = nullptr;     // workspace of the modular products (first use)
-  size_t mod_bytes = 0;
-  size_t mod_limit = SIZE_MAX;   // smallest size that could not be allocated (the CUDA-core kernels run instead)
+  // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
+  // fixed-point pair stage
+  LazyWs ws_mod, ws_bwd, ws_fx;
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)
@@ -141,6 +157,17 @@ cudaError_t launch_pair_planes(const chi0_plan_s* p, int iq, const void* psi_v, 
 // stage 3: D -> M rows (v0+iv)*ldc + (c0+ic)
 cudaError_t launch_pair_gather(const chi0_plan_s* p, int iq, const void* D, int nv, int nc,
                                int64_t row0, int64_t ldv, void* M, cudaStream_t s);
+// fixed-point pair stage of FP64 plans (kern_fx.cu): tables of a sphere, bands held at a time, workspace
+bool fx_fits(const chi0_plan_s* p, const SphereQ& s);
+cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s);
+int fx_bands(const chi0_plan_s* p);
+size_t fx_ws_bytes(const chi0_plan_s* p, int64_t bands);
+cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int32_t* idx, int b0, int nb, void* ws,
+                            int64_t bands, int first, cudaStream_t s);
+cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int vslots, int nv, int nc, void* D,
+                             cudaStream_t st);
+cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int nv, int nc, const void* D,
+                             int64_t row0, int64_t ldv, double2* M, cudaStream_t st);
 // frequency factors f[w][k] for pairs p0..p0+K of an (n_v x n_c) set
 cudaError_t launch_weights(const chi0_plan_s* p, int64_t p0, int64_t K, int n_c, const double* E_v,
                            const double* E_col, const double* w_col, double2* f, cudaStream_t s);

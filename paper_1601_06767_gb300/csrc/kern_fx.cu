@@ -1,0 +1,494 @@
+// Pair matrix elements of FP64 plans in fixed point on the integer pipe.
+//
+// GB300's FP64 pipe does two multiply-adds per clock and SM, so the direct FP64
+// sums (kern_pairs.cu) took 10.3 ms for the 8-atom workload's 3840 pairs.  Here
+// every number is a signed integer in two limbs and a multiply-add is four 32 x
+// 32 + 64-bit integer multiply-adds, thirty times the rate:
+//
+//   grids     57 bits relative to the largest component of the band (limbs 29 + 29)
+//   products  conj(psi_v) psi_c, and every transform's input, are rescaled to the
+//             largest component of the plane (55 bits, limbs 28 + 28): block
+//             floating point, one exponent per (pair, plane)
+//   twiddles  55 bits; the sums are exact, one rounding per output
+//
+// Roundings of 2^-56 of a plane's largest element against 2^-53 of every partial
+// sum: against quad precision, on the synthetic wavefunctions, 1.1e-16 (relative
+// Frobenius) on grids of 21 to 48 points, 4.7-6.6e-16 for the FP64 sums.
+//
+// 3840 pairs, 24^3, N_G 350: planes 10.32 -> 0.77 ms, gather 231 -> 71 us.
+//
+// A line of n points is transformed at the wanted frequencies only, with the
+// symmetries of the twiddles folded out first: with h = n / 2 and a_i = x_i +
+// x_{i+h}, b_i = x_i - x_{i+h},
+//   even k:  X(+-k) = E +- i O,  E = sum_i (a_i + a_{h-i}) cos,  O = sum_i (a_i - a_{h-i}) sin
+//   odd k:   the same with b_i - b_{h-i} and b_i + b_{h-i},
+// about n / 2 real multiplications per component and pair +-k where the direct sum
+// takes 4 n.  (Odd n: only the mirror i -> n - i.)  The folded values replace the
+// line in place: E(i) at i, O(i) at h - i (even k), E at h + i, O at n - i (odd k).
+#include <math.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "cplx.cuh"
+#include "internal.h"
+#include "modgemm.cuh"
+
+namespace chi0 {
+namespace {
+
+constexpr int QBITS = 57, QL = 29;    // grids: bits and limb width
+constexpr int WBITS = 55, WL = 28;    // transform inputs and twiddles
+constexpr int FX_MAX_N = 128;         // the 64-bit sums hold n / 4 + 1 products of 2^57
+
+// ---- grids to fixed point ----
+// mx[b] = largest magnitude word of band b (cleared by the caller)
+__global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ psi, const int32_t* __restrict__ idx, int b0,
+                                                int64_t nr, uint32_t* __restrict__ mx) {
+  const int64_t band = idx ? idx[b0 + blockIdx.y] : b0 + blockIdx.y;
+  const double2* x = psi + band * nr;
+  uint32_t m = 0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nr; e += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = x[e];
+    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(mx + blockIdx.y, m);
+}
+
+__device__ __forceinline__ int fx_scale(uint32_t w) {
+  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : QBITS - 1 - mod::word_exp(w));
+}
+
+// q[b][r] = (re1, re0, im1, im0): limbs of psi 2^scale
+__global__ void __launch_bounds__(256) k_fx_quant(const double2* __restrict__ psi, const int32_t* __restrict__ idx, int b0,
+                                                  int64_t nr, const uint32_t* __restrict__ mx, int4* __restrict__ q) {
+  const int64_t band = idx ? idx[b0 + blockIdx.y] : b0 + blockIdx.y;
+  const double2* x = psi + band * nr;
+  const int s = fx_scale(mx[blockIdx.y]);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nr; e += (int64_t)gridDim.x * blockDim.x) {
+    const double2 v = x[e];
+    const int64_t a = mod::quantise(v.x, s), b = mod::quantise(v.y, s);
+    const int a0 = ((int)a << (32 - QL)) >> (32 - QL), b0l = ((int)b << (32 - QL)) >> (32 - QL);
+    q[blockIdx.y * nr + e] = make_int4((int)((a - a0) >> QL), a0, (int)((b - b0l) >> QL), b0l);
+  }
+}
+
+// ---- line transforms ----
+// x 2^-s, rounded to nearest (s may be negative)
+__device__ __forceinline__ int64_t shift_round(int64_t x, int s) {
+  if (s <= 0) return x << -s;
+  return s > 62 ? 0 : (x + (1ll << (s - 1))) >> s;
+}
+__device__ __forceinline__ uint32_t abs_word(int64_t x) { return (uint32_t)((x ^ (x >> 63)) >> 32); }
+// bits of the magnitudes whose largest high word is m
+__device__ __forceinline__ int word_bits(uint32_t m) { return 64 - __clz((int)m); }
+
+__device__ __forceinline__ int4 limbs_w(int64_t re, int64_t im) {
+  const int r0 = ((int)re << (32 - WL)) >> (32 - WL), i0 = ((int)im << (32 - WL)) >> (32 - WL);
+  return make_int4((int)((re - r0) >> WL), r0, (int)((im - i0) >> WL), i0);
+}
+
+// units of one line's fold: i = 0 .. fold_units(n) - 1, each owns the slots it reads and writes
+__host__ __device__ __forceinline__ int fold_units(int n) { return n & 1 ? (n + 1) / 2 : n / 4 + 1; }
+
+__device__ __forceinline__ void fold_line(longlong2* __restrict__ r, int n, int i, int s) {
+  int4* w = reinterpret_cast<int4*>(r);
+  auto ld = [&](int k) {
+    const longlong2 v = r[k];
+    return make_longlong2(shift_round(v.x, s), shift_round(v.y, s));
+  };
+  if (n & 1) {
+    const longlong2 x = ld(i);
+    if (i == 0) {
+      w[0] = limbs_w(x.x, x.y);
+      return;
+    }
+    const longlong2 y = ld(n - i);
+    w[i] = limbs_w(x.x + y.x, x.y + y.y);
+    w[n - i] = limbs_w(x.x - y.x, x.y - y.y);
+    return;
+  }
+  const int h = n >> 1;
+  const longlong2 x1 = ld(i), x3 = ld(h + i);
+  if (i == 0 || 2 * i == h) {      // E even at i, E odd (i = 0) or O odd (i = h / 2) at h + i
+    w[i] = limbs_w(x1.x + x3.x, x1.y + x3.y);
+    w[h + i] = limbs_w(x1.x - x3.x, x1.y - x3.y);
+    return;
+  }
+  const longlong2 x2 = ld(h - i), x4 = ld(n - i);
+  const longlong2 a = make_longlong2(x1.x + x3.x, x1.y + x3.y), c = make_longlong2(x2.x + x4.x, x2.y + x4.y);
+  const longlong2 b = make_longlong2(x1.x - x3.x, x1.y - x3.y), d = make_longlong2(x2.x - x4.x, x2.y - x4.y);
+  w[i] = limbs_w(a.x + c.x, a.y + c.y);
+  w[h - i] = limbs_w(a.x - c.x, a.y - c.y);
+  w[h + i] = limbs_w(b.x - d.x, b.y - d.y);
+  w[n - i] = limbs_w(b.x + d.x, b.y + d.y);
+}
+
+struct Acc {
+  int64_t hh = 0, cr = 0, ll = 0;
+  __device__ __forceinline__ void add(int x1, int x0, int c1, int c0) {
+    hh += (int64_t)x1 * c1;
+    cr += (int64_t)x1 * c0;
+    cr += (int64_t)x0 * c1;
+    ll += (int64_t)x0 * c0;
+  }
+  // the sum over 2^55 (the twiddles' unit), rounded
+  __device__ __forceinline__ int64_t value() const {
+    return 2 * hh + ((cr + (ll >> WL) + (1ll << (WBITS - WL - 1))) >> (WBITS - WL));
+  }
+};
+
+// X(+k) and X(-k) of a folded line at item `it` of the axis
+__device__ __forceinline__ void line_pair(const int4* __restrict__ w, const FxAxis& ax, int it, int4 item,
+                                          longlong2& pos, longlong2& neg) {
+  const int n = ax.n, h = n >> 1;
+  const bool odd_k = item.x != 0;     // never for odd n
+  int ce, cb, oe, ob;                 // cosine terms w[cb + i], i < ce; sine terms w[ob - i], 1 <= i < oe
+  if (n & 1) {
+    ce = oe = (n + 1) / 2;
+    cb = 0;
+    ob = n;
+  } else if (!odd_k) {
+    ce = h / 2 + 1;
+    oe = (h + 1) / 2;
+    cb = 0;
+    ob = h;
+  } else {
+    ce = (h + 1) / 2;
+    oe = h / 2 + 1;
+    cb = h;
+    ob = n;
+  }
+  const int4* __restrict__ t = ax.coef + it * ax.units;     // (cos1, cos0, sin1, sin0)
+  Acc er, ei, sr, si;
+  for (int i = 0; i < ce; ++i) {
+    const int4 x = w[cb + i], c = t[i];
+    er.add(x.x, x.y, c.x, c.y);
+    ei.add(x.z, x.w, c.x, c.y);
+  }
+  for (int i = 1; i < oe; ++i) {
+    const int4 x = w[ob - i], c = t[i];
+    sr.add(x.x, x.y, c.z, c.w);
+    si.add(x.z, x.w, c.z, c.w);
+  }
+  const int64_t Er = er.value(), Ei = ei.value(), Or = sr.value(), Oi = si.value();
+  pos = make_longlong2(Er - Oi, Ei + Or);
+  neg = make_longlong2(Er + Oi, Ei - Or);
+}
+
+// largest magnitude word of the block: each thread gives its own, every thread gets the result
+__device__ __forceinline__ uint32_t block_max(uint32_t m, uint32_t* __restrict__ slot) {
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, m);
+  __syncthreads();
+  return *slot;
+}
+
+// Stages 1 and 2 of one plane i1: D[pair][i1][k2][k3] as 64-bit integers and their
+// exponents ex[pair][i1] = (unit, top): value = D 2^unit, |value| < 2^top.  A CTA
+// takes one valence band and a run of conduction bands.  Bound by the integer
+// multiplies (16 per grid point for the product, eight per folded point and
+// frequency pair).
+__global__ void k_fx_planes(const int4* __restrict__ qv, const uint32_t* __restrict__ mv, const int4* __restrict__ qc,
+                            const uint32_t* __restrict__ mc, int nc, int cpc, int n1, int n2, int n3, int nk2, int nk3,
+                            const __grid_constant__ FxAxis a3, const __grid_constant__ FxAxis a2,
+                            longlong2* __restrict__ D, int2* __restrict__ ex) {
+  extern __shared__ __align__(16) unsigned char smem_fx[];
+  __shared__ uint32_t slot[3];
+  const int ld3 = n3 | 1, ld2 = n2 | 1;
+  longlong2* A = reinterpret_cast<longlong2*>(smem_fx);    // [n2][ld3]
+  longlong2* X = A + (size_t)n2 * ld3;                     // [nk3][ld2]
+  const int i1 = blockIdx.x, jv = blockIdx.y, nt = blockDim.x, tid = threadIdx.x;
+  const int plane = n2 * n3;
+  const int64_t nr = (int64_t)n1 * plane, box = (int64_t)nk2 * nk3;
+  const int4* v0 = qv + jv * nr + (int64_t)i1 * plane;
+  const int sv = fx_scale(mv[jv]);
+  const int jc1 = min(nc, (int)(blockIdx.z + 1) * cpc);
+  for (int jc = blockIdx.z * cpc; jc < jc1; ++jc) {
+    const int4* c0 = qc + jc * nr + (int64_t)i1 * plane;
+    __syncthreads();                                       // the previous pair's readers are done
+    if (tid < 3) slot[tid] = 0;
+    __syncthreads();
+    uint32_t m = 0;
+    for (int e = tid; e < plane; e += nt) {                // conj(v) c / 2^54
+      const int i2 = e / n3, i3 = e - i2 * n3;
+      const int4 v = v0[e], c = c0[e];
+      const int64_t hr = (int64_t)v.x * c.x + (int64_t)v.z * c.z;
+      const int64_t xr = (int64_t)v.x * c.y + (int64_t)v.y * c.x + (int64_t)v.z * c.w + (int64_t)v.w * c.z;
+      const int64_t lr = (int64_t)v.y * c.y + (int64_t)v.w * c.w;
+      const int64_t hi = (int64_t)v.x * c.z - (int64_t)v.z * c.x;
+      const int64_t xi = (int64_t)v.x * c.w + (int64_t)v.y * c.z - (int64_t)v.z * c.y - (int64_t)v.w * c.x;
+      const int64_t li = (int64_t)v.y * c.w - (int64_t)v.w * c.y;
+      const longlong2 p = make_longlong2((hr << 4) + ((xr + (lr >> QL) + (1ll << 24)) >> 25),
+                                         (hi << 4) + ((xi + (li >> QL) + (1ll << 24)) >> 25));
+      A[i2 * ld3 + i3] = p;
+      m = max(m, max(abs_word(p.x), abs_word(p.y)));
+    }
+    const int s0 = word_bits(block_max(m, slot)) - WBITS;  // its barrier also orders A
+    const int u3 = fold_units(n3);
+    for (int e = tid; e < n2 * u3; e += nt) {
+      const int i2 = e % n2, i = e / n2;
+      fold_line(A + i2 * ld3, n3, i, s0);
+    }
+    __syncthreads();
+    m = 0;
+    for (int e = tid; e < n2 * a3.items; e += nt) {        // along i3
+      const int i2 = e % n2, it = e / n2;
+      const int4 item = a3.item[it];
+      longlong2 p, q;
+      line_pair(reinterpret_cast<const int4*>(A + i2 * ld3), a3, it, item, p, q);
+      if (item.y >= 0) {
+        X[item.y * ld2 + i2] = p;
+        m = max(m, max(abs_word(p.x), abs_word(p.y)));
+      }
+      if (item.z >= 0) {
+        X[item.z * ld2 + i2] = q;
+        m = max(m, max(abs_word(q.x), abs_word(q.y)));
+      }
+    }
+    const int s1 = word_bits(block_max(m, slot + 1)) - WBITS;
+    const int u2 = fold_units(n2);
+    for (int e = tid; e < nk3 * u2; e += nt) {
+      const int k3 = e % nk3, i = e / nk3;
+      fold_line(X + k3 * ld2, n2, i, s1);
+    }
+    __syncthreads();
+    m = 0;
+    const int64_t pair = (int64_t)jv * nc + jc;
+    longlong2* d = D + (pair * n1 + i1) * box;
+    for (int e = tid; e < nk3 * a2.items; e += nt) {       // along i2
+      const int k3 = e % nk3, it = e / nk3;
+      const int4 item = a2.item[it];
+      longlong2 p, q;
+      line_pair(reinterpret_cast<const int4*>(X + k3 * ld2), a2, it, item, p, q);
+      if (item.y >= 0) {
+        d[(int64_t)item.y * nk3 + k3] = p;
+        m = max(m, max(abs_word(p.x), abs_word(p.y)));
+      }
+      if (item.z >= 0) {
+        d[(int64_t)item.z * nk3 + k3] = q;
+        m = max(m, max(abs_word(q.x), abs_word(q.y)));
+      }
+    }
+    m = block_max(m, slot + 2);
+    if (tid == 0) {
+      const int sc = fx_scale(mc[jc]);
+      const int unit = 54 - sv - sc + s0 + s1;
+      ex[pair * n1 + i1] = sv == mod::NO_SCALE || sc == mod::NO_SCALE ? make_int2(mod::NO_SCALE, 0)
+                                                                      : make_int2(unit, unit + word_bits(m));
+    }
+  }
+}
+
+// y 2^k as a double, rounded to nearest
+__device__ __forceinline__ double to_double(int64_t y, int k) {
+  if (y == 0) return 0.0;
+  const uint64_t a = y < 0 ? 0ull - (uint64_t)y : (uint64_t)y;
+  const int z = __clzll((long long)a);
+  const uint64_t t = a << z;                              // top bit set
+  uint64_t man = (t >> 11) + ((t >> 10) & 1u);
+  int e = 1023 + 63 - z + k;
+  if (man >> 53) {
+    man >>= 1;
+    ++e;
+  }
+  const uint64_t sgn = y < 0 ? 0x8000000000000000ull : 0ull;
+  if (e >= 1 && e <= 2046) return __longlong_as_double((long long)(sgn | ((uint64_t)e << 52) | (man & 0xfffffffffffffull)));
+  return scalbn(__longlong_as_double((long long)(sgn | (1023ull << 52) | (man & 0xfffffffffffffull))), e - 1023);
+}
+
+// Stage 3: M[row][j] = (1/N_r) sum_i1 D(i1, k2_j, k3_j) e^{2 pi i k1_j i1 / n1} for a chunk of the
+// (k2, k3) columns of one pair; colmap[column][k1 - k1min] = j, or -1 off the sphere
+__global__ void __launch_bounds__(256) k_fx_gather(const longlong2* __restrict__ D, const int2* __restrict__ ex, int nc,
+                                                   int64_t row0, int64_t ldv, int n1, int64_t box, int nG, int ncol,
+                                                   int chunk, int nk1, const int* __restrict__ col_off,
+                                                   const int* __restrict__ colmap, const __grid_constant__ FxAxis a1,
+                                                   double scale, double2* __restrict__ M) {
+  extern __shared__ __align__(16) unsigned char smem_fx[];
+  __shared__ int unit[FX_MAX_N], s_top, s_bad;
+  const int ld1 = n1 | 1, tid = threadIdx.x, nt = blockDim.x;
+  longlong2* A = reinterpret_cast<longlong2*>(smem_fx);    // [chunk][ld1]
+  const int pl = blockIdx.x, jv = pl / nc, jc = pl - jv * nc;
+  const int c0 = blockIdx.y * chunk, cn = min(chunk, ncol - c0);
+  if (tid == 0) {
+    s_top = -(1 << 30);
+    s_bad = 0;
+  }
+  __syncthreads();
+  for (int i = tid; i < n1; i += nt) {
+    const int2 e = ex[(int64_t)pl * n1 + i];
+    unit[i] = e.x;
+    atomicMax(&s_top, e.y);
+    if (e.x == mod::NO_SCALE) s_bad = 1;
+  }
+  __syncthreads();
+  const int base = s_top - WBITS;                          // common unit of the planes: 2^base
+  const bool bad = s_bad != 0;
+  for (int e = tid; e < cn * n1; e += nt) {
+    const int c = e % cn, i = e / cn;
+    const longlong2 v = D[((int64_t)pl * n1 + i) * box + col_off[c0 + c]];
+    const int s = base - unit[i];
+    A[c * ld1 + i] = make_longlong2(shift_round(v.x, s), shift_round(v.y, s));
+  }
+  __syncthreads();
+  const int u1 = fold_units(n1);
+  for (int e = tid; e < cn * u1; e += nt) {
+    const int c = e % cn, i = e / cn;
+    fold_line(A + c * ld1, n1, i, 0);
+  }
+  __syncthreads();
+  double2* out = M + (row0 + (int64_t)jv * ldv + jc) * nG;
+  auto put = [&](int j, longlong2 y) {
+    out[j] = bad ? make_double2(nan(""), nan(""))
+                 : make_double2(to_double(y.x, base) * scale, to_double(y.y, base) * scale);
+  };
+  for (int e = tid; e < cn * a1.items; e += nt) {
+    const int c = e % cn, it = e / cn;
+    const int4 item = a1.item[it];
+    const int* cm = colmap + (int64_t)(c0 + c) * nk1;
+    const int jp = item.y >= 0 ? cm[item.y] : -1, jn = item.z >= 0 ? cm[item.z] : -1;
+    if (jp < 0 && jn < 0) continue;
+    longlong2 p, q;
+    line_pair(reinterpret_cast<const int4*>(A + c * ld1), a1, it, item, p, q);
+    if (jp >= 0) put(jp, p);
+    if (jn >= 0) put(jn, q);
+  }
+}
+
+size_t planes_smem(const chi0_plan_s* p, const SphereQ& s) {
+  return ((size_t)p->n2 * (p->n3 | 1) + (size_t)s.nk3 * (p->n2 | 1)) * 16;
+}
+constexpr size_t SMEM_CAP = 220 * 1024;
+constexpr int64_t QUANT_BYTES = (int64_t)2 << 30;         // quantised grids held at a time
+
+size_t al256(size_t x) { return (x + 255) / 256 * 256; }
+// the exponents of D in the workspace
+int2* fx_exponents(const chi0_plan_s* p, void* ws, int64_t bands) {
+  return reinterpret_cast<int2*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16) + al256((size_t)bands * 4));
+}
+
+// frequency pairs +-k of an axis (kmin .. kmin + nk - 1) and their twiddles
+cudaError_t make_axis(int n, int kmin, int nk, FxAxis* a) {
+  std::vector<int4> item, coef;
+  const int units = fold_units(n);
+  for (int k = 0; k <= n / 2; ++k) {
+    int pos = -1, neg = -1;
+    for (int c = 0; c < nk; ++c) {
+      int m = (kmin + c) % n;
+      if (m < 0) m += n;
+      if (m > n / 2) m -= n;
+      if (m == k) pos = c;
+      else if (m == -k) neg = c;
+    }
+    if (pos < 0 && neg < 0) continue;
+    item.push_back(make_int4(n % 2 == 0 ? k & 1 : 0, pos, neg, 0));
+    for (int i = 0; i < units; ++i) {
+      const long double ang = 2.0L * 3.14159265358979323846264338327950288L * (long double)((int64_t)k * i % n) / n;
+      int l[4];
+      for (int c = 0; c < 2; ++c) {
+        const int64_t q = llroundl((c ? sinl(ang) : cosl(ang)) * (long double)((int64_t)1 << WBITS));
+        int64_t q0 = q & (((int64_t)1 << WL) - 1);
+        if (q0 >= (int64_t)1 << (WL - 1)) q0 -= (int64_t)1 << WL;
+        l[2 * c] = (int)((q - q0) >> WL);
+        l[2 * c + 1] = (int)q0;
+      }
+      coef.push_back(make_int4(l[0], l[1], l[2], l[3]));
+    }
+  }
+  a->n = n;
+  a->units = units;
+  a->items = (int)item.size();
+  int4 *di = nullptr, *dc = nullptr;
+  cudaError_t e = cudaMalloc((void**)&di, item.size() * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&dc, coef.size() * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMemcpy(di, item.data(), item.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(dc, coef.data(), coef.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  a->item = di;
+  a->coef = dc;
+  return e;
+}
+
+}  // namespace
+
+// whether the plan's grid and a sphere fit the kernels (else the direct FP64 sums run)
+bool fx_fits(const chi0_plan_s* p, const SphereQ& s) {
+  return p->n1 <= FX_MAX_N && p->n2 <= FX_MAX_N && p->n3 <= FX_MAX_N && planes_smem(p, s) <= SMEM_CAP;
+}
+
+cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s) {
+  std::vector<int> map((size_t)s->ncol * s->nk1, -1), col((size_t)s->nk2 * s->nk3, -1);
+  int nc = 0;
+  for (int t = 0; t < s->nG; ++t) {         // columns in (k2, k3) order, as col_off lists them
+    const int32_t* g = &s->g_host[3 * t];
+    col[(size_t)(g[1] - s->k2min) * s->nk3 + (g[2] - s->k3min)] = 0;
+  }
+  for (int& c : col)
+    if (c == 0) c = nc++;
+  for (int t = 0; t < s->nG; ++t) {
+    const int32_t* g = &s->g_host[3 * t];
+    int& slot = map[(size_t)col[(size_t)(g[1] - s->k2min) * s->nk3 + (g[2] - s->k3min)] * s->nk1 + (g[0] - s->k1min)];
+    if (slot >= 0) return cudaSuccess;      // a G vector listed twice: the direct sums run (fx_map stays NULL)
+    slot = t;
+  }
+  cudaError_t e = cudaMalloc((void**)&s->fx_map, map.size() * sizeof(int));
+  if (e == cudaSuccess) e = cudaMemcpy(s->fx_map, map.data(), map.size() * sizeof(int), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = make_axis(p->n1, s->k1min, s->nk1, &s->fx[0]);
+  if (e == cudaSuccess) e = make_axis(p->n2, s->k2min, s->nk2, &s->fx[1]);
+  if (e == cudaSuccess) e = make_axis(p->n3, s->k3min, s->nk3, &s->fx[2]);
+  return e;
+}
+
+// bands whose quantised grids are held at a time, and the workspace: grids, magnitude words, exponents
+int fx_bands(const chi0_plan_s* p) { return (int)std::max<int64_t>(2, QUANT_BYTES / (16 * p->nr)); }
+size_t fx_ws_bytes(const chi0_plan_s* p, int64_t bands) {
+  return al256((size_t)bands * p->nr * 16) + al256((size_t)bands * 4) + al256((size_t)p->D_pairs * p->n1 * sizeof(int2));
+}
+
+// quantise bands idx[b0 ..] (or b0 ..) into slots first .. first + nb of the workspace
+cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int32_t* idx, int b0, int nb, void* ws,
+                            int64_t bands, int first, cudaStream_t s) {
+  int4* q = reinterpret_cast<int4*>(ws) + (int64_t)first * p->nr;
+  uint32_t* mx = reinterpret_cast<uint32_t*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16)) + first;
+  cudaError_t e = cudaMemsetAsync(mx, 0, (size_t)nb * 4, s);
+  if (e != cudaSuccess) return e;
+  const int gx = (int)std::min<int64_t>((p->nr + 1023) / 1024, std::max(1, 4096 / nb));
+  k_fx_max<<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx);
+  k_fx_quant<<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx, q);
+  return cudaGetLastError();
+}
+
+// stages 1 and 2 of the pairs of valence slots [0, nv) and conduction slots [vslots, vslots + nc) of
+// the workspace into D, and their exponents
+cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int vslots, int nv, int nc, void* D,
+                             cudaStream_t st) {
+  const SphereQ& s = p->q[iq];
+  const int4* q = reinterpret_cast<const int4*>(ws);
+  const uint32_t* mx = reinterpret_cast<const uint32_t*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16));
+  const size_t sm = planes_smem(p, s);
+  cudaError_t e = cudaFuncSetAttribute(k_fx_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  // threads: a line and frequency pair each; conduction bands in runs that leave enough CTAs
+  const int items = std::max(p->n2 * s.fx[2].items, s.nk3 * s.fx[1].items);
+  const int nt = items <= 128 ? 128 : (items <= 512 || sm <= 72 * 1024 ? 256 : 512);
+  int cpc = 8;
+  while (cpc > 1 && (int64_t)p->n1 * nv * ((nc + cpc - 1) / cpc) < 16 * 152) cpc >>= 1;
+  k_fx_planes<<<dim3(p->n1, nv, (nc + cpc - 1) / cpc), nt, sm, st>>>(q, mx, q + (int64_t)vslots * p->nr, mx + vslots, nc,
+                                                                  cpc, p->n1, p->n2, p->n3, s.nk2, s.nk3, s.fx[2],
+                                                                  s.fx[1], (longlong2*)D, fx_exponents(p, ws, bands));
+  return cudaGetLastError();
+}
+
+// stage 3: M rows row0 + iv ldv + ic
+cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int nv, int nc, const void* D,
+                             int64_t row0, int64_t ldv, double2* M, cudaStream_t st) {
+  const SphereQ& s = p->q[iq];
+  const int ld1 = p->n1 | 1;
+  const int chunk = std::min(s.ncol, std::max(1, 40 * 1024 / (ld1 * 16)));
+  k_fx_gather<<<dim3((unsigned)(nv * nc), (s.ncol + chunk - 1) / chunk), 256, (size_t)chunk * ld1 * 16, st>>>(
+      (const longlong2*)D, fx_exponents(p, ws, bands), nc, row0, ldv, p->n1, (int64_t)s.nk2 * s.nk3, s.nG, s.ncol, chunk,
+      s.nk1, s.col_off, s.fx_map, s.fx[0], 1.0 / (double)p->nr, M);
+  return cudaGetLastError();
+}
+
+}  // namespace chi0

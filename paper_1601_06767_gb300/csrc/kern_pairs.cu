@@ -4,8 +4,9 @@
 // then the transform along i1 evaluated only on the G sphere (stage 3).
 //
 // FP32 plans on cubic grids of 24, 36, 48 or 96 points transform with
-// register FFTs (length-Q FFTs of P interleaved sub-sequences); FP64 plans and
-// other grids use direct sums with exact twiddle tables.  Both are restricted
+// register FFTs (length-Q FFTs of P interleaved sub-sequences); other grids use
+// direct sums with exact twiddle tables, as do FP64 plans beyond 128 points per
+// axis or without workspace (kern_fx.cu has their usual path).  All are restricted
 // to the frequencies the sphere needs, and the three stages together equal
 // M(G) = (1/N_r) sum_r conj(psi_v(r)) psi_c(r) exp(2 pi i G.r).
 #include <algorithm>

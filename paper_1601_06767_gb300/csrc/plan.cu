@@ -88,7 +88,8 @@ cudaError_t make_table_t(int n, int kmin, int nk, double2** dd, float2** df) {
 void free_sphere(SphereQ& s) {
   cudaFree(s.ent_box); cudaFree(s.ent_k1); cudaFree(s.ent_j); cudaFree(s.col_off); cudaFree(s.col_start);
   cudaFree(s.T1d); cudaFree(s.T1f); cudaFree(s.T2d); cudaFree(s.T2f);
-  cudaFree(s.T3d); cudaFree(s.T3f);
+  cudaFree(s.T3d); cudaFree(s.T3f); cudaFree(s.fx_map);
+  for (auto& a : s.fx) { cudaFree((void*)a.item); cudaFree((void*)a.coef); }
   s = SphereQ();
 }
 
@@ -103,7 +104,7 @@ void free_plan(chi0_plan_s* p) {
   cudaFree(w.T3d); cudaFree(w.T3f);
   cudaFree(p->d_omega); cudaFree(p->d_D); cudaFree(p->d_M); cudaFree(p->d_f);
   cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->d_inv); cudaFree(p->wfn_ws);
-  cudaFree(p->d_mod);
+  cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
     cudaFree(p->bq_M[i]);
     cudaFree(p->bq_f[i]);
@@ -371,6 +372,12 @@ chi0_status chi0_plan_create(chi0_plan* out, const chi0_plan_desc* d) {
   }
   st = analyse_wfn(p, d->gw, d->npw);
   if (st != CHI0_OK) return bail(st);
+  if (!chi0::is_split(p))
+    for (auto& sq : p->q)
+      if (chi0::fx_fits(p, sq)) {
+        cudaError_t fe = chi0::fx_setup(p, &sq);
+        if (fe != cudaSuccess) { p->err = cudaGetErrorString(fe); return bail(fe == cudaErrorMemoryAllocation ? CHI0_ERR_OOM : CHI0_ERR_CUDA); }
+      }
 
   // workspace
   const size_t cb = chi0::cbytes(p);
@@ -703,11 +710,76 @@ chi0_status chi0_wfn_to_grid(chi0_plan p, const void* coeff, int nb, void* psi, 
   return CHI0_OK;
 }
 
+// A workspace of at least `need` bytes, allocated on first use and grown when a later call needs more:
+// not inside a stream capture (the CUDA-core kernels run there unless an earlier call has allocated
+// enough).  A size that could not be had is not asked for again.
+static bool ws_ready(chi0_plan p, LazyWs& w, size_t need, cudaStream_t s) {
+  if (need >= w.limit) return false;
+  if (need <= w.bytes) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  // the graph of a batched build holds the old address
+  if (p->graph_exec) {
+    cudaGraphExecDestroy(p->graph_exec);
+    p->graph_exec = nullptr;
+  }
+  cudaFree(w.p);   // waits for the work that uses it
+  w.p = nullptr;
+  p->ws_bytes -= w.bytes;
+  w.bytes = 0;
+  if (cudaMalloc(&w.p, need) != cudaSuccess) {
+    cudaGetLastError();
+    w.p = nullptr;
+    w.limit = need;
+    return false;
+  }
+  w.bytes = need;
+  p->ws_bytes += need;
+  return true;
+}
+
+// Pairs of FP64 plans in fixed point: valence and conduction grids quantised in chunks that fit the
+// workspace, then the pairs of the two chunks.  Same M rows as pairs_impl.
+static chi0_status pairs_fx(chi0_plan p, int iq, const void* psi_v, const int32_t* v_idx, int n_v, const void* psi_c,
+                            const int32_t* c_idx, int c_base, int n_c, void* M, int64_t ld_pairs_c, int64_t bands,
+                            cudaStream_t s) {
+  void* ws = p->ws_fx.p;
+  const int vchunk = (int)std::min<int64_t>({n_v, p->D_pairs, std::max<int64_t>(1, bands - std::min<int64_t>(n_c, bands / 2)), 65535});
+  const int cchunk = (int)std::min<int64_t>({n_c, std::max<int64_t>(1, p->D_pairs / vchunk), bands - vchunk, 65535});
+  for (int v0 = 0; v0 < n_v; v0 += vchunk) {
+    const int nv = std::min(vchunk, n_v - v0);
+    {
+      chi0::ProfScope ps(p, CHI0_K_PAIR_PLANES, s, 2);
+      CK(p, chi0::launch_fx_quant(p, (const double2*)psi_v, v_idx, v0, nv, ws, bands, 0, s));
+    }
+    for (int c0 = 0; c0 < n_c; c0 += cchunk) {
+      const int nc = std::min(cchunk, n_c - c0);
+      {
+        chi0::ProfScope ps(p, CHI0_K_PAIR_PLANES, s, 3);
+        CK(p, chi0::launch_fx_quant(p, (const double2*)psi_c, c_idx, c_base + c0, nc, ws, bands, vchunk, s));
+        CK(p, chi0::launch_fx_planes(p, iq, ws, bands, vchunk, nv, nc, p->d_D, s));
+      }
+      chi0::ProfScope ps(p, CHI0_K_PAIR_GATHER, s, 1);
+      CK(p, chi0::launch_fx_gather(p, iq, ws, bands, nv, nc, p->d_D, (int64_t)v0 * ld_pairs_c + c0, ld_pairs_c,
+                                   (double2*)M, s));
+    }
+  }
+  return CHI0_OK;
+}
+
 // Pairs of valence rows 0..n_v and conduction columns c_base..c_base+n_c (column ic of the
 // index space is band c_idx[ic], or ic when c_idx is NULL); M row = iv*ld_pairs_c + (ic - c_base).
 static chi0_status pairs_impl(chi0_plan p, int iq, const void* psi_v, const int32_t* v_idx, int n_v,
                               const void* psi_c, const int32_t* c_idx, int c_base, int n_c, void* M,
                               int64_t ld_pairs_c, cudaStream_t s) {
+  if (p->q[iq].fx_map) {
+    const int64_t bands = std::min<int64_t>(chi0::fx_bands(p), (int64_t)n_v + n_c);
+    if (bands >= 2 && ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, bands), s))
+      return pairs_fx(p, iq, psi_v, v_idx, n_v, psi_c, c_idx, c_base, n_c, M, ld_pairs_c, bands, s);
+  }
   // chunk over (v, c) so one chunk's per-plane transforms fit the D buffer
   int vchunk = (int)std::min<int64_t>(n_v, p->D_pairs);
   int cchunk = (int)std::max<int64_t>(1, std::min<int64_t>(n_c, p->D_pairs / vchunk));
@@ -752,37 +824,6 @@ static bool mod_pays(int nG, int n_freq, int64_t K) {
   return modular < direct;
 }
 
-// Workspace of the modular products (FP64 contraction, dense adjoint), at least `need` bytes,
-// allocated on first use and grown when a later call needs more: not inside a stream capture (the
-// CUDA-core kernels run there unless an earlier call has allocated enough).  A size that could not be
-// had is not asked for again.
-static bool mod_ready(chi0_plan p, size_t need, cudaStream_t s) {
-  if (need >= p->mod_limit || !chi0::mod_gemm_usable()) return false;
-  if (need <= p->mod_bytes) return true;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-    cudaGetLastError();
-    return false;
-  }
-  // graphs of batched builds hold the old address
-  if (p->graph_exec) {
-    cudaGraphExecDestroy(p->graph_exec);
-    p->graph_exec = nullptr;
-  }
-  if (p->d_mod) cudaFree(p->d_mod);   // waits for the work that uses it
-  p->d_mod = nullptr;
-  p->ws_bytes -= p->mod_bytes;
-  p->mod_bytes = 0;
-  if (cudaMalloc(&p->d_mod, need) != cudaSuccess) {
-    cudaGetLastError();
-    p->d_mod = nullptr;
-    p->mod_limit = need;
-    return false;
-  }
-  p->mod_bytes = need;
-  p->ws_bytes += need;
-  return true;
-}
 // bytes the contraction takes at most over the plan's spheres
 static size_t mod_contract_bytes(chi0_plan p) {
   size_t need = 0;
@@ -810,9 +851,9 @@ static chi0_status accumulate_impl(chi0_plan p, int iq, const void* M, int n_v, 
       if (e != cudaSuccess)
         return fail(p, CHI0_ERR_CUDA, "tensor-core contraction: " + why + " " + cudaGetErrorString(e));
     } else {
-      if (mod_pays(nG, p->n_freq, K) && mod_ready(p, mod_contract_bytes(p), s)) {
+      if (mod_pays(nG, p->n_freq, K) && chi0::mod_gemm_usable() && ws_ready(p, p->ws_mod, mod_contract_bytes(p), s)) {
         chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, chi0::mod_launches(p, nG));
-        CK(p, chi0::launch_contract_mod(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, p->d_mod, s));
+        CK(p, chi0::launch_contract_mod(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, p->ws_mod.p, s));
       } else {
         chi0::ProfScope ps(p, CHI0_K_CONTRACT_F64, s, 1);
         CK(p, chi0::launch_contract_f64(p, nG, (const double2*)M + p0 * nG, K, p->d_f, (double2*)chi, s));
@@ -971,9 +1012,10 @@ chi0_status chi0_backward(chi0_plan p, int iq, const void* M, int n_v, int n_c, 
   CK(p, cudaMemsetAsync(grad_Ev, 0, sizeof(double) * n_v, s));
   CK(p, cudaMemsetAsync(grad_Ecol, 0, sizeof(double) * n_c, s));
   const int64_t np = (int64_t)n_v * n_c;
-  if (grad_chi0 && chi0::bwd_mod_pays(p, nG, np) && mod_ready(p, chi0::bwd_mod_ws_bytes(p, nG, np), s)) {
+  if (grad_chi0 && chi0::bwd_mod_pays(p, nG, np) && chi0::mod_gemm_usable() &&
+      ws_ready(p, p->ws_bwd, chi0::bwd_mod_ws_bytes(p, nG, np), s)) {
     CK(p, chi0::launch_backward_mod(p, nG, M, np, n_c, E_v, E_col, w_col, (const double2*)grad_chi0, grad_M, grad_Ev,
-                                    grad_Ecol, p->d_bwd, p->d_mod, s));
+                                    grad_Ecol, p->d_bwd, p->ws_bwd.p, s));
     return CHI0_OK;
   }
   for (int64_t p0 = 0; p0 < np; p0 += p->max_pairs) {
@@ -1104,7 +1146,10 @@ chi0_status chi0_build_batched(chi0_plan p, const void* const* psi_v, int n_v, c
   key.push_back(psi_c); key.push_back(c_idx); key.push_back(E_col); key.push_back(w_col);
   key.push_back((const void*)(intptr_t)n_v); key.push_back((const void*)(intptr_t)n_c);
   if (!p->graph_exec || key != p->graph_key) {
-    if (!chi0::is_split(p)) mod_ready(p, mod_contract_bytes(p), s);   // its workspace cannot be allocated inside the capture
+    if (!chi0::is_split(p)) {   // workspaces cannot be allocated inside the capture
+      ws_ready(p, p->ws_mod, mod_contract_bytes(p), s);
+      ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, std::min<int64_t>(chi0::fx_bands(p), (int64_t)n_v + n_c)), s);
+    }
     if (p->graph_exec) { cudaGraphExecDestroy(p->graph_exec); p->graph_exec = nullptr; }
     if (!p->cap_stream) CK(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
     const bool timing = p->prof_timing;
