@@ -221,6 +221,7 @@ cudaError_t launch_backward(chi0_plan_s* p, int nG, const void* M, int64_t p0, i
                             const double* E_v, const double* E_col, const double* w_col, const double2* gamma,
                             const double* diag, void* gM, double* gEv, double* gEc, double* work, cudaStream_t s);
 int bwd_max_freq();
+size_t bwd_work_doubles(int nG, int n_freq, int64_t K);
 // dense adjoint of all pairs on the tensor cores (kern_bwd.cu): workspace, where it pays, the launches
 size_t bwd_mod_ws_bytes(const chi0_plan_s* p, int nG, int64_t n_pairs);
 bool bwd_mod_pays(const chi0_plan_s* p, int nG, int64_t n_pairs);

@@ -43,49 +43,145 @@ __device__ __forceinline__ void st_c(double2* p, int64_t i, double2 v) { p[i] = 
 
 constexpr int kMaxFreqBwd = 64;
 
-// one CTA per pair of the block p0..p0+K; g is [n_freq][nG] real
-template <typename C>
-__global__ void __launch_bounds__(256)
-k_bwd_diag(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
-           const double* __restrict__ E_col, const double* __restrict__ w_col, const double2* __restrict__ omega,
-           int n_freq, double delta, const double* __restrict__ g, C* __restrict__ gM, double* __restrict__ gdE) {
-  __shared__ double s_fr2[kMaxFreqBwd];   // 2 Re f
-  __shared__ double s_fpr[kMaxFreqBwd];   // Re f'
-  __shared__ double s_red[1][8];
-  const int64_t k = blockIdx.x;
-  const int64_t p = p0 + k;
-  const int64_t iv = p / n_c, ic = p - iv * n_c;
-  if (threadIdx.x < n_freq) {
-    double2 f, fp;
-    factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, omega[threadIdx.x], delta, &f, &fp);
-    s_fr2[threadIdx.x] = 2.0 * f.x;
-    s_fpr[threadIdx.x] = fp.x;
+// x^2 as a double, exact: from the mantissa's integer square (the FP64 pipe, two operations per clock
+// and SM, is what bounds the diagonal adjoint)
+__device__ __forceinline__ double square(float x) {
+  const uint32_t u = __float_as_uint(x) & 0x7fffffffu, e = u >> 23;
+  if (e - 1u >= 254u) return (double)x * (double)x;       // zero, subnormal, infinity, NaN
+  const uint32_t m = (u & 0x7fffffu) | 0x800000u;
+  const uint64_t p = (uint64_t)m * m;                     // in [2^46, 2^48)
+  const int t = (int)(p >> 47);
+  return __longlong_as_double((long long)(((uint64_t)(2 * e + (1023 - 254) + t) << 52) | ((p << (6 - t)) & 0xfffffffffffffull)));
+}
+__device__ __forceinline__ double square(double x) { return x * x; }
+
+// s m rounded to the output type, s = c g.  FP32: c and g as sums of two FP32 numbers (48 bits), the
+// product rounded once to within 2^-22 of half a unit, like the FP64 product rounded to FP32; `wide`
+// (c or g outside the range where that holds) takes the FP64 product.
+struct Split {
+  float hi, lo;
+  bool ok;
+};
+__device__ __forceinline__ Split split_of(double x) {     // integer operations: no FP64 subtraction
+  const uint32_t h = (uint32_t)__double2hiint(x), l = (uint32_t)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ff);
+  Split r;
+  r.ok = (e >= 1023 - 40 && e <= 1023 + 40) || x == 0.0;
+  const uint32_t sgn = h & 0x80000000u;
+  r.hi = __uint_as_float(sgn | ((uint32_t)(e - 1023 + 127) << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+  r.lo = (float)(l & 0x1fffffffu) * __uint_as_float(sgn | ((uint32_t)(e - 1023 - 52 + 127) << 23));
+  if (x == 0.0) r.hi = r.lo = 0.f;
+  return r;
+}
+__device__ __forceinline__ float2 scaled(double c, Split cs, double g, Split gs, float2 m) {
+  if (cs.ok && gs.ok) {
+    const float h = cs.hi * gs.hi;
+    const float l = fmaf(cs.hi, gs.hi, -h) + fmaf(cs.hi, gs.lo, cs.lo * gs.hi);
+    const float2 r = make_float2(fmaf(h, m.x, l * m.x), fmaf(h, m.y, l * m.y));
+    if (fabsf(r.x) < INFINITY && fabsf(r.y) < INFINITY) return r;   // not 0 x infinity
+  }
+  const double s = c * g;
+  return make_float2((float)(s * (double)m.x), (float)(s * (double)m.y));
+}
+__device__ __forceinline__ double2 scaled(double c, Split, double g, Split, double2 m) {
+  const double s = c * g;
+  return make_double2(s * m.x, s * m.y);
+}
+
+// fac[w][k] = (2 Re f, Re f') of pair p0 + k
+__global__ void __launch_bounds__(128) k_bwd_factors(int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
+                                                     const double* __restrict__ E_col, const double* __restrict__ w_col,
+                                                     const double2* __restrict__ omega, double delta,
+                                                     double2* __restrict__ fac) {
+  const int64_t k = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (k >= K) return;
+  const int64_t p = p0 + k, iv = p / n_c, ic = p - iv * n_c;
+  double2 f, fp;
+  factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, omega[blockIdx.y], delta, &f, &fp);
+  fac[blockIdx.y * K + k] = make_double2(2.0 * f.x, fp.x);
+}
+
+// A CTA per BD_PAIRS pairs of the block p0..p0+K, g [n_freq][nG] real, read once for
+// them:  gM = sum_w 2 Re f_w g_w M,  gdE = sum_w Re f'_w sum_G g_w |M|^2.
+// ONE: a single frequency, its factors out of the loop: two FP64 operations per
+// element in FP32 plans.  Bound by the FP64 pipe and the integer squares: 1.01 ms
+// for 128,000 pairs, N_G 1200 (2.4 TB/s); 3.97 ms with the square, both products,
+// the conversions and every CTA's own factors on the FP64 pipe, and 2.2 ms more for
+// the row sums by one thread per row.
+constexpr int BD_PAIRS = 4, BD_THREADS = 128;
+template <typename C, bool ONE>
+__global__ void __launch_bounds__(BD_THREADS)
+k_bwd_diag(const C* __restrict__ M, int nG, int64_t K, const double2* __restrict__ fac, int n_freq,
+           const double* __restrict__ g, C* __restrict__ gM, double* __restrict__ gdE) {
+  __shared__ double s_fr2[BD_PAIRS][kMaxFreqBwd];   // 2 Re f
+  __shared__ double s_fpr[BD_PAIRS][kMaxFreqBwd];   // Re f'
+  __shared__ double s_red[BD_THREADS / 32][BD_PAIRS];
+  const int64_t k0 = (int64_t)blockIdx.x * BD_PAIRS;
+  const int np = (int)min((int64_t)BD_PAIRS, K - k0);
+  for (int e = threadIdx.x; e < np * n_freq; e += BD_THREADS) {
+    const int j = e / n_freq, iw = e - j * n_freq;
+    const double2 f = fac[iw * K + k0 + j];
+    s_fr2[j][iw] = f.x;
+    s_fpr[j][iw] = f.y;
   }
   __syncthreads();
-  const C* Mp = M + k * nG;
-  C* gp = gM + k * nG;
-  // t = sum_G |M(G)|^2 sum_w Re f'(w) g_w(G)
-  double t = 0.0;
-  for (int G = threadIdx.x; G < nG; G += blockDim.x) {
-    const double2 m = ld_d(Mp, G);
-    const double m2 = m.x * m.x + m.y * m.y;
-    double s = 0.0, s2 = 0.0;
-    for (int iw = 0; iw < n_freq; ++iw) {
-      const double gw = g[(int64_t)iw * nG + G];
-      s = fma(s_fr2[iw], gw, s);
-      s2 = fma(s_fpr[iw], gw, s2);
+  double t[BD_PAIRS] = {}, c[BD_PAIRS];
+  Split cs[BD_PAIRS];
+  if (ONE)
+#pragma unroll
+    for (int j = 0; j < BD_PAIRS; ++j) {
+      c[j] = j < np ? s_fr2[j][0] : 0.0;
+      cs[j] = split_of(c[j]);
     }
-    t = fma(s2, m2, t);
-    st_c(gp, G, make_double2(s * m.x, s * m.y));
+  for (int G = threadIdx.x; G < nG; G += BD_THREADS) {
+    C m[BD_PAIRS];
+#pragma unroll
+    for (int j = 0; j < BD_PAIRS; ++j)
+      if (j < np) m[j] = M[(k0 + j) * nG + G];
+    if (ONE) {
+      const double gw = g[G];
+      const Split gs = split_of(gw);
+#pragma unroll
+      for (int j = 0; j < BD_PAIRS; ++j)
+        if (j < np) {
+          gM[(k0 + j) * nG + G] = scaled(c[j], cs[j], gw, gs, m[j]);
+          t[j] = fma(gw, square(m[j].x), t[j]);
+          t[j] = fma(gw, square(m[j].y), t[j]);
+        }
+    } else {
+      double s[BD_PAIRS] = {}, s2[BD_PAIRS] = {};
+      for (int iw = 0; iw < n_freq; ++iw) {
+        const double gw = g[(int64_t)iw * nG + G];
+#pragma unroll
+        for (int j = 0; j < BD_PAIRS; ++j)
+          if (j < np) {
+            s[j] = fma(s_fr2[j][iw], gw, s[j]);
+            s2[j] = fma(s_fpr[j][iw], gw, s2[j]);
+          }
+      }
+#pragma unroll
+      for (int j = 0; j < BD_PAIRS; ++j)
+        if (j < np) {
+          st_c(gM, (k0 + j) * nG + G, make_double2(s[j] * (double)m[j].x, s[j] * (double)m[j].y));
+          t[j] = fma(s2[j], square(m[j].x), t[j]);
+          t[j] = fma(s2[j], square(m[j].y), t[j]);
+        }
+    }
   }
-  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  // four sums over the warp in six additions: lanes keep two, then one of them
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) s_red[0][warp] = t;
+  static_assert(BD_PAIRS == 4, "reduction of four sums");
+  const bool hi = lane & 16, hi2 = lane & 8;
+  const double a0 = hi ? t[2] : t[0], a1 = hi ? t[3] : t[1], b0 = hi ? t[0] : t[2], b1 = hi ? t[1] : t[3];
+  const double u0 = a0 + __shfl_xor_sync(0xffffffffu, b0, 16), u1 = a1 + __shfl_xor_sync(0xffffffffu, b1, 16);
+  double r = (hi2 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 8);
+  for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  if ((lane & 7) == 0) s_red[warp][(hi ? 2 : 0) + (hi2 ? 1 : 0)] = r;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < np) {
     double sum = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += s_red[0][w];
-    gdE[k] = sum;
+    for (int w = 0; w < BD_THREADS / 32; ++w) sum += s_red[w][threadIdx.x];
+    gdE[k0 + threadIdx.x] = ONE ? s_fpr[threadIdx.x][0] * sum : sum;
   }
 }
 
@@ -281,25 +377,38 @@ __global__ void k_rowsum(const double* __restrict__ part, int64_t K, int ntile, 
   gdE[k] = s;
 }
 
-// grad E_v[iv] += sum of gdE over the block's pairs in row iv; grad E_col[ic] -= column sums
-__global__ void k_reduce_rows(const double* __restrict__ gdE, int64_t p0, int64_t K, int n_c, double* __restrict__ gEv) {
-  const int64_t iv = p0 / n_c + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t last = (p0 + K - 1) / n_c;
-  if (iv > last) return;
+// grad E_v[iv] += sum of gdE over the block's pairs in row iv; grad E_col[ic] -= column sums.  A CTA
+// per row, 32 x 32 threads per 32 columns, sums in a fixed order (one thread per row took 135 us for a
+// block of 8192 pairs in rows of 2000).
+__global__ void __launch_bounds__(128) k_reduce_rows(const double* __restrict__ gdE, int64_t p0, int64_t K, int n_c,
+                                                     double* __restrict__ gEv) {
+  __shared__ double red[4];
+  const int64_t iv = p0 / n_c + blockIdx.x;
   const int64_t a = max(p0, iv * n_c), b = min(p0 + K, (iv + 1) * n_c);
   double s = 0.0;
-  for (int64_t p = a; p < b; ++p) s += gdE[p - p0];
-  gEv[iv] += s;
+  for (int64_t p = a + threadIdx.x; p < b; p += 128) s += gdE[p - p0];
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) gEv[iv] += (red[0] + red[1]) + (red[2] + red[3]);
 }
-__global__ void k_reduce_cols(const double* __restrict__ gdE, int64_t p0, int64_t K, int n_c, double* __restrict__ gEc) {
-  const int64_t ic = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (ic >= n_c) return;
+__global__ void __launch_bounds__(1024) k_reduce_cols(const double* __restrict__ gdE, int64_t p0, int64_t K, int n_c,
+                                                      double* __restrict__ gEc) {
+  __shared__ double red[32][33];
+  const int64_t ic = (int64_t)blockIdx.x * 32 + threadIdx.x;
   double s = 0.0;
-  for (int64_t iv = p0 / n_c; iv * n_c + ic < p0 + K; ++iv) {
-    const int64_t p = iv * n_c + ic;
-    if (p >= p0) s += gdE[p - p0];
-  }
-  gEc[ic] -= s;
+  if (ic < n_c)
+    for (int64_t iv = p0 / n_c + threadIdx.y; iv * n_c + ic < p0 + K; iv += 32) {
+      const int64_t p = iv * n_c + ic;
+      if (p >= p0) s += gdE[p - p0];
+    }
+  red[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  // thread row y sums column y of the tile over the 32 partial rows
+  s = red[threadIdx.x][threadIdx.y];
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const int64_t c = (int64_t)blockIdx.x * 32 + threadIdx.y;
+  if (threadIdx.x == 0 && c < n_c) gEc[c] -= s;
 }
 
 // Eq. 4 step edge e_k = min(E_0 + k dE, E_max), rounded as written (no fused multiply-add, so the
@@ -354,6 +463,10 @@ cudaError_t launch_energy_substitution(const double* E_c, const double* sens, in
 }
 
 int bwd_max_freq() { return kMaxFreqBwd; }
+// doubles of work for K pairs at a time: grad dE, then per-tile sums (dense) or factors (diagonal)
+size_t bwd_work_doubles(int nG, int n_freq, int64_t K) {
+  return (size_t)(K + 1) / 2 * 2 + (size_t)K * std::max((nG + 63) / 64, 2 * std::min(n_freq, kMaxFreqBwd));
+}
 
 template <typename C>
 static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int64_t K, int n_c, const double* E_v,
@@ -361,8 +474,14 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
                             C* gM, double* gEv, double* gEc, double* work, cudaStream_t s) {
   double* gdE = work;
   if (diag) {
-    k_bwd_diag<C><<<(unsigned)K, 256, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, p->d_omega, p->n_freq, p->delta,
-                                              diag, gM, gdE);
+    double2* fac = reinterpret_cast<double2*>(work + (K + 1) / 2 * 2);
+    k_bwd_factors<<<dim3((unsigned)((K + 127) / 128), p->n_freq), 128, 0, s>>>(p0, K, n_c, E_v, E_col, w_col, p->d_omega,
+                                                                              p->delta, fac);
+    const unsigned grid = (unsigned)((K + BD_PAIRS - 1) / BD_PAIRS);
+    if (p->n_freq == 1)
+      k_bwd_diag<C, true><<<grid, BD_THREADS, 0, s>>>(M, nG, K, fac, p->n_freq, diag, gM, gdE);
+    else
+      k_bwd_diag<C, false><<<grid, BD_THREADS, 0, s>>>(M, nG, K, fac, p->n_freq, diag, gM, gdE);
   } else {
     const int ntile = (nG + 63) / 64;
     double* part = work + K;
@@ -379,8 +498,8 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
     k_rowsum<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(part, K, ntile, gdE);
   }
   const int64_t rows = (p0 + K - 1) / n_c - p0 / n_c + 1;
-  k_reduce_rows<<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEv);
-  k_reduce_cols<<<(unsigned)((n_c + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEc);
+  k_reduce_rows<<<(unsigned)rows, 128, 0, s>>>(gdE, p0, K, n_c, gEv);
+  k_reduce_cols<<<(unsigned)((n_c + 31) / 32), dim3(32, 32), 0, s>>>(gdE, p0, K, n_c, gEc);
   return cudaGetLastError();
 }
 
@@ -462,8 +581,8 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
     }
     k_rowsum<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(part, K, ntile, gdE);
     const int64_t rows = (p0 + K - 1) / n_c - p0 / n_c + 1;
-    k_reduce_rows<<<(unsigned)((rows + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEv);
-    k_reduce_cols<<<(unsigned)((n_c + 127) / 128), 128, 0, s>>>(gdE, p0, K, n_c, gEc);
+    k_reduce_rows<<<(unsigned)rows, 128, 0, s>>>(gdE, p0, K, n_c, gEv);
+    k_reduce_cols<<<(unsigned)((n_c + 31) / 32), dim3(32, 32), 0, s>>>(gdE, p0, K, n_c, gEc);
   }
   return cudaGetLastError();
 }

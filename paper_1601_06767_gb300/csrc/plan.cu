@@ -395,7 +395,7 @@ chi0_status chi0_plan_create(chi0_plan* out, const chi0_plan_desc* d) {
   size_t bytes_M = (size_t)mp * p->max_nG * cb;
   size_t bytes_f = (size_t)p->n_freq * mp * sizeof(double2);
   p->pack_bytes = chi0::is_split(p) ? chi0::tc_pack_bytes(p, mp, p->max_nG) : 0;
-  const size_t bytes_bwd = (size_t)mp * (1 + (p->max_nG + 63) / 64) * sizeof(double);
+  const size_t bytes_bwd = chi0::bwd_work_doubles(p->max_nG, p->n_freq, mp) * sizeof(double);
   if (env_fault("oom")) { p->err = "injected fault: oom"; return bail(CHI0_ERR_OOM); }
   cudaError_t e;
   if ((e = cudaMalloc(&p->d_D, bytes_D)) != cudaSuccess ||
@@ -1018,10 +1018,21 @@ chi0_status chi0_backward(chi0_plan p, int iq, const void* M, int n_v, int n_c, 
                                     grad_Ecol, p->d_bwd, p->ws_bwd.p, s));
     return CHI0_OK;
   }
-  for (int64_t p0 = 0; p0 < np; p0 += p->max_pairs) {
-    const int64_t K = std::min<int64_t>(p->max_pairs, np - p0);
+  // the diagonal adjoint is one short pass: all pairs in one launch where the work memory (three numbers
+  // per pair and frequency) can be had; the plan's own holds max_pairs
+  int64_t blk = p->max_pairs;
+  double* work = p->d_bwd;
+  if (diag_g && np > blk) {
+    const int64_t big = std::min<int64_t>(np, (int64_t)4 << 20);
+    if (ws_ready(p, p->ws_bwd, chi0::bwd_work_doubles(1, p->n_freq, big) * sizeof(double), s)) {
+      blk = big;
+      work = (double*)p->ws_bwd.p;
+    }
+  }
+  for (int64_t p0 = 0; p0 < np; p0 += blk) {
+    const int64_t K = std::min<int64_t>(blk, np - p0);
     CK(p, chi0::launch_backward(p, nG, M, p0, K, n_c, E_v, E_col, w_col, (const double2*)grad_chi0, diag_g,
-                                grad_M, grad_Ev, grad_Ecol, p->d_bwd, s));
+                                grad_M, grad_Ev, grad_Ecol, work, s));
   }
   return CHI0_OK;
 }
