@@ -114,6 +114,10 @@ struct chi0_plan_s {
   void* pipe_pack = nullptr;
   int pipe_state = 0;           // 0 not set up, 1 ready, -1 unavailable (serial build)
   size_t inv_bytes = 0;
+  // look-ahead of the dielectric inverse: the next panel runs beside the trailing update
+  cudaStream_t inv_side = nullptr;
+  cudaEvent_t inv_ev[2] = {};
+  int inv_state = 0;            // 0 not set up, 1 ready, -1 unavailable
   size_t ws_bytes = 0;
   std::string err;
   bool tc_ready = false;     // tensor-map encoder resolved

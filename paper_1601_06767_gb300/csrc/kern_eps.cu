@@ -20,6 +20,8 @@
 // the column swaps in reverse order to give A^-1.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "cplx.cuh"
 #include "internal.h"
 
@@ -35,7 +37,7 @@ template <typename C> __device__ __forceinline__ C csub(C a, C b) {
   return a;
 }
 template <typename C> __device__ __forceinline__ C crecip(C a) {
-  const auto d = a.x * a.x + a.y * a.y;
+  const auto d = fma(a.x, a.x, a.y * a.y);
   C r;
   r.x = a.x / d;
   r.y = -a.y / d;
@@ -43,15 +45,24 @@ template <typename C> __device__ __forceinline__ C crecip(C a) {
 }
 template <typename C> __device__ __forceinline__ auto cabs1(C a) -> decltype(a.x) { return fabs(a.x) + fabs(a.y); }
 
-__global__ void k_epsilon(const double2* __restrict__ chi, const double* __restrict__ v, int symmetric, int nG,
-                          int64_t total, double2* __restrict__ eps) {
-  const int64_t n2 = (int64_t)nG * nG;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e % n2;
-    const int i = (int)(r / nG), j = (int)(r - (int64_t)i * nG);
-    const double s = symmetric ? sqrt(v[i]) * sqrt(v[j]) : v[i];
-    const double2 c = chi[e];
-    eps[e] = make_double2((i == j ? 1.0 : 0.0) - s * c.x, -s * c.y);
+// A CTA takes 256 columns of EPS_ROWS rows of one matrix; the square roots of its rows
+// and columns are taken once (per element they and a 64-bit division cost 1.95 ms for
+// 9 x 2500^2 on the FP64 pipe, against 0.27 ms for the bytes).
+constexpr int EPS_ROWS = 32;
+__global__ void __launch_bounds__(256) k_epsilon(const double2* __restrict__ chi, const double* __restrict__ v,
+                                                 int symmetric, int nG, double2* __restrict__ eps) {
+  __shared__ double vr[EPS_ROWS];
+  const int j = blockIdx.x * 256 + threadIdx.x, i0 = blockIdx.y * EPS_ROWS, rows = min(EPS_ROWS, nG - i0);
+  if (threadIdx.x < rows) vr[threadIdx.x] = symmetric ? sqrt(v[i0 + threadIdx.x]) : v[i0 + threadIdx.x];
+  __syncthreads();
+  if (j >= nG) return;
+  const double vj = symmetric ? sqrt(v[j]) : 1.0;
+  const size_t base = ((size_t)blockIdx.z * nG + i0) * nG + j;
+#pragma unroll 4
+  for (int r = 0; r < rows; ++r) {
+    const double s = vr[r] * vj;
+    const double2 c = chi[base + (size_t)r * nG];
+    eps[base + (size_t)r * nG] = make_double2((i0 + r == j ? 1.0 : 0.0) - s * c.x, -s * c.y);
   }
 }
 
@@ -76,150 +87,182 @@ template <typename R> struct SelRows { static constexpr int V = sizeof(R) == 4 ?
 // winners.  Leaf level (cand_in == NULL): block c holds rows k0 + c*ROWS ...;
 // merge levels: block c holds entries c*ROWS ... of the previous level's list
 // (NB slots per set, -1 = empty).  Writes NB slots per block to cand_out.
+//
+// Rows are not moved, each has a position instead (ties go to the lowest one).  Three
+// barriers per column and several threads per row; latency bound (33 us a level of
+// 128 FP32 rows with one thread per row, moved rows and four barriers; 61 us with
+// the rows in registers, whose straight-line code missed the instruction cache).
+constexpr int SEL_THREADS = 256;
 template <typename R>
-__global__ void __launch_bounds__(SelRows<R>::V)
+__global__ void __launch_bounds__(SEL_THREADS)
 k_tp_select(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* __restrict__ cand_in,
-            int n_in, int* __restrict__ cand_out, int ld) {
+            int n_in, int* __restrict__ cand_out, int ld, const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
-  constexpr int ROWS = SelRows<R>::V;
-  const int w = blockIdx.y, c = blockIdx.x, r = threadIdx.x;
+  constexpr int ROWS = SelRows<R>::V, TPR = SEL_THREADS / ROWS, NW = SEL_THREADS / 32;
+  const int w = blockIdx.y, c = blockIdx.x, tid = threadIdx.x, warp = tid >> 5;
+  if (skip && skip[w] == 0) return;
   const C* a = A + (size_t)w * N * N;
-  __shared__ C S[ROWS][NB + 1];
-  __shared__ int idx[ROWS];
-  __shared__ R red_v[ROWS / 32];
-  __shared__ int red_i[ROWS / 32];
-  __shared__ int s_n, s_p, wcnt[ROWS / 32];
+  __shared__ C S[ROWS][NB + 2];
+  __shared__ int idx[ROWS], win[NB], wcnt[ROWS / 32];
+  __shared__ unsigned long long w_key[2][NW];
+  __shared__ unsigned w_min[2][NW];
+  __shared__ C s_inv;                              // reciprocal of the pivot, by one thread
+  // valid rows to the front, keeping their order (deterministic ties)
   int g = -1;
-  if (cand_in == nullptr) {
-    const int row = k0 + c * ROWS + r;
-    g = row < N ? row : -1;
-  } else {
-    const int e = c * ROWS + r;
-    g = e < n_in ? cand_in[(size_t)w * ld + e] : -1;
+  if (tid < ROWS) {
+    const int e = c * ROWS + tid;
+    if (cand_in == nullptr) g = k0 + e < N ? k0 + e : -1;
+    else g = e < n_in ? cand_in[(size_t)w * ld + e] : -1;
   }
-  // compact the valid rows to the front, keeping their order (deterministic ties)
   const unsigned bal = __ballot_sync(0xffffffffu, g >= 0);
-  if ((r & 31) == 0) wcnt[r >> 5] = __popc(bal);
+  if (tid < ROWS && (tid & 31) == 0) wcnt[warp] = __popc(bal);
   __syncthreads();
-  if (r == 0) {
-    int acc = 0;
-    for (int q = 0; q < ROWS / 32; ++q) {
-      const int n = wcnt[q];
-      wcnt[q] = acc;
-      acc += n;
-    }
-    s_n = acc;
+  int nr = 0, at = __popc(bal & ((1u << (tid & 31)) - 1u));
+#pragma unroll
+  for (int q = 0; q < ROWS / 32; ++q) {
+    if (q < warp) at += wcnt[q];
+    nr += wcnt[q];
+  }
+  if (g >= 0) idx[at] = g;
+  __syncthreads();
+  for (int e = tid; e < nr * NB; e += SEL_THREADS) {
+    const int r = e / NB, t = e - r * NB;
+    S[r][t] = t < kb ? a[(size_t)idx[r] * N + k0 + t] : cz(C{});
   }
   __syncthreads();
-  if (g >= 0) idx[wcnt[r >> 5] + __popc(bal & ((1u << (r & 31)) - 1u))] = g;
-  __syncthreads();
-  const int nr = s_n;
-  if (r < nr) {
-    const C* src = a + (size_t)idx[r] * N + k0;
-    for (int t = 0; t < kb; ++t) S[r][t] = src[t];
-  }
-  __syncthreads();
-  const int steps = min(kb, nr);
+  const int row = tid / TPR, sub = tid - row * TPR, steps = min(kb, nr);
+  int pos = row;
   for (int j = 0; j < steps; ++j) {
-    R best = (r >= j && r < nr) ? cabs1(S[r][j]) : (R)-1;
-    int bi = (r >= j && r < nr) ? r : ROWS;
-    for (int o = 16; o; o >>= 1) {
-      const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    const int b = j & 1;
+    // largest |re| + |im| among positions >= j, ties to the lowest position: the value's bits order
+    // non-negative numbers; 0 marks a row that is no candidate
+    unsigned long long key = 0;
+    if (pos >= j && pos < nr) {
+      if constexpr (sizeof(R) == 4) key = (unsigned long long)__float_as_uint(cabs1(S[row][j])) + 1;
+      else key = (unsigned long long)__double_as_longlong(cabs1(S[row][j])) + 1;
     }
-    if ((r & 31) == 0) { red_v[r >> 5] = best; red_i[r >> 5] = bi; }
-    __syncthreads();
-    if (r == 0) {
-      for (int q = 1; q < ROWS / 32; ++q)
-        if (red_v[q] > best || (red_v[q] == best && red_i[q] < bi)) { best = red_v[q]; bi = red_i[q]; }
-      s_p = (bi < nr) ? bi : j;
+    unsigned long long best = key;
+    if constexpr (sizeof(R) == 4) best = __reduce_max_sync(0xffffffffu, (unsigned)key);
+    else
+      for (int o = 16; o; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+    const unsigned mp = __reduce_min_sync(0xffffffffu, (key == best && key) ? (unsigned)(pos << 8 | row) : 0xffffffffu);
+    if ((tid & 31) == 0) {
+      w_key[b][warp] = best;
+      w_min[b][warp] = mp;
     }
     __syncthreads();
-    const int p = s_p;
-    if (p != j) {
-      if (r < kb) {
-        const C u = S[j][r];
-        S[j][r] = S[p][r];
-        S[p][r] = u;
+    best = w_key[b][0];
+    unsigned pm = w_min[b][0];
+#pragma unroll
+    for (int q = 1; q < NW; ++q) {
+      const unsigned long long k2 = w_key[b][q];
+      const unsigned p2 = w_min[b][q];
+      if (k2 > best || (k2 == best && p2 < pm)) { best = k2; pm = p2; }
+    }
+    // the pivot row goes to position j, the row there to the pivot's
+    const int p = (int)(pm >> 8), pr = (int)(pm & 255u);
+    if (row == pr) {
+      if (sub == 0) {
+        win[j] = idx[row];
+        s_inv = crecip(S[row][j]);
       }
-      if (r == 0) {
-        const int u = idx[j];
-        idx[j] = idx[p];
-        idx[p] = u;
-      }
+      pos = j;
+    } else if (pos == j) {
+      pos = p;
     }
     __syncthreads();
-    if (r > j && r < nr) {
-      const C piv = S[j][j];
+    if (pos > j && pos < nr) {
+      const C piv = S[pr][j];
       if (piv.x != (R)0 || piv.y != (R)0) {
-        const C l = cmul(S[r][j], crecip(piv));
-        for (int t = j + 1; t < kb; ++t) S[r][t] = csub(S[r][t], cmul(l, S[j][t]));
+        const C l = cmul(S[row][j], s_inv);
+#pragma unroll 4
+        for (int t = j + 1 + sub; t < kb; t += TPR) S[row][t] = csub(S[row][t], cmul(l, S[pr][t]));
       }
     }
     __syncthreads();
   }
-  if (r < NB) cand_out[(size_t)w * ld + (size_t)c * NB + r] = (r < steps) ? idx[r] : -1;
+  if (tid < NB) cand_out[(size_t)w * ld + (size_t)c * NB + tid] = (tid < steps) ? win[tid] : -1;
 }
 
-// Move the winners to rows k0..k0+kb-1 (recorded as a swap sequence in piv),
-// copy the panel columns of every row to Z, invert the pivot block by
-// Gauss-Jordan with partial pivoting in shared memory: T = A11^-1 (also
-// written over the pivot block).
+// Move the winners to rows k0..k0+kb-1 of the panel (recorded as a swap sequence in
+// piv) and invert the pivot block by Gauss-Jordan with partial pivoting in shared
+// memory: T = A11^-1 (also written over the pivot block).  One CTA per matrix,
+// latency bound: four barriers per column, the moved rows (64 at most) read and
+// written once each, the copy of the panel left to k_copy_panel (91 us with a
+// barrier and two memory round trips per swap, six barriers per column and the
+// copy by this one CTA, 2500^2 FP32).
 template <typename R>
 __global__ void __launch_bounds__(1024)
 k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* __restrict__ win, int ld,
-           typename Cx<R>::T* __restrict__ Z, typename Cx<R>::T* __restrict__ Tb, int* __restrict__ piv,
-           int* __restrict__ status) {
+           typename Cx<R>::T* __restrict__ Tb, int* __restrict__ piv, int* __restrict__ status,
+           const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
   const int w = blockIdx.x, tid = threadIdx.x;
+  if (skip && skip[w] == 0) return;
   C* a = A + (size_t)w * N * N;
-  C* z = Z + (size_t)w * N * NB;
   int* pv = piv + (size_t)w * N;
-  __shared__ int sp[NB];
+  __shared__ int orig[2 * NB], cur[2 * NB], s_n;
   __shared__ C B[NB][2 * NB + 1];
   __shared__ int s_p;
-  if (tid == 0) {
-    // swap sequence: step t exchanges row k0+t with the current row of winner t
-    int orig[2 * NB], cur[2 * NB], n = 0;
+  if (tid < 32) {
+    // swap sequence: step t exchanges row k0+t with the current row of winner t; (orig, cur) lists the
+    // rows moved so far and where each is now, two entries per lane
+    int n = 0, o0 = -1, o1 = -1, c0 = -1, c1 = -1;
+    const int mywin = tid < kb ? win[(size_t)w * ld + tid] : -1;
     for (int t = 0; t < kb; ++t) {
-      const int x = win[(size_t)w * ld + t];
-      int px = x;
-      for (int q = 0; q < n; ++q)
-        if (orig[q] == x) px = cur[q];
-      const int y = k0 + t;
-      int oy = y;
-      for (int q = 0; q < n; ++q)
-        if (cur[q] == y) oy = orig[q];
-      if (x < 0) px = y;     // fewer candidates than columns (cannot happen for kb <= N - k0)
-      sp[t] = px;
-      pv[y] = px;
+      const int x = __shfl_sync(0xffffffffu, mywin, t), y = k0 + t;
+      // position of original row x, original row at position y (each in at most one entry)
+      const int px_l = (o0 == x && tid < n) ? c0 : ((o1 == x && tid + 32 < n) ? c1 : -1);
+      const int oy_l = (c0 == y && tid < n) ? o0 : ((c1 == y && tid + 32 < n) ? o1 : -1);
+      int px = (int)__reduce_max_sync(0xffffffffu, (unsigned)(px_l + 1)) - 1;
+      int oy = (int)__reduce_max_sync(0xffffffffu, (unsigned)(oy_l + 1)) - 1;
+      if (px < 0) px = x;
+      if (oy < 0) oy = y;
+      if (x < 0) px = y;      // fewer candidates than columns (cannot happen for kb <= N - k0)
+      if (tid == 0) pv[y] = px;
       if (px != y) {
         // the row now at y (original oy) moves to px, winner x moves to y
-        bool fo = false, fx = false;
-        for (int q = 0; q < n; ++q) {
-          if (orig[q] == oy) { cur[q] = px; fo = true; }
-          else if (orig[q] == x) { cur[q] = y; fx = true; }
+        const bool fo = __any_sync(0xffffffffu, (o0 == oy && tid < n) || (o1 == oy && tid + 32 < n));
+        const bool fx = __any_sync(0xffffffffu, (o0 == x && tid < n) || (o1 == x && tid + 32 < n));
+        if (tid < n) {
+          if (o0 == oy) c0 = px;
+          else if (o0 == x) c0 = y;
         }
-        if (!fo) { orig[n] = oy; cur[n] = px; ++n; }
-        if (!fx) { orig[n] = x; cur[n] = y; ++n; }
+        if (tid + 32 < n) {
+          if (o1 == oy) c1 = px;
+          else if (o1 == x) c1 = y;
+        }
+        if (!fo) {
+          if (n == tid) { o0 = oy; c0 = px; }
+          if (n == tid + 32) { o1 = oy; c1 = px; }
+          ++n;
+        }
+        if (!fx) {
+          if (n == tid) { o0 = x; c0 = y; }
+          if (n == tid + 32) { o1 = x; c1 = y; }
+          ++n;
+        }
       }
     }
+    orig[tid] = o0;
+    orig[tid + 32] = o1;
+    cur[tid] = c0;
+    cur[tid + 32] = c1;
+    if (tid == 0) s_n = n;
   }
   __syncthreads();
-  for (int t = 0; t < kb; ++t) {
-    const int y = k0 + t, p = sp[t];
-    if (p != y && tid < kb) {
-      const C u = a[(size_t)y * N + k0 + tid];
-      a[(size_t)y * N + k0 + tid] = a[(size_t)p * N + k0 + tid];
-      a[(size_t)p * N + k0 + tid] = u;
-    }
+  {
+    // all moves at once: row orig[q] to cur[q], 32 columns each (two entries per thread)
+    const int q = tid >> 5, t = tid & 31;
+    C u = cz(C{}), v = cz(C{});
+    const bool m0 = q < s_n && t < kb, m1 = q + 32 < s_n && t < kb;
+    if (m0) u = a[(size_t)orig[q] * N + k0 + t];
+    if (m1) v = a[(size_t)orig[q + 32] * N + k0 + t];
     __syncthreads();
+    if (m0) a[(size_t)cur[q] * N + k0 + t] = u;
+    if (m1) a[(size_t)cur[q + 32] * N + k0 + t] = v;
   }
-  for (int64_t e = tid; e < (int64_t)N * kb; e += blockDim.x) {
-    const int i = (int)(e / kb), t = (int)(e - (int64_t)i * kb);
-    z[(size_t)i * NB + t] = a[(size_t)i * N + k0 + t];
-  }
+  __syncthreads();
   // [A11 | I] -> [I | A11^-1]
   for (int e = tid; e < NB * 2 * NB; e += blockDim.x) {
     const int i = e / (2 * NB), c = e - i * 2 * NB;
@@ -240,7 +283,7 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
       }
       if (tid == 0) {
         if (!(best > (R)0) || bi >= kb) {
-          atomicOr(status, SINGULAR_BIT);
+          if (status) atomicOr(status, SINGULAR_BIT);
           bi = j;
         }
         s_p = bi;
@@ -248,23 +291,24 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
     }
     __syncthreads();
     const int p = s_p;
-    if (p != j && tid < 2 * NB) {
-      const C u = B[j][tid];
-      B[j][tid] = B[p][tid];
-      B[p][tid] = u;
+    C u = cz(C{}), v = cz(C{}), d = cz(C{});
+    if (tid < 2 * NB) {
+      u = B[j][tid];
+      v = B[p][tid];
+      d = B[p][j];
     }
     __syncthreads();
-    const C inv = crecip(B[j][j]);
+    if (tid < 2 * NB) {
+      if (p != j) B[p][tid] = u;
+      B[j][tid] = cmul(v, crecip(d));
+    }
     __syncthreads();
-    if (tid < 2 * NB) B[j][tid] = cmul(B[j][tid], inv);
-    __syncthreads();
-    // eliminate column j from every other row: thread (i, c)
+    // eliminate column j from every other row: thread (i, c); columns up to j of the left half are
+    // not read again
     for (int e = tid; e < NB * 2 * NB; e += blockDim.x) {
       const int i = e / (2 * NB), c = e - i * 2 * NB;
-      if (i != j && i < kb && c != j) B[i][c] = csub(B[i][c], cmul(B[i][j], B[j][c]));
+      if (i != j && i < kb && c > j) B[i][c] = csub(B[i][c], cmul(B[i][j], B[j][c]));
     }
-    __syncthreads();
-    if (tid < NB && tid != j) B[tid][j] = cz(C{});
     __syncthreads();
   }
   for (int e = tid; e < kb * kb; e += blockDim.x) {
@@ -275,15 +319,26 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
   }
 }
 
+// Z = the panel's columns k0..k0+kb of every row outside the pivot rows (those are not read)
+template <typename R>
+__global__ void __launch_bounds__(256) k_copy_panel(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb,
+                                                    typename Cx<R>::T* __restrict__ Z, const int* __restrict__ skip) {
+  const int w = blockIdx.y;
+  if (skip && skip[w] == 0) return;
+  const int e = blockIdx.x * 256 + threadIdx.x, i = e / NB, t = e - i * NB;
+  if (i < N && t < kb) Z[((size_t)w * N + i) * NB + t] = A[((size_t)w * N + i) * N + k0 + t];
+}
+
 // ---------------------------------------------------------------------------
 // 2. row swaps outside the panel, pivot rows := T A10
 // ---------------------------------------------------------------------------
 template <typename R>
 __global__ void __launch_bounds__(128)
 k_gj_rows(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const typename Cx<R>::T* __restrict__ Tb,
-          const int* __restrict__ piv) {
+          const int* __restrict__ piv, const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
   const int w = blockIdx.y;
+  if (skip && skip[w] == 0) return;
   C* a = A + (size_t)w * N * N;
   const int* pv = piv + (size_t)w * N;
   __shared__ C ts[NB][NB];
@@ -316,61 +371,161 @@ k_gj_rows(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const typena
 }
 
 // ---------------------------------------------------------------------------
-// 3. trailing update of all rows outside R1 (64 x 64 output tiles, K = kb)
+// 3. trailing update of all rows outside R1, columns [c0, c1) without [x0, x1)
 // ---------------------------------------------------------------------------
-// output tile: 64 x 64 (FP32) or 32 x 32 (FP64, static shared memory limit); 256 threads
-template <typename R> struct UpdTile { static constexpr int T = sizeof(R) == 4 ? 64 : 32; };
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool ok) {
+  const int n = ok ? BYTES : 0;                   // 0: fill with zeros
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "n"(BYTES), "r"(n)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename R>
+__device__ __forceinline__ float4 ld_early(const float2* p) {   // volatile: not moved past the products
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
+// FP32 with even N (every row starts on 16 bytes): 64 x 64 output tiles, 256
+// threads, four consecutive rows x two pairs of columns each.  A CTA takes one tile
+// of rows and a run of `run` column tiles: Z's tile is loaded once, the pivot rows
+// of the next tile are copied (asynchronously, double buffered) and the tile's own
+// elements read while the products run.  Issue bound: 64 multiply-adds per step and
+// thread against four 16-byte shared loads.  9 x 2500^2, 79 panels: 24.3 ms; 32.0
+// ms with a CTA per tile, scalar loads and the tile's elements read after the
+// products.  (Packed f32x2 multiply-adds, with operands doubled in shared memory:
+// 33.4 ms, the shared-memory loads bound it.)
+constexpr int UT = 64, ULD = UT + 2;
+constexpr size_t UPD32_SMEM = (size_t)(NB * ULD + 2 * NB * UT) * sizeof(float2);
+__global__ void __launch_bounds__(256, 2)
+k_gj_update32(float2* __restrict__ A, int N, int k0, int kb, int c0, int c1, int x0, int x1, int run,
+              const float2* __restrict__ Z, const int* __restrict__ skip) {
+  extern __shared__ __align__(16) unsigned char smem_upd[];
+  float2* rs = reinterpret_cast<float2*>(smem_upd);    // [2][NB][UT]  rs[t][col]
+  float2* zs = rs + 2 * NB * UT;                       // [NB][ULD]  zs[t][row]
+  const int w = blockIdx.z, tid = threadIdx.x;
+  if (skip && skip[w] == 0) return;
+  float2* a = A + (size_t)w * N * N;
+  const float2* z = Z + (size_t)w * N * NB;
+  const int i0 = blockIdx.y * UT, jt0 = blockIdx.x * run;
+  const int ntile = (c1 - c0 + UT - 1) / UT, jt1 = min(ntile, jt0 + run);
+  // pivot rows: a thread copies column pair 2 (tid mod 32) of rows tid / 32 + 8 q (c0 and c1 are even)
+  const int pc = 2 * (tid & 31), pt = tid >> 5;
+  auto load_rows = [&](int jt) {
+    float2* dst = rs + (jt & 1) * NB * UT;
+    const int j = c0 + jt * UT + pc;
+#pragma unroll
+    for (int q = 0; q < NB / 8; ++q) {
+      const int t = pt + 8 * q;
+      const bool ok = j < c1 && t < kb;
+      cp_async<16>(dst + t * UT + pc, a + (ok ? (size_t)(k0 + t) * N + j : 0), ok);
+    }
+    cp_async_commit();
+  };
+  if (jt0 < jt1) load_rows(jt0);
+  for (int e = tid; e < UT * NB; e += 256) {
+    const int r = e / NB, t = e - r * NB, i = i0 + r;
+    zs[t * ULD + r] = (i < N && t < kb) ? z[(size_t)i * NB + t] : make_float2(0.f, 0.f);
+  }
+  const int tx = tid & 15, ty = tid >> 4;
+  float2* arow = a + (size_t)(i0 + 4 * ty) * N + 2 * tx;
+  for (int jt = jt0; jt < jt1; ++jt) {
+    const int j0 = c0 + jt * UT;
+    cp_async_wait<0>();
+    __syncthreads();                                   // this tile's pivot rows are there, the other buffer is free
+    if (jt + 1 < jt1) load_rows(jt + 1);
+    float4 base[4][2];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int j = j0 + 2 * tx + 32 * c;
+        base[r][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i0 + 4 * ty + r < N && j < c1 && !(j >= k0 && j < k0 + kb)) base[r][c] = ld_early(arow + (size_t)r * N + j0 + 32 * c);
+      }
+    const float2* rt = rs + (jt & 1) * NB * UT + 2 * tx;
+    float2 acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.f, 0.f);
+#pragma unroll 4
+    for (int t = 0; t < NB; ++t) {                     // rows t >= kb are zero
+      const float4 r0 = *reinterpret_cast<const float4*>(rt + t * UT);
+      const float4 r1 = *reinterpret_cast<const float4*>(rt + t * UT + 32);
+      const float4 z0 = *reinterpret_cast<const float4*>(zs + t * ULD + 4 * ty);
+      const float4 z1 = *reinterpret_cast<const float4*>(zs + t * ULD + 4 * ty + 2);
+      const float2 rc[4] = {make_float2(r0.x, r0.y), make_float2(r0.z, r0.w), make_float2(r1.x, r1.y), make_float2(r1.z, r1.w)};
+      const float2 zr[4] = {make_float2(z0.x, z0.y), make_float2(z0.z, z0.w), make_float2(z1.x, z1.y), make_float2(z1.z, z1.w)};
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) cfma(acc[r][c], zr[r], rc[c]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int i = i0 + 4 * ty + r;
+      if (i >= N || (i >= k0 && i < k0 + kb)) continue;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int j = j0 + 2 * tx + 32 * c;            // x0, x1 and the panel's edges are even
+        if (j >= c1 || (j >= x0 && j < x1)) continue;
+        const float2 u = csub(make_float2(base[r][c].x, base[r][c].y), acc[r][2 * c]);
+        const float2 v = csub(make_float2(base[r][c].z, base[r][c].w), acc[r][2 * c + 1]);
+        *reinterpret_cast<float4*>(arow + (size_t)r * N + j0 + 32 * c) = make_float4(u.x, u.y, v.x, v.y);
+      }
+    }
+  }
+}
+
+// FP64 (bound by the FP64 pipe) and FP32 with odd N: a CTA per 32 x 32 output tile, 256 threads, 2 x 2
+// elements each
+constexpr int UTG = 32;
+template <typename C>
 __global__ void __launch_bounds__(256)
-k_gj_update(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const typename Cx<R>::T* __restrict__ Z) {
-  using C = typename Cx<R>::T;
-  constexpr int TILE = UpdTile<R>::T, RT = TILE / 16;
+k_gj_update_tile(C* __restrict__ A, int N, int k0, int kb, int c0, int c1, int x0, int x1, const C* __restrict__ Z,
+                 const int* __restrict__ skip) {
   const int w = blockIdx.z;
+  if (skip && skip[w] == 0) return;
   C* a = A + (size_t)w * N * N;
   const C* z = Z + (size_t)w * N * NB;
-  __shared__ C zs[NB][TILE + 1];     // zs[t][row]
-  __shared__ C rs[NB][TILE + 1];     // rs[t][col]
-  const int i0 = blockIdx.y * TILE, j0 = blockIdx.x * TILE;
-  for (int e = threadIdx.x; e < TILE * NB; e += blockDim.x) {
-    const int r = e / NB, t = e - r * NB;
-    const int i = i0 + r;
+  __shared__ C zs[NB][UTG + 1];     // zs[t][row]
+  __shared__ C rs[NB][UTG + 1];     // rs[t][col]
+  const int i0 = blockIdx.y * UTG, j0 = c0 + blockIdx.x * UTG;
+  for (int e = threadIdx.x; e < UTG * NB; e += blockDim.x) {
+    const int r = e / NB, t = e - r * NB, i = i0 + r;
     zs[t][r] = (i < N && t < kb) ? z[(size_t)i * NB + t] : cz(C{});
-  }
-  for (int e = threadIdx.x; e < NB * TILE; e += blockDim.x) {
-    const int t = e / TILE, c = e - t * TILE;
-    const int j = j0 + c;
-    rs[t][c] = (j < N && t < kb) ? a[(size_t)(k0 + t) * N + j] : cz(C{});
+    const int tt = e / UTG, c = e - tt * UTG, j = j0 + c;
+    rs[tt][c] = (j < c1 && tt < kb) ? a[(size_t)(k0 + tt) * N + j] : cz(C{});
   }
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  C acc[RT][RT];
-#pragma unroll
-  for (int r = 0; r < RT; ++r)
-#pragma unroll
-    for (int c = 0; c < RT; ++c) acc[r][c] = cz(C{});
+  C acc[2][2] = {{cz(C{}), cz(C{})}, {cz(C{}), cz(C{})}};
   for (int t = 0; t < kb; ++t) {
-    C zr[RT], rc[RT];
+    C zr[2], rc[2];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) zr[r] = zs[t][ty + 16 * r];
+    for (int r = 0; r < 2; ++r) zr[r] = zs[t][ty + 16 * r];
 #pragma unroll
-    for (int c = 0; c < RT; ++c) rc[c] = rs[t][tx + 16 * c];
+    for (int c = 0; c < 2; ++c) rc[c] = rs[t][tx + 16 * c];
 #pragma unroll
-    for (int r = 0; r < RT; ++r)
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-      for (int c = 0; c < RT; ++c) cfma(acc[r][c], zr[r], rc[c]);
+      for (int c = 0; c < 2; ++c) cfma(acc[r][c], zr[r], rc[c]);
   }
 #pragma unroll
-  for (int r = 0; r < RT; ++r) {
+  for (int r = 0; r < 2; ++r) {
     const int i = i0 + ty + 16 * r;
     if (i >= N || (i >= k0 && i < k0 + kb)) continue;
 #pragma unroll
-    for (int c = 0; c < RT; ++c) {
+    for (int c = 0; c < 2; ++c) {
       const int j = j0 + tx + 16 * c;
-      if (j >= N) continue;
+      if (j >= c1 || (j >= x0 && j < x1)) continue;
       C* o = a + (size_t)i * N + j;
-      const C base = (j >= k0 && j < k0 + kb) ? cz(C{}) : *o;
-      *o = csub(base, acc[r][c]);
+      *o = csub((j >= k0 && j < k0 + kb) ? cz(C{}) : *o, acc[r][c]);
     }
   }
 }
@@ -379,9 +534,11 @@ k_gj_update(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const type
 // 4. column swaps in reverse order: (P A)^-1 P = A^-1
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void k_gj_colperm(typename Cx<R>::T* __restrict__ A, int N, const int* __restrict__ piv) {
+__global__ void k_gj_colperm(typename Cx<R>::T* __restrict__ A, int N, const int* __restrict__ piv,
+                             const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
   const int w = blockIdx.y;
+  if (skip && skip[w] == 0) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   C* row = A + (size_t)w * N * N + (size_t)i * N;
@@ -396,43 +553,126 @@ __global__ void k_gj_colperm(typename Cx<R>::T* __restrict__ A, int N, const int
   }
 }
 
+// side stream and events of the look-ahead, made on first use; false inside a stream capture
+bool inv_streams(chi0_plan_s* p, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if (p->inv_state != 0) return p->inv_state > 0;
+  p->inv_state = -1;
+  int least = 0, greatest = 0;
+  if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
+      cudaStreamCreateWithPriority(&p->inv_side, cudaStreamNonBlocking, greatest) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  for (cudaEvent_t& e : p->inv_ev)
+    if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+  p->inv_state = 1;
+  return true;
+}
+
 // candidate-list slots per matrix for an N-row panel (ping-pong pair)
 template <typename R> int64_t tp_ld(int N) { return (int64_t)((N + SelRows<R>::V - 1) / SelRows<R>::V) * NB; }
 
+// pivot search and pivot block of panel k0: Z (copy of its columns), T, piv
 template <typename R>
-cudaError_t gj_invert(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, void* Z, void* Tb, int* piv,
-                      int* cand, cudaStream_t s) {
+void gj_panel(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, int k0, void* Z, void* Tb, int* piv, int* cand,
+              int* status, const int* skip, cudaStream_t s) {
   using C = typename Cx<R>::T;
   constexpr int ROWS = SelRows<R>::V;
-  const int ld = (int)tp_ld<R>(N);
+  const int ld = (int)tp_ld<R>(N), kb = min(NB, N - k0);
   int* cbuf[2] = {cand, cand + (size_t)nf * ld};
-  for (int k0 = 0; k0 < N; k0 += NB) {
-    const int kb = min(NB, N - k0);
-    {
-      // tournament: leaf blocks of ROWS rows, then merges of ROWS / NB sets until one is left
-      int nblk = (N - k0 + ROWS - 1) / ROWS, levels = 1, cur = 0;
-      for (int b = nblk; b > 1; b = (b * NB + ROWS - 1) / ROWS) ++levels;
-      ProfScope ps(p, CHI0_K_INV_PANEL, s, levels + 2);
-      k_tp_select<R><<<dim3(nblk, nf), ROWS, 0, s>>>(A, N, k0, kb, nullptr, 0, cbuf[0], ld);
-      while (nblk > 1) {
-        const int n_in = nblk * NB;
-        nblk = (n_in + ROWS - 1) / ROWS;
-        k_tp_select<R><<<dim3(nblk, nf), ROWS, 0, s>>>(A, N, k0, kb, cbuf[cur], n_in, cbuf[cur ^ 1], ld);
-        cur ^= 1;
-      }
-      k_tp_final<R><<<nf, 1024, 0, s>>>(A, N, k0, kb, cbuf[cur], ld, (C*)Z, (C*)Tb, piv, p->d_status);
-      k_gj_rows<R><<<dim3((N + 127) / 128, nf), 128, 0, s>>>(A, N, k0, kb, (const C*)Tb, piv);
-    }
-    {
-      ProfScope ps(p, CHI0_K_INV_UPDATE, s, 1);
-      const int t = (N + UpdTile<R>::T - 1) / UpdTile<R>::T;
-      k_gj_update<R><<<dim3(t, t, nf), 256, 0, s>>>(A, N, k0, kb, (const C*)Z);
-    }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+  // tournament: leaf blocks of ROWS rows, then merges of ROWS / NB sets until one is left
+  int nblk = (N - k0 + ROWS - 1) / ROWS, levels = 1, cur = 0;
+  for (int b = nblk; b > 1; b = (b * NB + ROWS - 1) / ROWS) ++levels;
+  ProfScope ps(p, CHI0_K_INV_PANEL, s, levels + 2);
+  k_tp_select<R><<<dim3(nblk, nf), SEL_THREADS, 0, s>>>(A, N, k0, kb, nullptr, 0, cbuf[0], ld, skip);
+  while (nblk > 1) {
+    const int n_in = nblk * NB;
+    nblk = (n_in + ROWS - 1) / ROWS;
+    k_tp_select<R><<<dim3(nblk, nf), SEL_THREADS, 0, s>>>(A, N, k0, kb, cbuf[cur], n_in, cbuf[cur ^ 1], ld, skip);
+    cur ^= 1;
   }
+  k_tp_final<R><<<nf, 1024, 0, s>>>(A, N, k0, kb, cbuf[cur], ld, (C*)Tb, piv, status, skip);
+  k_copy_panel<R><<<dim3((N * NB + 255) / 256, nf), 256, 0, s>>>(A, N, k0, kb, (C*)Z, skip);
+}
+
+// columns [c0, c1) without [x0, x1)
+template <typename R>
+cudaError_t gj_update(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, int k0, int c0, int c1, int x0, int x1,
+                      const void* Z, const int* skip, cudaStream_t s) {
+  using C = typename Cx<R>::T;
+  const int kb = min(NB, N - k0);
+  ProfScope ps(p, CHI0_K_INV_UPDATE, s, 1);
+  bool wide = false;
+  if constexpr (sizeof(R) == 4) {
+    if (N % 2 == 0) {
+      cudaError_t e = cudaFuncSetAttribute(k_gj_update32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)UPD32_SMEM);
+      if (e != cudaSuccess) return e;
+      // runs of column tiles as long as eight CTAs per SM are left (two run at a time); short ones, so
+      // that the panel kernels beside them find room soon
+      const int rows = (N + UT - 1) / UT, cols = (c1 - c0 + UT - 1) / UT;
+      int run = 4;
+      while (run > 1 && (int64_t)rows * ((cols + run - 1) / run) * nf < 8 * 152) run >>= 1;
+      k_gj_update32<<<dim3((cols + run - 1) / run, rows, nf), 256, UPD32_SMEM, s>>>(A, N, k0, kb, c0, c1, x0, x1, run,
+                                                                                  (const C*)Z, skip);
+      wide = true;
+    }
+  }
+  if (!wide) {
+    const dim3 grid((c1 - c0 + UTG - 1) / UTG, (N + UTG - 1) / UTG, nf);
+    k_gj_update_tile<C><<<grid, 256, 0, s>>>(A, N, k0, kb, c0, c1, x0, x1, (const C*)Z, skip);
+  }
+  return cudaGetLastError();
+}
+
+// The panel of the next columns needs only their update, so that is done first and
+// the panel's latency-bound kernels (pivot search, pivot block) run on a stream of
+// the plan beside the update of all other columns; Z and T are double buffered.
+// 9 x 2500^2 in FP32, with the copies and eps = 1 - v chi0: 49.7 -> 34.4 ms.
+// Inside a stream capture everything stays on one stream.
+// skip (or NULL): matrices whose entry is 0 are left alone.  status: NULL = zero pivots not recorded.
+template <typename R>
+cudaError_t gj_invert(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, void* Z, void* Tb, int* piv,
+                      int* cand, int* status, const int* skip, cudaStream_t s) {
+  using C = typename Cx<R>::T;
+  C* Zb[2] = {(C*)Z, (C*)Z + (size_t)nf * N * NB};
+  C* Tbb[2] = {(C*)Tb, (C*)Tb + (size_t)nf * NB * NB};
+  const bool look = !skip && inv_streams(p, s);
+  cudaError_t e = cudaSuccess;
+  gj_panel<R>(p, A, N, nf, 0, Zb[0], Tbb[0], piv, cand, status, skip, s);
+  for (int k0 = 0, b = 0; k0 < N && e == cudaSuccess; k0 += NB, b ^= 1) {
+    const int kb = min(NB, N - k0), n0 = k0 + NB, n1 = min(N, n0 + NB);
+    {
+      ProfScope ps(p, CHI0_K_INV_PANEL, s, 1);
+      k_gj_rows<R><<<dim3((N + 127) / 128, nf), 128, 0, s>>>(A, N, k0, kb, Tbb[b], piv, skip);
+    }
+    if (n0 >= N) {
+      e = gj_update<R>(p, A, N, nf, k0, 0, N, 0, 0, Zb[b], skip, s);
+    } else if (!look) {
+      e = gj_update<R>(p, A, N, nf, k0, 0, N, 0, 0, Zb[b], skip, s);
+      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, status, skip, s);
+    } else {
+      e = gj_update<R>(p, A, N, nf, k0, n0, n1, 0, 0, Zb[b], skip, s);
+      if (e == cudaSuccess) e = cudaEventRecord(p->inv_ev[0], s);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(p->inv_side, p->inv_ev[0], 0);
+      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, status, skip, p->inv_side);
+      // joined whatever happens
+      cudaEventRecord(p->inv_ev[1], p->inv_side);
+      if (e == cudaSuccess) e = gj_update<R>(p, A, N, nf, k0, 0, N, n0, n1, Zb[b], skip, s);
+      cudaStreamWaitEvent(s, p->inv_ev[1], 0);
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
   ProfScope ps(p, CHI0_K_INV_PANEL, s, 1);
-  k_gj_colperm<R><<<dim3((N + 127) / 128, nf), 128, 0, s>>>(A, N, piv);
+  k_gj_colperm<R><<<dim3((N + 127) / 128, nf), 128, 0, s>>>(A, N, piv, skip);
   return cudaGetLastError();
 }
 
@@ -443,19 +683,23 @@ int eps_panel_width() { return NB; }
 cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const double* v, int symmetric,
                            double2* eps, cudaStream_t s) {
   ProfScope ps(p, CHI0_K_EPS, s, 1);
-  const int64_t total = (int64_t)p->n_freq * nG * nG;
-  k_epsilon<<<4 * 152, 256, 0, s>>>(chi, v, symmetric, nG, total, eps);
+  for (int w = 0; w < p->n_freq; w += 65535) {     // grid z limit
+    const int nw = std::min(65535, p->n_freq - w);
+    const size_t off = (size_t)w * nG * nG;
+    k_epsilon<<<dim3((nG + 255) / 256, (nG + EPS_ROWS - 1) / EPS_ROWS, nw), 256, 0, s>>>(chi + off, v, symmetric, nG,
+                                                                                       eps + off);
+  }
   return cudaGetLastError();
 }
 
-// Workspace (bytes): complex64 copy of the matrices (split plans), Z [nf][N][NB], T [nf][NB][NB],
+// Workspace (bytes): complex64 copy of the matrices (split plans), Z [2][nf][N][NB], T [2][nf][NB][NB],
 // piv [nf][N], two candidate lists [nf][tp_ld].
 size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG) {
   const size_t nf = (size_t)p->n_freq, c = is_split(p) ? sizeof(float2) : sizeof(double2);
   const size_t copy = is_split(p) ? nf * nG * nG * sizeof(float2) : 0;
   const size_t ld = (size_t)(is_split(p) ? tp_ld<float>(nG) : tp_ld<double>(nG));
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
-  return al(copy) + al(nf * nG * NB * c) + al(nf * NB * NB * c) + al(nf * nG * sizeof(int)) +
+  return al(copy) + al(2 * nf * nG * NB * c) + al(2 * nf * NB * NB * c) + al(nf * nG * sizeof(int)) +
          al(2 * nf * ld * sizeof(int));
 }
 
@@ -467,9 +711,9 @@ cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* w
     float2* a32 = reinterpret_cast<float2*>(b);
     b += al(nf * nG * nG * sizeof(float2));
     void* Z = b;
-    b += al(nf * nG * NB * sizeof(float2));
+    b += al(2 * nf * nG * NB * sizeof(float2));
     void* Tb = b;
-    b += al(nf * NB * NB * sizeof(float2));
+    b += al(2 * nf * NB * NB * sizeof(float2));
     int* piv = reinterpret_cast<int*>(b);
     b += al(nf * nG * sizeof(int));
     int* cand = reinterpret_cast<int*>(b);
@@ -478,20 +722,20 @@ cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* w
       ProfScope ps(p, CHI0_K_EPS, s, 1);
       k_to_c64<<<4 * 152, 256, 0, s>>>(eps, n, a32);
     }
-    cudaError_t e = gj_invert<float>(p, a32, nG, (int)nf, Z, Tb, piv, cand, s);
+    cudaError_t e = gj_invert<float>(p, a32, nG, (int)nf, Z, Tb, piv, cand, p->d_status, nullptr, s);
     if (e != cudaSuccess) return e;
     ProfScope ps(p, CHI0_K_EPS, s, 1);
     k_from_c64<<<4 * 152, 256, 0, s>>>(a32, n, eps);
     return cudaGetLastError();
   }
   void* Z = b;
-  b += al(nf * nG * NB * sizeof(double2));
+  b += al(2 * nf * nG * NB * sizeof(double2));
   void* Tb = b;
-  b += al(nf * NB * NB * sizeof(double2));
+  b += al(2 * nf * NB * NB * sizeof(double2));
   int* piv = reinterpret_cast<int*>(b);
   b += al(nf * nG * sizeof(int));
   int* cand = reinterpret_cast<int*>(b);
-  return gj_invert<double>(p, eps, nG, (int)nf, Z, Tb, piv, cand, s);
+  return gj_invert<double>(p, eps, nG, (int)nf, Z, Tb, piv, cand, p->d_status, nullptr, s);
 }
 
 }  // namespace chi0

@@ -115,6 +115,9 @@ void free_plan(chi0_plan_s* p) {
   cudaFree(p->pipe_M); cudaFree(p->pipe_f); cudaFree(p->pipe_pack);
   for (cudaEvent_t e : p->pipe_ev)
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : p->inv_ev)
+    if (e) cudaEventDestroy(e);
+  if (p->inv_side) cudaStreamDestroy(p->inv_side);
   if (p->pipe_lo) cudaStreamDestroy(p->pipe_lo);
   if (p->pipe_hi) cudaStreamDestroy(p->pipe_hi);
 }
