@@ -374,7 +374,9 @@ chi0_status chi0_epsilon(chi0_plan plan, int iq, const void* chi0, const double*
 
 /* In-place inverse of the n_freq matrices eps[w] ((device) [n_freq][n_G[iq]][n_G[iq]]
  * complex128, row-major) by blocked Gauss-Jordan elimination with partial
- * pivoting (largest |re| + |im| in the column).  FP64 plans compute in FP64;
+ * pivoting (largest |re| + |im| in the column).  FP64 plans compute to FP64 accuracy:
+ * an FP32 elimination refined by Newton steps in FP64, or, for matrices those do not
+ * bring to FP64 accuracy and small ones, the elimination in FP64;
  * split plans compute in FP32 on a complex64 copy and write the result back
  * as complex128 (forward error about cond(eps) x 1e-7).  Workspace (the
  * complex64 copy for split plans, panel buffers) is allocated at the first

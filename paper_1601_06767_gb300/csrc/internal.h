@@ -193,17 +193,19 @@ struct ModGemm {
   const uint16_t* B;               // [b_planes][cols][Kp]
   int16_t* R;                      // [planes][rows][ldR]
   int rows_a, row0, rows, cols, ldR, Kp, planes, a_planes, b_planes;
+  const int* todo;
 };
 cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s);
-// scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B
+// scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B.
+// todo (here, below and in ModGemm): not NULL = the kernels do nothing where it points at 0
 cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s);
+                                 uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
 cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s);
-// the same of the conjugate transpose of X [n][rows] (operand B; ws: mod_cols_ws_bytes)
+                                 uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
+// the same of the transpose (conj: conjugate transpose) of X [n][rows] (operand B; ws: mod_cols_ws_bytes)
 size_t mod_cols_ws_bytes(int n, int rows);
-cudaError_t launch_mod_pack_cols_conj(const double2* X, int n, int rows, int Kp, int* scale, uint16_t* planes,
-                                      void* ws, cudaStream_t s);
+cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, uint16_t* planes,
+                                 void* ws, cudaStream_t s, const int* todo = nullptr);
 // one q-point's share of a batched tensor-core contraction
 struct TcJob {
   int nG;
@@ -243,7 +245,9 @@ bool tc_supported(std::string* why);
 // dielectric matrix: eps = 1 - v chi0 (plain or symmetrised) and its in-place inverse
 cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const double* v, int symmetric,
                            double2* eps, cudaStream_t s);
-size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG);
+// workspace of the inverse; refined: with that of FP64 plans' refinement of an FP32 inverse
+size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG, bool refined);
+bool eps_inverse_refines(const chi0_plan_s* p, int nG);
 // COH self-energy with the plasmon-pole model
 cudaError_t launch_density(const chi0_plan_s* p, const void* psi_v, int n_v, double* dens, cudaStream_t s);
 size_t density_ft_ws_bytes(const chi0_plan_s* p, int s2, int s3);
@@ -255,6 +259,6 @@ size_t sigma_coh_ws_bytes(const chi0_plan_s* p, int nG, int n_t);
 cudaError_t launch_sigma_coh(const chi0_plan_s* p, int nG, const void* m, int n_t, int n_b, const double* x,
                              const double* w, const double2* Om2, const double2* wt, const double* v, double delta,
                              void* ws, double2* partial, int* n_tiles, cudaStream_t s);
-cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* ws, cudaStream_t s);
+cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* ws, bool refined, cudaStream_t s);
 
 }  // namespace chi0

@@ -568,11 +568,11 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
           const double2* G = gamma + (size_t)(w0 + w) * nG * nG;
           e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG, Bp + 2 * w * set, s);
           if (e == cudaSuccess)
-            e = launch_mod_pack_cols_conj(G, nG, nG, z.Kp, sB + (size_t)(2 * w + 1) * nG, Bp + (2 * w + 1) * set,
+            e = launch_mod_pack_cols(G, nG, nG, z.Kp, true, sB + (size_t)(2 * w + 1) * nG, Bp + (2 * w + 1) * set,
                                           b + z.off_ws, s);
           if (e != cudaSuccess) return e;
         }
-      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL};
+      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
       k_bwd_mod<C><<<dim3(ntile, (K + 15) / 16), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,

@@ -24,6 +24,7 @@
 
 #include "cplx.cuh"
 #include "internal.h"
+#include "modgemm.cuh"
 
 namespace chi0 {
 namespace {
@@ -692,18 +693,171 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// FP64 plans: FP32 inverse refined in FP64
+// ---------------------------------------------------------------------------
+// The FP64 elimination is bound by the FP64 pipe (two multiply-adds per clock and SM):
+// 42 ms for one 1200^2.  Here X is the FP32 inverse and every step takes
+//   R = I - A X,  X += X R   (Newton; the error is squared)
+// with both products exact modular ones on the tensor cores (modgemm.cuh).  A step
+// whose largest |R| is at most 2^-32 is a matrix's last: the error left is below
+// the rounding of X.  A matrix that has no such step within STEPS (ill conditioned
+// beyond FP32, out of its range, singular, not finite) is inverted by the FP64
+// elimination from the untouched A, whose kernels skip the others.
+//
+// 1200^2: 42.6 -> 7.9 ms (FP32 inverse 6.2, one matrix's latency; two steps 0.8,
+// skipped kernels 0.7); 9 x 2500^2: 1047 ms at first, 72 ms.  Against quad precision
+// 1.8e-16 (relative Frobenius, eps-like matrices), 3.3e-16 by the elimination.
+namespace {
+constexpr int STEPS = 3;
+constexpr uint32_t LAST_STEP = (uint32_t)(1023 - 32) << 20;     // magnitude word of 2^-32
+
+__global__ void k_ref_init(int* __restrict__ todo, uint32_t* __restrict__ rmax, int nf) {
+  for (int w = threadIdx.x; w < nf; w += blockDim.x) {
+    todo[w] = 1;
+    rmax[w] = 0;
+  }
+}
+
+// values of the residue planes of one N x N product.  LAST = false: R = I - value and the largest
+// magnitude word of R; true: X += value.  A warp takes 16 rows x 8 columns (as k_mod_add).
+template <bool ADD>
+__global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P, int N, int ldR,
+                                                   const int* __restrict__ sA, const int* __restrict__ sB,
+                                                   double2* __restrict__ out, uint32_t* __restrict__ rmax,
+                                                   const int* __restrict__ todo) {
+  if (*todo == 0) return;
+  const int lane = threadIdx.x & 31;
+  const int j0 = 8 * (blockIdx.x * 4 + (threadIdx.x >> 5)), i = blockIdx.y * 16 + (lane >> 1);
+  uint32_t big = 0;
+  if (j0 < N && i < N) {
+    double2* o = out + (size_t)i * N + j0 + (lane & 1);
+    double2 v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (ADD && j0 + 2 * c + (lane & 1) < N) v[c] = o[2 * c];
+    mod::Frac re[4] = {}, im[4] = {};
+    mod::gather_fractions(P + mod::res_index(N, ldR, 0, i, j0), mod::res_plane(N, ldR), lane & 1 ? mod::ODD : mod::EVEN, re, im);
+    const int sa = sA[i];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = j0 + 2 * c + (lane & 1);
+      if (j >= N) break;
+      const int sb = sB[j];
+      const bool bad = sa == mod::NO_SCALE || sb == mod::NO_SCALE;
+      const double x = bad ? nan("") : mod::frac_value(re[c], -sa - sb), y = bad ? nan("") : mod::frac_value(im[c], -sa - sb);
+      const double2 r = ADD ? make_double2(v[c].x + x, v[c].y + y) : make_double2((i == j ? 1.0 : 0.0) - x, -y);
+      if (!ADD) big = max(big, max(mod::mag_word(r.x), mod::mag_word(r.y)));
+      o[2 * c] = r;
+    }
+  }
+  if (!ADD) {
+    big = __reduce_max_sync(0xffffffffu, big);
+    if (lane == 0) atomicMax(rmax, big);
+  }
+}
+
+// after a step: the matrix is done when its R was small enough; the next step starts from 0
+__global__ void k_ref_decide(uint32_t* __restrict__ rmax, int* __restrict__ todo) {
+  if (*todo && *rmax <= LAST_STEP) *todo = 0;
+  *rmax = 0;
+}
+
+// eps = X where the matrix is done (todo 0)
+__global__ void __launch_bounds__(256) k_ref_store(const double2* __restrict__ X, int64_t n, double2* __restrict__ eps,
+                                                   const int* __restrict__ todo) {
+  if (*todo != 0) return;
+  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (int64_t)gridDim.x * 256) eps[e] = X[e];
+}
+
+// offsets of the refinement's workspace: FP32 copies of all matrices, then for one matrix at a time X, R,
+// planes of A, planes of X rows, planes of a transposed operand, residues, scales
+struct RefSizes {
+  int Kp, ldR;
+  size_t x, r, pa, px, pt, res, sa, sx, st, cols, todo, rmax, bytes;
+};
+RefSizes ref_sizes(int N, int nf) {
+  auto al = [](size_t v) { return (v + 255) / 256 * 256; };
+  RefSizes z;
+  z.Kp = (N + 63) / 64 * 64;
+  z.ldR = (N + 7) / 8 * 8;
+  const size_t planes = al((size_t)mod::NPL * 2 * N * z.Kp), mat = al((size_t)N * N * sizeof(double2)), sc = al((size_t)N * sizeof(int));
+  z.x = al((size_t)nf * N * N * sizeof(float2));
+  z.r = z.x + mat;
+  z.pa = z.r + mat;
+  z.px = z.pa + planes;
+  z.pt = z.px + planes;
+  z.res = z.pt + planes;
+  z.sa = z.res + al((size_t)mod::NPL * 2 * mod::res_plane(N, z.ldR));
+  z.sx = z.sa + sc;
+  z.st = z.sx + sc;
+  z.cols = z.st + sc;
+  z.todo = z.cols + al(mod_cols_ws_bytes(N, N));
+  z.rmax = z.todo + al((size_t)nf * sizeof(int));
+  z.bytes = z.rmax + al((size_t)nf * sizeof(uint32_t));
+  return z;
+}
+
+cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z, void* Tb, int* piv, int* cand, void* ws,
+                            cudaStream_t s) {
+  const RefSizes z = ref_sizes(N, nf);
+  unsigned char* b = reinterpret_cast<unsigned char*>(ws);
+  float2* a32 = reinterpret_cast<float2*>(b);
+  double2 *X = reinterpret_cast<double2*>(b + z.x), *R = reinterpret_cast<double2*>(b + z.r);
+  uint16_t *PA = (uint16_t*)(b + z.pa), *PX = (uint16_t*)(b + z.px), *PT = (uint16_t*)(b + z.pt);
+  int16_t* res = (int16_t*)(b + z.res);
+  int *sA = (int*)(b + z.sa), *sX = (int*)(b + z.sx), *sT = (int*)(b + z.st), *todo = (int*)(b + z.todo);
+  uint32_t* rmax = (uint32_t*)(b + z.rmax);
+  const int64_t n2 = (int64_t)N * N;
+  {
+    ProfScope ps(p, CHI0_K_EPS, s, 2);
+    k_ref_init<<<1, 128, 0, s>>>(todo, rmax, nf);
+    k_to_c64<<<4 * 152, 256, 0, s>>>(eps, nf * n2, a32);
+  }
+  cudaError_t e = gj_invert<float>(p, a32, N, nf, Z, Tb, piv, cand, nullptr, nullptr, s);
+  const dim3 gv((z.ldR / 8 + 3) / 4, (N + 15) / 16);
+  for (int w = 0; w < nf && e == cudaSuccess; ++w) {
+    ProfScope ps(p, CHI0_K_INV_UPDATE, s, 4 + STEPS * 15);
+    const double2* A = eps + w * n2;
+    k_from_c64<<<4 * 152, 256, 0, s>>>(a32 + w * n2, n2, X);
+    e = launch_mod_pack_rows(A, N, N, N, z.Kp, true, sA, PA, s);
+    for (int it = 0; it < STEPS && e == cudaSuccess; ++it) {
+      e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
+      if (e == cudaSuccess)
+        e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
+      k_ref_value<false><<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, rmax + w, todo + w);
+      if (e == cudaSuccess) e = launch_mod_pack_rows(X, N, N, N, z.Kp, true, sX, PX, s, todo + w);
+      if (e == cudaSuccess) e = launch_mod_pack_cols(R, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
+      if (e == cudaSuccess)
+        e = launch_mod_gemm(p, ModGemm{PX, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
+      k_ref_value<true><<<gv, 128, 0, s>>>(res, N, z.ldR, sX, sT, X, nullptr, todo + w);
+      k_ref_decide<<<1, 1, 0, s>>>(rmax + w, todo + w);
+    }
+    k_ref_store<<<4 * 152, 256, 0, s>>>(X, n2, eps + w * n2, todo + w);
+    if (e == cudaSuccess) e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  return gj_invert<double>(p, eps, N, nf, Z, Tb, piv, cand, p->d_status, todo, s);
+}
+}  // namespace
+
+// Where the refined inverse runs: FP64 plans from REF_MIN_N on, two panels (128^2: 2.5 ms by the
+// elimination, 0.7 ms refined; a single panel has nothing to gain)
+constexpr int REF_MIN_N = 64;
+bool eps_inverse_refines(const chi0_plan_s* p, int nG) { return !is_split(p) && nG >= REF_MIN_N && mod_gemm_usable(); }
+
 // Workspace (bytes): complex64 copy of the matrices (split plans), Z [2][nf][N][NB], T [2][nf][NB][NB],
 // piv [nf][N], two candidate lists [nf][tp_ld].
-size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG) {
+size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG, bool refined) {
   const size_t nf = (size_t)p->n_freq, c = is_split(p) ? sizeof(float2) : sizeof(double2);
   const size_t copy = is_split(p) ? nf * nG * nG * sizeof(float2) : 0;
   const size_t ld = (size_t)(is_split(p) ? tp_ld<float>(nG) : tp_ld<double>(nG));
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   return al(copy) + al(2 * nf * nG * NB * c) + al(2 * nf * NB * NB * c) + al(nf * nG * sizeof(int)) +
-         al(2 * nf * ld * sizeof(int));
+         al(2 * nf * ld * sizeof(int)) + (refined ? ref_sizes(nG, (int)nf).bytes : 0);
 }
 
-cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* ws, cudaStream_t s) {
+cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* ws, bool refined, cudaStream_t s) {
   const size_t nf = (size_t)p->n_freq;
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   unsigned char* b = reinterpret_cast<unsigned char*>(ws);
@@ -735,6 +889,8 @@ cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* w
   int* piv = reinterpret_cast<int*>(b);
   b += al(nf * nG * sizeof(int));
   int* cand = reinterpret_cast<int*>(b);
+  b += al(2 * nf * tp_ld<double>(nG) * sizeof(int));
+  if (refined) return refined_inverse(p, eps, nG, (int)nf, Z, Tb, piv, cand, b, s);
   return gj_invert<double>(p, eps, nG, (int)nf, Z, Tb, piv, cand, p->d_status, nullptr, s);
 }
 

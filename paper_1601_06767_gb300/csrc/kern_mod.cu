@@ -60,7 +60,8 @@ constexpr int ST_COLS = 64, ST_ROWS = 128;   // a statistics block: 64 sphere po
 
 // eg[G] = largest magnitude word of M[0..K)[G] (eg cleared by the caller)
 __global__ void __launch_bounds__(256) k_mod_rowmax(const double2* __restrict__ M, int nG, int64_t K,
-                                                    uint32_t* __restrict__ eg) {
+                                                    uint32_t* __restrict__ eg, const int* __restrict__ todo) {
+  if (todo && *todo == 0) return;
   const int G = blockIdx.x * ST_COLS + (threadIdx.x & 63);
   if (G >= nG) return;
   const int64_t k1 = min(K, (int64_t)(blockIdx.y + 1) * ST_ROWS);
@@ -125,6 +126,30 @@ __global__ void __launch_bounds__(256) k_mod_norms(const double2* __restrict__ M
   }
 }
 
+// slot 0 alone, relative to the column's own largest element: FP32 sums do (what underflows is below
+// 2^-126 of the norm), without the FP64 pipe
+__global__ void __launch_bounds__(256) k_mod_col_norms(const double2* __restrict__ M, int nG, int64_t K,
+                                                       const uint32_t* __restrict__ eg, double* __restrict__ part,
+                                                       const int* __restrict__ todo) {
+  if (todo && *todo == 0) return;
+  __shared__ float red[4][ST_COLS];
+  const int g = threadIdx.x & 63, r = threadIdx.x >> 6, G = blockIdx.x * ST_COLS + g;
+  const int64_t k0 = (int64_t)blockIdx.y * ST_ROWS;
+  const uint32_t wg = G < nG ? eg[G] : 0;
+  float s = 0.f;
+  if (wg >= 0x00100000u && wg < 0x7ff00000u) {
+    const int e = mod::word_exp(wg);
+    for (int j = r; j < ST_ROWS && k0 + j < K; j += 4) {
+      const double2 v = M[(k0 + j) * nG + G];
+      const float x = mod::scaled_abs(v.x, e), y = mod::scaled_abs(v.y, e);
+      s = fmaf(x, x, fmaf(y, y, s));
+    }
+  }
+  red[r][g] = s;
+  __syncthreads();
+  if (r == 0 && G < nG) part[(size_t)blockIdx.y * nG + G] = (double)((red[0][g] + red[1][g]) + (red[2][g] + red[3][g]));
+}
+
 // scale exponents: slot 0 (conj(M), operand B) and 1 + w (W_w, operand A)
 __global__ void __launch_bounds__(256) k_mod_scales(const double* __restrict__ part, int n_part, int nG, int n_freq,
                                                     const uint32_t* __restrict__ eg, const uint32_t* __restrict__ ef,
@@ -145,13 +170,14 @@ __global__ void __launch_bounds__(256) k_mod_scales(const double* __restrict__ p
 // ---------------------------------------------------------------------------
 constexpr int PK_G = 16, PK_K = 64;   // tile: 16 sphere points x 64 pairs, transposed through shared memory
 
-// Planes [26][nG][Kp] (FP16) of conj(M) into Bp (when not NULL) and of W_w = f(w) M,
+// Planes [26][nG][Kp] (FP16) of conj(M) (of M: conj = false) into Bp (when not NULL) and of W_w = f(w) M,
 // w = w0 .. w0 + nw, into Ap (26 planes per frequency).  A warp holds one sphere
 // point, a lane two neighbouring pairs: 128-byte stores per plane.
 __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M, int nG, int64_t K, int Kp,
                                                   const double2* __restrict__ f, int w0, int nw,
-                                                  const int* __restrict__ scale, uint32_t* __restrict__ Bp,
-                                                  uint32_t* __restrict__ Ap) {
+                                                  const int* __restrict__ scale, bool conj, uint32_t* __restrict__ Bp,
+                                                  uint32_t* __restrict__ Ap, const int* __restrict__ todo) {
+  if (todo && *todo == 0) return;
   __shared__ double2 tile[PK_K][PK_G + 1];
   __shared__ double2 fs[PK_K];
   const int G0 = blockIdx.x * PK_G;
@@ -183,7 +209,7 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
         b = cmul(fs[2 * lane + 1], b);
       }
       mod::store_residues(mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s)),
-                          mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), slot < 0,
+                          mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), slot < 0 && conj,
                           dst + (size_t)G * (Kp / 2) + p0 / 2 + lane, plane);
     }
   }
@@ -197,7 +223,8 @@ __device__ __forceinline__ double2 ld_wide(const double2* p, size_t i) { return 
 // largest: what underflows there does not count), summed in a fixed order
 template <typename C>
 __global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X, int n, size_t ld, int beta,
-                                                        int* __restrict__ scale) {
+                                                        int* __restrict__ scale, const int* __restrict__ todo) {
+  if (todo && *todo == 0) return;
   __shared__ uint32_t mx[4];
   __shared__ float sm[4];
   const C* x = X + blockIdx.x * ld;
@@ -230,7 +257,9 @@ __global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X,
 // planes [26][rows][Kp] of X; a warp takes 64 elements of a row
 template <typename C>
 __global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, int rows, int n, size_t ld, int Kp,
-                                                       const int* __restrict__ scale, uint32_t* __restrict__ dst) {
+                                                       const int* __restrict__ scale, uint32_t* __restrict__ dst,
+                                                       const int* __restrict__ todo) {
+  if (todo && *todo == 0) return;
   const int lane = threadIdx.x & 31, segs = Kp / 64;
   const int64_t unit = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (unit >= (int64_t)rows * segs) return;
@@ -277,6 +306,7 @@ struct GemmArgs {
   int tiles_m, tiles_n, n_b;   // tiles and planes
   int a_planes, b_planes;      // planes of A and B (a plane index is taken modulo these)
   int nK;                      // stages of GK
+  const int* todo;             // not NULL: nothing is done where it points at 0
 };
 
 struct GemmBars {
@@ -308,6 +338,7 @@ __constant__ float c_mod[NM] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f,
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
+  if (P.todo && *P.todo == 0) return;   // the same for both CTAs of a pair
   extern __shared__ __align__(1024) unsigned char smem_mod[];
   unsigned char* tiles = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_mod) + 1023) & ~uintptr_t(1023));
@@ -583,6 +614,7 @@ cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s) {
   P.a_planes = g.a_planes;
   P.b_planes = g.b_planes;
   P.nK = g.Kp / GK;
+  P.todo = g.todo;
   int dev = 0, nsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -618,36 +650,36 @@ ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
 
 template <typename C>
 static cudaError_t pack_rows(const C* X, int rows, int n, size_t ld, int Kp, int beta, int* scale, uint16_t* planes,
-                             cudaStream_t s) {
-  k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale);
+                             const int* todo, cudaStream_t s) {
+  k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale, todo);
   const int64_t units = (int64_t)rows * (Kp / 64);
-  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, (uint32_t*)planes);
+  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, (uint32_t*)planes, todo);
   return cudaGetLastError();
 }
 cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, s);
+                                 uint16_t* planes, cudaStream_t s, const int* todo) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, todo, s);
 }
 cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, s);
+                                 uint16_t* planes, cudaStream_t s, const int* todo) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, todo, s);
 }
 size_t mod_cols_ws_bytes(int n, int rows) {
   return al256(sizeof(uint32_t) * rows) + sizeof(double) * ((n + ST_ROWS - 1) / ST_ROWS) * (size_t)rows;
 }
-cudaError_t launch_mod_pack_cols_conj(const double2* X, int n, int rows, int Kp, int* scale, uint16_t* planes,
-                                      void* ws, cudaStream_t s) {
+cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, uint16_t* planes,
+                                 void* ws, cudaStream_t s, const int* todo) {
   uint32_t* eg = reinterpret_cast<uint32_t*>(ws);
   double* part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(ws) + al256(sizeof(uint32_t) * rows));
   cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * rows, s);
   if (e != cudaSuccess) return e;
   const int n_part = (n + ST_ROWS - 1) / ST_ROWS;
   const dim3 gst((rows + ST_COLS - 1) / ST_COLS, n_part);
-  k_mod_rowmax<<<gst, 256, 0, s>>>(X, rows, n, eg);
-  k_mod_norms<<<gst, 256, 0, s>>>(X, rows, n, nullptr, 0, eg, nullptr, part);
+  k_mod_rowmax<<<gst, 256, 0, s>>>(X, rows, n, eg, todo);
+  k_mod_col_norms<<<gst, 256, 0, s>>>(X, rows, n, eg, part, todo);
   k_mod_scales<<<dim3((rows + 255) / 256, 1), 256, 0, s>>>(part, n_part, rows, 0, eg, nullptr, scale);
-  k_mod_pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale,
-                                                                     (uint32_t*)planes, nullptr);
+  k_mod_pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale, conj,
+                                                                     (uint32_t*)planes, nullptr, todo);
   return cudaGetLastError();
 }
 
@@ -675,16 +707,16 @@ cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_
   const int n_part = (int)((K + ST_ROWS - 1) / ST_ROWS);
   const dim3 gst((nG + ST_COLS - 1) / ST_COLS, n_part);
   k_mod_fmax<<<nf, 256, 0, s>>>(f, K, ef);
-  k_mod_rowmax<<<gst, 256, 0, s>>>(M, nG, K, eg);
+  k_mod_rowmax<<<gst, 256, 0, s>>>(M, nG, K, eg, nullptr);
   k_mod_norms<<<gst, 256, 0, s>>>(M, nG, K, f, nf, eg, ef, part);
   k_mod_scales<<<dim3((nG + 255) / 256, nf + 1), 256, 0, s>>>(part, n_part, nG, nf, eg, ef, scale);
   for (int w0 = 0; w0 < nf; w0 += z.nw) {
     const int nw = std::min(z.nw, nf - w0);
-    k_mod_pack<<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(M, nG, K, Kp, f, w0, nw, scale,
-                                                                     w0 == 0 ? (uint32_t*)Bp : nullptr, (uint32_t*)Ap);
+    k_mod_pack<<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(
+        M, nG, K, Kp, f, w0, nw, scale, true, w0 == 0 ? (uint32_t*)Bp : nullptr, (uint32_t*)Ap, nullptr);
     for (int r0 = 0; r0 < nG; r0 += z.rows) {
       const int rows = std::min(z.rows, nG - r0);
-      ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, NPL * nw, NPL * nw, NPL};
+      ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, NPL * nw, NPL * nw, NPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
       k_mod_add<<<dim3((z.ldR / 8 + 3) / 4, (rows + 15) / 16, nw), 128, 0, s>>>(R, rows, r0, nG, z.ldR, scale, w0, chi);

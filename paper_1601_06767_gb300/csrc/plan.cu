@@ -528,17 +528,28 @@ chi0_status chi0_epsilon_inverse(chi0_plan p, int iq, void* eps, void* stream) {
   if (iq < 0 || iq >= (int)p->q.size()) return fail(p, CHI0_ERR_INVALID, "iq out of range");
   if (!eps) return fail(p, CHI0_ERR_INVALID, "NULL buffer");
   const int nG = p->q[iq].nG;
-  const size_t need = chi0::eps_inverse_ws_bytes(p, nG);
-  if (need > p->inv_bytes) {
+  // with the memory of the refinement where that can be had, else without
+  bool refined = chi0::eps_inverse_refines(p, nG);
+  for (;;) {
+    const size_t need = chi0::eps_inverse_ws_bytes(p, nG, refined);
+    if (need <= p->inv_bytes) break;
     CK(p, cudaStreamSynchronize((cudaStream_t)stream));
     cudaFree(p->d_inv);
     p->d_inv = nullptr;
+    p->ws_bytes -= p->inv_bytes;
     p->inv_bytes = 0;
-    CK(p, cudaMalloc(&p->d_inv, need));
-    p->inv_bytes = need;
-    p->ws_bytes += need;
+    const cudaError_t e = cudaMalloc(&p->d_inv, need);
+    if (e == cudaSuccess) {
+      p->inv_bytes = need;
+      p->ws_bytes += need;
+      break;
+    }
+    cudaGetLastError();
+    p->d_inv = nullptr;
+    if (!refined) CK(p, e);
+    refined = false;
   }
-  CK(p, chi0::launch_epsilon_inverse(p, nG, (double2*)eps, p->d_inv, (cudaStream_t)stream));
+  CK(p, chi0::launch_epsilon_inverse(p, nG, (double2*)eps, p->d_inv, refined, (cudaStream_t)stream));
   return CHI0_OK;
 }
 
