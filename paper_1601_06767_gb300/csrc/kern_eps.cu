@@ -89,10 +89,11 @@ template <typename R> struct SelRows { static constexpr int V = sizeof(R) == 4 ?
 // merge levels: block c holds entries c*ROWS ... of the previous level's list
 // (NB slots per set, -1 = empty).  Writes NB slots per block to cand_out.
 //
-// Rows are not moved, each has a position instead (ties go to the lowest one).  Three
-// barriers per column and several threads per row; latency bound (33 us a level of
-// 128 FP32 rows with one thread per row, moved rows and four barriers; 61 us with
-// the rows in registers, whose straight-line code missed the instruction cache).
+// Rows are not moved, each has a position instead (ties go to the lowest one).  Two
+// barriers per column (FP64: three) and several threads per row; latency bound (33
+// us a level of 128 FP32 rows with one thread per row, moved rows and four barriers;
+// 61 us with the rows in registers, whose straight-line code missed the
+// instruction cache).
 constexpr int SEL_THREADS = 256;
 template <typename R>
 __global__ void __launch_bounds__(SEL_THREADS)
@@ -105,9 +106,8 @@ k_tp_select(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, cons
   const C* a = A + (size_t)w * N * N;
   __shared__ C S[ROWS][NB + 2];
   __shared__ int idx[ROWS], win[NB], wcnt[ROWS / 32];
-  __shared__ unsigned long long w_key[2][NW];
-  __shared__ unsigned w_min[2][NW];
-  __shared__ C s_inv;                              // reciprocal of the pivot, by one thread
+  __shared__ ulonglong2 w_best[2][NW];             // a warp's largest key and the complement of its position
+  __shared__ C s_inv[ROWS];                        // reciprocals of the candidates
   // valid rows to the front, keeping their order (deterministic ties)
   int g = -1;
   if (tid < ROWS) {
@@ -126,9 +126,10 @@ k_tp_select(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, cons
   }
   if (g >= 0) idx[at] = g;
   __syncthreads();
-  for (int e = tid; e < nr * NB; e += SEL_THREADS) {
-    const int r = e / NB, t = e - r * NB;
-    S[r][t] = t < kb ? a[(size_t)idx[r] * N + k0 + t] : cz(C{});
+#pragma unroll
+  for (int q = 0; q < ROWS * NB / SEL_THREADS; ++q) {   // all loads in flight
+    const int e = tid + q * SEL_THREADS, r = e / NB, t = e - r * NB;
+    if (r < nr) S[r][t] = t < kb ? a[(size_t)idx[r] * N + k0 + t] : cz(C{});
   }
   __syncthreads();
   const int row = tid / TPR, sub = tid - row * TPR, steps = min(kb, nr);
@@ -138,44 +139,49 @@ k_tp_select(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, cons
     // largest |re| + |im| among positions >= j, ties to the lowest position: the value's bits order
     // non-negative numbers; 0 marks a row that is no candidate
     unsigned long long key = 0;
-    if (pos >= j && pos < nr) {
-      if constexpr (sizeof(R) == 4) key = (unsigned long long)__float_as_uint(cabs1(S[row][j])) + 1;
-      else key = (unsigned long long)__double_as_longlong(cabs1(S[row][j])) + 1;
+    const bool cand = pos >= j && pos < nr;
+    if (cand) {
+      const C d = S[row][j];
+      if constexpr (sizeof(R) == 4) key = (unsigned long long)__float_as_uint(cabs1(d)) + 1;
+      else key = (unsigned long long)__double_as_longlong(cabs1(d)) + 1;
+      // FP32: every candidate's reciprocal, beside the search (FP64: the pivot's alone, by one thread, after it)
+      if (sizeof(R) == 4 && sub == 0) s_inv[row] = crecip(d);
     }
     unsigned long long best = key;
     if constexpr (sizeof(R) == 4) best = __reduce_max_sync(0xffffffffu, (unsigned)key);
     else
       for (int o = 16; o; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
     const unsigned mp = __reduce_min_sync(0xffffffffu, (key == best && key) ? (unsigned)(pos << 8 | row) : 0xffffffffu);
-    if ((tid & 31) == 0) {
-      w_key[b][warp] = best;
-      w_min[b][warp] = mp;
-    }
+    if ((tid & 31) == 0) w_best[b][warp] = make_ulonglong2(best, ~mp);
     __syncthreads();
-    best = w_key[b][0];
-    unsigned pm = w_min[b][0];
-#pragma unroll
-    for (int q = 1; q < NW; ++q) {
-      const unsigned long long k2 = w_key[b][q];
-      const unsigned p2 = w_min[b][q];
-      if (k2 > best || (k2 == best && p2 < pm)) { best = k2; pm = p2; }
+    // the warps' answers, one per lane
+    ulonglong2 top = w_best[b][tid & (NW - 1)];
+    if constexpr (sizeof(R) == 4) {
+      const unsigned k = (unsigned)top.x, m = __reduce_max_sync(0xffffffffu, k);
+      top.y = __reduce_max_sync(0xffffffffu, k == m ? (unsigned)top.y : 0u);
+    } else {
+      for (int o = NW / 2; o; o >>= 1) {
+        const unsigned long long ox = __shfl_xor_sync(0xffffffffu, top.x, o), oy = __shfl_xor_sync(0xffffffffu, top.y, o);
+        if (ox > top.x || (ox == top.x && oy > top.y)) top = make_ulonglong2(ox, oy);
+      }
     }
     // the pivot row goes to position j, the row there to the pivot's
+    const unsigned pm = ~(unsigned)top.y;
     const int p = (int)(pm >> 8), pr = (int)(pm & 255u);
     if (row == pr) {
       if (sub == 0) {
         win[j] = idx[row];
-        s_inv = crecip(S[row][j]);
+        if (sizeof(R) == 8) s_inv[row] = crecip(S[row][j]);
       }
       pos = j;
     } else if (pos == j) {
       pos = p;
     }
-    __syncthreads();
+    if (sizeof(R) == 8) __syncthreads();
     if (pos > j && pos < nr) {
       const C piv = S[pr][j];
       if (piv.x != (R)0 || piv.y != (R)0) {
-        const C l = cmul(S[row][j], s_inv);
+        const C l = cmul(S[row][j], s_inv[pr]);
 #pragma unroll 4
         for (int t = j + 1 + sub; t < kb; t += TPR) S[row][t] = csub(S[row][t], cmul(l, S[pr][t]));
       }
@@ -186,17 +192,20 @@ k_tp_select(const typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, cons
 }
 
 // Move the winners to rows k0..k0+kb-1 of the panel (recorded as a swap sequence in
-// piv) and invert the pivot block by Gauss-Jordan with partial pivoting in shared
+// piv, and for k_gj_rows as the moves themselves: mv[t] = the row that comes to k0 + t,
+// mv[NB + t] = where row k0 + t goes to, -1 = within the pivot rows) and invert the pivot block by Gauss-Jordan with partial pivoting in shared
 // memory: T = A11^-1 (also written over the pivot block).  One CTA per matrix,
-// latency bound: four barriers per column, the moved rows (64 at most) read and
-// written once each, the copy of the panel left to k_copy_panel (91 us with a
-// barrier and two memory round trips per swap, six barriers per column and the
-// copy by this one CTA, 2500^2 FP32).
+// latency bound: three barriers per column, the reciprocals taken beside the pivot
+// search, the moved rows (64 at most) read and written once each, the copy of the
+// panel left to k_copy_panel (2500^2 FP32: 91 us with a barrier and two memory
+// round trips per swap, six barriers of 1024 threads per column and the copy by
+// this one CTA; 33 us with four barriers of 1024 threads).
+constexpr int FIN_THREADS = 256;
 template <typename R>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(FIN_THREADS)
 k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* __restrict__ win, int ld,
-           typename Cx<R>::T* __restrict__ Tb, int* __restrict__ piv, int* __restrict__ status,
-           const int* __restrict__ skip) {
+           typename Cx<R>::T* __restrict__ Tb, int* __restrict__ piv, int* __restrict__ moves,
+           int* __restrict__ status, const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
   const int w = blockIdx.x, tid = threadIdx.x;
   if (skip && skip[w] == 0) return;
@@ -205,6 +214,7 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
   __shared__ int orig[2 * NB], cur[2 * NB], s_n;
   __shared__ C B[NB][2 * NB + 1];
   __shared__ int s_p;
+  __shared__ C s_inv;
   if (tid < 32) {
     // swap sequence: step t exchanges row k0+t with the current row of winner t; (orig, cur) lists the
     // rows moved so far and where each is now, two entries per lane
@@ -253,15 +263,26 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
   }
   __syncthreads();
   {
-    // all moves at once: row orig[q] to cur[q], 32 columns each (two entries per thread)
-    const int q = tid >> 5, t = tid & 31;
-    C u = cz(C{}), v = cz(C{});
-    const bool m0 = q < s_n && t < kb, m1 = q + 32 < s_n && t < kb;
-    if (m0) u = a[(size_t)orig[q] * N + k0 + t];
-    if (m1) v = a[(size_t)orig[q + 32] * N + k0 + t];
+    // all moves at once: row orig[q] to cur[q], 32 columns each
+    C u[2 * NB * 32 / FIN_THREADS];
+    int* mv = moves + (size_t)w * 2 * NB;
+    if (tid < 2 * NB) mv[tid] = tid < NB ? k0 + tid : -1;
+#pragma unroll
+    for (int x = 0; x < 2 * NB * 32 / FIN_THREADS; ++x) {
+      const int q = (tid >> 5) + x * (FIN_THREADS / 32), t = tid & 31;
+      u[x] = q < s_n && t < kb ? a[(size_t)orig[q] * N + k0 + t] : cz(C{});
+    }
     __syncthreads();
-    if (m0) a[(size_t)cur[q] * N + k0 + t] = u;
-    if (m1) a[(size_t)cur[q + 32] * N + k0 + t] = v;
+#pragma unroll
+    for (int x = 0; x < 2 * NB * 32 / FIN_THREADS; ++x) {
+      const int q = (tid >> 5) + x * (FIN_THREADS / 32), t = tid & 31;
+      if (q < s_n && t < kb) a[(size_t)cur[q] * N + k0 + t] = u[x];
+    }
+    if (tid < s_n) {
+      const int o = orig[tid] - k0, c = cur[tid] - k0;
+      if (c < kb) mv[c] = orig[tid];
+      else if (o < kb) mv[NB + o] = cur[tid];
+    }
   }
   __syncthreads();
   // [A11 | I] -> [I | A11^-1]
@@ -275,39 +296,46 @@ k_tp_final(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const int* 
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
     if (tid < 32) {
-      R best = (tid >= j && tid < kb) ? cabs1(B[tid][j]) : (R)-1;
-      int bi = (tid >= j && tid < kb) ? tid : NB;
-      for (int o = 16; o; o >>= 1) {
-        const R ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      if (tid == 0) {
-        if (!(best > (R)0) || bi >= kb) {
-          if (status) atomicOr(status, SINGULAR_BIT);
-          bi = j;
+      const bool in = tid >= j && tid < kb;
+      const C d = in ? B[tid][j] : cz(C{});
+      const C inv = crecip(d);                     // of every candidate, beside the search
+      int bi;
+      bool none;                                   // no candidate above zero (or not a number)
+      if constexpr (sizeof(R) == 4) {
+        const unsigned key = in ? __float_as_uint(cabs1(d)) + 1u : 0u, m = __reduce_max_sync(0xffffffffu, key);
+        bi = __ffs(__ballot_sync(0xffffffffu, key == m)) - 1;
+        none = m <= 1u || m > 0x7f800001u;
+      } else {
+        R best = in ? cabs1(d) : (R)-1;
+        bi = in ? tid : NB;
+        for (int o = 16; o; o >>= 1) {
+          const R ob = __shfl_xor_sync(0xffffffffu, best, o);
+          const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+          if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
         }
+        none = __shfl_sync(0xffffffffu, !(best > (R)0) || bi >= kb, 0);
+        bi = __shfl_sync(0xffffffffu, bi, 0);
+      }
+      if (none) bi = j;
+      if (tid == 0) {
+        if (none && status) atomicOr(status, SINGULAR_BIT);
         s_p = bi;
       }
+      if (tid == bi) s_inv = inv;
     }
     __syncthreads();
     const int p = s_p;
-    C u = cz(C{}), v = cz(C{}), d = cz(C{});
-    if (tid < 2 * NB) {
-      u = B[j][tid];
-      v = B[p][tid];
-      d = B[p][j];
-    }
-    __syncthreads();
-    if (tid < 2 * NB) {
+    if (tid < 2 * NB) {                            // a thread per column: swap rows j and p, scale row j
+      const C u = B[j][tid], v = B[p][tid];
       if (p != j) B[p][tid] = u;
-      B[j][tid] = cmul(v, crecip(d));
+      B[j][tid] = cmul(v, s_inv);
     }
     __syncthreads();
     // eliminate column j from every other row: thread (i, c); columns up to j of the left half are
     // not read again
-    for (int e = tid; e < NB * 2 * NB; e += blockDim.x) {
-      const int i = e / (2 * NB), c = e - i * 2 * NB;
+#pragma unroll
+    for (int x = 0; x < NB * 2 * NB / FIN_THREADS; ++x) {
+      const int e = tid + x * FIN_THREADS, i = e / (2 * NB), c = e - i * 2 * NB;
       if (i != j && i < kb && c > j) B[i][c] = csub(B[i][c], cmul(B[i][j], B[j][c]));
     }
     __syncthreads();
@@ -333,40 +361,59 @@ __global__ void __launch_bounds__(256) k_copy_panel(const typename Cx<R>::T* __r
 // ---------------------------------------------------------------------------
 // 2. row swaps outside the panel, pivot rows := T A10
 // ---------------------------------------------------------------------------
+// A CTA takes 32 columns: the pivot rows and the rows that come to them are read at
+// once, the moved pivot rows written out, and four threads per column form eight
+// rows of the product each (38 panels of 1200^2 FP32: 443 us with a thread per
+// column doing one swap after another).
+constexpr int GR_COLS = 32;
 template <typename R>
 __global__ void __launch_bounds__(128)
 k_gj_rows(typename Cx<R>::T* __restrict__ A, int N, int k0, int kb, const typename Cx<R>::T* __restrict__ Tb,
-          const int* __restrict__ piv, const int* __restrict__ skip) {
+          const int* __restrict__ moves, const int* __restrict__ skip) {
   using C = typename Cx<R>::T;
   const int w = blockIdx.y;
   if (skip && skip[w] == 0) return;
   C* a = A + (size_t)w * N * N;
-  const int* pv = piv + (size_t)w * N;
+  const int* mv = moves + (size_t)w * 2 * NB;
   __shared__ C ts[NB][NB];
+  __shared__ C xs[NB][GR_COLS + 1];
+  const int c = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int j = blockIdx.x * GR_COLS + c;
+  const bool in = j < N && !(j >= k0 && j < k0 + kb);
   // entries outside the kb x kb block are never written by the panel kernel: use zeros
-  for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-    const int r = e / NB, c = e - r * NB;
-    ts[r][c] = (r < kb && c < kb) ? Tb[(size_t)w * NB * NB + e] : cz(C{});
+  for (int e = threadIdx.x; e < NB * NB; e += 128) {
+    const int r = e / NB, t = e - r * NB;
+    ts[r][t] = (r < kb && t < kb) ? Tb[(size_t)w * NB * NB + e] : cz(C{});
   }
-  __syncthreads();
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= N || (j >= k0 && j < k0 + kb)) return;
-  for (int t = 0; t < kb; ++t) {
-    const int p = pv[k0 + t];
-    if (p != k0 + t) {
-      const C u = a[(size_t)(k0 + t) * N + j];
-      a[(size_t)(k0 + t) * N + j] = a[(size_t)p * N + j];
-      a[(size_t)p * N + j] = u;
+  C old[NB / 4], nw[NB / 4];
+#pragma unroll
+  for (int q = 0; q < NB / 4; ++q) {
+    const int t = g + 4 * q;
+    old[q] = nw[q] = cz(C{});
+    if (in && t < kb) {
+      old[q] = a[(size_t)(k0 + t) * N + j];
+      nw[q] = a[(size_t)mv[t] * N + j];
     }
   }
-  C x[NB];
 #pragma unroll
-  for (int t = 0; t < NB; ++t) x[t] = t < kb ? a[(size_t)(k0 + t) * N + j] : cz(C{});
-#pragma unroll 4
-  for (int i = 0; i < kb; ++i) {
+  for (int q = 0; q < NB / 4; ++q) xs[g + 4 * q][c] = nw[q];
+  __syncthreads();                                 // every row that moves has been read
+#pragma unroll
+  for (int q = 0; q < NB / 4; ++q) {
+    const int t = g + 4 * q;
+    if (in && t < kb) {
+      const int d = mv[NB + t];
+      if (d >= 0) a[(size_t)d * N + j] = old[q];
+    }
+  }
+  if (!in) return;
+#pragma unroll 2
+  for (int q = 0; q < NB / 4; ++q) {
+    const int i = g + 4 * q;
+    if (i >= kb) break;
     C s = cz(C{});
 #pragma unroll
-    for (int t = 0; t < NB; ++t) cfma(s, ts[i][t], x[t]);
+    for (int t = 0; t < NB; ++t) cfma(s, ts[i][t], xs[t][c]);
     a[(size_t)(k0 + i) * N + j] = s;
   }
 }
@@ -584,7 +631,7 @@ template <typename R> int64_t tp_ld(int N) { return (int64_t)((N + SelRows<R>::V
 // pivot search and pivot block of panel k0: Z (copy of its columns), T, piv
 template <typename R>
 void gj_panel(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, int k0, void* Z, void* Tb, int* piv, int* cand,
-              int* status, const int* skip, cudaStream_t s) {
+              int* moves, int* status, const int* skip, cudaStream_t s) {
   using C = typename Cx<R>::T;
   constexpr int ROWS = SelRows<R>::V;
   const int ld = (int)tp_ld<R>(N), kb = min(NB, N - k0);
@@ -600,7 +647,7 @@ void gj_panel(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, int k0, void*
     k_tp_select<R><<<dim3(nblk, nf), SEL_THREADS, 0, s>>>(A, N, k0, kb, cbuf[cur], n_in, cbuf[cur ^ 1], ld, skip);
     cur ^= 1;
   }
-  k_tp_final<R><<<nf, 1024, 0, s>>>(A, N, k0, kb, cbuf[cur], ld, (C*)Tb, piv, status, skip);
+  k_tp_final<R><<<nf, FIN_THREADS, 0, s>>>(A, N, k0, kb, cbuf[cur], ld, (C*)Tb, piv, moves, status, skip);
   k_copy_panel<R><<<dim3((N * NB + 255) / 256, nf), 256, 0, s>>>(A, N, k0, kb, (C*)Z, skip);
 }
 
@@ -645,25 +692,26 @@ cudaError_t gj_invert(chi0_plan_s* p, typename Cx<R>::T* A, int N, int nf, void*
   using C = typename Cx<R>::T;
   C* Zb[2] = {(C*)Z, (C*)Z + (size_t)nf * N * NB};
   C* Tbb[2] = {(C*)Tb, (C*)Tb + (size_t)nf * NB * NB};
+  int* mvb[2] = {cand + (size_t)2 * nf * tp_ld<R>(N), cand + (size_t)2 * nf * tp_ld<R>(N) + (size_t)nf * 2 * NB};
   const bool look = !skip && inv_streams(p, s);
   cudaError_t e = cudaSuccess;
-  gj_panel<R>(p, A, N, nf, 0, Zb[0], Tbb[0], piv, cand, status, skip, s);
+  gj_panel<R>(p, A, N, nf, 0, Zb[0], Tbb[0], piv, cand, mvb[0], status, skip, s);
   for (int k0 = 0, b = 0; k0 < N && e == cudaSuccess; k0 += NB, b ^= 1) {
     const int kb = min(NB, N - k0), n0 = k0 + NB, n1 = min(N, n0 + NB);
     {
       ProfScope ps(p, CHI0_K_INV_PANEL, s, 1);
-      k_gj_rows<R><<<dim3((N + 127) / 128, nf), 128, 0, s>>>(A, N, k0, kb, Tbb[b], piv, skip);
+      k_gj_rows<R><<<dim3((N + GR_COLS - 1) / GR_COLS, nf), 128, 0, s>>>(A, N, k0, kb, Tbb[b], mvb[b], skip);
     }
     if (n0 >= N) {
       e = gj_update<R>(p, A, N, nf, k0, 0, N, 0, 0, Zb[b], skip, s);
     } else if (!look) {
       e = gj_update<R>(p, A, N, nf, k0, 0, N, 0, 0, Zb[b], skip, s);
-      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, status, skip, s);
+      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, mvb[b ^ 1], status, skip, s);
     } else {
       e = gj_update<R>(p, A, N, nf, k0, n0, n1, 0, 0, Zb[b], skip, s);
       if (e == cudaSuccess) e = cudaEventRecord(p->inv_ev[0], s);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(p->inv_side, p->inv_ev[0], 0);
-      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, status, skip, p->inv_side);
+      if (e == cudaSuccess) gj_panel<R>(p, A, N, nf, n0, Zb[b ^ 1], Tbb[b ^ 1], piv, cand, mvb[b ^ 1], status, skip, p->inv_side);
       // joined whatever happens
       cudaEventRecord(p->inv_ev[1], p->inv_side);
       if (e == cudaSuccess) e = gj_update<R>(p, A, N, nf, k0, 0, N, n0, n1, Zb[b], skip, s);
@@ -847,14 +895,14 @@ constexpr int REF_MIN_N = 64;
 bool eps_inverse_refines(const chi0_plan_s* p, int nG) { return !is_split(p) && nG >= REF_MIN_N && mod_gemm_usable(); }
 
 // Workspace (bytes): complex64 copy of the matrices (split plans), Z [2][nf][N][NB], T [2][nf][NB][NB],
-// piv [nf][N], two candidate lists [nf][tp_ld].
+// piv [nf][N], two candidate lists [nf][tp_ld], two lists of row moves [nf][2 NB].
 size_t eps_inverse_ws_bytes(const chi0_plan_s* p, int nG, bool refined) {
   const size_t nf = (size_t)p->n_freq, c = is_split(p) ? sizeof(float2) : sizeof(double2);
   const size_t copy = is_split(p) ? nf * nG * nG * sizeof(float2) : 0;
   const size_t ld = (size_t)(is_split(p) ? tp_ld<float>(nG) : tp_ld<double>(nG));
   auto al = [](size_t x) { return (x + 255) / 256 * 256; };
   return al(copy) + al(2 * nf * nG * NB * c) + al(2 * nf * NB * NB * c) + al(nf * nG * sizeof(int)) +
-         al(2 * nf * ld * sizeof(int)) + (refined ? ref_sizes(nG, (int)nf).bytes : 0);
+         al((2 * nf * ld + 4 * NB * nf) * sizeof(int)) + (refined ? ref_sizes(nG, (int)nf).bytes : 0);
 }
 
 cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* ws, bool refined, cudaStream_t s) {
@@ -889,7 +937,7 @@ cudaError_t launch_epsilon_inverse(chi0_plan_s* p, int nG, double2* eps, void* w
   int* piv = reinterpret_cast<int*>(b);
   b += al(nf * nG * sizeof(int));
   int* cand = reinterpret_cast<int*>(b);
-  b += al(2 * nf * tp_ld<double>(nG) * sizeof(int));
+  b += al((2 * nf * tp_ld<double>(nG) + 4 * NB * nf) * sizeof(int));
   if (refined) return refined_inverse(p, eps, nG, (int)nf, Z, Tb, piv, cand, b, s);
   return gj_invert<double>(p, eps, nG, (int)nf, Z, Tb, piv, cand, p->d_status, nullptr, s);
 }
