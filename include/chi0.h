@@ -417,8 +417,8 @@ chi0_status chi0_gpp(chi0_plan plan, int iq, const void* psi_v, int n_v, const v
  * as the second; x: (device) [n_t][n_b] FP64, E_t - E_b (E_b the grid energy for an energy-grid
  * state); w: (device) [n_b] FP64 or NULL (= 1); Omega2, wt from chi0_gpp; v: (device) [N_G] FP64;
  * sigma: (host) [n_t] complex128.  Split plans compute the terms in FP32 and sum them in FP64,
- * FP64 plans in FP64; the tile sums are added on the host in a fixed order.  Allocates a
- * workspace (two N_G x N_G tables) and synchronises `stream`. */
+ * FP64 plans in FP64; the tile sums are added on the host in a fixed order.  Keeps a
+ * workspace (two N_G x N_G tables) in the plan from the first call on and synchronises `stream`. */
 chi0_status chi0_sigma_coh(chi0_plan plan, int iq, const void* m, int n_t, int n_b, const double* x,
                            const double* w, const void* Omega2, const void* wt, const double* v,
                            double* sigma, void* stream);

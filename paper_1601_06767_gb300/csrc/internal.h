@@ -102,8 +102,8 @@ struct chi0_plan_s {
   size_t wfn_ws_bytes = 0;
   void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
   // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
-  // fixed-point pair stage
-  LazyWs ws_mod, ws_bwd, ws_fx;
+  // fixed-point pair stage, COH
+  LazyWs ws_mod, ws_bwd, ws_fx, ws_coh;
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)

@@ -167,9 +167,11 @@ k_sigma_coh(const typename Cx<R>::T* __restrict__ m, int n_b, int nG, const doub
   constexpr int CB = CohBands<R>::V;
   const int t = blockIdx.z;
   const int i0 = blockIdx.y * CT, j0 = blockIdx.x * CT;
+  constexpr bool F32 = sizeof(R) == 4;
   __shared__ C cs[CT][CT + 1], ws[CT][CT + 1];
   __shared__ C mi[CB][CT + 1], mj[CB][CT + 1];
-  __shared__ R xs[CB];
+  __shared__ R xs[CB], wgts[CB];
+  __shared__ R s_xmax;
   __shared__ double2 red[8];
   for (int e = threadIdx.x; e < CT * CT; e += blockDim.x) {
     const int a = e / CT, b = e - a * CT;
@@ -182,21 +184,34 @@ k_sigma_coh(const typename Cx<R>::T* __restrict__ m, int n_b, int nG, const doub
   const C* mt = m + (size_t)t * n_b * nG;
   for (int b0 = 0; b0 < n_b; b0 += CB) {
     __syncthreads();
-    for (int e = threadIdx.x; e < CB * CT; e += blockDim.x) {
-      const int bb = e / CT, g = e - bb * CT;
-      const int b = b0 + bb;
-      const bool okb = b < n_b;
-      // the band weight rides on the G side: w_b m(G)
-      const R wgt = okb ? (R)(wb ? wb[b] : 1.0) : (R)0;
-      C u = (okb && i0 + g < nG) ? mt[(size_t)b * nG + i0 + g] : cz(C{});
-      u.x *= wgt;
-      u.y *= wgt;
-      mi[bb][g] = u;
-      mj[bb][g] = (okb && j0 + g < nG) ? mt[(size_t)b * nG + j0 + g] : cz(C{});
-    }
     if (threadIdx.x < CB) {
       const int b = b0 + threadIdx.x;
-      xs[threadIdx.x] = b < n_b ? (R)x[(size_t)t * n_b + b] : (R)0;
+      const R xv = b < n_b ? (R)x[(size_t)t * n_b + b] : (R)0;
+      xs[threadIdx.x] = xv;
+      wgts[threadIdx.x] = b < n_b ? (R)(wb ? wb[b] : 1.0) : (R)0;
+      if constexpr (F32) {
+        const unsigned big = __reduce_max_sync(0xffffffffu, __float_as_uint(xv) & 0x7fffffffu);   // CB = 32: one warp
+        if (threadIdx.x == 0) s_xmax = __uint_as_float(big);
+      }
+    }
+    C ui[CB * CT / 256], uj[CB * CT / 256];
+#pragma unroll
+    for (int k = 0; k < CB * CT / 256; ++k) {
+      const int e = threadIdx.x + 256 * k, bb = e / CT, g = e - bb * CT, b = b0 + bb;
+      const bool okb = b < n_b;
+      ui[k] = (okb && i0 + g < nG) ? mt[(size_t)b * nG + i0 + g] : cz(C{});
+      uj[k] = (okb && j0 + g < nG) ? mt[(size_t)b * nG + j0 + g] : cz(C{});
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < CB * CT / 256; ++k) {
+      const int e = threadIdx.x + 256 * k, bb = e / CT, g = e - bb * CT;
+      // the band weight rides on the G side: w_b m(G)
+      C u = ui[k];
+      u.x *= wgts[bb];
+      u.y *= wgts[bb];
+      mi[bb][g] = u;
+      mj[bb][g] = uj[k];
     }
     __syncthreads();
     // the thread's four elements share the column G' (rows a = tid/32 + 8q): m(G') and x are
@@ -211,26 +226,64 @@ k_sigma_coh(const typename Cx<R>::T* __restrict__ m, int n_b, int nG, const doub
       wv[q] = ws[a0 + 8 * q][bcol];
       dy[q] = (R)delta - wv[q].y;
     }
-#pragma unroll 2
-    for (int bb = 0; bb < CB; ++bb) {
-      const C mjv = mj[bb][bcol];
-      const R xb = xs[bb];
+    // FP32: |d|^2 of every term lies well inside the normal range (from the largest |x| of the chunk and
+    // dy): the bare reciprocal then has the bits of the division's, which also scales subnormal and huge
+    // divisors.  4 targets, 663 bands, N_G 2500:
+    // 12.0 -> 9.9 ms.  (Two rows per packed f32x2 instruction ran slower: 11.6 ms.)
+    bool plain = F32;
+    if constexpr (F32) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        // c / (x - wt + i delta) = c conj(d) / |d|^2,  d = dx + i dy (c = 0: no pole, adds 0)
-        const R dx = xb - wv[q].x;
-        R inv;
-        if constexpr (sizeof(R) == 4)
-          inv = __fdividef(1.0f, dx * dx + dy[q] * dy[q]);   // 2-ulp reciprocal: terms carry FP32 errors anyway
-        else
-          inv = (R)1 / (dx * dx + dy[q] * dy[q]);
-        C cr;                                                 // c conj(d)
-        cr.x = fma(cc[q].x, dx, cc[q].y * dy[q]);
-        cr.y = fma(cc[q].y, dx, -(cc[q].x * dy[q]));
-        const C mm = cconjmul(mjv, mi[bb][a0 + 8 * q]);       // w_b m(G) conj(m(G'))
-        const C t2 = cmul(mm, cr);
-        part.x = fma(t2.x, inv, part.x);
-        part.y = fma(t2.y, inv, part.y);
+      for (int q = 0; q < 4; ++q)
+        plain = plain && s_xmax + fabsf(wv[q].x) < 4.6e18f && fabsf(dy[q]) > 1e-15f && fabsf(dy[q]) < 4.6e18f;
+      plain = __all_sync(0xffffffffu, plain);
+    }
+    if (plain) {
+      if constexpr (F32) {
+        float dy2[4], k1[4], k2[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          dy2[q] = dy[q] * dy[q];
+          k1[q] = cc[q].y * dy[q];
+          k2[q] = -(cc[q].x * dy[q]);
+        }
+#pragma unroll 4
+        for (int bb = 0; bb < CB; ++bb) {
+          const float2 mjv = mj[bb][bcol];
+          const float xb = xs[bb];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float dx = xb - wv[q].x;
+            float inv;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(fmaf(dx, dx, dy2[q])));
+            const float2 cr = make_float2(fmaf(cc[q].x, dx, k1[q]), fmaf(cc[q].y, dx, k2[q]));
+            const float2 t2 = cmul(cconjmul(mjv, mi[bb][a0 + 8 * q]), cr);
+            part.x = fmaf(t2.x, inv, part.x);
+            part.y = fmaf(t2.y, inv, part.y);
+          }
+        }
+      }
+    } else {
+#pragma unroll 2
+      for (int bb = 0; bb < CB; ++bb) {
+        const C mjv = mj[bb][bcol];
+        const R xb = xs[bb];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          // c / (x - wt + i delta) = c conj(d) / |d|^2,  d = dx + i dy (c = 0: no pole, adds 0)
+          const R dx = xb - wv[q].x;
+          R inv;
+          if constexpr (F32)
+            inv = __fdividef(1.0f, dx * dx + dy[q] * dy[q]);   // 2-ulp reciprocal: terms carry FP32 errors anyway
+          else
+            inv = (R)1 / (dx * dx + dy[q] * dy[q]);
+          C cr;                                                 // c conj(d)
+          cr.x = fma(cc[q].x, dx, cc[q].y * dy[q]);
+          cr.y = fma(cc[q].y, dx, -(cc[q].x * dy[q]));
+          const C mm = cconjmul(mjv, mi[bb][a0 + 8 * q]);       // w_b m(G) conj(m(G'))
+          const C t2 = cmul(mm, cr);
+          part.x = fma(t2.x, inv, part.x);
+          part.y = fma(t2.y, inv, part.y);
+        }
       }
     }
     acc.x += (double)part.x;
