@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -21,16 +22,20 @@ __device__ __forceinline__ double2 cinv(double a, double b) {
 
 // f[w][k] = (w_p/2) [1/(dE_p - omega_w + i delta) + 1/(dE_p + omega_w + i delta)],
 // dE_p = E_v[p / n_c] - E_col[p % n_c], w_p = w_col[p % n_c] (or 1), p = p0 + k.
-__global__ void k_weights(int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
-                          const double* __restrict__ E_col, const double* __restrict__ w_col,
-                          const double2* __restrict__ omega, int n_freq, double delta, double2* __restrict__ f) {
+// One thread per pair and frequency: the divisions are a long FP64 chain, and few
+// pairs with many frequencies (512 x 32: 102 us with a thread per pair) would leave
+// most of the GPU idle.
+__global__ void __launch_bounds__(128) k_weights(int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
+                                                 const double* __restrict__ E_col, const double* __restrict__ w_col,
+                                                 const double2* __restrict__ omega, int n_freq, double delta,
+                                                 double2* __restrict__ f) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= K) return;
   const int64_t p = p0 + k;
   const int64_t iv = p / n_c, ic = p - iv * n_c;
   const double dE = E_v[iv] - E_col[ic];
   const double w = w_col ? w_col[ic] : 1.0;
-  for (int iw = 0; iw < n_freq; ++iw) {
+  for (int iw = blockIdx.y; iw < n_freq; iw += gridDim.y) {
     const double2 om = omega[iw];
     const double2 a = cinv(dE - om.x, delta - om.y);
     const double2 b = cinv(dE + om.x, delta + om.y);
@@ -107,9 +112,9 @@ k_contract_f64(int nG, const double2* __restrict__ M, int64_t K, const double2* 
 cudaError_t launch_weights(const chi0_plan_s* p, int64_t p0, int64_t K, int n_c, const double* E_v,
                            const double* E_col, const double* w_col, double2* f, cudaStream_t s) {
   if (K <= 0) return cudaSuccess;
-  const int bs = 256;
-  k_weights<<<(unsigned)((K + bs - 1) / bs), bs, 0, s>>>(p0, K, n_c, E_v, E_col, w_col, p->d_omega, p->n_freq,
-                                                         p->delta, f);
+  const int bs = 128;
+  k_weights<<<dim3((unsigned)((K + bs - 1) / bs), std::min(p->n_freq, 65535)), bs, 0, s>>>(
+      p0, K, n_c, E_v, E_col, w_col, p->d_omega, p->n_freq, p->delta, f);
   return cudaGetLastError();
 }
 

@@ -120,11 +120,8 @@ __device__ __forceinline__ float float_of_ord(unsigned int o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// largest |component| of the M block -> amax[0]; largest |Re f(w)| -> amax[1 + 2w],
-// largest |Im f(w)| -> amax[2 + 2w]; Hermitian mode: the smallest and largest
-// Im f / Re f over the block (order-mapped) -> tr[2w], tr[2w + 1]
-__global__ void k_absmax(const float2* __restrict__ M, int64_t n, const double2* __restrict__ f, int64_t K,
-                         int n_freq, unsigned int* __restrict__ amax, unsigned int* __restrict__ tr) {
+// largest |component| of the M block -> amax[0]
+__global__ void __launch_bounds__(256) k_absmax(const float2* __restrict__ M, int64_t n, unsigned int* __restrict__ amax) {
   float m = 0.f;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float2 v = M[i];
@@ -132,35 +129,37 @@ __global__ void k_absmax(const float2* __restrict__ M, int64_t n, const double2*
   }
   for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) atomicMax(amax, __float_as_uint(m));
-  for (int iw = 0; iw < n_freq; ++iw) {
-    float gr = 0.f, gi = 0.f;
+}
+
+// largest |Re f(w)| -> amax[1 + 2w], largest |Im f(w)| -> amax[2 + 2w]; Hermitian
+// mode: the smallest and largest Im f / Re f over the block (order-mapped) ->
+// tr[2w], tr[2w + 1].  A row of CTAs per frequency (frequency after frequency in
+// every CTA of k_absmax took most of its 103 us for 512 pairs and 32 frequencies).
+__global__ void __launch_bounds__(128) k_factor_range(const double2* __restrict__ f, int64_t K, int n_freq,
+                                                      unsigned int* __restrict__ amax, unsigned int* __restrict__ tr) {
+  for (int iw = blockIdx.y; iw < n_freq; iw += gridDim.y) {
+    float gr = 0.f, gi = 0.f, tlo = INFINITY, thi = -INFINITY;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += (int64_t)gridDim.x * blockDim.x) {
       const double2 v = f[(int64_t)iw * K + i];
       gr = fmaxf(gr, (float)fabs(v.x));
       gi = fmaxf(gi, (float)fabs(v.y));
-    }
-    for (int o = 16; o; o >>= 1) {
-      gr = fmaxf(gr, __shfl_xor_sync(0xffffffffu, gr, o));
-      gi = fmaxf(gi, __shfl_xor_sync(0xffffffffu, gi, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicMax(amax + 1 + 2 * iw, __float_as_uint(gr));
-      atomicMax(amax + 2 + 2 * iw, __float_as_uint(gi));
-    }
-    if (tr) {
-      float tlo = INFINITY, thi = -INFINITY;
-      for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = f[(int64_t)iw * K + i];
+      if (tr) {
         const float t = (float)(v.y / v.x);   // +-inf or NaN where Re f vanishes: the range is then unusable
         tlo = fminf(tlo, t);
         thi = fmaxf(thi, t);
         if (t != t) thi = INFINITY;
       }
-      for (int o = 16; o; o >>= 1) {
-        tlo = fminf(tlo, __shfl_xor_sync(0xffffffffu, tlo, o));
-        thi = fmaxf(thi, __shfl_xor_sync(0xffffffffu, thi, o));
-      }
-      if ((threadIdx.x & 31) == 0) {
+    }
+    for (int o = 16; o; o >>= 1) {
+      gr = fmaxf(gr, __shfl_xor_sync(0xffffffffu, gr, o));
+      gi = fmaxf(gi, __shfl_xor_sync(0xffffffffu, gi, o));
+      tlo = fminf(tlo, __shfl_xor_sync(0xffffffffu, tlo, o));
+      thi = fmaxf(thi, __shfl_xor_sync(0xffffffffu, thi, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+      atomicMax(amax + 1 + 2 * iw, __float_as_uint(gr));
+      atomicMax(amax + 2 + 2 * iw, __float_as_uint(gi));
+      if (tr) {
         atomicMin(tr + 2 * iw, ord_of(tlo));
         atomicMax(tr + 2 * iw + 1, ord_of(thi));
       }
@@ -1336,7 +1335,7 @@ static PackWs pack_ws(const chi0_plan_s* p, void* base, int nGp, int Kp) {
 template <bool BF16, int NT>
 static cudaError_t pack_one(chi0_plan_s* p, int nG, const float2* M, int64_t K, const double2* f, const PackWs& w,
                             int nGp, int Kp, cudaStream_t s) {
-  ProfScope ps(p, CHI0_K_PACK, s, p->tc_herm ? 4 : 3);
+  ProfScope ps(p, CHI0_K_PACK, s, p->tc_herm ? 5 : 4);
   cudaError_t e = cudaMemsetAsync(w.amax, 0, sizeof(unsigned int) * (2 * p->n_freq + 1), s);
   if (e != cudaSuccess) return e;
   if (p->tc_herm) {
@@ -1345,7 +1344,9 @@ static cudaError_t pack_one(chi0_plan_s* p, int nG, const float2* M, int64_t K, 
     if (e == cudaSuccess) e = fill_ratio_min(w.tr, p->n_freq, s);
     if (e != cudaSuccess) return e;
   }
-  k_absmax<<<2 * 152, 256, 0, s>>>(M, K * nG, f, K, p->n_freq, w.amax, p->tc_herm ? w.tr : nullptr);
+  k_absmax<<<4 * 152, 256, 0, s>>>(M, K * nG, w.amax);
+  k_factor_range<<<dim3((unsigned)((K + 127) / 128), std::min(p->n_freq, 65535)), 128, 0, s>>>(
+      f, K, p->n_freq, w.amax, p->tc_herm ? w.tr : nullptr);
   k_scales<<<1, 128, 0, s>>>(w.amax, w.tr, p->n_freq, p->tc_herm ? 1 : 0, p->n_products, BF16 ? 1 : 0, w.scale,
                              w.inv, w.h2np, w.tbar);
   e = cudaMemsetAsync(w.diag, 0, sizeof(double2) * p->n_freq * nGp, s);
