@@ -54,6 +54,8 @@ struct WfnSphere {
   double2* T1d = nullptr; float2* T1f = nullptr;   // [n1][nw1]
   double2* T2d = nullptr; float2* T2f = nullptr;   // [n2][nw2]
   double2* T3d = nullptr; float2* T3f = nullptr;   // [nw3][n3] (transposed)
+  FxAxis fx[2];                       // FP64 plans: axes 2 and 3 of the fixed-point synthesis (items = largest |g|)
+  const int4* fx_tw = nullptr;        // [n1] twiddles of axis 1
 };
 
 }  // namespace chi0
@@ -102,8 +104,8 @@ struct chi0_plan_s {
   size_t wfn_ws_bytes = 0;
   void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
   // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
-  // fixed-point pair stage, COH
-  LazyWs ws_mod, ws_bwd, ws_fx, ws_coh;
+  // fixed-point pair stage, fixed-point wavefunctions, COH
+  LazyWs ws_mod, ws_bwd, ws_fx, ws_wfn, ws_coh;
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)
@@ -164,6 +166,11 @@ cudaError_t launch_pair_gather(const chi0_plan_s* p, int iq, const void* D, int 
 // fixed-point pair stage of FP64 plans (kern_fx.cu): tables of a sphere, bands held at a time, workspace
 bool fx_fits(const chi0_plan_s* p, const SphereQ& s);
 cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s);
+// the same for the wavefunctions (w->fx_tw stays NULL where they do not fit)
+cudaError_t fx_setup_wfn(const chi0_plan_s* p, WfnSphere* w);
+size_t fx_wfn_ws_bytes(const chi0_plan_s* p, int64_t bands);
+cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, int64_t bands,
+                          cudaStream_t s);
 int fx_bands(const chi0_plan_s* p);
 size_t fx_ws_bytes(const chi0_plan_s* p, int64_t bands);
 cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int32_t* idx, int b0, int nb, void* ws,

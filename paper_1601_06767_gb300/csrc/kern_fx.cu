@@ -1,4 +1,5 @@
-// Pair matrix elements of FP64 plans in fixed point on the integer pipe.
+// Wavefunctions on the grid and pair matrix elements of FP64 plans in fixed point on
+// the integer pipe.
 //
 // GB300's FP64 pipe does two multiply-adds per clock and SM, so the direct FP64
 // sums (kern_pairs.cu) took 10.3 ms for the 8-atom workload's 3840 pairs.  Here
@@ -15,7 +16,8 @@
 // sum: against quad precision, on the synthetic wavefunctions, 1.1e-16 (relative
 // Frobenius) on grids of 21 to 48 points, 4.7-6.6e-16 for the FP64 sums.
 //
-// 3840 pairs, 24^3, N_G 350: planes 10.32 -> 0.77 ms, gather 231 -> 71 us.
+// 3840 pairs, 24^3, N_G 350: planes 10.32 -> 0.77 ms, gather 231 -> 71 us; 256
+// wavefunctions: 703 -> 165 us, 6.1e-16 -> 9.6e-17.
 //
 // A line of n points is transformed at the wanted frequencies only, with the
 // symmetries of the twiddles folded out first: with h = n / 2 and a_i = x_i +
@@ -40,6 +42,7 @@ namespace {
 constexpr int QBITS = 57, QL = 29;    // grids: bits and limb width
 constexpr int WBITS = 55, WL = 28;    // transform inputs and twiddles
 constexpr int FX_MAX_N = 128;         // the 64-bit sums hold n / 4 + 1 products of 2^57
+constexpr int FX_MAX_W = 64;          // wavefunction sphere: 64 coefficients per column (4 products of 2^54 each)
 
 // ---- grids to fixed point ----
 // mx[b] = largest magnitude word of band b (cleared by the caller)
@@ -56,21 +59,23 @@ __global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ psi,
   if ((threadIdx.x & 31) == 0 && m) atomicMax(mx + blockIdx.y, m);
 }
 
+template <int BITS = QBITS>
 __device__ __forceinline__ int fx_scale(uint32_t w) {
-  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : QBITS - 1 - mod::word_exp(w));
+  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : BITS - 1 - mod::word_exp(w));
 }
 
 // q[b][r] = (re1, re0, im1, im0): limbs of psi 2^scale
+template <int BITS, int LIMB>
 __global__ void __launch_bounds__(256) k_fx_quant(const double2* __restrict__ psi, const int32_t* __restrict__ idx, int b0,
                                                   int64_t nr, const uint32_t* __restrict__ mx, int4* __restrict__ q) {
   const int64_t band = idx ? idx[b0 + blockIdx.y] : b0 + blockIdx.y;
   const double2* x = psi + band * nr;
-  const int s = fx_scale(mx[blockIdx.y]);
+  const int s = fx_scale<BITS>(mx[blockIdx.y]);
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nr; e += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = x[e];
     const int64_t a = mod::quantise(v.x, s), b = mod::quantise(v.y, s);
-    const int a0 = ((int)a << (32 - QL)) >> (32 - QL), b0l = ((int)b << (32 - QL)) >> (32 - QL);
-    q[blockIdx.y * nr + e] = make_int4((int)((a - a0) >> QL), a0, (int)((b - b0l) >> QL), b0l);
+    const int a0 = ((int)a << (32 - LIMB)) >> (32 - LIMB), b0l = ((int)b << (32 - LIMB)) >> (32 - LIMB);
+    q[blockIdx.y * nr + e] = make_int4((int)((a - a0) >> LIMB), a0, (int)((b - b0l) >> LIMB), b0l);
   }
 }
 
@@ -87,6 +92,23 @@ __device__ __forceinline__ int word_bits(uint32_t m) { return 64 - __clz((int)m)
 __device__ __forceinline__ int4 limbs_w(int64_t re, int64_t im) {
   const int r0 = ((int)re << (32 - WL)) >> (32 - WL), i0 = ((int)im << (32 - WL)) >> (32 - WL);
   return make_int4((int)((re - r0) >> WL), r0, (int)((im - i0) >> WL), i0);
+}
+
+// y 2^k as a double, rounded to nearest
+__device__ __forceinline__ double to_double(int64_t y, int k) {
+  if (y == 0) return 0.0;
+  const uint64_t a = y < 0 ? 0ull - (uint64_t)y : (uint64_t)y;
+  const int z = __clzll((long long)a);
+  const uint64_t t = a << z;                              // top bit set
+  uint64_t man = (t >> 11) + ((t >> 10) & 1u);
+  int e = 1023 + 63 - z + k;
+  if (man >> 53) {
+    man >>= 1;
+    ++e;
+  }
+  const uint64_t sgn = y < 0 ? 0x8000000000000000ull : 0ull;
+  if (e >= 1 && e <= 2046) return __longlong_as_double((long long)(sgn | ((uint64_t)e << 52) | (man & 0xfffffffffffffull)));
+  return scalbn(__longlong_as_double((long long)(sgn | (1023ull << 52) | (man & 0xfffffffffffffull))), e - 1023);
 }
 
 // units of one line's fold: i = 0 .. fold_units(n) - 1, each owns the slots it reads and writes
@@ -281,23 +303,6 @@ __global__ void k_fx_planes(const int4* __restrict__ qv, const uint32_t* __restr
   }
 }
 
-// y 2^k as a double, rounded to nearest
-__device__ __forceinline__ double to_double(int64_t y, int k) {
-  if (y == 0) return 0.0;
-  const uint64_t a = y < 0 ? 0ull - (uint64_t)y : (uint64_t)y;
-  const int z = __clzll((long long)a);
-  const uint64_t t = a << z;                              // top bit set
-  uint64_t man = (t >> 11) + ((t >> 10) & 1u);
-  int e = 1023 + 63 - z + k;
-  if (man >> 53) {
-    man >>= 1;
-    ++e;
-  }
-  const uint64_t sgn = y < 0 ? 0x8000000000000000ull : 0ull;
-  if (e >= 1 && e <= 2046) return __longlong_as_double((long long)(sgn | ((uint64_t)e << 52) | (man & 0xfffffffffffffull)));
-  return scalbn(__longlong_as_double((long long)(sgn | (1023ull << 52) | (man & 0xfffffffffffffull))), e - 1023);
-}
-
 // Stage 3: M[row][j] = (1/N_r) sum_i1 D(i1, k2_j, k3_j) e^{2 pi i k1_j i1 / n1} for a chunk of the
 // (k2, k3) columns of one pair; colmap[column][k1 - k1min] = j, or -1 off the sphere
 __global__ void __launch_bounds__(256) k_fx_gather(const longlong2* __restrict__ D, const int2* __restrict__ ex, int nc,
@@ -356,6 +361,138 @@ __global__ void __launch_bounds__(256) k_fx_gather(const longlong2* __restrict__
   }
 }
 
+// ---- wavefunctions ----
+// Synthesis of a line of n points from coefficients c(g), |g| <= G, with the same
+// symmetries: P = c(g) + c(-g), M = c(g) - c(-g), sums over even and odd g apart,
+//   X(i) = (Ee + Eo) + i (Oe + Oo),  X(n - i) = (Ee + Eo) - i (Oe + Oo),
+//   X(i + h) = (Ee - Eo) + i (Oe - Oo),  X(h - i) = (Ee - Eo) - i (Oe - Oo),  h = n / 2,
+// E = sum P cos, O = sum M sin, for i = 0 .. n / 4 (odd n: i = 0 .. (n - 1) / 2, the
+// first row only).  The line is kept as slots G + g, folded in place (P at +g, M at -g).
+__device__ __forceinline__ void fold_synth(longlong2* __restrict__ r, int G, int g, int s) {
+  int4* w = reinterpret_cast<int4*>(r);
+  const longlong2 p = r[G + g], m = r[G - g];
+  const int64_t px = shift_round(p.x, s), py = shift_round(p.y, s), mx = shift_round(m.x, s), my = shift_round(m.y, s);
+  if (g == 0) {
+    w[G] = limbs_w(px, py);
+    return;
+  }
+  w[G + g] = limbs_w(px + mx, py + my);
+  w[G - g] = limbs_w(px - mx, py - my);
+}
+
+// calls put(index, value) for the outputs of unit i
+template <class Put>
+__device__ __forceinline__ void synth_unit(const int4* __restrict__ w, const FxAxis& ax, int i, Put put) {
+  const int n = ax.n, h = n >> 1, G = ax.items;
+  const int4* __restrict__ t = ax.coef + i;            // [g][units]
+  const bool even = !(n & 1);
+  int64_t E[2][2] = {}, O[2][2] = {};                  // [parity of g][re, im]
+#pragma unroll
+  for (int par = 0; par < 2; ++par) {
+    if (par && !even) break;
+    Acc er, ei, sr, si;
+    for (int g = par; g <= G; g += even ? 2 : 1) {
+      const int4 p = w[G + g], c = t[g * ax.units];
+      er.add(p.x, p.y, c.x, c.y);
+      ei.add(p.z, p.w, c.x, c.y);
+      if (g) {
+        const int4 m = w[G - g];
+        sr.add(m.x, m.y, c.z, c.w);
+        si.add(m.z, m.w, c.z, c.w);
+      }
+    }
+    E[par][0] = er.value();
+    E[par][1] = ei.value();
+    O[par][0] = sr.value();
+    O[par][1] = si.value();
+  }
+  const int64_t er = E[0][0] + E[1][0], ei = E[0][1] + E[1][1], orr = O[0][0] + O[1][0], oi = O[0][1] + O[1][1];
+  put(i, make_longlong2(er - oi, ei + orr));
+  if (i) put(n - i, make_longlong2(er + oi, ei - orr));
+  if (even) {
+    const int64_t fr = E[0][0] - E[1][0], fi = E[0][1] - E[1][1], pr = O[0][0] - O[1][0], pi = O[0][1] - O[1][1];
+    if (2 * i != h || i == 0) put(i + h, make_longlong2(fr - pi, fi + pr));
+    if (i && 2 * i != h) put(h - i, make_longlong2(fr + pi, fi - pr));
+  }
+}
+
+// psi[band][i1] for one plane and band: along g1 for every (g2, g3) column of the sphere (direct sums
+// over its few coefficients), along g2 for every g3, along g3 for every i2.
+__global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict__ mx, int npw, int n1, int n2, int n3,
+                         int nw1, int w2min, int w3min, int nw2, int nw3, const int* __restrict__ col_start,
+                         const int* __restrict__ col_pw, const int* __restrict__ col_g1, int w1min,
+                         const int4* __restrict__ tw1, const __grid_constant__ FxAxis a2, const __grid_constant__ FxAxis a3,
+                         double2* __restrict__ psi) {
+  extern __shared__ __align__(16) unsigned char smem_fx[];
+  __shared__ uint32_t slot[2];
+  __shared__ int4 tws[FX_MAX_W];
+  const int G2 = a2.items, G3 = a3.items, lda = 2 * G2 + 1, ldb = 2 * G3 + 1;   // odd
+  longlong2* A = reinterpret_cast<longlong2*>(smem_fx);    // [2 G3 + 1][lda]: slot of g3, slot of g2
+  longlong2* B = A + (size_t)(2 * G3 + 1) * lda;           // [n2][ldb]
+  const int i1 = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
+  const int64_t b = blockIdx.y;
+  double2* out = psi + (b * n1 + i1) * (int64_t)n2 * n3;
+  const int s = fx_scale<WBITS>(mx[b]);
+  if (s == mod::NO_SCALE) {                                // an infinity or a NaN among the coefficients
+    for (int e = tid; e < n2 * n3; e += nt) out[e] = make_double2(nan(""), nan(""));
+    return;
+  }
+  if (tid < 2) slot[tid] = 0;
+  for (int g = tid; g < nw1; g += nt) {
+    int k = (int)((int64_t)(w1min + g) * i1 % n1);
+    tws[g] = tw1[k < 0 ? k + n1 : k];
+  }
+  for (int e = tid; e < (2 * G3 + 1) * lda; e += nt) A[e] = make_longlong2(0, 0);
+  __syncthreads();
+  const int4* qb = q + b * npw;
+  uint32_t m = 0;
+  for (int c = tid; c < nw2 * nw3; c += nt) {
+    const int r = c / nw3, g3 = w3min + c - r * nw3, g2 = w2min + r, k1 = col_start[c + 1];
+    Acc re, im;
+    for (int k = col_start[c]; k < k1; ++k) {
+      const int4 x = qb[col_pw[k]], t = tws[col_g1[k]];    // t = (cos, sin) in two limbs each
+      re.add(x.x, x.y, t.x, t.y);
+      re.add(-x.z, -x.w, t.z, t.w);
+      im.add(x.z, x.w, t.x, t.y);
+      im.add(x.x, x.y, t.z, t.w);
+    }
+    const longlong2 v = make_longlong2(re.value(), im.value());
+    A[(G3 + g3) * lda + G2 + g2] = v;
+    m = max(m, max(abs_word(v.x), abs_word(v.y)));
+  }
+  const int sa = word_bits(block_max(m, slot)) - WBITS;
+  for (int e = tid; e < (2 * G3 + 1) * (G2 + 1); e += nt) {
+    const int c = e % (2 * G3 + 1), g = e / (2 * G3 + 1);
+    fold_synth(A + c * lda, G2, g, sa);
+  }
+  __syncthreads();
+  m = 0;
+  for (int e = tid; e < (2 * G3 + 1) * a2.units; e += nt) {    // along g2
+    const int c = e % (2 * G3 + 1), i = e / (2 * G3 + 1);
+    synth_unit(reinterpret_cast<const int4*>(A + c * lda), a2, i, [&](int i2, longlong2 v) {
+      B[i2 * ldb + c] = v;
+      m = max(m, max(abs_word(v.x), abs_word(v.y)));
+    });
+  }
+  const int sb = word_bits(block_max(m, slot + 1)) - WBITS;
+  for (int e = tid; e < n2 * (G3 + 1); e += nt) {
+    const int i2 = e % n2, g = e / n2;
+    fold_synth(B + i2 * ldb, G3, g, sb);
+  }
+  __syncthreads();
+  const int unit = -s + sa + sb;
+  for (int e = tid; e < n2 * a3.units; e += nt) {              // along g3
+    const int i = e % a3.units, i2 = e / a3.units;
+    synth_unit(reinterpret_cast<const int4*>(B + i2 * ldb), a3, i, [&](int i3, longlong2 v) {
+      out[i2 * n3 + i3] = make_double2(to_double(v.x, unit), to_double(v.y, unit));
+    });
+  }
+}
+
+size_t wfn_smem(const chi0_plan_s* p, const WfnSphere& w) {
+  return ((size_t)(2 * w.fx[1].items + 1) * (2 * w.fx[0].items + 1) + (size_t)p->n2 * (2 * w.fx[1].items + 1)) * 16;
+}
+
 size_t planes_smem(const chi0_plan_s* p, const SphereQ& s) {
   return ((size_t)p->n2 * (p->n3 | 1) + (size_t)s.nk3 * (p->n2 | 1)) * 16;
 }
@@ -368,10 +505,50 @@ int2* fx_exponents(const chi0_plan_s* p, void* ws, int64_t bands) {
   return reinterpret_cast<int2*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16) + al256((size_t)bands * 4));
 }
 
+// (cos, sin) of 2 pi m / n, m < n, in two limbs each; evaluated on the first octant only (long double
+// is software on the Arm hosts)
+std::vector<int4> twiddle_table(int n) {
+  const long double two_pi = 2.0L * 3.14159265358979323846264338327950288L;
+  std::vector<int64_t> c(n / 8 + 1), s(n / 8 + 1);
+  for (int m = 0; m <= n / 8; ++m) {
+    c[m] = llroundl(cosl(two_pi * m / n) * (long double)((int64_t)1 << WBITS));
+    s[m] = llroundl(sinl(two_pi * m / n) * (long double)((int64_t)1 << WBITS));
+  }
+  std::vector<int4> t(n);
+  for (int m = 0; m < n; ++m) {
+    // angle 2 pi m / n = (quarter turns) + 2 pi r / (4 n): r = 4 m mod n quarters of a step
+    const int quarter = 4 * m / n, r = 4 * m - quarter * n;
+    int64_t co, si;
+    if (r % 4 == 0 && 8 * (r / 4) <= n) {                    // r / 4 whole steps past the quarter turn
+      co = c[r / 4];
+      si = s[r / 4];
+    } else if ((n - r) % 4 == 0 && 8 * ((n - r) / 4) <= n) { // before the next quarter turn
+      co = s[(n - r) / 4];
+      si = c[(n - r) / 4];
+    } else {                                                 // n not a multiple of 4: no symmetric point
+      co = llroundl(cosl(two_pi * r / (4.0L * n)) * (long double)((int64_t)1 << WBITS));
+      si = llroundl(sinl(two_pi * r / (4.0L * n)) * (long double)((int64_t)1 << WBITS));
+    }
+    const int64_t re = quarter == 0 ? co : quarter == 1 ? -si : quarter == 2 ? -co : si;
+    const int64_t im = quarter == 0 ? si : quarter == 1 ? co : quarter == 2 ? -si : -co;
+    int l[4];
+    for (int k = 0; k < 2; ++k) {
+      const int64_t q = k ? im : re;
+      int64_t q0 = q & (((int64_t)1 << WL) - 1);
+      if (q0 >= (int64_t)1 << (WL - 1)) q0 -= (int64_t)1 << WL;
+      l[2 * k] = (int)((q - q0) >> WL);
+      l[2 * k + 1] = (int)q0;
+    }
+    t[m] = make_int4(l[0], l[1], l[2], l[3]);
+  }
+  return t;
+}
+
 // frequency pairs +-k of an axis (kmin .. kmin + nk - 1) and their twiddles
 cudaError_t make_axis(int n, int kmin, int nk, FxAxis* a) {
   std::vector<int4> item, coef;
   const int units = fold_units(n);
+  const std::vector<int4> tw = twiddle_table(n);
   for (int k = 0; k <= n / 2; ++k) {
     int pos = -1, neg = -1;
     for (int c = 0; c < nk; ++c) {
@@ -383,18 +560,7 @@ cudaError_t make_axis(int n, int kmin, int nk, FxAxis* a) {
     }
     if (pos < 0 && neg < 0) continue;
     item.push_back(make_int4(n % 2 == 0 ? k & 1 : 0, pos, neg, 0));
-    for (int i = 0; i < units; ++i) {
-      const long double ang = 2.0L * 3.14159265358979323846264338327950288L * (long double)((int64_t)k * i % n) / n;
-      int l[4];
-      for (int c = 0; c < 2; ++c) {
-        const int64_t q = llroundl((c ? sinl(ang) : cosl(ang)) * (long double)((int64_t)1 << WBITS));
-        int64_t q0 = q & (((int64_t)1 << WL) - 1);
-        if (q0 >= (int64_t)1 << (WL - 1)) q0 -= (int64_t)1 << WL;
-        l[2 * c] = (int)((q - q0) >> WL);
-        l[2 * c + 1] = (int)q0;
-      }
-      coef.push_back(make_int4(l[0], l[1], l[2], l[3]));
-    }
+    for (int i = 0; i < units; ++i) coef.push_back(tw[(int64_t)k * i % n]);
   }
   a->n = n;
   a->units = units;
@@ -410,6 +576,70 @@ cudaError_t make_axis(int n, int kmin, int nk, FxAxis* a) {
 }
 
 }  // namespace
+
+static cudaError_t upload4(const int4** dst, const std::vector<int4>& v) {
+  int4* d = nullptr;
+  cudaError_t e = cudaMalloc((void**)&d, v.size() * sizeof(int4));
+  if (e == cudaSuccess) e = cudaMemcpy(d, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  *dst = d;
+  return e;
+}
+
+// tables of the wavefunction sphere where the fixed-point synthesis fits (else w->fx_tw stays NULL and the
+// direct FP64 sums run): axis g2 in fx[0], g3 in fx[1] (items = largest |g|), plane twiddles
+cudaError_t fx_setup_wfn(const chi0_plan_s* p, WfnSphere* w) {
+  if (w->npw <= 0 || p->n1 > FX_MAX_N || p->n2 > FX_MAX_N || p->n3 > FX_MAX_N || w->nw1 > FX_MAX_W) return cudaSuccess;
+  const int n[2] = {p->n2, p->n3}, lo[2] = {w->w2min, w->w3min}, cnt[2] = {w->nw2, w->nw3};
+  for (int a = 0; a < 2; ++a) {
+    const int G = std::max(std::abs(lo[a]), std::abs(lo[a] + cnt[a] - 1));
+    if (G > FX_MAX_W) return cudaSuccess;                   // a sphere far from the origin
+    w->fx[a].n = n[a];
+    w->fx[a].units = fold_units(n[a]);
+    w->fx[a].items = G;
+  }
+  if (wfn_smem(p, *w) > SMEM_CAP) return cudaSuccess;
+  std::vector<int> start((size_t)w->nw2 * w->nw3 + 1);
+  cudaError_t e = cudaMemcpy(start.data(), w->col_start, start.size() * sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return e;
+  for (size_t c = 0; c + 1 < start.size(); ++c)             // (a vector listed twice counts twice)
+    if (start[c + 1] - start[c] > FX_MAX_W) return cudaSuccess;
+  for (int a = 0; a < 2 && e == cudaSuccess; ++a) {
+    const std::vector<int4> tw = twiddle_table(n[a]);
+    std::vector<int4> t;
+    for (int g = 0; g <= w->fx[a].items; ++g)
+      for (int i = 0; i < w->fx[a].units; ++i) t.push_back(tw[(int64_t)g * i % n[a]]);
+    e = upload4(&w->fx[a].coef, t);
+  }
+  if (e == cudaSuccess) e = upload4(&w->fx_tw, twiddle_table(p->n1));
+  return e;
+}
+
+size_t fx_wfn_ws_bytes(const chi0_plan_s* p, int64_t bands) {
+  return al256((size_t)bands * p->w.npw * 16) + al256((size_t)bands * 4);
+}
+
+cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, int64_t bands,
+                          cudaStream_t s) {
+  const WfnSphere& w = p->w;
+  int4* q = reinterpret_cast<int4*>(ws);
+  uint32_t* mx = reinterpret_cast<uint32_t*>((unsigned char*)ws + al256((size_t)bands * w.npw * 16));
+  const size_t sm = wfn_smem(p, w);
+  cudaError_t e = cudaFuncSetAttribute(k_fx_wfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  for (int b0 = 0; b0 < nb; b0 += (int)bands) {
+    const int n = (int)std::min<int64_t>(bands, nb - b0);
+    e = cudaMemsetAsync(mx, 0, (size_t)n * 4, s);
+    if (e != cudaSuccess) return e;
+    const int gx = (int)std::min<int64_t>((w.npw + 1023) / 1024, std::max(1, 4096 / n));
+    k_fx_max<<<dim3(gx, n), 256, 0, s>>>(coeff, nullptr, b0, w.npw, mx);
+    k_fx_quant<WBITS, WL><<<dim3(gx, n), 256, 0, s>>>(coeff, nullptr, b0, w.npw, mx, q);
+    const int nt = sm <= 32 * 1024 ? 128 : (sm <= 72 * 1024 ? 256 : 512);
+    k_fx_wfn<<<dim3(p->n1, n), nt, sm, s>>>(q, mx, w.npw, p->n1, p->n2, p->n3, w.nw1, w.w2min, w.w3min, w.nw2, w.nw3,
+                                            w.col_start, w.col_pw, w.col_g1, w.w1min, w.fx_tw, w.fx[0], w.fx[1],
+                                            psi + (int64_t)b0 * p->nr);
+  }
+  return cudaGetLastError();
+}
 
 // whether the plan's grid and a sphere fit the kernels (else the direct FP64 sums run)
 bool fx_fits(const chi0_plan_s* p, const SphereQ& s) {
@@ -454,7 +684,7 @@ cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int3
   if (e != cudaSuccess) return e;
   const int gx = (int)std::min<int64_t>((p->nr + 1023) / 1024, std::max(1, 4096 / nb));
   k_fx_max<<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx);
-  k_fx_quant<<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx, q);
+  k_fx_quant<QBITS, QL><<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx, q);
   return cudaGetLastError();
 }
 

@@ -101,10 +101,12 @@ void free_plan(chi0_plan_s* p) {
   chi0::WfnSphere& w = p->w;
   cudaFree(w.col_start); cudaFree(w.col_pw); cudaFree(w.col_g1);
   cudaFree(w.T1d); cudaFree(w.T1f); cudaFree(w.T2d); cudaFree(w.T2f);
-  cudaFree(w.T3d); cudaFree(w.T3f);
+  cudaFree(w.T3d); cudaFree(w.T3f); cudaFree((void*)w.fx_tw);
+  for (auto& a : w.fx) cudaFree((void*)a.coef);
   cudaFree(p->d_omega); cudaFree(p->d_D); cudaFree(p->d_M); cudaFree(p->d_f);
   cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->d_inv); cudaFree(p->wfn_ws);
-  cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p); cudaFree(p->ws_coh.p);
+  cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p); cudaFree(p->ws_wfn.p);
+  cudaFree(p->ws_coh.p);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
     cudaFree(p->bq_M[i]);
     cudaFree(p->bq_f[i]);
@@ -406,6 +408,10 @@ chi0_status chi0_plan_create(chi0_plan* out, const chi0_plan_desc* d) {
   }
   st = analyse_wfn(p, d->gw, d->npw);
   if (st != CHI0_OK) return bail(st);
+  if (!chi0::is_split(p)) {
+    cudaError_t fe = chi0::fx_setup_wfn(p, &p->w);
+    if (fe != cudaSuccess) { p->err = cudaGetErrorString(fe); return bail(fe == cudaErrorMemoryAllocation ? CHI0_ERR_OOM : CHI0_ERR_CUDA); }
+  }
   if (!chi0::is_split(p))
     for (auto& sq : p->q)
       if (chi0::fx_fits(p, sq)) {
@@ -747,6 +753,15 @@ chi0_status chi0_wfn_to_grid(chi0_plan p, const void* coeff, int nb, void* psi, 
   if (p->w.npw <= 0) return fail(p, CHI0_ERR_INVALID, "the plan has no wavefunction sphere");
   if (nb < 0 || (nb > 0 && (!coeff || !psi))) return fail(p, CHI0_ERR_INVALID, "bad band count or NULL buffer");
   if (nb == 0) return CHI0_OK;
+  if (p->w.fx_tw) {
+    // coefficients in fixed point for up to 1 GiB (and 65535) bands at a time
+    const int64_t bands = std::min<int64_t>({nb, 65535, std::max<int64_t>(1, ((int64_t)1 << 30) / (16 * (int64_t)p->w.npw))});
+    if (ws_ready(p, p->ws_wfn, chi0::fx_wfn_ws_bytes(p, bands), (cudaStream_t)stream)) {
+      chi0::ProfScope ps(p, CHI0_K_WFN, (cudaStream_t)stream, 3 * (int)((nb + bands - 1) / bands));
+      CK(p, chi0::launch_fx_wfn(p, (const double2*)coeff, nb, (double2*)psi, p->ws_wfn.p, bands, (cudaStream_t)stream));
+      return CHI0_OK;
+    }
+  }
   chi0::ProfScope ps(p, CHI0_K_WFN, (cudaStream_t)stream, 1);
   CK(p, chi0::launch_wfn_to_grid(p, (const double2*)coeff, nb, psi, (cudaStream_t)stream));
   return CHI0_OK;

@@ -1,4 +1,4 @@
-"""Pair elements of FP64 plans in fixed point, where the line transforms change
+"""Wavefunctions and pair elements of FP64 plans in fixed point, where the line transforms change
 form: odd axes, even axes with odd and even halves, mixed grids, spheres away
 from the origin (frequencies beyond n / 2, both ends of the range), pair blocks
 in several chunks, and bands without a usable scale.
@@ -77,3 +77,30 @@ def test_scales_zero_and_nonfinite_bands():
     good = np.ones((4, 5), bool)
     good[1] = good[:, 3] = False
     assert np.all(fin[good]) and not fin[~good].any()
+
+
+@pytest.mark.parametrize("n,lo,hi", [
+    ((2, 2, 2), (0, 0, 0), (1, 1, 1)), ((3, 4, 5), (-1, -1, -2), (1, 2, 2)), ((6, 10, 22), (-2, -4, -10), (3, 5, 11)),
+    ((24, 24, 24), (-7, -7, -7), (7, 7, 7)), ((21, 27, 30), (-6, 3, 11), (6, 11, 19)), ((48, 20, 33), (-14, -9, -16), (14, 6, 16)),
+    ((130, 4, 4), (-3, -1, -1), (3, 1, 2)), ((70, 6, 4), (-34, -1, -1), (34, 1, 1)),
+])
+def test_wavefunctions_all_axis_forms(n, lo, hi):
+    """psi(r) = sum_g c(g) exp(2 pi i g.r) against NumPy, bands far apart in magnitude, a zero band and one
+    holding an infinity.  Three roundings to 2^-56 of a plane's largest value: bar 2e-15 as above."""
+    rng = np.random.default_rng(sum(n) + 1)
+    g = np.stack(np.meshgrid(*[np.arange(a, b + 1) for a, b in zip(lo, hi)], indexing="ij"), -1).reshape(-1, 3)
+    g = g[rng.permutation(len(g))[: max(1, (2 * len(g)) // 3)]].astype(np.int32)
+    c = rng.standard_normal((5, len(g))) + 1j * rng.standard_normal((5, len(g)))
+    c *= np.array([1.0, 1e-120, 1e100, 0.0, 1.0])[:, None]
+    ref = np.zeros((5,) + n, complex)
+    for b in range(5):
+        np.add.at(ref[b], tuple(np.mod(g, n).T), c[b])
+        ref[b] = np.fft.ifftn(ref[b], norm="forward")
+    c[4, 0] = np.inf
+    from paper_1601_06767_gb300 import Chi0Plan
+    with Chi0Plan(n, [np.zeros((1, 3), np.int32)], [0.0], 1e-3, precision="fp64", gw=g) as plan:
+        psi = plan.wfn_to_grid(_dev(c)).cpu().numpy()
+        plan.sync_status()
+    for b in range(3):
+        assert np.linalg.norm(psi[b] - ref[b]) <= 2e-15 * np.linalg.norm(ref[b])
+    assert not psi[3].any() and not np.isfinite(psi[4]).any()
