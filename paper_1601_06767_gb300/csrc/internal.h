@@ -65,6 +65,7 @@ struct LazyWs {
   void* p = nullptr;
   size_t bytes = 0;
   size_t limit = SIZE_MAX;            // smallest size that could not be had (not asked for again)
+  bool captured = false;              // a caller's stream capture holds the address
 };
 
 struct chi0_plan_s {
@@ -106,6 +107,8 @@ struct chi0_plan_s {
   // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
   // fixed-point pair stage, fixed-point wavefunctions, COH
   LazyWs ws_mod, ws_bwd, ws_fx, ws_wfn, ws_coh;
+  std::vector<void*> ws_kept;          // outgrown workspaces that a caller's captured graph still names
+  cudaEvent_t wfn_ev = nullptr;        // last use of ws_wfn
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)

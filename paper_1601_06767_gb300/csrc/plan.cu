@@ -107,6 +107,8 @@ void free_plan(chi0_plan_s* p) {
   cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->d_inv); cudaFree(p->wfn_ws);
   cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p); cudaFree(p->ws_wfn.p);
   cudaFree(p->ws_coh.p);
+  for (void* w : p->ws_kept) cudaFree(w);
+  if (p->wfn_ev) cudaEventDestroy(p->wfn_ev);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
     cudaFree(p->bq_M[i]);
     cudaFree(p->bq_f[i]);
@@ -295,25 +297,41 @@ static bool herm_pays(const chi0_plan_s* p, const chi0_plan_desc* d) {
 
 // A workspace of at least `need` bytes, allocated on first use and grown when a later call needs more:
 // not inside a stream capture (the CUDA-core kernels run there unless an earlier call has allocated
-// enough).  A size that could not be had is not asked for again.
+// enough).  A size that could not be had is not asked for again.  A workspace that a caller's capture
+// has used is kept until the plan is destroyed when it is outgrown: the caller's graph names its address.
 static bool ws_ready(chi0_plan_s* p, LazyWs& w, size_t need, cudaStream_t s) {
   if (need >= w.limit) return false;
-  if (need <= w.bytes) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
+  if (cap != cudaStreamCaptureStatusNone) {
+    if (need > w.bytes) return false;
+    w.captured = w.captured || s != p->cap_stream;
+    return true;
+  }
+  if (need <= w.bytes) return true;
+  // a capture on some other stream does not see the allocation
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
   // the graph of a batched build holds the old address
   if (p->graph_exec) {
     cudaGraphExecDestroy(p->graph_exec);
     p->graph_exec = nullptr;
   }
-  cudaFree(w.p);   // waits for the work that uses it
+  if (w.captured) {
+    p->ws_kept.push_back(w.p);
+    w.captured = false;
+  } else {
+    cudaFree(w.p);   // waits for the work that uses it
+    p->ws_bytes -= w.bytes;
+  }
   w.p = nullptr;
-  p->ws_bytes -= w.bytes;
   w.bytes = 0;
-  if (cudaMalloc(&w.p, need) != cudaSuccess) {
+  const cudaError_t e = cudaMalloc(&w.p, need);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
     cudaGetLastError();
     w.p = nullptr;
     w.limit = need;
@@ -702,6 +720,7 @@ chi0_status chi0_sigma_coh(chi0_plan p, int iq, const void* m, int n_t, int n_b,
   cudaStream_t s = (cudaStream_t)stream;
   const size_t bytes = chi0::sigma_coh_ws_bytes(p, nG, n_t);
   // kept by the plan: an allocation and a release per call took 0.2 ms of a 12 ms sum
+  p->ws_coh.limit = SIZE_MAX;   // nothing else computes the sum: ask again after a refusal
   if (!ws_ready(p, p->ws_coh, bytes, s)) return fail(p, CHI0_ERR_OOM, "chi0_sigma_coh: workspace");
   void* ws = p->ws_coh.p;
   cudaError_t e = cudaSuccess;
@@ -756,9 +775,24 @@ chi0_status chi0_wfn_to_grid(chi0_plan p, const void* coeff, int nb, void* psi, 
   if (p->w.fx_tw) {
     // coefficients in fixed point for up to 1 GiB (and 65535) bands at a time
     const int64_t bands = std::min<int64_t>({nb, 65535, std::max<int64_t>(1, ((int64_t)1 << 30) / (16 * (int64_t)p->w.npw))});
-    if (ws_ready(p, p->ws_wfn, chi0::fx_wfn_ws_bytes(p, bands), (cudaStream_t)stream)) {
-      chi0::ProfScope ps(p, CHI0_K_WFN, (cudaStream_t)stream, 3 * (int)((nb + bands - 1) / bands));
-      CK(p, chi0::launch_fx_wfn(p, (const double2*)coeff, nb, (double2*)psi, p->ws_wfn.p, bands, (cudaStream_t)stream));
+    // Calls on several streams share the workspace one after the other.  A captured call could run beside
+    // any of them when its graph is launched: it keeps the direct sums, which need none.
+    cudaStream_t s = (cudaStream_t)stream;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(p, cudaStreamIsCapturing(s, &cap));
+    if (cap == cudaStreamCaptureStatusNone && ws_ready(p, p->ws_wfn, chi0::fx_wfn_ws_bytes(p, bands), s)) {
+      if (!p->wfn_ev)
+        CK(p, cudaEventCreateWithFlags(&p->wfn_ev, cudaEventDisableTiming));
+      else
+        CK(p, cudaStreamWaitEvent(s, p->wfn_ev, 0));
+      cudaError_t e;
+      {
+        chi0::ProfScope ps(p, CHI0_K_WFN, s, 3 * (int)((nb + bands - 1) / bands));
+        e = chi0::launch_fx_wfn(p, (const double2*)coeff, nb, (double2*)psi, p->ws_wfn.p, bands, s);
+      }
+      const cudaError_t er = cudaEventRecord(p->wfn_ev, s);
+      CK(p, e);
+      CK(p, er);
       return CHI0_OK;
     }
   }
