@@ -367,17 +367,21 @@ static_assert(SMEM_BYTES <= 227 * 1024, "shared memory above the per-block limit
 // to one stage and ordered smallest-first: every term product t_i t_j with
 // i + j > 0 goes in while the accumulator is still small, and the t0 t0
 // products (the only large ones) come last.
-template <bool BF16, int NT, bool PAIR, int NPROD>
+// COMP: both components (COMP_BOTH), or Re or Im alone into d_re over COMP_N columns
+// (k_contract_tc_narrow); an accumulator sees the same products in the same order.
+constexpr int COMP_BOTH = 0, COMP_RE = 1, COMP_IM = 2, COMP_N = 64;
+template <bool BF16, int NT, bool PAIR, int NPROD, int COMP = COMP_BOTH>
 __device__ __forceinline__ void issue_stage_np(const unsigned char* st, uint32_t d_re, uint32_t d_im, bool first) {
   constexpr int P = 2 * NT;
   // in a CTA pair each CTA holds 128 rows of A and 64 rows of B; the MMA spans 256 rows
-  constexpr int B_BYTES = PAIR ? TILE_BYTES / 2 : TILE_BYTES;
-  const uint32_t id_pos = tc::idesc_f16(BF16, false, PAIR ? 2 * BM : BM, BN);
-  const uint32_t id_neg = tc::idesc_f16(BF16, true, PAIR ? 2 * BM : BM, BN);
+  constexpr int B_BYTES = PAIR || COMP ? TILE_BYTES / 2 : TILE_BYTES;
+  const uint32_t id_pos = tc::idesc_f16(BF16, false, PAIR ? 2 * BM : BM, COMP ? COMP_N : BN);
+  [[maybe_unused]] const uint32_t id_neg = tc::idesc_f16(BF16, true, PAIR ? 2 * BM : BM, COMP ? COMP_N : BN);
   // one descriptor for the stage; tiles and K steps are constant offsets of its address field
   const uint64_t d0 = tc::sdesc_kmajor_sw64(st);
   constexpr uint64_t kTile = TILE_BYTES >> 4, kBTile = B_BYTES >> 4, kB0 = (uint64_t)(P * TILE_BYTES) >> 4;
-  uint32_t acc_re = first ? 0u : 1u, acc_im = acc_re;
+  uint32_t acc_re = first ? 0u : 1u;
+  [[maybe_unused]] uint32_t acc_im = acc_re;
 #pragma unroll
   for (int order = 2 * NT - 2; order >= 0; --order) {
 #pragma unroll
@@ -402,6 +406,14 @@ __device__ __forceinline__ void issue_stage_np(const unsigned char* st, uint32_t
           tc::mma_f16_pair(d_im, ai, br, id_pos, acc_im);
           acc_im = 1u;
           tc::mma_f16_pair(d_im, ar, bi, id_neg, 1u);
+        } else if constexpr (COMP == COMP_RE) {
+          tc::mma_f16(d_re, ar, br, id_pos, acc_re);
+          acc_re = 1u;
+          tc::mma_f16(d_re, ai, bi, id_pos, 1u);
+        } else if constexpr (COMP == COMP_IM) {
+          tc::mma_f16(d_re, ai, br, id_pos, acc_re);
+          acc_re = 1u;
+          tc::mma_f16(d_re, ar, bi, id_neg, 1u);
         } else {
           // Re += Wr Mr + Wi Mi
           tc::mma_f16(d_re, ar, br, id_pos, acc_re);
@@ -457,13 +469,13 @@ __device__ __forceinline__ void issue_stage_1p(const unsigned char* st, uint32_t
 }
 
 // the product count as a compile-time constant: no per-MMA test in the issue loop
-template <bool BF16, int NT, bool PAIR = false>
+template <bool BF16, int NT, bool PAIR = false, int COMP = COMP_BOTH>
 __device__ __forceinline__ void issue_stage(const unsigned char* st, uint32_t d_re, uint32_t d_im, bool first,
                                             int n_products) {
-  if (n_products == 6) issue_stage_np<BF16, NT, PAIR, 6>(st, d_re, d_im, first);
-  else if (n_products == 4) issue_stage_np<BF16, NT, PAIR, 4>(st, d_re, d_im, first);
-  else if (n_products == 1) issue_stage_np<BF16, NT, PAIR, 1>(st, d_re, d_im, first);
-  else issue_stage_np<BF16, NT, PAIR, 3>(st, d_re, d_im, first);
+  if (n_products == 6) issue_stage_np<BF16, NT, PAIR, 6, COMP>(st, d_re, d_im, first);
+  else if (n_products == 4) issue_stage_np<BF16, NT, PAIR, 4, COMP>(st, d_re, d_im, first);
+  else if (n_products == 1) issue_stage_np<BF16, NT, PAIR, 1, COMP>(st, d_re, d_im, first);
+  else issue_stage_np<BF16, NT, PAIR, 3, COMP>(st, d_re, d_im, first);
 }
 
 // One persistent launch over a list of work items (q-point, frequency, 128x128
@@ -1028,6 +1040,189 @@ template <int NT> struct Ring2 {
   static constexpr int STAGES = RING2_BYTES / STAGE_BYTES;   // 4 for NT = 2, 3 for NT = 3
 };
 
+// ---------------------------------------------------------------------------
+// Narrow items (plain mode): 128 rows x 64 columns of Re chi0 or of Im chi0.  With a
+// handful of 128 x 128 tiles most of the chip has no work, and a tile's time is its
+// own MMAs' (N_G 350, 3840 pairs, one frequency, six BF16 products: 9 tiles,
+// 254 us).  The sums over pairs cannot be shared out (their FP32 order is
+// fixed), but the components and columns can: a stage's MMAs take a quarter of
+// the math (N = 64 reads the same A: about 0.38 of the time), for three quarters of the
+// loads, which then set the pace (64-byte rows).  Same bits; whole accumulate calls, N_G 350,
+// one frequency: 3840 pairs BF16 286 -> 160 us, 4096 pairs FP16 201 -> 131 us, 256
+// pairs 62 -> 46 us; 500 points and two frequencies (128 items): 311 -> 173 us.
+// Roles, barriers and bounded waits as in k_contract_tc, the ring as in the
+// CTA-pair kernel (B tiles of 64 rows).
+// ---------------------------------------------------------------------------
+template <bool BF16, int NT>
+__global__ void __launch_bounds__(THREADS, 1)
+k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status) {
+  using RG = Ring2<NT>;
+  constexpr int STAGES = RG::STAGES, STAGE_BYTES = RG::STAGE_BYTES, PL = RG::PLANES;
+  extern __shared__ __align__(1024) unsigned char smem_tcn[];
+  unsigned char* tiles = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_tcn) + 1023) & ~uintptr_t(1023));
+  struct Bars {
+    uint64_t full[4], empty[4], tfull[2], tempty[2], done;
+    uint32_t tmem_base;
+  };
+  static_assert(STAGES <= 4 && sizeof(Bars) <= BAR_BYTES, "barriers overlap");
+  Bars* bar = reinterpret_cast<Bars*>(tiles + RING2_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nK = P.nK, np = P.n_products, ck = P.chain_k;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&bar->tfull[b], 1);
+      tc::mbar_init(&bar->tempty[b], EPI_WARPS);
+    }
+    tc::mbar_init(&bar->done, 1);
+    tc::fence_mbar_init();
+    for (int q = 0; q < P.n_q; ++q) {
+      tc::prefetch_tmap(&P.tmA[q]);
+      tc::prefetch_tmap(&P.tmB[q]);
+    }
+  }
+  if (warp == 1) {
+    tc::tmem_alloc(&bar->tmem_base, TMEM_COLS);
+    tc::tmem_relinquish();
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tbase = bar->tmem_base;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer ----------------
+      const int nt = (NT == 3 && np != 6) ? 2 : NT;
+      int64_t gs = 0;
+      int slot = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int64_t item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
+        int q, iw, tm, tn;
+        decode_item(P, item >> 1, q, iw, tm, tn);
+        const int plane0 = iw * PL;
+        for (int kc = 0; kc < nK; ++kc, ++gs) {
+          const int s = slot;
+          if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, status, 1, WAIT_BUDGET_NS)) { ok = false; break; }
+          if (++slot == STAGES) {
+            slot = 0;
+            ph ^= 1u;
+          }
+          tc::mbar_arrive_expect_tx(&bar->full[s], 2 * nt * (RG::A_BYTES + RG::B_BYTES));
+          unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+#pragma unroll
+          for (int j = 0; j < PL; ++j) {
+            if (j % NT >= nt) continue;
+            tc::tma_load_3d(st + j * RG::A_BYTES, &P.tmA[q], &bar->full[s], kc * BK, tm * BM, plane0 + j);
+            tc::tma_load_3d(st + PL * RG::A_BYTES + j * RG::B_BYTES, &P.tmB[q], &bar->full[s], kc * BK, tn * COMP_N,
+                            j);
+          }
+        }
+      }
+      // copies still in flight must land before the CTA may exit
+      for (int64_t g = max((int64_t)0, gs - STAGES); g < gs; ++g)
+        tc::mbar_wait(&bar->full[g % STAGES], (uint32_t)((g / STAGES) & 1), status, 1, WAIT_BUDGET_NS);
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      // ---------------- MMA issuer ----------------
+      int64_t gc = 0;
+      int slot = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int64_t item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
+        const bool im = (item & 1) != 0;
+        for (int kc = 0, pos = 0; kc < nK; ++kc) {
+          const int buf = (int)(gc & 1);
+          const bool first = pos == 0;
+          if (first) {
+            if (!tc::mbar_wait(&bar->tempty[buf], (uint32_t)(((gc >> 1) & 1) ^ 1), status, 1, WAIT_BUDGET_NS)) {
+              ok = false;
+              break;
+            }
+            tc::fence_after();
+          }
+          const int s = slot;
+          if (!tc::mbar_wait(&bar->full[s], ph, status, 1, WAIT_BUDGET_NS)) {
+            ok = false;
+            break;
+          }
+          if (++slot == STAGES) {
+            slot = 0;
+            ph ^= 1u;
+          }
+          tc::fence_after();
+          const unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+          const uint32_t d = tbase + buf * 256;
+          if (im) issue_stage<BF16, NT, false, COMP_IM>(st, d, d, first, np);
+          else issue_stage<BF16, NT, false, COMP_RE>(st, d, d, first, np);
+          tc::mma_commit(&bar->empty[s]);
+          if (++pos == ck || kc == nK - 1) {
+            tc::mma_commit(&bar->tfull[buf]);
+            ++gc;
+            pos = 0;
+          }
+        }
+      }
+      tc::mma_commit(&bar->done);
+      tc::mbar_wait(&bar->done, 0, status, 1, WAIT_BUDGET_NS);
+    }
+  } else if (warp >= EPI_WARP0) {
+    // ---------------- epilogue: 32 columns per warp ----------------
+    const int quad = warp & 3, half = (warp - EPI_WARP0) >> 2;
+    const int nch = (nK + ck - 1) / ck;
+    int64_t gc = 0;
+    bool ok = true;
+    for (int64_t item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
+      float sum[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) sum[i] = 0.f;
+      for (int c = 0; c < nch; ++c, ++gc) {
+        const int buf = (int)(gc & 1);
+        if (!tc::mbar_wait(&bar->tfull[buf], (uint32_t)((gc >> 1) & 1), status, 1, WAIT_BUDGET_NS)) {
+          ok = false;
+          break;
+        }
+        tc::fence_after();
+        float v[32];
+        tc::tmem_ld32(tbase + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * 32, v);
+        tc::tmem_ld_wait();
+        tc::reg_after_wait(v);
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&bar->tempty[buf]);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) sum[i] += v[i];
+      }
+      if (!ok) break;
+      int q, iw, tm, tn;
+      decode_item(P, item >> 1, q, iw, tm, tn);
+      const int comp = (int)(item & 1), nG = P.nG[q], G = tm * BM + quad * 32 + lane, Hb = tn * COMP_N + half * 32;
+      if (G < nG) {
+        const int k = exponent_of_pow2(P.inv[q][iw]);
+        double* row = reinterpret_cast<double*>(P.chi[q] + ((size_t)iw * nG + G) * nG) + comp;
+#pragma unroll
+        for (int i = 0; i < 32; ++i)
+          if (Hb + i < nG && Hb + i != G) red_add_pow2(row + 2 * (Hb + i), sum[i], k);
+        if ((unsigned)(G - Hb) < 32u) {
+          const double2 d = P.diag[q][(size_t)iw * P.tiles_m[q] * BM + G];
+          atomicAdd(row + 2 * G, comp ? d.y : d.x);
+        }
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == 1) tc::tmem_dealloc(tbase, TMEM_COLS);
+}
+
 template <bool BF16, int NT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_contract_tc2(const __grid_constant__ TcBatch P, int* __restrict__ status) {
@@ -1389,6 +1584,18 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
   memset(P, 0, sizeof(TcBatch));
   int64_t items = 0;
   const bool pair = p->tc_pair != 0;
+  int dev = 0, nsm = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  // Narrow items where all of them run at once: at 128 and 144 items of 152 SMs still 1.8x (BF16), and
+  // below that 1.2x (256 pairs) to 2x; a second round of them takes as long as one round of whole tiles.
+  bool narrow = !pair && !p->tc_herm;
+  if (narrow) {
+    int64_t n = 0;
+    for (int j = 0; j < n_jobs; ++j)
+      n += 2 * (int64_t)p->n_freq * ((jobs[j].nG + BM - 1) / BM) * ((jobs[j].nG + COMP_N - 1) / COMP_N);
+    narrow = n <= nsm;
+  }
   for (int j = 0; j < n_jobs; ++j) {
     const TcJob& jb = jobs[j];
     const int nGp = round_up_i(jb.nG, pair ? 2 * BM : BM);
@@ -1398,7 +1605,7 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
       if (e != cudaSuccess) { delete P; return e; }
       if (mode == 1) continue;
     }
-    if (!encode_planes(&P->tmB[j], w.Bp, BF16, Kp, nGp, b_planes(p), why, pair ? BN / 2 : BN) ||
+    if (!encode_planes(&P->tmB[j], w.Bp, BF16, Kp, nGp, b_planes(p), why, pair || narrow ? BN / 2 : BN) ||
         !encode_planes(&P->tmA[j], w.Ap, BF16, Kp, nGp, 2 * NT * n_parts(p) * p->n_freq, why, BM)) {
       delete P;
       return cudaErrorInvalidValue;
@@ -1409,13 +1616,13 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
     P->tbar[j] = w.tbar;
     P->diag[j] = w.diag;
     P->nG[j] = jb.nG;
-    const int TM = nGp / (pair ? 2 * BM : BM), TN = nGp / BN;
+    const int TM = nGp / (pair ? 2 * BM : BM), TN = narrow ? (jb.nG + COMP_N - 1) / COMP_N : nGp / BN;
     P->tiles_m[j] = TM;
     P->tiles_n[j] = TN;
     // Hermitian mode: row tm holds the TN - rr tm tiles from column rr tm on
     P->tpf[j] = p->tc_herm ? (int64_t)(TN / TM) * TM * (TM + 1) / 2 : (int64_t)TM * TN;
     P->item0[j] = items;
-    items += P->tpf[j] * p->n_freq;
+    items += P->tpf[j] * p->n_freq;   // narrow items: two (Re, Im) each
   }
   if (mode == 1) {
     delete P;
@@ -1430,10 +1637,7 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
   P->chain_k = std::max(1, p->chain_pairs / BK);
   P->n_products = p->n_products;
   P->group = p->tc_group > 0 ? p->tc_group : 8;
-  P->total_items = items;
-  int dev = 0, nsm = 152;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  P->total_items = narrow ? 2 * items : items;
   cudaError_t e;
   if (pair) {
     if (!regs_match(k_contract_tc2<BF16, NT>, why)) { delete P; return cudaErrorNotSupported; }
@@ -1443,6 +1647,12 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
     const int pairs = (int)std::min<int64_t>(items, (int64_t)(nsm / 2));
     ProfScope ps(p, CHI0_K_CONTRACT_TC, s, 1);
     k_contract_tc2<BF16, NT><<<2 * pairs, THREADS, SMEM2_BYTES, s>>>(*P, p->d_status);
+  } else if (narrow) {
+    e = cudaFuncSetAttribute(k_contract_tc_narrow<BF16, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)SMEM2_BYTES);
+    if (e != cudaSuccess) { delete P; return e; }
+    ProfScope ps(p, CHI0_K_CONTRACT_TC, s, 1);
+    k_contract_tc_narrow<BF16, NT><<<(int)P->total_items, THREADS, SMEM2_BYTES, s>>>(*P, p->d_status);
   } else {
     if (!regs_match(k_contract_tc<BF16, NT>, why)) { delete P; return cudaErrorNotSupported; }
     e = cudaFuncSetAttribute(k_contract_tc<BF16, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
