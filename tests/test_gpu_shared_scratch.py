@@ -1,3 +1,4 @@
+"""Workspaces that FP64 plans allocate on demand: a captured call keeps its memory when a
 later call outgrows it, and wavefunction transforms on several streams do not
 overwrite each other's.  Equal calls give equal bits."""
 import numpy as np
