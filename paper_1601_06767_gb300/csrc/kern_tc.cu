@@ -1040,14 +1040,188 @@ template <int NT> struct Ring2 {
   static constexpr int STAGES = RING2_BYTES / STAGE_BYTES;   // 4 for NT = 2, 3 for NT = 3
 };
 
+template <bool BF16, int NT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+k_contract_tc2(const __grid_constant__ TcBatch P, int* __restrict__ status) {
+  using RG = Ring2<NT>;
+  constexpr int STAGES = RG::STAGES, STAGE_BYTES = RG::STAGE_BYTES, PL = RG::PLANES;
+  static_assert(STAGES <= MAX_STAGES + 1, "barrier array too small");
+  extern __shared__ __align__(1024) unsigned char smem_tc2[];
+  unsigned char* tiles = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_tc2) + 1023) & ~uintptr_t(1023));
+  struct Bars {
+    uint64_t full[4], empty[4], tfull[2], tempty[2], done;
+    uint32_t tmem_base;
+  };
+  static_assert(sizeof(Bars) <= BAR_BYTES, "barriers overlap the transpose buffers");
+  Bars* bar = reinterpret_cast<Bars*>(tiles + RING2_BYTES);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = tc::cluster_rank();
+  const bool leader = rank == 0;
+  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int nK = P.nK;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      tc::mbar_init(&bar->full[s], 1);
+      tc::mbar_init(&bar->empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&bar->tfull[b], 1);
+      tc::mbar_init(&bar->tempty[b], 2 * EPI_WARPS);
+    }
+    tc::mbar_init(&bar->done, 1);
+    tc::fence_mbar_init();
+    for (int q = 0; q < P.n_q; ++q) {
+      tc::prefetch_tmap(&P.tmA[q]);
+      tc::prefetch_tmap(&P.tmB[q]);
+    }
+  }
+  if (warp == 1) {
+    tc::tmem_alloc_pair(&bar->tmem_base, TMEM_COLS);
+    tc::tmem_relinquish_pair();
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();      // barriers of both CTAs initialised before any remote use
+  tc::fence_after();
+  const uint32_t tbase = bar->tmem_base;
+
+  // warpgroup 0 (producer, issuer, two idle warps) runs on REG_LOW registers,
+  // the epilogue warpgroups on REG_HIGH
+  if (warp < EPI_WARP0) {
+  tc::setmaxnreg_dec<REG_LOW>();
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer (both CTAs) ----------------
+      int64_t gs = 0;
+      int slot = 0;        // ring slot of stage gs and its phase parity
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
+        int q, iw, tm, tn;
+        decode_item(P, item, q, iw, tm, tn);
+        const int arow = tm * 2 * BM + (int)rank * BM;     // this CTA's 128 rows of A
+        const int brow = tn * BN + (int)rank * (BN / 2);   // this CTA's 64 rows of B
+        for (int part = 0; part < P.n_parts && ok; ++part) {
+          const int npp = part_products(P, q, iw, part);
+          const bool one = npp == 1;                  // k-slices of term 0 in the term slots
+          const int nt = one ? 1 : ((NT == 3 && npp != 6) ? 2 : NT);
+          const int nks = part_stages<NT>(P, q, iw, part);
+          const int plane0 = (part * P.n_freq + iw) * PL;
+          for (int kc = 0; kc < nks; ++kc, ++gs) {
+            const int s = slot;
+            if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, status, 1, WAIT_BUDGET_NS)) { ok = false; break; }
+            if (++slot == STAGES) {
+              slot = 0;
+              ph ^= 1u;
+            }
+            const int ns = one ? min(NT, nK - kc * NT) : nt;
+            // the first CTA's barrier counts the loads of both CTAs
+            if (leader) tc::mbar_arrive_expect_tx(&bar->full[s], 4 * ns * (RG::A_BYTES + RG::B_BYTES));
+            const uint32_t fb = tc::mapa(&bar->full[s], 0);
+            unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+#pragma unroll
+            for (int j = 0; j < PL; ++j) {
+              const int t = j % NT;
+              if (t >= ns) continue;
+              const int pa = one ? (j / NT) * NT : j;
+              const int pb = (BF16 && one) ? 2 * NT + j / NT : pa;
+              const int kx = one ? (kc * NT + t) * BK : kc * BK;
+              tc::tma_load_3d_pair(st + j * RG::A_BYTES, &P.tmA[q], fb, kx, arow, plane0 + pa);
+              tc::tma_load_3d_pair(st + PL * RG::A_BYTES + j * RG::B_BYTES, &P.tmB[q], fb, kx, brow, pb);
+            }
+          }
+        }
+      }
+      // copies of this CTA still in flight land before it may exit: wait until the
+      // pair's MMA has released the stages it issued last
+      for (int64_t g = max((int64_t)0, gs - STAGES); g < gs; ++g)
+        tc::mbar_wait(&bar->empty[g % STAGES], (uint32_t)((g / STAGES) & 1), status, 1, WAIT_BUDGET_NS);
+    }
+  } else if (warp == 1) {
+    if (lane == 0 && leader) {
+      // ---------------- MMA issuer (first CTA of the pair) ----------------
+      int64_t gs = 0, gc = 0;
+      int slot = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
+        int q, iw, tm, tn;
+        decode_item(P, item, q, iw, tm, tn);
+        for (int part = 0; part < P.n_parts && ok; ++part) {
+          const int np = part_products(P, q, iw, part), nks = part_stages<NT>(P, q, iw, part);
+          const int ck = part_chain(P, q, iw, part, nks);
+          // pos: stage within the accumulation chain; s, ph: ring slot and its phase (counters,
+          // not divisions, on this single issuing thread)
+          for (int kc = 0, pos = 0; kc < nks; ++kc, ++gs) {
+            const int buf = (int)(gc & 1);
+            const bool first = pos == 0;
+            if (first) {
+              if (!tc::mbar_wait(&bar->tempty[buf], (uint32_t)(((gc >> 1) & 1) ^ 1), status, 1, WAIT_BUDGET_NS)) {
+                ok = false;
+                break;
+              }
+              tc::fence_after();
+            }
+            const int s = slot;
+            if (!tc::mbar_wait(&bar->full[s], ph, status, 1, WAIT_BUDGET_NS)) {
+              ok = false;
+              break;
+            }
+            if (++slot == STAGES) {
+              slot = 0;
+              ph ^= 1u;
+            }
+            tc::fence_after();
+            const unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
+            const uint32_t d_re = tbase + buf * 256, d_im = d_re + 128;
+            if (np == 1) issue_stage_1p<false, NT, true>(st, d_re, d_im, first, min(NT, nK - kc * NT));
+            else issue_stage<BF16, NT, true>(st, d_re, d_im, first, np);
+            tc::mma_commit_pair(&bar->empty[s], 0x3);
+            if (++pos == ck || kc == nks - 1) {
+              tc::mma_commit_pair(&bar->tfull[buf], 0x3);
+              ++gc;
+              pos = 0;
+            }
+          }
+        }
+      }
+      tc::mma_commit_pair(&bar->done, 0x1);
+      tc::mbar_wait(&bar->done, 0, status, 1, WAIT_BUDGET_NS);
+    }
+  }
+  } else {
+    tc::setmaxnreg_inc<REG_HIGH>();
+    // ---------------- epilogue (both CTAs, own 128 rows) ----------------
+    const int ew = warp - EPI_WARP0, quad = warp & 3, half = ew >> 2;
+    const int row = quad * 32 + lane;
+    float* xb = reinterpret_cast<float*>(tiles + RING2_BYTES + BAR_BYTES) + ew * XBUF_FLOATS;
+    int64_t gc = 0;
+    bool ok = true;
+    for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
+      int q, iw, tm, tn;
+      decode_item(P, item, q, iw, tm, tn);
+      ok = epilogue_item<NT, true>(P, bar, tbase, quad, half, lane, q, iw, tm * 2 * BM + (int)rank * BM + row, tn, gc,
+                                   status, xb);
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::cluster_sync();      // neither CTA leaves while the pair's MMAs may still read its operands
+  tc::fence_after();
+  if (warp == 1) tc::tmem_dealloc_pair(tbase, TMEM_COLS);
+}
+
 // ---------------------------------------------------------------------------
 // Narrow items (plain mode): 128 rows x 64 columns of Re chi0 or of Im chi0.  With a
 // handful of 128 x 128 tiles most of the chip has no work, and a tile's time is its
 // own MMAs' (N_G 350, 3840 pairs, one frequency, six BF16 products: 9 tiles,
 // 254 us).  The sums over pairs cannot be shared out (their FP32 order is
-// fixed), but the components and columns can: a stage's MMAs take a quarter of
-// the math (N = 64 reads the same A: about 0.38 of the time), for three quarters of the
-// loads, which then set the pace (64-byte rows).  Same bits; whole accumulate calls, N_G 350,
+// fixed), but the components and columns can: a stage has half the MMAs, of half the
+// columns.  A stage still takes about half the time, 1.0 us for its 24 MMAs (six products):
+// loads of 512-byte rows, one load per operand and four accumulators left that
+// as it was, so what remains is the MMAs' own time.  Same bits; whole accumulate calls, N_G 350,
 // one frequency: 3840 pairs BF16 286 -> 160 us, 4096 pairs FP16 201 -> 131 us, 256
 // pairs 62 -> 46 us; 500 points and two frequencies (128 items): 311 -> 173 us.
 // Roles, barriers and bounded waits as in k_contract_tc, the ring as in the
@@ -1221,179 +1395,6 @@ k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status
   __syncthreads();
   tc::fence_after();
   if (warp == 1) tc::tmem_dealloc(tbase, TMEM_COLS);
-}
-
-template <bool BF16, int NT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
-k_contract_tc2(const __grid_constant__ TcBatch P, int* __restrict__ status) {
-  using RG = Ring2<NT>;
-  constexpr int STAGES = RG::STAGES, STAGE_BYTES = RG::STAGE_BYTES, PL = RG::PLANES;
-  static_assert(STAGES <= MAX_STAGES + 1, "barrier array too small");
-  extern __shared__ __align__(1024) unsigned char smem_tc2[];
-  unsigned char* tiles = reinterpret_cast<unsigned char*>(
-      (reinterpret_cast<uintptr_t>(smem_tc2) + 1023) & ~uintptr_t(1023));
-  struct Bars {
-    uint64_t full[4], empty[4], tfull[2], tempty[2], done;
-    uint32_t tmem_base;
-  };
-  static_assert(sizeof(Bars) <= BAR_BYTES, "barriers overlap the transpose buffers");
-  Bars* bar = reinterpret_cast<Bars*>(tiles + RING2_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = tc::cluster_rank();
-  const bool leader = rank == 0;
-  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
-  const int nK = P.nK;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      tc::mbar_init(&bar->full[s], 1);
-      tc::mbar_init(&bar->empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      tc::mbar_init(&bar->tfull[b], 1);
-      tc::mbar_init(&bar->tempty[b], 2 * EPI_WARPS);
-    }
-    tc::mbar_init(&bar->done, 1);
-    tc::fence_mbar_init();
-    for (int q = 0; q < P.n_q; ++q) {
-      tc::prefetch_tmap(&P.tmA[q]);
-      tc::prefetch_tmap(&P.tmB[q]);
-    }
-  }
-  if (warp == 1) {
-    tc::tmem_alloc_pair(&bar->tmem_base, TMEM_COLS);
-    tc::tmem_relinquish_pair();
-  }
-  tc::fence_before();
-  __syncthreads();
-  tc::cluster_sync();      // barriers of both CTAs initialised before any remote use
-  tc::fence_after();
-  const uint32_t tbase = bar->tmem_base;
-
-  // warpgroup 0 (producer, issuer, two idle warps) runs on REG_LOW registers,
-  // the epilogue warpgroups on REG_HIGH
-  if (warp < EPI_WARP0) {
-  tc::setmaxnreg_dec<REG_LOW>();
-  if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer (both CTAs) ----------------
-      int64_t gs = 0;
-      int slot = 0;        // ring slot of stage gs and its phase parity
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
-        int q, iw, tm, tn;
-        decode_item(P, item, q, iw, tm, tn);
-        const int arow = tm * 2 * BM + (int)rank * BM;     // this CTA's 128 rows of A
-        const int brow = tn * BN + (int)rank * (BN / 2);   // this CTA's 64 rows of B
-        for (int part = 0; part < P.n_parts && ok; ++part) {
-          const int npp = part_products(P, q, iw, part);
-          const bool one = npp == 1;                  // k-slices of term 0 in the term slots
-          const int nt = one ? 1 : ((NT == 3 && npp != 6) ? 2 : NT);
-          const int nks = part_stages<NT>(P, q, iw, part);
-          const int plane0 = (part * P.n_freq + iw) * PL;
-          for (int kc = 0; kc < nks; ++kc, ++gs) {
-            const int s = slot;
-            if (!tc::mbar_wait(&bar->empty[s], ph ^ 1u, status, 1, WAIT_BUDGET_NS)) { ok = false; break; }
-            if (++slot == STAGES) {
-              slot = 0;
-              ph ^= 1u;
-            }
-            const int ns = one ? min(NT, nK - kc * NT) : nt;
-            // the first CTA's barrier counts the loads of both CTAs
-            if (leader) tc::mbar_arrive_expect_tx(&bar->full[s], 4 * ns * (RG::A_BYTES + RG::B_BYTES));
-            const uint32_t fb = tc::mapa(&bar->full[s], 0);
-            unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
-#pragma unroll
-            for (int j = 0; j < PL; ++j) {
-              const int t = j % NT;
-              if (t >= ns) continue;
-              const int pa = one ? (j / NT) * NT : j;
-              const int pb = (BF16 && one) ? 2 * NT + j / NT : pa;
-              const int kx = one ? (kc * NT + t) * BK : kc * BK;
-              tc::tma_load_3d_pair(st + j * RG::A_BYTES, &P.tmA[q], fb, kx, arow, plane0 + pa);
-              tc::tma_load_3d_pair(st + PL * RG::A_BYTES + j * RG::B_BYTES, &P.tmB[q], fb, kx, brow, pb);
-            }
-          }
-        }
-      }
-      // copies of this CTA still in flight land before it may exit: wait until the
-      // pair's MMA has released the stages it issued last
-      for (int64_t g = max((int64_t)0, gs - STAGES); g < gs; ++g)
-        tc::mbar_wait(&bar->empty[g % STAGES], (uint32_t)((g / STAGES) & 1), status, 1, WAIT_BUDGET_NS);
-    }
-  } else if (warp == 1) {
-    if (lane == 0 && leader) {
-      // ---------------- MMA issuer (first CTA of the pair) ----------------
-      int64_t gs = 0, gc = 0;
-      int slot = 0;
-      uint32_t ph = 0;
-      bool ok = true;
-      for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
-        int q, iw, tm, tn;
-        decode_item(P, item, q, iw, tm, tn);
-        for (int part = 0; part < P.n_parts && ok; ++part) {
-          const int np = part_products(P, q, iw, part), nks = part_stages<NT>(P, q, iw, part);
-          const int ck = part_chain(P, q, iw, part, nks);
-          // pos: stage within the accumulation chain; s, ph: ring slot and its phase (counters,
-          // not divisions, on this single issuing thread)
-          for (int kc = 0, pos = 0; kc < nks; ++kc, ++gs) {
-            const int buf = (int)(gc & 1);
-            const bool first = pos == 0;
-            if (first) {
-              if (!tc::mbar_wait(&bar->tempty[buf], (uint32_t)(((gc >> 1) & 1) ^ 1), status, 1, WAIT_BUDGET_NS)) {
-                ok = false;
-                break;
-              }
-              tc::fence_after();
-            }
-            const int s = slot;
-            if (!tc::mbar_wait(&bar->full[s], ph, status, 1, WAIT_BUDGET_NS)) {
-              ok = false;
-              break;
-            }
-            if (++slot == STAGES) {
-              slot = 0;
-              ph ^= 1u;
-            }
-            tc::fence_after();
-            const unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
-            const uint32_t d_re = tbase + buf * 256, d_im = d_re + 128;
-            if (np == 1) issue_stage_1p<false, NT, true>(st, d_re, d_im, first, min(NT, nK - kc * NT));
-            else issue_stage<BF16, NT, true>(st, d_re, d_im, first, np);
-            tc::mma_commit_pair(&bar->empty[s], 0x3);
-            if (++pos == ck || kc == nks - 1) {
-              tc::mma_commit_pair(&bar->tfull[buf], 0x3);
-              ++gc;
-              pos = 0;
-            }
-          }
-        }
-      }
-      tc::mma_commit_pair(&bar->done, 0x1);
-      tc::mbar_wait(&bar->done, 0, status, 1, WAIT_BUDGET_NS);
-    }
-  }
-  } else {
-    tc::setmaxnreg_inc<REG_HIGH>();
-    // ---------------- epilogue (both CTAs, own 128 rows) ----------------
-    const int ew = warp - EPI_WARP0, quad = warp & 3, half = ew >> 2;
-    const int row = quad * 32 + lane;
-    float* xb = reinterpret_cast<float*>(tiles + RING2_BYTES + BAR_BYTES) + ew * XBUF_FLOATS;
-    int64_t gc = 0;
-    bool ok = true;
-    for (int64_t item = pair; item < P.total_items && ok; item += npairs) {
-      int q, iw, tm, tn;
-      decode_item(P, item, q, iw, tm, tn);
-      ok = epilogue_item<NT, true>(P, bar, tbase, quad, half, lane, q, iw, tm * 2 * BM + (int)rank * BM + row, tn, gc,
-                                   status, xb);
-    }
-  }
-  tc::fence_before();
-  __syncthreads();
-  tc::cluster_sync();      // neither CTA leaves while the pair's MMAs may still read its operands
-  tc::fence_after();
-  if (warp == 1) tc::tmem_dealloc_pair(tbase, TMEM_COLS);
 }
 
 // Diagnostic: wait on an mbarrier that nothing arrives on, with the same
