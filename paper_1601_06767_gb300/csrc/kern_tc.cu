@@ -367,16 +367,16 @@ static_assert(SMEM_BYTES <= 227 * 1024, "shared memory above the per-block limit
 // to one stage and ordered smallest-first: every term product t_i t_j with
 // i + j > 0 goes in while the accumulator is still small, and the t0 t0
 // products (the only large ones) come last.
-// COMP: both components (COMP_BOTH), or Re or Im alone into d_re over COMP_N columns
+// COMP: both components (COMP_BOTH), or Re or Im alone into d_re over CN columns
 // (k_contract_tc_narrow); an accumulator sees the same products in the same order.
-constexpr int COMP_BOTH = 0, COMP_RE = 1, COMP_IM = 2, COMP_N = 64;
-template <bool BF16, int NT, bool PAIR, int NPROD, int COMP = COMP_BOTH>
+constexpr int COMP_BOTH = 0, COMP_RE = 1, COMP_IM = 2;
+template <bool BF16, int NT, bool PAIR, int NPROD, int COMP = COMP_BOTH, int CN = BN>
 __device__ __forceinline__ void issue_stage_np(const unsigned char* st, uint32_t d_re, uint32_t d_im, bool first) {
   constexpr int P = 2 * NT;
   // in a CTA pair each CTA holds 128 rows of A and 64 rows of B; the MMA spans 256 rows
-  constexpr int B_BYTES = PAIR || COMP ? TILE_BYTES / 2 : TILE_BYTES;
-  const uint32_t id_pos = tc::idesc_f16(BF16, false, PAIR ? 2 * BM : BM, COMP ? COMP_N : BN);
-  [[maybe_unused]] const uint32_t id_neg = tc::idesc_f16(BF16, true, PAIR ? 2 * BM : BM, COMP ? COMP_N : BN);
+  constexpr int B_BYTES = PAIR ? TILE_BYTES / 2 : CN * BK * 2;
+  const uint32_t id_pos = tc::idesc_f16(BF16, false, PAIR ? 2 * BM : BM, CN);
+  [[maybe_unused]] const uint32_t id_neg = tc::idesc_f16(BF16, true, PAIR ? 2 * BM : BM, CN);
   // one descriptor for the stage; tiles and K steps are constant offsets of its address field
   const uint64_t d0 = tc::sdesc_kmajor_sw64(st);
   constexpr uint64_t kTile = TILE_BYTES >> 4, kBTile = B_BYTES >> 4, kB0 = (uint64_t)(P * TILE_BYTES) >> 4;
@@ -469,13 +469,13 @@ __device__ __forceinline__ void issue_stage_1p(const unsigned char* st, uint32_t
 }
 
 // the product count as a compile-time constant: no per-MMA test in the issue loop
-template <bool BF16, int NT, bool PAIR = false, int COMP = COMP_BOTH>
+template <bool BF16, int NT, bool PAIR = false, int COMP = COMP_BOTH, int CN = BN>
 __device__ __forceinline__ void issue_stage(const unsigned char* st, uint32_t d_re, uint32_t d_im, bool first,
                                             int n_products) {
-  if (n_products == 6) issue_stage_np<BF16, NT, PAIR, 6, COMP>(st, d_re, d_im, first);
-  else if (n_products == 4) issue_stage_np<BF16, NT, PAIR, 4, COMP>(st, d_re, d_im, first);
-  else if (n_products == 1) issue_stage_np<BF16, NT, PAIR, 1, COMP>(st, d_re, d_im, first);
-  else issue_stage_np<BF16, NT, PAIR, 3, COMP>(st, d_re, d_im, first);
+  if (n_products == 6) issue_stage_np<BF16, NT, PAIR, 6, COMP, CN>(st, d_re, d_im, first);
+  else if (n_products == 4) issue_stage_np<BF16, NT, PAIR, 4, COMP, CN>(st, d_re, d_im, first);
+  else if (n_products == 1) issue_stage_np<BF16, NT, PAIR, 1, COMP, CN>(st, d_re, d_im, first);
+  else issue_stage_np<BF16, NT, PAIR, 3, COMP, CN>(st, d_re, d_im, first);
 }
 
 // One persistent launch over a list of work items (q-point, frequency, 128x128
@@ -1214,24 +1214,24 @@ k_contract_tc2(const __grid_constant__ TcBatch P, int* __restrict__ status) {
 }
 
 // ---------------------------------------------------------------------------
-// Narrow items (plain mode): 128 rows x 64 columns of Re chi0 or of Im chi0.  With a
+// Narrow items (plain mode): 128 rows x CN (64 or 128) columns of Re chi0 or of Im chi0.  With a
 // handful of 128 x 128 tiles most of the chip has no work, and a tile's time is its
 // own MMAs' (N_G 350, 3840 pairs, one frequency, six BF16 products: 9 tiles,
 // 254 us).  The sums over pairs cannot be shared out (their FP32 order is
 // fixed), but the components and columns can: a stage has half the MMAs, of half the
-// columns.  A stage still takes about half the time, 1.0 us for its 24 MMAs (six products):
-// loads of 512-byte rows, one load per operand and four accumulators left that
-// as it was, so what remains is the MMAs' own time.  Same bits; whole accumulate calls, N_G 350,
+// columns.  It takes 1.0 us of 2.1 (six products; about 1.5 with 128 columns, whose ring has two
+// stages): loads of 512-byte rows, one load per operand and four accumulators did
+// not shorten it.  Same bits; whole accumulate calls with 64 columns, N_G 350,
 // one frequency: 3840 pairs BF16 286 -> 160 us, 4096 pairs FP16 201 -> 131 us, 256
 // pairs 62 -> 46 us; 500 points and two frequencies (128 items): 311 -> 173 us.
-// Roles, barriers and bounded waits as in k_contract_tc, the ring as in the
-// CTA-pair kernel (B tiles of 64 rows).
+// Roles, barriers and bounded waits as in k_contract_tc, the ring's memory as
+// in the CTA-pair kernel.
 // ---------------------------------------------------------------------------
-template <bool BF16, int NT>
+template <bool BF16, int NT, int CN>
 __global__ void __launch_bounds__(THREADS, 1)
 k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status) {
-  using RG = Ring2<NT>;
-  constexpr int STAGES = RG::STAGES, STAGE_BYTES = RG::STAGE_BYTES, PL = RG::PLANES;
+  constexpr int PL = 2 * NT, A_BYTES = TILE_BYTES, B_BYTES = CN * BK * 2;
+  constexpr int STAGE_BYTES = PL * (A_BYTES + B_BYTES), STAGES = RING2_BYTES / STAGE_BYTES;
   extern __shared__ __align__(1024) unsigned char smem_tcn[];
   unsigned char* tiles = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_tcn) + 1023) & ~uintptr_t(1023));
@@ -1288,13 +1288,13 @@ k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status
             slot = 0;
             ph ^= 1u;
           }
-          tc::mbar_arrive_expect_tx(&bar->full[s], 2 * nt * (RG::A_BYTES + RG::B_BYTES));
+          tc::mbar_arrive_expect_tx(&bar->full[s], 2 * nt * (A_BYTES + B_BYTES));
           unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
 #pragma unroll
           for (int j = 0; j < PL; ++j) {
             if (j % NT >= nt) continue;
-            tc::tma_load_3d(st + j * RG::A_BYTES, &P.tmA[q], &bar->full[s], kc * BK, tm * BM, plane0 + j);
-            tc::tma_load_3d(st + PL * RG::A_BYTES + j * RG::B_BYTES, &P.tmB[q], &bar->full[s], kc * BK, tn * COMP_N,
+            tc::tma_load_3d(st + j * A_BYTES, &P.tmA[q], &bar->full[s], kc * BK, tm * BM, plane0 + j);
+            tc::tma_load_3d(st + PL * A_BYTES + j * B_BYTES, &P.tmB[q], &bar->full[s], kc * BK, tn * CN,
                             j);
           }
         }
@@ -1334,8 +1334,8 @@ k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status
           tc::fence_after();
           const unsigned char* st = tiles + (size_t)s * STAGE_BYTES;
           const uint32_t d = tbase + buf * 256;
-          if (im) issue_stage<BF16, NT, false, COMP_IM>(st, d, d, first, np);
-          else issue_stage<BF16, NT, false, COMP_RE>(st, d, d, first, np);
+          if (im) issue_stage<BF16, NT, false, COMP_IM, CN>(st, d, d, first, np);
+          else issue_stage<BF16, NT, false, COMP_RE, CN>(st, d, d, first, np);
           tc::mma_commit(&bar->empty[s]);
           if (++pos == ck || kc == nK - 1) {
             tc::mma_commit(&bar->tfull[buf]);
@@ -1348,15 +1348,16 @@ k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status
       tc::mbar_wait(&bar->done, 0, status, 1, WAIT_BUDGET_NS);
     }
   } else if (warp >= EPI_WARP0) {
-    // ---------------- epilogue: 32 columns per warp ----------------
+    // ---------------- epilogue: CN / 2 columns per warp ----------------
+    constexpr int W = CN / 2;
     const int quad = warp & 3, half = (warp - EPI_WARP0) >> 2;
     const int nch = (nK + ck - 1) / ck;
     int64_t gc = 0;
     bool ok = true;
     for (int64_t item = blockIdx.x; item < P.total_items && ok; item += gridDim.x) {
-      float sum[32];
+      float sum[W];
 #pragma unroll
-      for (int i = 0; i < 32; ++i) sum[i] = 0.f;
+      for (int i = 0; i < W; ++i) sum[i] = 0.f;
       for (int c = 0; c < nch; ++c, ++gc) {
         const int buf = (int)(gc & 1);
         if (!tc::mbar_wait(&bar->tfull[buf], (uint32_t)((gc >> 1) & 1), status, 1, WAIT_BUDGET_NS)) {
@@ -1364,27 +1365,30 @@ k_contract_tc_narrow(const __grid_constant__ TcBatch P, int* __restrict__ status
           break;
         }
         tc::fence_after();
-        float v[32];
-        tc::tmem_ld32(tbase + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * 32, v);
+        float v[W / 32][32];
+#pragma unroll
+        for (int h = 0; h < W / 32; ++h)
+          tc::tmem_ld32(tbase + ((uint32_t)(quad * 32) << 16) + buf * 256 + half * W + 32 * h, v[h]);
         tc::tmem_ld_wait();
-        tc::reg_after_wait(v);
+#pragma unroll
+        for (int h = 0; h < W / 32; ++h) tc::reg_after_wait(v[h]);
         tc::fence_before();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(&bar->tempty[buf]);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) sum[i] += v[i];
+        for (int i = 0; i < W; ++i) sum[i] += v[i / 32][i % 32];
       }
       if (!ok) break;
       int q, iw, tm, tn;
       decode_item(P, item >> 1, q, iw, tm, tn);
-      const int comp = (int)(item & 1), nG = P.nG[q], G = tm * BM + quad * 32 + lane, Hb = tn * COMP_N + half * 32;
+      const int comp = (int)(item & 1), nG = P.nG[q], G = tm * BM + quad * 32 + lane, Hb = tn * CN + half * W;
       if (G < nG) {
         const int k = exponent_of_pow2(P.inv[q][iw]);
         double* row = reinterpret_cast<double*>(P.chi[q] + ((size_t)iw * nG + G) * nG) + comp;
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
+        for (int i = 0; i < W; ++i)
           if (Hb + i < nG && Hb + i != G) red_add_pow2(row + 2 * (Hb + i), sum[i], k);
-        if ((unsigned)(G - Hb) < 32u) {
+        if ((unsigned)(G - Hb) < (unsigned)W) {
           const double2 d = P.diag[q][(size_t)iw * P.tiles_m[q] * BM + G];
           atomicAdd(row + 2 * G, comp ? d.y : d.x);
         }
@@ -1588,14 +1592,18 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
   int dev = 0, nsm = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  // Narrow items where all of them run at once: at 128 and 144 items of 152 SMs still 1.8x (BF16), and
-  // below that 1.2x (256 pairs) to 2x; a second round of them takes as long as one round of whole tiles.
-  bool narrow = !pair && !p->tc_herm;
-  if (narrow) {
-    int64_t n = 0;
-    for (int j = 0; j < n_jobs; ++j)
-      n += 2 * (int64_t)p->n_freq * ((jobs[j].nG + BM - 1) / BM) * ((jobs[j].nG + COMP_N - 1) / COMP_N);
-    narrow = n <= nsm;
+  // Narrow items where all of them run at once, of 64 columns (cn) or else of 128: at 128 and 144 items of
+  // 152 SMs still 1.8x (BF16), and below that 1.2x (256 pairs) to 2x; with 128 columns 1.4-1.5x up to 144
+  // items (N_G 350, eight frequencies, BF16: 363 -> 239 us, 4096 pairs FP16 268 -> 171 us), 1.1-1.8x with 256 pairs.
+  // A second round of items takes as long as one round of whole tiles.
+  int cn = 0;
+  if (!pair && !p->tc_herm) {
+    for (int c = 64; c <= BN && !cn; c += 64) {
+      int64_t n = 0;
+      for (int j = 0; j < n_jobs; ++j)
+        n += 2 * (int64_t)p->n_freq * ((jobs[j].nG + BM - 1) / BM) * ((jobs[j].nG + c - 1) / c);
+      if (n <= nsm) cn = c;
+    }
   }
   for (int j = 0; j < n_jobs; ++j) {
     const TcJob& jb = jobs[j];
@@ -1606,7 +1614,7 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
       if (e != cudaSuccess) { delete P; return e; }
       if (mode == 1) continue;
     }
-    if (!encode_planes(&P->tmB[j], w.Bp, BF16, Kp, nGp, b_planes(p), why, pair || narrow ? BN / 2 : BN) ||
+    if (!encode_planes(&P->tmB[j], w.Bp, BF16, Kp, nGp, b_planes(p), why, pair ? BN / 2 : cn ? cn : BN) ||
         !encode_planes(&P->tmA[j], w.Ap, BF16, Kp, nGp, 2 * NT * n_parts(p) * p->n_freq, why, BM)) {
       delete P;
       return cudaErrorInvalidValue;
@@ -1617,7 +1625,7 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
     P->tbar[j] = w.tbar;
     P->diag[j] = w.diag;
     P->nG[j] = jb.nG;
-    const int TM = nGp / (pair ? 2 * BM : BM), TN = narrow ? (jb.nG + COMP_N - 1) / COMP_N : nGp / BN;
+    const int TM = nGp / (pair ? 2 * BM : BM), TN = cn ? (jb.nG + cn - 1) / cn : nGp / BN;
     P->tiles_m[j] = TM;
     P->tiles_n[j] = TN;
     // Hermitian mode: row tm holds the TN - rr tm tiles from column rr tm on
@@ -1638,7 +1646,7 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
   P->chain_k = std::max(1, p->chain_pairs / BK);
   P->n_products = p->n_products;
   P->group = p->tc_group > 0 ? p->tc_group : 8;
-  P->total_items = narrow ? 2 * items : items;
+  P->total_items = cn ? 2 * items : items;
   cudaError_t e;
   if (pair) {
     if (!regs_match(k_contract_tc2<BF16, NT>, why)) { delete P; return cudaErrorNotSupported; }
@@ -1648,12 +1656,12 @@ static cudaError_t run_tc(chi0_plan_s* p, const TcJob* jobs, int n_jobs, int64_t
     const int pairs = (int)std::min<int64_t>(items, (int64_t)(nsm / 2));
     ProfScope ps(p, CHI0_K_CONTRACT_TC, s, 1);
     k_contract_tc2<BF16, NT><<<2 * pairs, THREADS, SMEM2_BYTES, s>>>(*P, p->d_status);
-  } else if (narrow) {
-    e = cudaFuncSetAttribute(k_contract_tc_narrow<BF16, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)SMEM2_BYTES);
+  } else if (cn) {
+    auto* kern = cn == 64 ? k_contract_tc_narrow<BF16, NT, 64> : k_contract_tc_narrow<BF16, NT, 128>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM2_BYTES);
     if (e != cudaSuccess) { delete P; return e; }
     ProfScope ps(p, CHI0_K_CONTRACT_TC, s, 1);
-    k_contract_tc_narrow<BF16, NT><<<(int)P->total_items, THREADS, SMEM2_BYTES, s>>>(*P, p->d_status);
+    kern<<<(int)P->total_items, THREADS, SMEM2_BYTES, s>>>(*P, p->d_status);
   } else {
     if (!regs_match(k_contract_tc<BF16, NT>, why)) { delete P; return cudaErrorNotSupported; }
     e = cudaFuncSetAttribute(k_contract_tc<BF16, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -1,5 +1,6 @@
-"""Small contractions of split plans run as narrow items (128 x 64 columns of one component).  A
-plan with one frequency more than fit the chip that way uses 128 x 128 tiles: the same
+"""Small contractions of split plans run as narrow items (128 x 64 or, with more
+tiles, 128 x 128 of one component).  A plan with one frequency more than fit the chip that way
+uses the next larger items (128 x 128 of one component, then of both): the same
 sums in the same order, so the shared frequencies agree bit for bit off the diagonal
 (whose FP64 sums are atomics).  The first frequency is compared with the FP64 sum."""
 import numpy as np
@@ -10,14 +11,15 @@ from oracle import chi0_from_pairs, freq_factor
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("columns", [64, 128])
 @pytest.mark.parametrize("precision,n_products,chain_pairs", [("bf16", 6, 0), ("bf16", 3, 96), ("fp16", 4, 0), ("fp16", 3, 64)])
 @pytest.mark.parametrize("n_G,n_c", [(1, 1), (2, 40), (63, 33), (64, 7), (65, 160), (128, 32), (129, 301), (257, 64), (350, 96)])
-def test_narrow_items_equal_full_tiles(n_G, n_c, precision, n_products, chain_pairs):
+def test_narrow_items_equal_full_tiles(n_G, n_c, precision, n_products, chain_pairs, columns):
     import torch
     from paper_1601_06767_gb300 import Chi0Plan
     from synth.mgo import g_sphere
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    fit = sms // (2 * ((n_G + 127) // 128) * ((n_G + 63) // 64))
+    fit = sms // (2 * ((n_G + 127) // 128) * ((n_G + columns - 1) // columns))
     assert fit >= 1
     rng = np.random.default_rng(n_G)
     g, n_v = g_sphere(n_G, (0.0, 0.0, 0.0)), 3
