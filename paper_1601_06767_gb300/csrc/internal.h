@@ -166,7 +166,7 @@ cudaError_t launch_pair_planes(const chi0_plan_s* p, int iq, const void* psi_v, 
 // stage 3: D -> M rows (v0+iv)*ldc + (c0+ic)
 cudaError_t launch_pair_gather(const chi0_plan_s* p, int iq, const void* D, int nv, int nc,
                                int64_t row0, int64_t ldv, void* M, cudaStream_t s);
-// fixed-point pair stage of FP64 plans (kern_fx.cu): tables of a sphere, bands held at a time, workspace
+// fixed-point pair stage of FP64 plans (kern_fx.cu): tables of a sphere, workspace, stages 1 and 2, stage 3
 bool fx_fits(const chi0_plan_s* p, const SphereQ& s);
 cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s);
 // the same for the wavefunctions (w->fx_tw stays NULL where they do not fit)
@@ -174,14 +174,12 @@ cudaError_t fx_setup_wfn(const chi0_plan_s* p, WfnSphere* w);
 size_t fx_wfn_ws_bytes(const chi0_plan_s* p, int64_t bands);
 cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, int64_t bands,
                           cudaStream_t s);
-int fx_bands(const chi0_plan_s* p);
-size_t fx_ws_bytes(const chi0_plan_s* p, int64_t bands);
-cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int32_t* idx, int b0, int nb, void* ws,
-                            int64_t bands, int first, cudaStream_t s);
-cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int vslots, int nv, int nc, void* D,
+size_t fx_ws_bytes(const chi0_plan_s* p, int64_t pairs);
+cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, const double2* psi_v, const int32_t* v_idx, int v0, int nv,
+                             const double2* psi_c, const int32_t* c_idx, int c0, int nc, void* D, void* ex,
                              cudaStream_t st);
-cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int nv, int nc, const void* D,
-                             int64_t row0, int64_t ldv, double2* M, cudaStream_t st);
+cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, int nv, int nc, const void* D, const void* ex, int64_t row0,
+                             int64_t ldv, double2* M, cudaStream_t st);
 // frequency factors f[w][k] for pairs p0..p0+K of an (n_v x n_c) set
 cudaError_t launch_weights(const chi0_plan_s* p, int64_t p0, int64_t K, int n_c, const double* E_v,
                            const double* E_col, const double* w_col, double2* f, cudaStream_t s);

@@ -6,18 +6,15 @@
 // every number is a signed integer in two limbs and a multiply-add is four 32 x
 // 32 + 64-bit integer multiply-adds, thirty times the rate:
 //
-//   grids     57 bits relative to the largest component of the band (limbs 29 + 29)
-//   products  conj(psi_v) psi_c, and every transform's input, are rescaled to the
-//             largest component of the plane (55 bits, limbs 28 + 28): block
-//             floating point, one exponent per (pair, plane)
+//   inputs    55 bits (limbs 28 + 28) relative to the largest one: of the plane's
+//             products conj(psi_v) psi_c, which are formed in FP64, or of a column's
+//             coefficients.  Each further transform rescales to the plane's largest
+//             element (block floating point, one exponent per plane)
 //   twiddles  55 bits; the sums are exact, one rounding per output
 //
-// Roundings of 2^-56 of a plane's largest element against 2^-53 of every partial
-// sum: against quad precision, on the synthetic wavefunctions, 1.1e-16 (relative
-// Frobenius) on grids of 21 to 48 points, 4.7-6.6e-16 for the FP64 sums.
-//
-// 3840 pairs, 24^3, N_G 350: planes 10.32 -> 0.77 ms, gather 231 -> 71 us; 256
-// wavefunctions: 703 -> 165 us, 6.1e-16 -> 9.6e-17.
+// The unit follows the products and not the bands, so bands that overlap little lose
+// nothing: what a plane holds is rounded to 2^-56 of its own largest product, against
+// 2^-53 of every partial sum in FP64.
 //
 // A line of n points is transformed at the wanted frequencies only, with the
 // symmetries of the twiddles folded out first: with h = n / 2 and a_i = x_i +
@@ -39,19 +36,30 @@
 namespace chi0 {
 namespace {
 
-constexpr int QBITS = 57, QL = 29;    // grids: bits and limb width
-constexpr int WBITS = 55, WL = 28;    // transform inputs and twiddles
+constexpr int WBITS = 55, WL = 28;    // transform inputs and twiddles: bits and limb width
 constexpr int FX_MAX_N = 128;         // the 64-bit sums hold n / 4 + 1 products of 2^57
 constexpr int FX_MAX_W = 64;          // wavefunction sphere: 64 coefficients per column (4 products of 2^54 each)
 
-// ---- grids to fixed point ----
+// ---- doubles to fixed point ----
+// biased exponent of a set's largest magnitude word; its integers are below 2^55 in units of
+// 2^fx_unit(exponent)
+__device__ __forceinline__ int fx_exp(uint32_t w) { return max((int)(w >> 20), 1); }
+__device__ __forceinline__ int fx_unit(int emax) { return emax - 1023 - (WBITS - 1); }
+// x in that unit, rounded (subnormal numbers included)
+__device__ __forceinline__ int64_t fx_int(double x, int emax) {
+  const int64_t b = __double_as_longlong(x);
+  const int e = (int)((b >> 52) & 0x7ff);
+  const uint64_t man = ((uint64_t)b & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
+  const int64_t q = (int64_t)(((man << (WBITS - 52)) >> min(emax - max(e, 1), 63)) + 1) >> 1;
+  return b < 0 ? -q : q;
+}
+
 // mx[b] = largest magnitude word of band b (cleared by the caller)
-__global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ psi, const int32_t* __restrict__ idx, int b0,
-                                                int64_t nr, uint32_t* __restrict__ mx) {
-  const int64_t band = idx ? idx[b0 + blockIdx.y] : b0 + blockIdx.y;
-  const double2* x = psi + band * nr;
+__global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ c, int b0, int64_t n,
+                                                uint32_t* __restrict__ mx) {
+  const double2* x = c + (int64_t)(b0 + blockIdx.y) * n;
   uint32_t m = 0;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nr; e += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = x[e];
     m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
   }
@@ -59,23 +67,20 @@ __global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ psi,
   if ((threadIdx.x & 31) == 0 && m) atomicMax(mx + blockIdx.y, m);
 }
 
-template <int BITS = QBITS>
 __device__ __forceinline__ int fx_scale(uint32_t w) {
-  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : BITS - 1 - mod::word_exp(w));
+  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : WBITS - 1 - mod::word_exp(w));
 }
 
-// q[b][r] = (re1, re0, im1, im0): limbs of psi 2^scale
-template <int BITS, int LIMB>
-__global__ void __launch_bounds__(256) k_fx_quant(const double2* __restrict__ psi, const int32_t* __restrict__ idx, int b0,
-                                                  int64_t nr, const uint32_t* __restrict__ mx, int4* __restrict__ q) {
-  const int64_t band = idx ? idx[b0 + blockIdx.y] : b0 + blockIdx.y;
-  const double2* x = psi + band * nr;
-  const int s = fx_scale<BITS>(mx[blockIdx.y]);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nr; e += (int64_t)gridDim.x * blockDim.x) {
+// q[b][r] = (re1, re0, im1, im0): limbs of the coefficients 2^scale
+__global__ void __launch_bounds__(256) k_fx_quant(const double2* __restrict__ c, int b0, int64_t n,
+                                                  const uint32_t* __restrict__ mx, int4* __restrict__ q) {
+  const double2* x = c + (int64_t)(b0 + blockIdx.y) * n;
+  const int s = fx_scale(mx[blockIdx.y]);
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
     const double2 v = x[e];
     const int64_t a = mod::quantise(v.x, s), b = mod::quantise(v.y, s);
-    const int a0 = ((int)a << (32 - LIMB)) >> (32 - LIMB), b0l = ((int)b << (32 - LIMB)) >> (32 - LIMB);
-    q[blockIdx.y * nr + e] = make_int4((int)((a - a0) >> LIMB), a0, (int)((b - b0l) >> LIMB), b0l);
+    const int a0 = ((int)a << (32 - WL)) >> (32 - WL), b0l = ((int)b << (32 - WL)) >> (32 - WL);
+    q[blockIdx.y * n + e] = make_int4((int)((a - a0) >> WL), a0, (int)((b - b0l) >> WL), b0l);
   }
 }
 
@@ -114,12 +119,16 @@ __device__ __forceinline__ double to_double(int64_t y, int k) {
 // units of one line's fold: i = 0 .. fold_units(n) - 1, each owns the slots it reads and writes
 __host__ __device__ __forceinline__ int fold_units(int n) { return n & 1 ? (n + 1) / 2 : n / 4 + 1; }
 
-__device__ __forceinline__ void fold_line(longlong2* __restrict__ r, int n, int i, int s) {
+// elements of a line as integers below 2^55: integers x 2^-s, doubles of a set with exponent s
+__device__ __forceinline__ longlong2 line_int(longlong2 v, int s) {
+  return make_longlong2(shift_round(v.x, s), shift_round(v.y, s));
+}
+__device__ __forceinline__ longlong2 line_int(double2 v, int s) { return make_longlong2(fx_int(v.x, s), fx_int(v.y, s)); }
+
+template <class T>
+__device__ __forceinline__ void fold_line(T* __restrict__ r, int n, int i, int s) {
   int4* w = reinterpret_cast<int4*>(r);
-  auto ld = [&](int k) {
-    const longlong2 v = r[k];
-    return make_longlong2(shift_round(v.x, s), shift_round(v.y, s));
-  };
+  auto ld = [&](int k) { return line_int(r[k], s); };
   if (n & 1) {
     const longlong2 x = ld(i);
     if (i == 0) {
@@ -209,45 +218,42 @@ __device__ __forceinline__ uint32_t block_max(uint32_t m, uint32_t* __restrict__
 
 // Stages 1 and 2 of one plane i1: D[pair][i1][k2][k3] as 64-bit integers and their
 // exponents ex[pair][i1] = (unit, top): value = D 2^unit, |value| < 2^top.  A CTA
-// takes one valence band and a run of conduction bands.  Bound by the integer
-// multiplies (16 per grid point for the product, eight per folded point and
-// frequency pair).
-__global__ void k_fx_planes(const int4* __restrict__ qv, const uint32_t* __restrict__ mv, const int4* __restrict__ qc,
-                            const uint32_t* __restrict__ mc, int nc, int cpc, int n1, int n2, int n3, int nk2, int nk3,
-                            const __grid_constant__ FxAxis a3, const __grid_constant__ FxAxis a2,
-                            longlong2* __restrict__ D, int2* __restrict__ ex) {
+// takes one valence band and a run of conduction bands.  The products run on the
+// FP64 pipe (four operations per grid point), beside the integer multiplies of other
+// CTAs' transforms (eight per folded point and frequency pair).
+__global__ void k_fx_planes(const double2* __restrict__ psi_v, const int32_t* __restrict__ v_idx, int v_base,
+                            const double2* __restrict__ psi_c, const int32_t* __restrict__ c_idx, int c_base, int nc,
+                            int cpc, int n1, int n2, int n3, int nk2, int nk3, const __grid_constant__ FxAxis a3,
+                            const __grid_constant__ FxAxis a2, longlong2* __restrict__ D, int2* __restrict__ ex) {
   extern __shared__ __align__(16) unsigned char smem_fx[];
   __shared__ uint32_t slot[3];
   const int ld3 = n3 | 1, ld2 = n2 | 1;
-  longlong2* A = reinterpret_cast<longlong2*>(smem_fx);    // [n2][ld3]
-  longlong2* X = A + (size_t)n2 * ld3;                     // [nk3][ld2]
+  double2* A = reinterpret_cast<double2*>(smem_fx);        // [n2][ld3]
+  longlong2* X = reinterpret_cast<longlong2*>(A + (size_t)n2 * ld3);   // [nk3][ld2]
   const int i1 = blockIdx.x, jv = blockIdx.y, nt = blockDim.x, tid = threadIdx.x;
   const int plane = n2 * n3;
   const int64_t nr = (int64_t)n1 * plane, box = (int64_t)nk2 * nk3;
-  const int4* v0 = qv + jv * nr + (int64_t)i1 * plane;
-  const int sv = fx_scale(mv[jv]);
+  const double2* v0 = psi_v + (v_idx ? v_idx[v_base + jv] : v_base + jv) * nr + (int64_t)i1 * plane;
   const int jc1 = min(nc, (int)(blockIdx.z + 1) * cpc);
   for (int jc = blockIdx.z * cpc; jc < jc1; ++jc) {
-    const int4* c0 = qc + jc * nr + (int64_t)i1 * plane;
+    const double2* c0 = psi_c + (c_idx ? c_idx[c_base + jc] : c_base + jc) * nr + (int64_t)i1 * plane;
+    const int64_t pair = (int64_t)jv * nc + jc;
     __syncthreads();                                       // the previous pair's readers are done
     if (tid < 3) slot[tid] = 0;
     __syncthreads();
     uint32_t m = 0;
-    for (int e = tid; e < plane; e += nt) {                // conj(v) c / 2^54
+    for (int e = tid; e < plane; e += nt) {
       const int i2 = e / n3, i3 = e - i2 * n3;
-      const int4 v = v0[e], c = c0[e];
-      const int64_t hr = (int64_t)v.x * c.x + (int64_t)v.z * c.z;
-      const int64_t xr = (int64_t)v.x * c.y + (int64_t)v.y * c.x + (int64_t)v.z * c.w + (int64_t)v.w * c.z;
-      const int64_t lr = (int64_t)v.y * c.y + (int64_t)v.w * c.w;
-      const int64_t hi = (int64_t)v.x * c.z - (int64_t)v.z * c.x;
-      const int64_t xi = (int64_t)v.x * c.w + (int64_t)v.y * c.z - (int64_t)v.z * c.y - (int64_t)v.w * c.x;
-      const int64_t li = (int64_t)v.y * c.w - (int64_t)v.w * c.y;
-      const longlong2 p = make_longlong2((hr << 4) + ((xr + (lr >> QL) + (1ll << 24)) >> 25),
-                                         (hi << 4) + ((xi + (li >> QL) + (1ll << 24)) >> 25));
+      const double2 p = cconjmul(v0[e], c0[e]);
       A[i2 * ld3 + i3] = p;
-      m = max(m, max(abs_word(p.x), abs_word(p.y)));
+      m = max(m, max(mod::mag_word(p.x), mod::mag_word(p.y)));
     }
-    const int s0 = word_bits(block_max(m, slot)) - WBITS;  // its barrier also orders A
+    m = block_max(m, slot);                                // its barrier also orders A
+    if (m >= 0x7ff00000u) {                                // an infinity or a NaN: the pair's elements are NaN
+      if (tid == 0) ex[pair * n1 + i1] = make_int2(mod::NO_SCALE, 0);
+      continue;
+    }
+    const int s0 = fx_exp(m);
     const int u3 = fold_units(n3);
     for (int e = tid; e < n2 * u3; e += nt) {
       const int i2 = e % n2, i = e / n2;
@@ -277,7 +283,6 @@ __global__ void k_fx_planes(const int4* __restrict__ qv, const uint32_t* __restr
     }
     __syncthreads();
     m = 0;
-    const int64_t pair = (int64_t)jv * nc + jc;
     longlong2* d = D + (pair * n1 + i1) * box;
     for (int e = tid; e < nk3 * a2.items; e += nt) {       // along i2
       const int k3 = e % nk3, it = e / nk3;
@@ -295,10 +300,8 @@ __global__ void k_fx_planes(const int4* __restrict__ qv, const uint32_t* __restr
     }
     m = block_max(m, slot + 2);
     if (tid == 0) {
-      const int sc = fx_scale(mc[jc]);
-      const int unit = 54 - sv - sc + s0 + s1;
-      ex[pair * n1 + i1] = sv == mod::NO_SCALE || sc == mod::NO_SCALE ? make_int2(mod::NO_SCALE, 0)
-                                                                      : make_int2(unit, unit + word_bits(m));
+      const int unit = fx_unit(s0) + s1;
+      ex[pair * n1 + i1] = make_int2(unit, unit + word_bits(m));
     }
   }
 }
@@ -432,7 +435,7 @@ __global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict_
   const int i1 = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const int64_t b = blockIdx.y;
   double2* out = psi + (b * n1 + i1) * (int64_t)n2 * n3;
-  const int s = fx_scale<WBITS>(mx[b]);
+  const int s = fx_scale(mx[b]);
   if (s == mod::NO_SCALE) {                                // an infinity or a NaN among the coefficients
     for (int e = tid; e < n2 * n3; e += nt) out[e] = make_double2(nan(""), nan(""));
     return;
@@ -497,13 +500,7 @@ size_t planes_smem(const chi0_plan_s* p, const SphereQ& s) {
   return ((size_t)p->n2 * (p->n3 | 1) + (size_t)s.nk3 * (p->n2 | 1)) * 16;
 }
 constexpr size_t SMEM_CAP = 220 * 1024;
-constexpr int64_t QUANT_BYTES = (int64_t)2 << 30;         // quantised grids held at a time
-
 size_t al256(size_t x) { return (x + 255) / 256 * 256; }
-// the exponents of D in the workspace
-int2* fx_exponents(const chi0_plan_s* p, void* ws, int64_t bands) {
-  return reinterpret_cast<int2*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16) + al256((size_t)bands * 4));
-}
 
 // (cos, sin) of 2 pi m / n, m < n, in two limbs each; evaluated on the first octant only (long double
 // is software on the Arm hosts)
@@ -631,8 +628,8 @@ cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, do
     e = cudaMemsetAsync(mx, 0, (size_t)n * 4, s);
     if (e != cudaSuccess) return e;
     const int gx = (int)std::min<int64_t>((w.npw + 1023) / 1024, std::max(1, 4096 / n));
-    k_fx_max<<<dim3(gx, n), 256, 0, s>>>(coeff, nullptr, b0, w.npw, mx);
-    k_fx_quant<WBITS, WL><<<dim3(gx, n), 256, 0, s>>>(coeff, nullptr, b0, w.npw, mx, q);
+    k_fx_max<<<dim3(gx, n), 256, 0, s>>>(coeff, b0, w.npw, mx);
+    k_fx_quant<<<dim3(gx, n), 256, 0, s>>>(coeff, b0, w.npw, mx, q);
     const int nt = sm <= 32 * 1024 ? 128 : (sm <= 72 * 1024 ? 256 : 512);
     k_fx_wfn<<<dim3(p->n1, n), nt, sm, s>>>(q, mx, w.npw, p->n1, p->n2, p->n3, w.nw1, w.w2min, w.w3min, w.nw2, w.nw3,
                                             w.col_start, w.col_pw, w.col_g1, w.w1min, w.fx_tw, w.fx[0], w.fx[1],
@@ -669,32 +666,15 @@ cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s) {
   return e;
 }
 
-// bands whose quantised grids are held at a time, and the workspace: grids, magnitude words, exponents
-int fx_bands(const chi0_plan_s* p) { return (int)std::max<int64_t>(2, QUANT_BYTES / (16 * p->nr)); }
-size_t fx_ws_bytes(const chi0_plan_s* p, int64_t bands) {
-  return al256((size_t)bands * p->nr * 16) + al256((size_t)bands * 4) + al256((size_t)p->D_pairs * p->n1 * sizeof(int2));
-}
+// workspace of the exponents of D for `pairs` pairs at a time
+size_t fx_ws_bytes(const chi0_plan_s* p, int64_t pairs) { return (size_t)pairs * p->n1 * sizeof(int2); }
 
-// quantise bands idx[b0 ..] (or b0 ..) into slots first .. first + nb of the workspace
-cudaError_t launch_fx_quant(const chi0_plan_s* p, const double2* psi, const int32_t* idx, int b0, int nb, void* ws,
-                            int64_t bands, int first, cudaStream_t s) {
-  int4* q = reinterpret_cast<int4*>(ws) + (int64_t)first * p->nr;
-  uint32_t* mx = reinterpret_cast<uint32_t*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16)) + first;
-  cudaError_t e = cudaMemsetAsync(mx, 0, (size_t)nb * 4, s);
-  if (e != cudaSuccess) return e;
-  const int gx = (int)std::min<int64_t>((p->nr + 1023) / 1024, std::max(1, 4096 / nb));
-  k_fx_max<<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx);
-  k_fx_quant<QBITS, QL><<<dim3(gx, nb), 256, 0, s>>>(psi, idx, b0, p->nr, mx, q);
-  return cudaGetLastError();
-}
-
-// stages 1 and 2 of the pairs of valence slots [0, nv) and conduction slots [vslots, vslots + nc) of
-// the workspace into D, and their exponents
-cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int vslots, int nv, int nc, void* D,
+// stages 1 and 2 of the pairs of valence rows v0 .. v0 + nv and conduction columns c0 .. c0 + nc into D, and
+// their exponents
+cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, const double2* psi_v, const int32_t* v_idx, int v0, int nv,
+                             const double2* psi_c, const int32_t* c_idx, int c0, int nc, void* D, void* ex,
                              cudaStream_t st) {
   const SphereQ& s = p->q[iq];
-  const int4* q = reinterpret_cast<const int4*>(ws);
-  const uint32_t* mx = reinterpret_cast<const uint32_t*>((unsigned char*)ws + al256((size_t)bands * p->nr * 16));
   const size_t sm = planes_smem(p, s);
   cudaError_t e = cudaFuncSetAttribute(k_fx_planes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
@@ -703,20 +683,20 @@ cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, void* ws, int64_t ban
   const int nt = items <= 128 ? 128 : (items <= 512 || sm <= 72 * 1024 ? 256 : 512);
   int cpc = 8;
   while (cpc > 1 && (int64_t)p->n1 * nv * ((nc + cpc - 1) / cpc) < 16 * 152) cpc >>= 1;
-  k_fx_planes<<<dim3(p->n1, nv, (nc + cpc - 1) / cpc), nt, sm, st>>>(q, mx, q + (int64_t)vslots * p->nr, mx + vslots, nc,
-                                                                  cpc, p->n1, p->n2, p->n3, s.nk2, s.nk3, s.fx[2],
-                                                                  s.fx[1], (longlong2*)D, fx_exponents(p, ws, bands));
+  k_fx_planes<<<dim3(p->n1, nv, (nc + cpc - 1) / cpc), nt, sm, st>>>(psi_v, v_idx, v0, psi_c, c_idx, c0, nc, cpc, p->n1,
+                                                                    p->n2, p->n3, s.nk2, s.nk3, s.fx[2], s.fx[1],
+                                                                    (longlong2*)D, (int2*)ex);
   return cudaGetLastError();
 }
 
 // stage 3: M rows row0 + iv ldv + ic
-cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, void* ws, int64_t bands, int nv, int nc, const void* D,
-                             int64_t row0, int64_t ldv, double2* M, cudaStream_t st) {
+cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, int nv, int nc, const void* D, const void* ex, int64_t row0,
+                             int64_t ldv, double2* M, cudaStream_t st) {
   const SphereQ& s = p->q[iq];
   const int ld1 = p->n1 | 1;
   const int chunk = std::min(s.ncol, std::max(1, 40 * 1024 / (ld1 * 16)));
   k_fx_gather<<<dim3((unsigned)(nv * nc), (s.ncol + chunk - 1) / chunk), 256, (size_t)chunk * ld1 * 16, st>>>(
-      (const longlong2*)D, fx_exponents(p, ws, bands), nc, row0, ldv, p->n1, (int64_t)s.nk2 * s.nk3, s.nG, s.ncol, chunk,
+      (const longlong2*)D, (const int2*)ex, nc, row0, ldv, p->n1, (int64_t)s.nk2 * s.nk3, s.nG, s.ncol, chunk,
       s.nk1, s.col_off, s.fx_map, s.fx[0], 1.0 / (double)p->nr, M);
   return cudaGetLastError();
 }

@@ -801,59 +801,34 @@ chi0_status chi0_wfn_to_grid(chi0_plan p, const void* coeff, int nb, void* psi, 
   return CHI0_OK;
 }
 
-// Pairs of FP64 plans in fixed point: valence and conduction grids quantised in chunks that fit the
-// workspace, then the pairs of the two chunks.  Same M rows as pairs_impl.
-static chi0_status pairs_fx(chi0_plan p, int iq, const void* psi_v, const int32_t* v_idx, int n_v, const void* psi_c,
-                            const int32_t* c_idx, int c_base, int n_c, void* M, int64_t ld_pairs_c, int64_t bands,
-                            cudaStream_t s) {
-  void* ws = p->ws_fx.p;
-  const int vchunk = (int)std::min<int64_t>({n_v, p->D_pairs, std::max<int64_t>(1, bands - std::min<int64_t>(n_c, bands / 2)), 65535});
-  const int cchunk = (int)std::min<int64_t>({n_c, std::max<int64_t>(1, p->D_pairs / vchunk), bands - vchunk, 65535});
-  for (int v0 = 0; v0 < n_v; v0 += vchunk) {
-    const int nv = std::min(vchunk, n_v - v0);
-    {
-      chi0::ProfScope ps(p, CHI0_K_PAIR_PLANES, s, 2);
-      CK(p, chi0::launch_fx_quant(p, (const double2*)psi_v, v_idx, v0, nv, ws, bands, 0, s));
-    }
-    for (int c0 = 0; c0 < n_c; c0 += cchunk) {
-      const int nc = std::min(cchunk, n_c - c0);
-      {
-        chi0::ProfScope ps(p, CHI0_K_PAIR_PLANES, s, 3);
-        CK(p, chi0::launch_fx_quant(p, (const double2*)psi_c, c_idx, c_base + c0, nc, ws, bands, vchunk, s));
-        CK(p, chi0::launch_fx_planes(p, iq, ws, bands, vchunk, nv, nc, p->d_D, s));
-      }
-      chi0::ProfScope ps(p, CHI0_K_PAIR_GATHER, s, 1);
-      CK(p, chi0::launch_fx_gather(p, iq, ws, bands, nv, nc, p->d_D, (int64_t)v0 * ld_pairs_c + c0, ld_pairs_c,
-                                   (double2*)M, s));
-    }
-  }
-  return CHI0_OK;
-}
-
 // Pairs of valence rows 0..n_v and conduction columns c_base..c_base+n_c (column ic of the
 // index space is band c_idx[ic], or ic when c_idx is NULL); M row = iv*ld_pairs_c + (ic - c_base).
 static chi0_status pairs_impl(chi0_plan p, int iq, const void* psi_v, const int32_t* v_idx, int n_v,
                               const void* psi_c, const int32_t* c_idx, int c_base, int n_c, void* M,
                               int64_t ld_pairs_c, cudaStream_t s) {
-  if (p->q[iq].fx_map) {
-    const int64_t bands = std::min<int64_t>(chi0::fx_bands(p), (int64_t)n_v + n_c);
-    if (bands >= 2 && ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, bands), s))
-      return pairs_fx(p, iq, psi_v, v_idx, n_v, psi_c, c_idx, c_base, n_c, M, ld_pairs_c, bands, s);
-  }
-  // chunk over (v, c) so one chunk's per-plane transforms fit the D buffer
-  int vchunk = (int)std::min<int64_t>(n_v, p->D_pairs);
-  int cchunk = (int)std::max<int64_t>(1, std::min<int64_t>(n_c, p->D_pairs / vchunk));
+  // FP64 plans transform in fixed point where the sphere fits and the exponents' memory can be had
+  const bool fx = p->q[iq].fx_map &&
+                  ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, std::min<int64_t>((int64_t)n_v * n_c, p->D_pairs)), s);
+  // chunk over (v, c) so one chunk's per-plane transforms fit the D buffer (and the launches' grids)
+  const int vchunk = (int)std::min<int64_t>({n_v, p->D_pairs, 65535});
+  const int cchunk = (int)std::max<int64_t>(1, std::min<int64_t>({n_c, p->D_pairs / vchunk, 65535}));
   for (int v0 = 0; v0 < n_v; v0 += vchunk) {
     int nv = std::min(vchunk, n_v - v0);
     for (int c0 = 0; c0 < n_c; c0 += cchunk) {
       int nc = std::min(cchunk, n_c - c0);
+      const int64_t row0 = (int64_t)v0 * ld_pairs_c + c0;
       {
         chi0::ProfScope ps(p, CHI0_K_PAIR_PLANES, s, 1);
-        CK(p, chi0::launch_pair_planes(p, iq, psi_v, v_idx, v0, nv, psi_c, c_idx, c_base + c0, nc, p->d_D, s));
+        if (fx)
+          CK(p, chi0::launch_fx_planes(p, iq, (const double2*)psi_v, v_idx, v0, nv, (const double2*)psi_c, c_idx,
+                                       c_base + c0, nc, p->d_D, p->ws_fx.p, s));
+        else
+          CK(p, chi0::launch_pair_planes(p, iq, psi_v, v_idx, v0, nv, psi_c, c_idx, c_base + c0, nc, p->d_D, s));
       }
       {
         chi0::ProfScope ps(p, CHI0_K_PAIR_GATHER, s, 1);
-        CK(p, chi0::launch_pair_gather(p, iq, p->d_D, nv, nc, (int64_t)v0 * ld_pairs_c + c0, ld_pairs_c, M, s));
+        if (fx) CK(p, chi0::launch_fx_gather(p, iq, nv, nc, p->d_D, p->ws_fx.p, row0, ld_pairs_c, (double2*)M, s));
+        else CK(p, chi0::launch_pair_gather(p, iq, p->d_D, nv, nc, row0, ld_pairs_c, M, s));
       }
     }
   }
@@ -1219,7 +1194,7 @@ chi0_status chi0_build_batched(chi0_plan p, const void* const* psi_v, int n_v, c
   if (!p->graph_exec || key != p->graph_key) {
     if (!chi0::is_split(p)) {   // workspaces cannot be allocated inside the capture
       ws_ready(p, p->ws_mod, mod_contract_bytes(p), s);
-      ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, std::min<int64_t>(chi0::fx_bands(p), (int64_t)n_v + n_c)), s);
+      ws_ready(p, p->ws_fx, chi0::fx_ws_bytes(p, std::min<int64_t>((int64_t)n_v * n_c, p->D_pairs)), s);
     }
     if (p->graph_exec) { cudaGraphExecDestroy(p->graph_exec); p->graph_exec = nullptr; }
     if (!p->cap_stream) CK(p, cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
