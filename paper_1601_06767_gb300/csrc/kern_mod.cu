@@ -589,8 +589,7 @@ size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 bool mod_gemm_usable() {
   static const bool ok = [] {
     cudaFuncAttributes a;
-    if (!encoder() || cudaFuncGetAttributes(&a, k_mod_gemm) != cudaSuccess || a.numRegs != REG_LAUNCH ||
-        cudaFuncSetAttribute(k_mod_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess) {
+    if (!encoder() || cudaFuncGetAttributes(&a, k_mod_gemm) != cudaSuccess || a.numRegs != REG_LAUNCH) {
       cudaGetLastError();
       return false;
     }
@@ -600,6 +599,9 @@ bool mod_gemm_usable() {
 }
 
 cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s) {
+  // before every launch: the attribute belongs to the current device
+  const cudaError_t ea = cudaFuncSetAttribute(k_mod_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+  if (ea != cudaSuccess) return ea;
   GemmArgs P{};
   if (!encode(&P.tmA, g.A, g.Kp, g.rows_a, g.a_planes) || !encode(&P.tmB, g.B, g.Kp, g.cols, g.b_planes))
     return cudaErrorInvalidValue;
