@@ -64,7 +64,7 @@ struct WfnSphere {
 struct LazyWs {
   void* p = nullptr;
   size_t bytes = 0;
-  size_t limit = SIZE_MAX;            // smallest size that could not be had (not asked for again)
+  size_t refused = SIZE_MAX;          // size that the last attempt could not have
   bool captured = false;              // a caller's stream capture holds the address
 };
 
@@ -103,10 +103,9 @@ struct chi0_plan_s {
   double* d_bwd = nullptr;   // adjoint work: per-pair grad dE and per-tile partial sums
   void* wfn_ws = nullptr;    // scratch of the three-pass wavefunction transform (FP32 plans on 96^3)
   size_t wfn_ws_bytes = 0;
-  void* d_inv = nullptr;     // dielectric-inverse workspace (grown on demand)
   // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
-  // fixed-point pair stage, fixed-point wavefunctions, COH
-  LazyWs ws_mod, ws_bwd, ws_fx, ws_wfn, ws_coh;
+  // fixed-point pair stage, fixed-point wavefunctions, COH, dielectric inverse
+  LazyWs ws_mod, ws_bwd, ws_fx, ws_wfn, ws_coh, ws_inv;
   std::vector<void*> ws_kept;          // outgrown workspaces that a caller's captured graph still names
   cudaEvent_t wfn_ev = nullptr;        // last use of ws_wfn
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
@@ -118,7 +117,6 @@ struct chi0_plan_s {
   double2* pipe_f = nullptr;
   void* pipe_pack = nullptr;
   int pipe_state = 0;           // 0 not set up, 1 ready, -1 unavailable (serial build)
-  size_t inv_bytes = 0;
   // look-ahead of the dielectric inverse: the next panel runs beside the trailing update
   cudaStream_t inv_side = nullptr;
   cudaEvent_t inv_ev[2] = {};

@@ -104,9 +104,9 @@ void free_plan(chi0_plan_s* p) {
   cudaFree(w.T3d); cudaFree(w.T3f); cudaFree((void*)w.fx_tw);
   for (auto& a : w.fx) cudaFree((void*)a.coef);
   cudaFree(p->d_omega); cudaFree(p->d_D); cudaFree(p->d_M); cudaFree(p->d_f);
-  cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->d_inv); cudaFree(p->wfn_ws);
+  cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->wfn_ws);
   cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p); cudaFree(p->ws_wfn.p);
-  cudaFree(p->ws_coh.p);
+  cudaFree(p->ws_coh.p); cudaFree(p->ws_inv.p);
   for (void* w : p->ws_kept) cudaFree(w);
   if (p->wfn_ev) cudaEventDestroy(p->wfn_ev);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
@@ -220,6 +220,12 @@ bool env_fault(const char* what) {
   return e && strcmp(e, what) == 0;
 }
 
+// CHI0_FAULT=ws:N refuses workspaces of N bytes and more
+bool ws_fault(size_t need) {
+  const char* e = getenv("CHI0_FAULT");
+  return e && strncmp(e, "ws:", 3) == 0 && need >= strtoull(e + 3, nullptr, 10);
+}
+
 chi0_status check_plan(chi0_plan_s* p) {
   if (!p) return CHI0_ERR_INVALID;
   int dev = -1;
@@ -295,12 +301,29 @@ static bool herm_pays(const chi0_plan_s* p, const chi0_plan_desc* d) {
   return herm < plain;
 }
 
+static void ws_drop(chi0_plan_s* p, LazyWs& w) {
+  // the graph of a batched build holds the address
+  if (p->graph_exec && w.p && (&w == &p->ws_mod || &w == &p->ws_fx)) {
+    cudaGraphExecDestroy(p->graph_exec);
+    p->graph_exec = nullptr;
+  }
+  if (w.captured) {
+    p->ws_kept.push_back(w.p);
+  } else {
+    cudaFree(w.p);   // waits for the work that uses it
+    p->ws_bytes -= w.bytes;
+  }
+  w.p = nullptr;
+  w.bytes = 0;
+  w.captured = false;
+}
+
 // A workspace of at least `need` bytes, allocated on first use and grown when a later call needs more:
 // not inside a stream capture (the CUDA-core kernels run there unless an earlier call has allocated
-// enough).  A size that could not be had is not asked for again.  A workspace that a caller's capture
-// has used is kept until the plan is destroyed when it is outgrown: the caller's graph names its address.
+// enough).  After a refusal the size is asked for again once the device has that much free.  A
+// workspace that a caller's capture has used is kept until the plan is destroyed when it is outgrown:
+// the caller's graph names its address.
 static bool ws_ready(chi0_plan_s* p, LazyWs& w, size_t need, cudaStream_t s) {
-  if (need >= w.limit) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
     cudaGetLastError();
@@ -312,34 +335,34 @@ static bool ws_ready(chi0_plan_s* p, LazyWs& w, size_t need, cudaStream_t s) {
     return true;
   }
   if (need <= w.bytes) return true;
+  if (ws_fault(need)) return false;
   // a capture on some other stream does not see the allocation
   cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
   cudaThreadExchangeStreamCaptureMode(&mode);
-  // the graph of a batched build holds the old address
-  if (p->graph_exec) {
-    cudaGraphExecDestroy(p->graph_exec);
-    p->graph_exec = nullptr;
+  const size_t reuse = w.captured ? 0 : w.bytes;   // freed below when the new one does not fit beside it
+  size_t avail = 0, total = 0;
+  void* fresh = nullptr;
+  bool ok = need < w.refused || (cudaMemGetInfo(&avail, &total) == cudaSuccess && avail + reuse >= need);
+  if (ok) {
+    ok = cudaMalloc(&fresh, need) == cudaSuccess;
+    if (!ok && reuse) {
+      cudaGetLastError();
+      ws_drop(p, w);
+      ok = cudaMalloc(&fresh, need) == cudaSuccess;
+    }
+    if (!ok) w.refused = need;
   }
-  if (w.captured) {
-    p->ws_kept.push_back(w.p);
-    w.captured = false;
+  if (ok) {
+    ws_drop(p, w);
+    w.p = fresh;
+    w.bytes = need;
+    w.refused = SIZE_MAX;
+    p->ws_bytes += need;
   } else {
-    cudaFree(w.p);   // waits for the work that uses it
-    p->ws_bytes -= w.bytes;
-  }
-  w.p = nullptr;
-  w.bytes = 0;
-  const cudaError_t e = cudaMalloc(&w.p, need);
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  if (e != cudaSuccess) {
     cudaGetLastError();
-    w.p = nullptr;
-    w.limit = need;
-    return false;
   }
-  w.bytes = need;
-  p->ws_bytes += need;
-  return true;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return ok;
 }
 
 extern "C" {
@@ -584,27 +607,11 @@ chi0_status chi0_epsilon_inverse(chi0_plan p, int iq, void* eps, void* stream) {
   if (!eps) return fail(p, CHI0_ERR_INVALID, "NULL buffer");
   const int nG = p->q[iq].nG;
   // with the memory of the refinement where that can be had, else without
-  bool refined = chi0::eps_inverse_refines(p, nG);
-  for (;;) {
-    const size_t need = chi0::eps_inverse_ws_bytes(p, nG, refined);
-    if (need <= p->inv_bytes) break;
-    CK(p, cudaStreamSynchronize((cudaStream_t)stream));
-    cudaFree(p->d_inv);
-    p->d_inv = nullptr;
-    p->ws_bytes -= p->inv_bytes;
-    p->inv_bytes = 0;
-    const cudaError_t e = cudaMalloc(&p->d_inv, need);
-    if (e == cudaSuccess) {
-      p->inv_bytes = need;
-      p->ws_bytes += need;
-      break;
-    }
-    cudaGetLastError();
-    p->d_inv = nullptr;
-    if (!refined) CK(p, e);
-    refined = false;
-  }
-  CK(p, chi0::launch_epsilon_inverse(p, nG, (double2*)eps, p->d_inv, refined, (cudaStream_t)stream));
+  const bool refined = chi0::eps_inverse_refines(p, nG) &&
+                       ws_ready(p, p->ws_inv, chi0::eps_inverse_ws_bytes(p, nG, true), (cudaStream_t)stream);
+  if (!refined && !ws_ready(p, p->ws_inv, chi0::eps_inverse_ws_bytes(p, nG, false), (cudaStream_t)stream))
+    return fail(p, CHI0_ERR_OOM, "chi0_epsilon_inverse: workspace (a captured call needs one before it)");
+  CK(p, chi0::launch_epsilon_inverse(p, nG, (double2*)eps, p->ws_inv.p, refined, (cudaStream_t)stream));
   return CHI0_OK;
 }
 
@@ -720,7 +727,6 @@ chi0_status chi0_sigma_coh(chi0_plan p, int iq, const void* m, int n_t, int n_b,
   cudaStream_t s = (cudaStream_t)stream;
   const size_t bytes = chi0::sigma_coh_ws_bytes(p, nG, n_t);
   // kept by the plan: an allocation and a release per call took 0.2 ms of a 12 ms sum
-  p->ws_coh.limit = SIZE_MAX;   // nothing else computes the sum: ask again after a refusal
   if (!ws_ready(p, p->ws_coh, bytes, s)) return fail(p, CHI0_ERR_OOM, "chi0_sigma_coh: workspace");
   void* ws = p->ws_coh.p;
   cudaError_t e = cudaSuccess;
