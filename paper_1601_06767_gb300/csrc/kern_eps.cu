@@ -748,8 +748,9 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 // 42 ms for one 1200^2.  Here X is the FP32 inverse and every step takes
 //   R = I - A X,  X += X R   (Newton; the error is squared)
 // with both products exact modular ones on the tensor cores (modgemm.cuh).  A step
-// whose largest |R| is at most 2^-32 is a matrix's last: the error left is below
-// the rounding of X.  A matrix that has no such step within STEPS (ill conditioned
+// with |R| <= 2^-26.5 in the Frobenius norm is a matrix's last: the error left, X R^2,
+// is at most 2^-53 of X.  (A bound on the largest element alone leaves up to N^2
+// times its square.)  A matrix that has no such step within STEPS (ill conditioned
 // beyond FP32, out of its range, singular, not finite) is inverted by the FP64
 // elimination from the untouched A, whose kernels skip the others.
 //
@@ -758,26 +759,24 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 // 1.8e-16 (relative Frobenius, eps-like matrices), 3.3e-16 by the elimination.
 namespace {
 constexpr int STEPS = 3;
-constexpr uint32_t LAST_STEP = (uint32_t)(1023 - 32) << 20;     // magnitude word of 2^-32
+constexpr double LAST_STEP = 1.1102230246251565e-16;            // |R|^2 = 2^-53
 
-__global__ void k_ref_init(int* __restrict__ todo, uint32_t* __restrict__ rmax, int nf) {
-  for (int w = threadIdx.x; w < nf; w += blockDim.x) {
-    todo[w] = 1;
-    rmax[w] = 0;
-  }
+__global__ void k_ref_init(int* __restrict__ todo, int nf) {
+  for (int w = threadIdx.x; w < nf; w += blockDim.x) todo[w] = 1;
 }
 
-// values of the residue planes of one N x N product.  LAST = false: R = I - value and the largest
-// magnitude word of R; true: X += value.  A warp takes 16 rows x 8 columns (as k_mod_add).
+// values of the residue planes of one N x N product.  ADD = false: R = I - value and the sum of
+// |R|^2 over the block's elements; true: X += value.  A warp takes 16 rows x 8 columns (as k_mod_add).
 template <bool ADD>
 __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P, int N, int ldR,
                                                    const int* __restrict__ sA, const int* __restrict__ sB,
-                                                   double2* __restrict__ out, uint32_t* __restrict__ rmax,
+                                                   double2* __restrict__ out, float* __restrict__ part,
                                                    const int* __restrict__ todo) {
   if (*todo == 0) return;
+  __shared__ float red[4];
   const int lane = threadIdx.x & 31;
   const int j0 = 8 * (blockIdx.x * 4 + (threadIdx.x >> 5)), i = blockIdx.y * 16 + (lane >> 1);
-  uint32_t big = 0;
+  float sq = 0.f;
   if (j0 < N && i < N) {
     double2* o = out + (size_t)i * N + j0 + (lane & 1);
     double2 v[4];
@@ -795,20 +794,32 @@ __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P
       const bool bad = sa == mod::NO_SCALE || sb == mod::NO_SCALE;
       const double x = bad ? nan("") : mod::frac_value(re[c], -sa - sb), y = bad ? nan("") : mod::frac_value(im[c], -sa - sb);
       const double2 r = ADD ? make_double2(v[c].x + x, v[c].y + y) : make_double2((i == j ? 1.0 : 0.0) - x, -y);
-      if (!ADD) big = max(big, max(mod::mag_word(r.x), mod::mag_word(r.y)));
+      if (!ADD) sq = fmaf((float)r.x, (float)r.x, fmaf((float)r.y, (float)r.y, sq));
       o[2 * c] = r;
     }
   }
   if (!ADD) {
-    big = __reduce_max_sync(0xffffffffu, big);
-    if (lane == 0) atomicMax(rmax, big);
+    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane == 0) red[threadIdx.x >> 5] = sq;
+    __syncthreads();
+    if (threadIdx.x == 0) part[blockIdx.y * gridDim.x + blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
   }
 }
 
-// after a step: the matrix is done when its R was small enough; the next step starts from 0
-__global__ void k_ref_decide(uint32_t* __restrict__ rmax, int* __restrict__ todo) {
-  if (*todo && *rmax <= LAST_STEP) *todo = 0;
-  *rmax = 0;
+// after a step: the matrix is done when its R was small enough (sums in a fixed order; an infinity or a
+// NaN is not small)
+__global__ void __launch_bounds__(256) k_ref_decide(const float* __restrict__ part, int n, int* __restrict__ todo) {
+  __shared__ double red[8];
+  if (*todo == 0) return;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < n; i += 256) s += (double)part[i];
+  for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) s += red[w];
+    if (s <= LAST_STEP) *todo = 0;
+  }
 }
 
 // eps = X where the matrix is done (todo 0)
@@ -822,8 +833,9 @@ __global__ void __launch_bounds__(256) k_ref_store(const double2* __restrict__ X
 // planes of A, planes of X rows, planes of a transposed operand, residues, scales
 struct RefSizes {
   int Kp, ldR;
-  size_t x, r, pa, px, pt, res, sa, sx, st, cols, todo, rmax, bytes;
+  size_t x, r, pa, px, pt, res, sa, sx, st, cols, todo, part, bytes;
 };
+dim3 ref_grid(int N) { return dim3(((N + 7) / 8 + 3) / 4, (N + 15) / 16); }   // k_ref_value
 RefSizes ref_sizes(int N, int nf) {
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
   RefSizes z;
@@ -841,8 +853,9 @@ RefSizes ref_sizes(int N, int nf) {
   z.st = z.sx + sc;
   z.cols = z.st + sc;
   z.todo = z.cols + al(mod_cols_ws_bytes(N, N));
-  z.rmax = z.todo + al((size_t)nf * sizeof(int));
-  z.bytes = z.rmax + al((size_t)nf * sizeof(uint32_t));
+  z.part = z.todo + al((size_t)nf * sizeof(int));
+  const dim3 g = ref_grid(N);
+  z.bytes = z.part + al((size_t)g.x * g.y * sizeof(float));
   return z;
 }
 
@@ -855,15 +868,15 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
   uint16_t *PA = (uint16_t*)(b + z.pa), *PX = (uint16_t*)(b + z.px), *PT = (uint16_t*)(b + z.pt);
   int16_t* res = (int16_t*)(b + z.res);
   int *sA = (int*)(b + z.sa), *sX = (int*)(b + z.sx), *sT = (int*)(b + z.st), *todo = (int*)(b + z.todo);
-  uint32_t* rmax = (uint32_t*)(b + z.rmax);
+  float* part = (float*)(b + z.part);
   const int64_t n2 = (int64_t)N * N;
   {
     ProfScope ps(p, CHI0_K_EPS, s, 2);
-    k_ref_init<<<1, 128, 0, s>>>(todo, rmax, nf);
+    k_ref_init<<<1, 128, 0, s>>>(todo, nf);
     k_to_c64<<<4 * 152, 256, 0, s>>>(eps, nf * n2, a32);
   }
   cudaError_t e = gj_invert<float>(p, a32, N, nf, Z, Tb, piv, cand, nullptr, nullptr, s);
-  const dim3 gv((z.ldR / 8 + 3) / 4, (N + 15) / 16);
+  const dim3 gv = ref_grid(N);
   for (int w = 0; w < nf && e == cudaSuccess; ++w) {
     ProfScope ps(p, CHI0_K_INV_UPDATE, s, 4 + STEPS * 15);
     const double2* A = eps + w * n2;
@@ -873,13 +886,13 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
       e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
       if (e == cudaSuccess)
         e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
-      k_ref_value<false><<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, rmax + w, todo + w);
+      k_ref_value<false><<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, part, todo + w);
       if (e == cudaSuccess) e = launch_mod_pack_rows(X, N, N, N, z.Kp, true, sX, PX, s, todo + w);
       if (e == cudaSuccess) e = launch_mod_pack_cols(R, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
       if (e == cudaSuccess)
         e = launch_mod_gemm(p, ModGemm{PX, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
       k_ref_value<true><<<gv, 128, 0, s>>>(res, N, z.ldR, sX, sT, X, nullptr, todo + w);
-      k_ref_decide<<<1, 1, 0, s>>>(rmax + w, todo + w);
+      k_ref_decide<<<1, 256, 0, s>>>(part, (int)(gv.x * gv.y), todo + w);
     }
     k_ref_store<<<4 * 152, 256, 0, s>>>(X, n2, eps + w * n2, todo + w);
     if (e == cudaSuccess) e = cudaGetLastError();
