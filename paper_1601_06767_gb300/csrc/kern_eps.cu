@@ -752,7 +752,12 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 // is at most 2^-53 of X.  (A bound on the largest element alone leaves up to N^2
 // times its square.)  A matrix that has no such step within STEPS (ill conditioned
 // beyond FP32, out of its range, singular, not finite) is inverted by the FP64
-// elimination from the untouched A, whose kernels skip the others.
+// elimination from A, whose kernels skip the others.
+//
+// All of this is done on A with its columns scaled to the same power of two, and the
+// rows of the result scaled back: both exact.  The products are rounded relative to
+// |row of A| |column of X|, where a graded A would lose the ratio of its columns (an
+// elimination does not: it gives the same digits for any column scaling).
 //
 // 1200^2: 42.6 -> 7.9 ms (FP32 inverse 6.2, one matrix's latency; two steps 0.8,
 // skipped kernels 0.7); 9 x 2500^2: 1047 ms at first, 72 ms.  Against quad precision
@@ -760,6 +765,38 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 namespace {
 constexpr int STEPS = 3;
 constexpr double LAST_STEP = 1.1102230246251565e-16;            // |R|^2 = 2^-53
+
+// cmax[w][j] = largest magnitude word of column j (cleared by the caller); a CTA takes 64 columns x 128 rows
+__global__ void __launch_bounds__(256) k_ref_colmax(const double2* __restrict__ A, int N, uint32_t* __restrict__ cmax) {
+  const int j = blockIdx.x * 64 + (threadIdx.x & 63), w = blockIdx.z;
+  if (j >= N) return;
+  const double2* a = A + (size_t)w * N * N;
+  const int i1 = min(N, (int)(blockIdx.y + 1) * 128);
+  uint32_t m = 0;
+  for (int i = blockIdx.y * 128 + (threadIdx.x >> 6); i < i1; i += 4) {
+    const double2 v = a[(size_t)i * N + j];
+    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  atomicMax(cmax + (size_t)w * N + j, m);
+}
+// 2^-e of a column: e the exponent of its largest component (0 for zeros, subnormal and non-finite columns)
+__device__ __forceinline__ double col_scale(uint32_t w) {
+  return w >= 0x00100000u && w < 0x7ff00000u ? mod::pow2d(-min(mod::word_exp(w), 1022)) : 1.0;
+}
+// A = A diag(2^-e) in place, and its complex64 copy
+__global__ void __launch_bounds__(256) k_ref_scale_cols(double2* __restrict__ A, int N, const uint32_t* __restrict__ cmax,
+                                                        float2* __restrict__ a32) {
+  const int j = blockIdx.x * 256 + threadIdx.x, w = blockIdx.z;
+  if (j >= N) return;
+  const double s = col_scale(cmax[(size_t)w * N + j]);
+  const int i1 = min(N, (int)(blockIdx.y + 1) * 16);
+  for (int i = blockIdx.y * 16; i < i1; ++i) {
+    const size_t o = ((size_t)w * N + i) * N + j;
+    const double2 v = make_double2(A[o].x * s, A[o].y * s);
+    A[o] = v;
+    a32[o] = make_float2((float)v.x, (float)v.y);
+  }
+}
 
 __global__ void k_ref_init(int* __restrict__ todo, int nf) {
   for (int w = threadIdx.x; w < nf; w += blockDim.x) todo[w] = 1;
@@ -822,18 +859,27 @@ __global__ void __launch_bounds__(256) k_ref_decide(const float* __restrict__ pa
   }
 }
 
-// eps = X where the matrix is done (todo 0)
-__global__ void __launch_bounds__(256) k_ref_store(const double2* __restrict__ X, int64_t n, double2* __restrict__ eps,
-                                                   const int* __restrict__ todo) {
-  if (*todo != 0) return;
-  for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < n; e += (int64_t)gridDim.x * 256) eps[e] = X[e];
+// eps = diag(2^-e) Y of matrix blockIdx.y, Y = X where the matrix is done (todo 0), else the elimination's result in eps itself
+__global__ void __launch_bounds__(256) k_ref_store(const double2* X, int N, const uint32_t* __restrict__ cmax,
+                                                   double2* eps, const int* __restrict__ todo, int if_todo) {
+  if ((todo[blockIdx.y] != 0) != (if_todo != 0)) return;
+  X += (size_t)blockIdx.y * N * N;
+  eps += (size_t)blockIdx.y * N * N;
+  cmax += (size_t)blockIdx.y * N;
+  for (int i = blockIdx.x; i < N; i += gridDim.x) {
+    const double s = col_scale(cmax[i]);
+    for (int j = threadIdx.x; j < N; j += 256) {
+      const double2 v = X[(size_t)i * N + j];
+      eps[(size_t)i * N + j] = make_double2(v.x * s, v.y * s);
+    }
+  }
 }
 
 // offsets of the refinement's workspace: FP32 copies of all matrices, then for one matrix at a time X, R,
 // planes of A, planes of X rows, planes of a transposed operand, residues, scales
 struct RefSizes {
   int Kp, ldR;
-  size_t x, r, pa, px, pt, res, sa, sx, st, cols, todo, part, bytes;
+  size_t x, r, pa, px, pt, res, sa, sx, st, cols, todo, part, cmax, bytes;
 };
 dim3 ref_grid(int N) { return dim3(((N + 7) / 8 + 3) / 4, (N + 15) / 16); }   // k_ref_value
 RefSizes ref_sizes(int N, int nf) {
@@ -855,7 +901,8 @@ RefSizes ref_sizes(int N, int nf) {
   z.todo = z.cols + al(mod_cols_ws_bytes(N, N));
   z.part = z.todo + al((size_t)nf * sizeof(int));
   const dim3 g = ref_grid(N);
-  z.bytes = z.part + al((size_t)g.x * g.y * sizeof(float));
+  z.cmax = z.part + al((size_t)g.x * g.y * sizeof(float));
+  z.bytes = z.cmax + al((size_t)nf * N * sizeof(uint32_t));
   return z;
 }
 
@@ -869,11 +916,15 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
   int16_t* res = (int16_t*)(b + z.res);
   int *sA = (int*)(b + z.sa), *sX = (int*)(b + z.sx), *sT = (int*)(b + z.st), *todo = (int*)(b + z.todo);
   float* part = (float*)(b + z.part);
+  uint32_t* cmax = (uint32_t*)(b + z.cmax);
   const int64_t n2 = (int64_t)N * N;
   {
-    ProfScope ps(p, CHI0_K_EPS, s, 2);
+    ProfScope ps(p, CHI0_K_EPS, s, 3);
     k_ref_init<<<1, 128, 0, s>>>(todo, nf);
-    k_to_c64<<<4 * 152, 256, 0, s>>>(eps, nf * n2, a32);
+    const cudaError_t em = cudaMemsetAsync(cmax, 0, (size_t)nf * N * sizeof(uint32_t), s);
+    if (em != cudaSuccess) return em;
+    k_ref_colmax<<<dim3((N + 63) / 64, (N + 127) / 128, nf), 256, 0, s>>>(eps, N, cmax);
+    k_ref_scale_cols<<<dim3((N + 255) / 256, (N + 15) / 16, nf), 256, 0, s>>>(eps, N, cmax, a32);
   }
   cudaError_t e = gj_invert<float>(p, a32, N, nf, Z, Tb, piv, cand, nullptr, nullptr, s);
   const dim3 gv = ref_grid(N);
@@ -894,11 +945,15 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
       k_ref_value<true><<<gv, 128, 0, s>>>(res, N, z.ldR, sX, sT, X, nullptr, todo + w);
       k_ref_decide<<<1, 256, 0, s>>>(part, (int)(gv.x * gv.y), todo + w);
     }
-    k_ref_store<<<4 * 152, 256, 0, s>>>(X, n2, eps + w * n2, todo + w);
+    k_ref_store<<<4 * 152, 256, 0, s>>>(X, N, cmax + (size_t)w * N, eps + w * n2, todo + w, 0);
     if (e == cudaSuccess) e = cudaGetLastError();
   }
   if (e != cudaSuccess) return e;
-  return gj_invert<double>(p, eps, N, nf, Z, Tb, piv, cand, p->d_status, todo, s);
+  e = gj_invert<double>(p, eps, N, nf, Z, Tb, piv, cand, p->d_status, todo, s);
+  if (e != cudaSuccess) return e;
+  ProfScope ps(p, CHI0_K_EPS, s, 1);
+  k_ref_store<<<dim3(4 * 152, nf), 256, 0, s>>>(eps, N, cmax, eps, todo, 1);
+  return cudaGetLastError();
 }
 }  // namespace
 
