@@ -297,6 +297,7 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
 // (reconstruction of two values from 52 residues), the FP64 pipe a third of it: 356 us for 4096
 // pairs, N_G 1200, one frequency (530 us with one CTA per SM, before its registers were bounded).
 // The whole adjoint of that size: 77.0 -> 1.02 ms.
+constexpr int BM_PAIRS = 16;
 template <typename C>
 __global__ void __launch_bounds__(256, 2)
 k_bwd_mod(const int16_t* __restrict__ R, int rows, int ldR, const int* __restrict__ sA, const int* __restrict__ sB,
@@ -528,7 +529,8 @@ static BwdMod bwd_mod_sizes(const chi0_plan_s* p, int nG, int64_t n_pairs) {
   const int64_t gam = (int64_t)2 * mod::NPL * 2 * nG * z.Kp;                  // one frequency's planes
   z.nw = (int)std::max<int64_t>(1, std::min<int64_t>(p->n_freq, kMem / gam));
   const int64_t per_pair = (int64_t)2 * z.nw * mod::NPL * 2 * z.ldR;           // residues of one pair
-  z.kc = (int)std::min<int64_t>({n_pairs, p->max_pairs, std::max<int64_t>(256, kMem / per_pair / 256 * 256)});
+  z.kc = (int)std::min<int64_t>({n_pairs, p->max_pairs, std::max<int64_t>(256, kMem / per_pair / 256 * 256),
+                                 (int64_t)65535 * BM_PAIRS});   // grid y of k_bwd_mod
   z.off_a = al((size_t)gam * z.nw);
   z.off_r = z.off_a + al((size_t)mod::NPL * 2 * z.kc * z.Kp);
   z.off_sa = z.off_r + al((size_t)2 * z.nw * mod::NPL * 2 * mod::res_plane(z.kc, z.ldR));
@@ -575,7 +577,7 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
       ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
-      k_bwd_mod<C><<<dim3(ntile, (K + 15) / 16), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,
+      k_bwd_mod<C><<<dim3(ntile, (K + BM_PAIRS - 1) / BM_PAIRS), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,
                                                               w_col, p->d_omega, w0, nw, p->delta, gM + p0 * nG, part,
                                                               ntile);
     }

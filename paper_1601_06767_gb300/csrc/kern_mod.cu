@@ -579,7 +579,7 @@ bool encode(CUtensorMap* tm, const void* base, int Kp, int rows, int planes) {
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int round64(int64_t x) { return (int)((x + 63) / 64 * 64); }
+int64_t round64(int64_t x) { return (x + 63) / 64 * 64; }
 size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
@@ -631,7 +631,8 @@ ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
   ModSizes z;
   z.ldR = (nG + 7) / 8 * 8;
   const int64_t per_pair = (int64_t)NPL * 2 * nG;
-  z.Kc = (int)std::min<int64_t>(round64(p->max_pairs), std::max<int64_t>(64, kPlanes / per_pair / 64 * 64));
+  z.Kc = (int)std::min<int64_t>({round64(p->max_pairs), std::max<int64_t>(64, kPlanes / per_pair / 64 * 64),
+                                 (int64_t)65535 * PK_K});   // grid y of k_mod_pack
   // enough frequencies per launch for 40 waves of CTA pairs, within the same memory
   const int64_t tiles = (int64_t)((nG + GM - 1) / GM) * ((nG + GN - 1) / GN) * NPL;
   int64_t nw = std::min<int64_t>(p->n_freq, std::max<int64_t>(1, (40 * 76 + tiles - 1) / tiles));
@@ -703,7 +704,7 @@ cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_
   int* scale = reinterpret_cast<int*>(b + z.off_scale);
   uint32_t* eg = reinterpret_cast<uint32_t*>(b + z.off_exp);
   uint32_t* ef = eg + nG;
-  const int nf = p->n_freq, Kp = round64(K);
+  const int nf = p->n_freq, Kp = (int)round64(K);
   cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * nG, s);
   if (e != cudaSuccess) return e;
   const int n_part = (int)((K + ST_ROWS - 1) / ST_ROWS);
