@@ -181,37 +181,39 @@ cudaError_t launch_fx_gather(const chi0_plan_s* p, int iq, int nv, int nc, const
 // frequency factors f[w][k] for pairs p0..p0+K of an (n_v x n_c) set
 cudaError_t launch_weights(const chi0_plan_s* p, int64_t p0, int64_t K, int n_c, const double* E_v,
                            const double* E_col, const double* w_col, double2* f, cudaStream_t s);
+// flags: not NULL = only the 64 x 64 tiles [n_freq][tiles][tiles] of chi0 that are not 0 there
 cudaError_t launch_contract_f64(const chi0_plan_s* p, int nG, const double2* M, int64_t K,
-                                const double2* f, double2* chi, cudaStream_t s);
+                                const double2* f, double2* chi, cudaStream_t s, const int* flags = nullptr);
 // FP64 contraction by exact modular products on the tensor cores (kern_mod.cu)
 struct ModSizes {
   int Kc, nw, rows, ldR, n_part;   // pairs, frequencies and chi0 rows at a time; row stride of the residues
-  size_t off_a, off_r, off_part, off_scale, off_exp, bytes;
+  size_t off_a, off_r, off_part, off_scale, off_exp, off_norm, off_flag, bytes_flag, bytes;
 };
 ModSizes mod_sizes(const chi0_plan_s* p, int nG);
 int mod_launches(const chi0_plan_s* p, int nG);   // kernels per block of pairs
 bool mod_gemm_usable();
 cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_t K, const double2* f, double2* chi,
                                 void* ws, cudaStream_t s);
-// residue products R[plane][rows][cols] = A[plane mod a_planes] B[plane mod b_planes]^T
+// residue products (set: planes of a product, modgemm.cuh) R[plane][rows][cols] = A[plane mod a_planes] B[plane mod b_planes]^T
 struct ModGemm {
   const uint16_t* A;               // [a_planes][rows_a][Kp]
   const uint16_t* B;               // [b_planes][cols][Kp]
   int16_t* R;                      // [planes][rows][ldR]
-  int rows_a, row0, rows, cols, ldR, Kp, planes, a_planes, b_planes;
+  int rows_a, row0, rows, cols, ldR, Kp, planes, a_planes, b_planes, set;
   const int* todo;
 };
 cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s);
-// scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B.
+// scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B; norm not
+// NULL: scaled norms [rows] and a 27th plane of magnitudes.
 // todo (here, below and in ModGemm): not NULL = the kernels do nothing where it points at 0
 cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
+                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
 cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
+                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
 // the same of the transpose (conj: conjugate transpose) of X [n][rows] (operand B; ws: mod_cols_ws_bytes)
 size_t mod_cols_ws_bytes(int n, int rows);
-cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, uint16_t* planes,
-                                 void* ws, cudaStream_t s, const int* todo = nullptr);
+cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, float* norm,
+                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo = nullptr);
 // one q-point's share of a batched tensor-core contraction
 struct TcJob {
   int nG;

@@ -561,20 +561,20 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
     const int K = (int)std::min<int64_t>(z.kc, n_pairs - p0);
     double* gdE = work;
     double* part = work + K;
-    e = launch_mod_pack_rows(M + p0 * nG, K, nG, nG, z.Kp, true, sA, Ap, s);
+    e = launch_mod_pack_rows(M + p0 * nG, K, nG, nG, z.Kp, true, sA, nullptr, Ap, s);
     if (e != cudaSuccess) return e;
     for (int w0 = 0; w0 < p->n_freq; w0 += z.nw) {
       const int nw = std::min(z.nw, p->n_freq - w0);
       if (p0 == 0 || z.nw < p->n_freq)
         for (int w = 0; w < nw; ++w) {
           const double2* G = gamma + (size_t)(w0 + w) * nG * nG;
-          e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG, Bp + 2 * w * set, s);
+          e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG, nullptr, Bp + 2 * w * set, s);
           if (e == cudaSuccess)
-            e = launch_mod_pack_cols(G, nG, nG, z.Kp, true, sB + (size_t)(2 * w + 1) * nG, Bp + (2 * w + 1) * set,
+            e = launch_mod_pack_cols(G, nG, nG, z.Kp, true, sB + (size_t)(2 * w + 1) * nG, nullptr, Bp + (2 * w + 1) * set,
                                           b + z.off_ws, s);
           if (e != cudaSuccess) return e;
         }
-      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL, nullptr};
+      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL, mod::NPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
       k_bwd_mod<C><<<dim3(ntile, (K + BM_PAIRS - 1) / BM_PAIRS), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,

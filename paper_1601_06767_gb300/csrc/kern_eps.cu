@@ -932,16 +932,16 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
     ProfScope ps(p, CHI0_K_INV_UPDATE, s, 4 + STEPS * 15);
     const double2* A = eps + w * n2;
     k_from_c64<<<4 * 152, 256, 0, s>>>(a32 + w * n2, n2, X);
-    e = launch_mod_pack_rows(A, N, N, N, z.Kp, true, sA, PA, s);
+    e = launch_mod_pack_rows(A, N, N, N, z.Kp, true, sA, nullptr, PA, s);
     for (int it = 0; it < STEPS && e == cudaSuccess; ++it) {
-      e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
+      e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, nullptr, PT, b + z.cols, s, todo + w);
       if (e == cudaSuccess)
-        e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
+        e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
       k_ref_value<false><<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, part, todo + w);
-      if (e == cudaSuccess) e = launch_mod_pack_rows(X, N, N, N, z.Kp, true, sX, PX, s, todo + w);
-      if (e == cudaSuccess) e = launch_mod_pack_cols(R, N, N, z.Kp, false, sT, PT, b + z.cols, s, todo + w);
+      if (e == cudaSuccess) e = launch_mod_pack_rows(X, N, N, N, z.Kp, true, sX, nullptr, PX, s, todo + w);
+      if (e == cudaSuccess) e = launch_mod_pack_cols(R, N, N, z.Kp, false, sT, nullptr, PT, b + z.cols, s, todo + w);
       if (e == cudaSuccess)
-        e = launch_mod_gemm(p, ModGemm{PX, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
+        e = launch_mod_gemm(p, ModGemm{PX, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
       k_ref_value<true><<<gv, 128, 0, s>>>(res, N, z.ldR, sX, sT, X, nullptr, todo + w);
       k_ref_decide<<<1, 256, 0, s>>>(part, (int)(gv.x * gv.y), todo + w);
     }

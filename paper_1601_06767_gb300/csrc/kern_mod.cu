@@ -28,6 +28,7 @@ namespace {
 
 using mod::NM;
 using mod::NPL;
+using mod::CPL;
 using mod::gather_fractions;
 using mod::res_index;
 using mod::res_plane;
@@ -150,19 +151,21 @@ __global__ void __launch_bounds__(256) k_mod_col_norms(const double2* __restrict
   if (r == 0 && G < nG) part[(size_t)blockIdx.y * nG + G] = (double)((red[0][g] + red[1][g]) + (red[2][g] + red[3][g]));
 }
 
-// scale exponents: slot 0 (conj(M), operand B) and 1 + w (W_w, operand A)
+// scale exponents and, where norm is not NULL, scaled norms: slot 0 (conj(M), operand B) and 1 + w (W_w, operand A)
 __global__ void __launch_bounds__(256) k_mod_scales(const double* __restrict__ part, int n_part, int nG, int n_freq,
                                                     const uint32_t* __restrict__ eg, const uint32_t* __restrict__ ef,
-                                                    int* __restrict__ scale) {
+                                                    int* __restrict__ scale, float* __restrict__ norm) {
   const int G = blockIdx.x * blockDim.x + threadIdx.x, slot = blockIdx.y;
   if (G >= nG) return;
   double s = 0.0;
   for (int b = 0; b < n_part; ++b) s += part[((size_t)b * (n_freq + 1) + slot) * nG + G];
   const uint32_t wg = eg[G], wf = slot ? ef[slot - 1] : 0x3ff00000u;
   int r;
+  const int e = mod::word_exp(wg) + (slot ? mod::word_exp(wf) : 0), beta = slot ? mod::BETA_A : mod::BETA_B;
   if (wg >= 0x7ff00000u || wf >= 0x7ff00000u) r = mod::NO_SCALE;   // the result row is NaN
-  else r = mod::scale_exp(s, mod::word_exp(wg) + (slot ? mod::word_exp(wf) : 0), slot ? mod::BETA_A : mod::BETA_B);
+  else r = mod::scale_exp(s, e, beta);
   scale[(size_t)slot * nG + G] = r;
+  if (norm) norm[(size_t)slot * nG + G] = mod::scaled_norm(s, r, e, beta);
 }
 
 // ---------------------------------------------------------------------------
@@ -171,8 +174,10 @@ __global__ void __launch_bounds__(256) k_mod_scales(const double* __restrict__ p
 constexpr int PK_G = 16, PK_K = 64;   // tile: 16 sphere points x 64 pairs, transposed through shared memory
 
 // Planes [26][nG][Kp] (FP16) of conj(M) (of M: conj = false) into Bp (when not NULL) and of W_w = f(w) M,
-// w = w0 .. w0 + nw, into Ap (26 planes per frequency).  A warp holds one sphere
-// point, a lane two neighbouring pairs: 128-byte stores per plane.
+// w = w0 .. w0 + nw, into Ap (26 planes per frequency; CHECK: 27, with the
+// magnitudes).  A warp holds one sphere point, a lane two neighbouring pairs:
+// 128-byte stores per plane.
+template <bool CHECK>
 __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M, int nG, int64_t K, int Kp,
                                                   const double2* __restrict__ f, int w0, int nw,
                                                   const int* __restrict__ scale, bool conj, uint32_t* __restrict__ Bp,
@@ -198,7 +203,7 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
     }
     __syncthreads();
     const int* sc = scale + (size_t)(slot < 0 ? 0 : 1 + w0 + slot) * nG;
-    uint32_t* dst = slot < 0 ? Bp : Ap + (size_t)slot * NPL * plane;
+    uint32_t* dst = slot < 0 ? Bp : Ap + (size_t)slot * (CHECK ? CPL : NPL) * plane;
     for (int g = warp; g < PK_G; g += 8) {
       const int G = G0 + g;
       if (G >= nG) break;
@@ -208,9 +213,11 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
         a = cmul(fs[2 * lane], a);
         b = cmul(fs[2 * lane + 1], b);
       }
-      mod::store_residues(mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s)),
-                          mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), slot < 0 && conj,
-                          dst + (size_t)G * (Kp / 2) + p0 / 2 + lane, plane);
+      const mod::Limbs x = mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s));
+      const mod::Limbs y = mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s));
+      uint32_t* o = dst + (size_t)G * (Kp / 2) + p0 / 2 + lane;
+      mod::store_residues(x, y, slot < 0 && conj, o, plane);
+      if (CHECK) mod::store_magnitudes(x, y, slot < 0 ? mod::BETA_B : mod::BETA_A, o, plane);
     }
   }
 }
@@ -223,7 +230,8 @@ __device__ __forceinline__ double2 ld_wide(const double2* p, size_t i) { return 
 // largest: what underflows there does not count), summed in a fixed order
 template <typename C>
 __global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X, int n, size_t ld, int beta,
-                                                        int* __restrict__ scale, const int* __restrict__ todo) {
+                                                        int* __restrict__ scale, float* __restrict__ norm,
+                                                        const int* __restrict__ todo) {
   if (todo && *todo == 0) return;
   __shared__ uint32_t mx[4];
   __shared__ float sm[4];
@@ -249,16 +257,19 @@ __global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X,
   for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) sm[warp] = s;
   __syncthreads();
-  if (threadIdx.x == 0)
-    scale[blockIdx.x] = m >= 0x7ff00000u ? mod::NO_SCALE
-                                         : mod::scale_exp((double)((sm[0] + sm[1]) + (sm[2] + sm[3])), e, beta);
+  if (threadIdx.x == 0) {
+    const double n2 = (double)((sm[0] + sm[1]) + (sm[2] + sm[3]));
+    const int r = m >= 0x7ff00000u ? mod::NO_SCALE : mod::scale_exp(n2, e, beta);
+    scale[blockIdx.x] = r;
+    if (norm) norm[blockIdx.x] = mod::scaled_norm(n2, r, e, beta);
+  }
 }
 
-// planes [26][rows][Kp] of X; a warp takes 64 elements of a row
+// planes [26][rows][Kp] of X (beta not 0: 27, with the magnitudes); a warp takes 64 elements of a row
 template <typename C>
 __global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, int rows, int n, size_t ld, int Kp,
-                                                       const int* __restrict__ scale, uint32_t* __restrict__ dst,
-                                                       const int* __restrict__ todo) {
+                                                       const int* __restrict__ scale, int beta,
+                                                       uint32_t* __restrict__ dst, const int* __restrict__ todo) {
   if (todo && *todo == 0) return;
   const int lane = threadIdx.x & 31, segs = Kp / 64;
   const int64_t unit = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -268,15 +279,18 @@ __global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, 
   const int s = scale[r];
   const double2 a = k < n ? ld_wide(x, k) : make_double2(0.0, 0.0);
   const double2 b = k + 1 < n ? ld_wide(x, k + 1) : make_double2(0.0, 0.0);
-  mod::store_residues(mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s)),
-                      mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s)), false,
-                      dst + (size_t)r * (Kp / 2) + k / 2, (size_t)rows * (Kp / 2));
+  const mod::Limbs u = mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s));
+  const mod::Limbs v = mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s));
+  uint32_t* o = dst + (size_t)r * (Kp / 2) + k / 2;
+  mod::store_residues(u, v, false, o, (size_t)rows * (Kp / 2));
+  if (beta) mod::store_magnitudes(u, v, beta, o, (size_t)rows * (Kp / 2));
 }
 
 // ---------------------------------------------------------------------------
 // modular products
 // ---------------------------------------------------------------------------
-// R[b][i][j] = sum_k A[b][i][k] B[b][j][k] (mod m of plane b), |R| <= 257.
+// R[b][i][j] = sum_k A[b][i][k] B[b][j][k] (mod m of plane b), |R| <= 257; of the magnitudes' plane
+// the sum itself, rounded.
 // A CTA pair computes a 256 x 256 tile with tcgen05.mma.cta_group::2 (each CTA
 // holds 128 rows of A and 128 of B: 32 KB per 512 MMA cycles, half the operand
 // traffic per flop of two single-CTA 128 x 128 tiles).  Warp 0 issues the TMA
@@ -305,6 +319,7 @@ struct GemmArgs {
   int row0;                    // first row of A
   int tiles_m, tiles_n, n_b;   // tiles and planes
   int a_planes, b_planes;      // planes of A and B (a plane index is taken modulo these)
+  int set;                     // planes of a product: NPL, or CPL with the magnitudes
   int nK;                      // stages of GK
   const int* todo;             // not NULL: nothing is done where it points at 0
 };
@@ -334,7 +349,9 @@ __device__ __forceinline__ void gemm_item(const GemmArgs& P, int item, int& b, i
   tn = within / rows;
 }
 
-__constant__ float c_mod[NM] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f, 433.f, 421.f, 409.f, 401.f, 397.f, 389.f};
+// the moduli; for the magnitudes' plane one that their sums (below 2^14) never reach
+__constant__ float c_mod[NM + 1] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f,
+                                    433.f, 421.f, 409.f, 401.f, 397.f, 389.f, 1048576.f};
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
@@ -462,7 +479,7 @@ k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
     for (int item = pair; item < n_items && ok; item += npairs) {
       int b, tm, tn;
       gemm_item(P, item, b, tm, tn);
-      const float m = c_mod[(b % NPL) >> 1], im = 1.0f / m;
+      const float m = c_mod[(b % P.set) >> 1], im = 1.0f / m;
       const uint64_t inv2 = pack2(im, im), neg2 = pack2(-m, -m);
       const uint64_t magic = pack2(12582912.f, 12582912.f), nmagic = pack2(-12582912.f, -12582912.f);
       uint64_t acc[64];
@@ -524,23 +541,53 @@ k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
 // ---------------------------------------------------------------------------
 // reconstruction
 // ---------------------------------------------------------------------------
+// flags[z flag_step + tile] = 1 for the 64 x 64 tiles with an element whose S (modgemm.cuh) is below CHECK_MIN of its
+// rows' norms; R holds the products z = 0 .. gridDim.z of CPL planes each.  Grid (column tiles, row tiles, products);
+// tile row0 / 64 is the first of flag_cols tiles a row.  Zeros and non-finite rows raise no flag.
+__global__ void __launch_bounds__(128) k_mod_check(const int16_t* __restrict__ R, int rows, int cols, int ldR, int row0,
+                                                   const float* __restrict__ nA, size_t stepA,
+                                                   const float* __restrict__ nB, size_t stepB, int* __restrict__ flags,
+                                                   size_t flag_step) {
+  const int z = blockIdx.z, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int16_t* S = R + (size_t)z * CPL * res_plane(rows, ldR);
+  const float t = mod::CHECK_MIN * (float)(1 << 2 * mod::CHECK_BITS);
+  bool low = false;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {                     // a warp reads blocks of 32 rows x 8 columns
+    const int i = blockIdx.y * 64 + (q & 1) * 32 + lane, j0 = blockIdx.x * 64 + (warp + 4 * (q >> 1)) * 8;
+    if (i >= rows || j0 >= cols) continue;
+    const uint4 v = *reinterpret_cast<const uint4*>(S + res_index(rows, ldR, mod::CHECK_PLANE, i, j0));
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    const float ta = t * nA[z * stepA + row0 + i];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const float s = (float)(int16_t)(u[c >> 1] >> 16 * (c & 1));
+      if (j0 + c < cols && s < ta * nB[z * stepB + j0 + c]) low = true;
+    }
+  }
+  if (__syncthreads_or(low) && threadIdx.x == 0)
+    flags[z * flag_step + (size_t)(row0 / 64 + blockIdx.y) * gridDim.x + blockIdx.x] = 1;
+}
+
 // chi[w][row0 + i][j] += the value of R's planes (w, i, j).  A warp takes 16 rows x 8
 // columns (half a residue block); two neighbouring lanes share a row and take its
 // even and odd columns, so that each access to chi covers whole 32-byte sectors.
-// Grid (column blocks / 4, half row blocks, frequencies).
+// Grid (column blocks / 4, half row blocks, frequencies).  Flagged tiles are left out.
 __global__ void __launch_bounds__(128) k_mod_add(const int16_t* __restrict__ R, int rows, int row0, int nG, int ldR,
-                                                 const int* __restrict__ scale, int w0, double2* __restrict__ chi) {
+                                                 const int* __restrict__ scale, int w0, const int* __restrict__ flags,
+                                                 double2* __restrict__ chi) {
   const int lane = threadIdx.x & 31, w = blockIdx.z;
   const int j0 = 8 * (blockIdx.x * 4 + (threadIdx.x >> 5)), i = blockIdx.y * 16 + (lane >> 1);
   if (j0 >= nG || i >= rows) return;
-  const int G = row0 + i, sa = scale[(size_t)(1 + w0 + w) * nG + G];
+  const int G = row0 + i, sa = scale[(size_t)(1 + w0 + w) * nG + G], nt = (nG + 63) / 64;
+  if (flags[((size_t)(w0 + w) * nt + (G >> 6)) * nt + (j0 >> 6)]) return;
   double2* o = chi + ((size_t)(w0 + w) * nG + G) * nG + j0 + (lane & 1);
   double2 v[4];                                  // read early: the loads run beside those of the residues
 #pragma unroll
   for (int c = 0; c < 4; ++c)
     if (j0 + 2 * c + (lane & 1) < nG) v[c] = o[2 * c];
   mod::Frac re[4] = {}, im[4] = {};
-  gather_fractions(R + res_index(rows, ldR, w * NPL, i, j0), res_plane(rows, ldR), lane & 1 ? mod::ODD : mod::EVEN, re, im);
+  gather_fractions(R + res_index(rows, ldR, w * CPL, i, j0), res_plane(rows, ldR), lane & 1 ? mod::ODD : mod::EVEN, re, im);
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int j = j0 + 2 * c + (lane & 1);
@@ -615,6 +662,7 @@ cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s) {
   P.n_b = g.planes;
   P.a_planes = g.a_planes;
   P.b_planes = g.b_planes;
+  P.set = g.set;
   P.nK = g.Kp / GK;
   P.todo = g.todo;
   int dev = 0, nsm = 0;
@@ -630,48 +678,53 @@ ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
   constexpr int64_t kPlanes = (int64_t)4 << 30, kRes = (int64_t)4 << 30;   // operand planes, residues
   ModSizes z;
   z.ldR = (nG + 7) / 8 * 8;
-  const int64_t per_pair = (int64_t)NPL * 2 * nG;
+  const int64_t per_pair = (int64_t)CPL * 2 * nG;
   z.Kc = (int)std::min<int64_t>({round64(p->max_pairs), std::max<int64_t>(64, kPlanes / per_pair / 64 * 64),
                                  (int64_t)65535 * PK_K});   // grid y of k_mod_pack
   // enough frequencies per launch for 40 waves of CTA pairs, within the same memory
-  const int64_t tiles = (int64_t)((nG + GM - 1) / GM) * ((nG + GN - 1) / GN) * NPL;
+  const int64_t tiles = (int64_t)((nG + GM - 1) / GM) * ((nG + GN - 1) / GN) * CPL;
   int64_t nw = std::min<int64_t>(p->n_freq, std::max<int64_t>(1, (40 * 76 + tiles - 1) / tiles));
   nw = std::max<int64_t>(1, std::min(nw, kPlanes / (per_pair * z.Kc)));
-  nw = std::max<int64_t>(1, std::min(nw, kRes / ((int64_t)NPL * 2 * nG * z.ldR)));
+  nw = std::max<int64_t>(1, std::min(nw, kRes / ((int64_t)CPL * 2 * nG * z.ldR)));
   z.nw = (int)nw;
-  z.rows = (int)std::min<int64_t>(nG, std::max<int64_t>(GM, kRes / ((int64_t)NPL * 2 * z.ldR * nw) / GM * GM));
+  z.rows = (int)std::min<int64_t>(nG, std::max<int64_t>(GM, kRes / ((int64_t)CPL * 2 * z.ldR * nw) / GM * GM));
   z.n_part = (z.Kc + ST_ROWS - 1) / ST_ROWS;
   const size_t nf1 = (size_t)p->n_freq + 1;
   z.off_a = al256((size_t)per_pair * z.Kc);
   z.off_r = z.off_a + al256((size_t)per_pair * z.Kc * nw);
-  z.off_part = z.off_r + al256((size_t)NPL * 2 * nw * res_plane(z.rows, z.ldR));
+  z.off_part = z.off_r + al256((size_t)CPL * 2 * nw * res_plane(z.rows, z.ldR));
   z.off_scale = z.off_part + al256(nf1 * z.n_part * nG * sizeof(double));
   z.off_exp = z.off_scale + al256(nf1 * nG * sizeof(int));
-  z.bytes = z.off_exp + al256((nG + nf1) * sizeof(uint32_t));
+  z.off_norm = z.off_exp + al256((nG + nf1) * sizeof(uint32_t));
+  z.off_flag = z.off_norm + al256(nf1 * nG * sizeof(float));
+  const size_t nt = (nG + 63) / 64;
+  z.bytes_flag = (size_t)p->n_freq * nt * nt * sizeof(int);
+  z.bytes = z.off_flag + al256(z.bytes_flag);
   return z;
 }
 
 template <typename C>
-static cudaError_t pack_rows(const C* X, int rows, int n, size_t ld, int Kp, int beta, int* scale, uint16_t* planes,
-                             const int* todo, cudaStream_t s) {
-  k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale, todo);
+static cudaError_t pack_rows(const C* X, int rows, int n, size_t ld, int Kp, int beta, int* scale, float* norm,
+                             uint16_t* planes, const int* todo, cudaStream_t s) {
+  k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale, norm, todo);
   const int64_t units = (int64_t)rows * (Kp / 64);
-  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, (uint32_t*)planes, todo);
+  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, norm ? beta : 0,
+                                                                      (uint32_t*)planes, todo);
   return cudaGetLastError();
 }
-cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale, float* norm,
                                  uint16_t* planes, cudaStream_t s, const int* todo) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, todo, s);
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, planes, todo, s);
 }
-cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
+cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale, float* norm,
                                  uint16_t* planes, cudaStream_t s, const int* todo) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, planes, todo, s);
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, planes, todo, s);
 }
 size_t mod_cols_ws_bytes(int n, int rows) {
   return al256(sizeof(uint32_t) * rows) + sizeof(double) * ((n + ST_ROWS - 1) / ST_ROWS) * (size_t)rows;
 }
-cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, uint16_t* planes,
-                                 void* ws, cudaStream_t s, const int* todo) {
+cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, float* norm,
+                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo) {
   uint32_t* eg = reinterpret_cast<uint32_t*>(ws);
   double* part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(ws) + al256(sizeof(uint32_t) * rows));
   cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * rows, s);
@@ -680,16 +733,17 @@ cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool
   const dim3 gst((rows + ST_COLS - 1) / ST_COLS, n_part);
   k_mod_rowmax<<<gst, 256, 0, s>>>(X, rows, n, eg, todo);
   k_mod_col_norms<<<gst, 256, 0, s>>>(X, rows, n, eg, part, todo);
-  k_mod_scales<<<dim3((rows + 255) / 256, 1), 256, 0, s>>>(part, n_part, rows, 0, eg, nullptr, scale);
-  k_mod_pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale, conj,
-                                                                     (uint32_t*)planes, nullptr, todo);
+  k_mod_scales<<<dim3((rows + 255) / 256, 1), 256, 0, s>>>(part, n_part, rows, 0, eg, nullptr, scale, norm);
+  auto* pack = norm ? k_mod_pack<true> : k_mod_pack<false>;
+  pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale, conj,
+                                                               (uint32_t*)planes, nullptr, todo);
   return cudaGetLastError();
 }
 
 int mod_launches(const chi0_plan_s* p, int nG) {
   const ModSizes z = mod_sizes(p, nG);
   const int groups = (p->n_freq + z.nw - 1) / z.nw, panels = (nG + z.rows - 1) / z.rows;
-  return 4 + groups * (1 + 2 * panels);
+  return 5 + groups * (1 + 3 * panels);
 }
 
 // K <= mod_sizes().Kc pairs of M with factors f [n_freq][K]
@@ -704,28 +758,35 @@ cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_
   int* scale = reinterpret_cast<int*>(b + z.off_scale);
   uint32_t* eg = reinterpret_cast<uint32_t*>(b + z.off_exp);
   uint32_t* ef = eg + nG;
+  float* norm = reinterpret_cast<float*>(b + z.off_norm);
+  int* flags = reinterpret_cast<int*>(b + z.off_flag);
   const int nf = p->n_freq, Kp = (int)round64(K);
   cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * nG, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(flags, 0, z.bytes_flag, s);
   if (e != cudaSuccess) return e;
-  const int n_part = (int)((K + ST_ROWS - 1) / ST_ROWS);
+  const int n_part = (int)((K + ST_ROWS - 1) / ST_ROWS), nt = (nG + 63) / 64;
   const dim3 gst((nG + ST_COLS - 1) / ST_COLS, n_part);
   k_mod_fmax<<<nf, 256, 0, s>>>(f, K, ef);
   k_mod_rowmax<<<gst, 256, 0, s>>>(M, nG, K, eg, nullptr);
   k_mod_norms<<<gst, 256, 0, s>>>(M, nG, K, f, nf, eg, ef, part);
-  k_mod_scales<<<dim3((nG + 255) / 256, nf + 1), 256, 0, s>>>(part, n_part, nG, nf, eg, ef, scale);
+  k_mod_scales<<<dim3((nG + 255) / 256, nf + 1), 256, 0, s>>>(part, n_part, nG, nf, eg, ef, scale, norm);
   for (int w0 = 0; w0 < nf; w0 += z.nw) {
     const int nw = std::min(z.nw, nf - w0);
-    k_mod_pack<<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(
+    k_mod_pack<true><<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(
         M, nG, K, Kp, f, w0, nw, scale, true, w0 == 0 ? (uint32_t*)Bp : nullptr, (uint32_t*)Ap, nullptr);
     for (int r0 = 0; r0 < nG; r0 += z.rows) {
       const int rows = std::min(z.rows, nG - r0);
-      ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, NPL * nw, NPL * nw, NPL, nullptr};
+      ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, CPL * nw, CPL * nw, CPL, CPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
-      k_mod_add<<<dim3((z.ldR / 8 + 3) / 4, (rows + 15) / 16, nw), 128, 0, s>>>(R, rows, r0, nG, z.ldR, scale, w0, chi);
+      k_mod_check<<<dim3(nt, (rows + 63) / 64, nw), 128, 0, s>>>(R, rows, nG, z.ldR, r0, norm + (size_t)(1 + w0) * nG, nG,
+                                                                 norm, 0, flags + (size_t)w0 * nt * nt, (size_t)nt * nt);
+      k_mod_add<<<dim3((z.ldR / 8 + 3) / 4, (rows + 15) / 16, nw), 128, 0, s>>>(R, rows, r0, nG, z.ldR, scale, w0, flags,
+                                                                               chi);
     }
   }
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  return e == cudaSuccess ? launch_contract_f64(p, nG, M, K, f, chi, s, flags) : e;
 }
 
 }  // namespace chi0

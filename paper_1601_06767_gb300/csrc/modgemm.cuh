@@ -17,6 +17,13 @@
 // order and rounding.  The only error is the rounding to integers, about 0.08 x
 // 2^-53 of |A_m| |B_n| (0.3 x 2^-53 for the same sum by FP64 fused multiply-adds
 // over Gaussian rows).
+//
+// That is FP64 accuracy while S = sum_k |A[m][k]| |B[n][k]|, what FP64 sums are accurate
+// to, is not far below |A_m| |B_n|; rows that live on different k have a smaller S.
+// One more plane per operand (CHECK_PLANE) carries the elements' magnitudes, its
+// product is S, and tiles with an S below CHECK_MIN of the norms are computed by
+// FP64 multiply-adds instead (k_mod_check; dense Gaussian rows have 0.6, the largest
+// error let through is 0.08 x 32 x 2^-53 of S).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -26,6 +33,10 @@ namespace mod {
 
 constexpr int NM = 13;               // moduli
 constexpr int NPL = 2 * NM;          // residue planes (u and v of every modulus)
+constexpr int CHECK_PLANE = NPL;     // magnitudes, norm below 2^CHECK_BITS
+constexpr int CPL = NPL + 1;         // planes of a checked product
+constexpr int CHECK_BITS = 7;
+constexpr float CHECK_MIN = 1.0f / 32;
 constexpr int BETA_A = 57, BETA_B = 56;   // bits of the rows' norms after scaling
 constexpr int NO_SCALE = -(1 << 28);      // scale exponent of a row holding an infinity or a NaN
 
@@ -117,6 +128,13 @@ __device__ __forceinline__ int scale_exp(double n2, int e, int beta) {
   int k;
   frexp(n2 * (1.0 + 2e-5), &k);                   // n2 < 2^k
   return beta - e - ((k + 1) >> 1);               // norm < 2^(e + k / 2)
+}
+
+// norm 2^(s - beta) in [0.5, 1), s the scale exponent of a row with norm^2 = n2 4^e (0 for zeros, NaN
+// for non-finite rows)
+__device__ __forceinline__ float scaled_norm(double n2, int s, int e, int beta) {
+  if (s == NO_SCALE) return nanf("");
+  return n2 > 0.0 ? (float)scalbn(sqrt(n2), s + e - beta) : 0.f;
 }
 
 // |x| 2^-e truncated to FP32, for |x| < 2^(e + 1) (integer operations; zero below 2^(e - 126))
@@ -220,6 +238,20 @@ __device__ __forceinline__ void store_residues(const Limbs& x, const Limbs& y, b
   dst[(2 * I) * plane] = conj ? v : u;
   dst[(2 * I + 1) * plane] = conj ? u : v;
   if constexpr (I + 1 < NM) store_residues<I + 1>(x, y, conj, dst, plane);
+}
+
+// largest component of each of the two elements, scaled to norms of at most 2^CHECK_BITS (beta: BETA_A or
+// BETA_B), into the plane after the residues: no more than the magnitude and 2^-21 of the norm, no
+// less than 0.7 of it
+__device__ __forceinline__ void store_magnitudes(const Limbs& x, const Limbs& y, int beta, uint32_t* __restrict__ dst,
+                                                 size_t plane) {
+  float a, b, c, d;
+  unpack2(fma2(x.l[4], both(4096.f), x.l[3]), a, b);          // 2^-36 of the integers
+  unpack2(fma2(y.l[4], both(4096.f), y.l[3]), c, d);
+  const float s = __int_as_float((127 + 36 + CHECK_BITS - beta) << 23);
+  uint32_t r;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(s * fmaxf(fabsf(b), fabsf(d))), "f"(s * fmaxf(fabsf(a), fabsf(c))));
+  dst[CHECK_PLANE * plane] = r;
 }
 
 // ---------------------------------------------------------------------------
