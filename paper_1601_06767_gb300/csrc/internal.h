@@ -214,6 +214,9 @@ cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, in
 size_t mod_cols_ws_bytes(int n, int rows);
 cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, float* norm,
                                  uint16_t* planes, void* ws, cudaStream_t s, const int* todo = nullptr);
+// flags[z flag_step + tile] = 1 for the 64 x 64 tiles of the products z that want FP64 multiply-adds (modgemm.cuh)
+cudaError_t launch_mod_check(const int16_t* R, int rows, int cols, int ldR, int row0, const float* nA, size_t stepA,
+                             const float* nB, size_t stepB, int* flags, size_t flag_step, int products, cudaStream_t s);
 // one q-point's share of a batched tensor-core contraction
 struct TcJob {
   int nG;

@@ -188,11 +188,14 @@ k_bwd_diag(const C* __restrict__ M, int nG, int64_t K, const double2* __restrict
 // dense upstream, one frequency: tile of 32 pairs x 64 sphere points, K loop over H
 //   Y[p][G] = sum_H M[p][H] Gam[G][H],  Z[p][G] = sum_H M[p][H] conj(Gam[H][G])
 //   gM[p][G] += conj(f_p) Y + f_p Z;  part[p][gt] += Re( f'_p conj(sum_{G in tile} conj(M[p][G]) Y[p][G]) )
+// flags (or NULL): [pairs / 64][ntile], only the tiles that are not 0.  first: = in place of +=
 template <typename C>
 __global__ void __launch_bounds__(256)
 k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
             const double* __restrict__ E_col, const double* __restrict__ w_col, double2 om, double delta,
-            const double2* __restrict__ Gam, C* __restrict__ gM, double* __restrict__ part, int ntile) {
+            const double2* __restrict__ Gam, C* __restrict__ gM, double* __restrict__ part, int ntile,
+            const int* __restrict__ flags, bool first) {
+  if (flags && flags[(blockIdx.y >> 1) * ntile + blockIdx.x] == 0) return;
   constexpr int TP = 32, TG = 64, TH = 16;
   __shared__ double2 Ms[TP][TH + 1];
   __shared__ double2 Gs[TG][TH + 1];     // Gam[G][H]
@@ -263,7 +266,7 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
       for (int c = 0; c < 4; ++c) {
         const int G = G0 + tx + 16 * c;
         if (G >= nG) continue;
-        double2 gv = ld_d(gM, k * nG + G);
+        double2 gv = first ? make_double2(0, 0) : ld_d(gM, k * nG + G);
         const double2 t1 = cmul(fc, y[r][c]), t2 = cmul(f, z[r][c]);
         gv.x += t1.x + t2.x;
         gv.y += t1.y + t2.y;
@@ -284,13 +287,15 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
     if (k < K) {
       double sum = 0.0;
       for (int t = 0; t < 16; ++t) sum += sq[threadIdx.x][t];
-      part[k * ntile + blockIdx.x] += sum;
+      double* o = part + k * ntile + blockIdx.x;
+      *o = first ? sum : *o + sum;
     }
   }
 }
 
 // Dense upstream from the residues of Y and Z (modgemm.cuh), frequencies w0 .. w0 + nw: plane set
-// 2 w holds Y, 2 w + 1 holds Z of the block's pairs.
+// 2 w holds Y, 2 w + 1 holds Z of the block's pairs.  (Tiles that k_mod_check flagged for any of them are
+// overwritten by k_bwd_dense.)
 //   gM[k][G] (+)= sum_w conj(f) Y + f Z;  part[k][tile] (+)= Re( f' conj(sum_{G in tile} conj(M) Y) )
 // A CTA takes 16 pairs x 64 sphere points, a warp 16 x 8 of them (half a residue block): two
 // neighbouring lanes share a pair and take its even and odd points.  Bound by the integer pipe
@@ -334,7 +339,7 @@ k_bwd_mod(const int16_t* __restrict__ R, int rows, int ldR, const int* __restric
 #pragma unroll
     for (int part2 = 0; part2 < 2; ++part2) {
       mod::Frac re[4] = {}, im[4] = {};
-      mod::gather_fractions(R + mod::res_index(rows, ldR, (2 * w + part2) * mod::NPL, i, j0), plane, odd ? mod::ODD : mod::EVEN, re, im);
+      mod::gather_fractions(R + mod::res_index(rows, ldR, (2 * w + part2) * mod::CPL, i, j0), plane, odd ? mod::ODD : mod::EVEN, re, im);
       const int sa = sA[k];
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -469,6 +474,20 @@ size_t bwd_work_doubles(int nG, int n_freq, int64_t K) {
   return (size_t)(K + 1) / 2 * 2 + (size_t)K * std::max((nG + 63) / 64, 2 * std::min(n_freq, kMaxFreqBwd));
 }
 
+// all frequencies of the pairs' dense adjoint (flags: the flagged tiles') by FP64 multiply-adds
+template <typename C>
+static void dense_direct(chi0_plan_s* p, int nG, const C* M, int64_t p0, int64_t K, int n_c, const double* E_v,
+                         const double* E_col, const double* w_col, const double2* gamma, C* gM, double* part,
+                         const int* flags, cudaStream_t s) {
+  const int ntile = (nG + 63) / 64;
+  const dim3 grid(ntile, (unsigned)((K + 31) / 32));
+  for (int iw = 0; iw < p->n_freq; ++iw) {
+    const double2 om = make_double2(p->om_re[iw], p->om_im[iw]);
+    k_bwd_dense<C><<<grid, 256, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, om, p->delta,
+                                        gamma + (size_t)iw * nG * nG, gM, part, ntile, flags, iw == 0);
+  }
+}
+
 template <typename C>
 static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int64_t K, int n_c, const double* E_v,
                             const double* E_col, const double* w_col, const double2* gamma, const double* diag,
@@ -486,16 +505,7 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
   } else {
     const int ntile = (nG + 63) / 64;
     double* part = work + K;
-    cudaError_t e = cudaMemsetAsync(part, 0, sizeof(double) * (size_t)K * ntile, s);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(gM, 0, sizeof(C) * (size_t)K * nG, s);
-    if (e != cudaSuccess) return e;
-    dim3 grid(ntile, (unsigned)((K + 31) / 32));
-    for (int iw = 0; iw < p->n_freq; ++iw) {
-      const double2 om = make_double2(p->om_re[iw], p->om_im[iw]);
-      k_bwd_dense<C><<<grid, 256, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, om, p->delta,
-                                          gamma + (size_t)iw * nG * nG, gM, part, ntile);
-    }
+    dense_direct<C>(p, nG, M, p0, K, n_c, E_v, E_col, w_col, gamma, gM, part, nullptr, s);
     k_rowsum<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(part, K, ntile, gdE);
   }
   const int64_t rows = (p0 + K - 1) / n_c - p0 / n_c + 1;
@@ -518,7 +528,7 @@ bool bwd_mod_pays(const chi0_plan_s* p, int nG, int64_t n_pairs) {
 // residues of Y and Z for kc pairs, scales
 struct BwdMod {
   int Kp, ldR, nw, kc;
-  size_t off_a, off_r, off_sa, off_sb, off_ws, bytes;
+  size_t off_a, off_r, off_sa, off_sb, off_na, off_nb, off_flag, off_ws, bytes;
 };
 static BwdMod bwd_mod_sizes(const chi0_plan_s* p, int nG, int64_t n_pairs) {
   constexpr int64_t kMem = (int64_t)4 << 30;
@@ -526,16 +536,19 @@ static BwdMod bwd_mod_sizes(const chi0_plan_s* p, int nG, int64_t n_pairs) {
   BwdMod z;
   z.Kp = (nG + 63) / 64 * 64;
   z.ldR = (nG + 7) / 8 * 8;
-  const int64_t gam = (int64_t)2 * mod::NPL * 2 * nG * z.Kp;                  // one frequency's planes
+  const int64_t gam = (int64_t)2 * mod::CPL * 2 * nG * z.Kp;                  // one frequency's planes
   z.nw = (int)std::max<int64_t>(1, std::min<int64_t>(p->n_freq, kMem / gam));
-  const int64_t per_pair = (int64_t)2 * z.nw * mod::NPL * 2 * z.ldR;           // residues of one pair
+  const int64_t per_pair = (int64_t)2 * z.nw * mod::CPL * 2 * z.ldR;           // residues of one pair
   z.kc = (int)std::min<int64_t>({n_pairs, p->max_pairs, std::max<int64_t>(256, kMem / per_pair / 256 * 256),
                                  (int64_t)65535 * BM_PAIRS});   // grid y of k_bwd_mod
   z.off_a = al((size_t)gam * z.nw);
-  z.off_r = z.off_a + al((size_t)mod::NPL * 2 * z.kc * z.Kp);
-  z.off_sa = z.off_r + al((size_t)2 * z.nw * mod::NPL * 2 * mod::res_plane(z.kc, z.ldR));
+  z.off_r = z.off_a + al((size_t)mod::CPL * 2 * z.kc * z.Kp);
+  z.off_sa = z.off_r + al((size_t)2 * z.nw * mod::CPL * 2 * mod::res_plane(z.kc, z.ldR));
   z.off_sb = z.off_sa + al(sizeof(int) * (size_t)z.kc);
-  z.off_ws = z.off_sb + al(sizeof(int) * (size_t)2 * z.nw * nG);
+  z.off_na = z.off_sb + al(sizeof(int) * (size_t)2 * z.nw * nG);
+  z.off_nb = z.off_na + al(sizeof(float) * (size_t)z.kc);
+  z.off_flag = z.off_nb + al(sizeof(float) * (size_t)2 * z.nw * nG);
+  z.off_ws = z.off_flag + al(sizeof(int) * (size_t)((z.kc + 63) / 64) * ((nG + 63) / 64));
   z.bytes = z.off_ws + al(mod_cols_ws_bytes(nG, nG));
   return z;
 }
@@ -552,7 +565,10 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
   int16_t* R = reinterpret_cast<int16_t*>(b + z.off_r);
   int* sA = reinterpret_cast<int*>(b + z.off_sa);
   int* sB = reinterpret_cast<int*>(b + z.off_sb);
-  const size_t set = (size_t)mod::NPL * nG * z.Kp;       // 16-bit words of one operand's planes
+  float* nA = reinterpret_cast<float*>(b + z.off_na);
+  float* nB = reinterpret_cast<float*>(b + z.off_nb);
+  int* flags = reinterpret_cast<int*>(b + z.off_flag);
+  const size_t set = (size_t)mod::CPL * nG * z.Kp;       // 16-bit words of one operand's planes
   const int ntile = (nG + 63) / 64;
   cudaError_t e;
   // every pair block keeps its sums over the frequencies in gM and part: with several groups of
@@ -561,26 +577,30 @@ static cudaError_t bwd_mod_impl(chi0_plan_s* p, int nG, const C* M, int64_t n_pa
     const int K = (int)std::min<int64_t>(z.kc, n_pairs - p0);
     double* gdE = work;
     double* part = work + K;
-    e = launch_mod_pack_rows(M + p0 * nG, K, nG, nG, z.Kp, true, sA, nullptr, Ap, s);
+    e = cudaMemsetAsync(flags, 0, sizeof(int) * (size_t)((K + 63) / 64) * ntile, s);
+    if (e == cudaSuccess) e = launch_mod_pack_rows(M + p0 * nG, K, nG, nG, z.Kp, true, sA, nA, Ap, s);
     if (e != cudaSuccess) return e;
     for (int w0 = 0; w0 < p->n_freq; w0 += z.nw) {
       const int nw = std::min(z.nw, p->n_freq - w0);
       if (p0 == 0 || z.nw < p->n_freq)
         for (int w = 0; w < nw; ++w) {
           const double2* G = gamma + (size_t)(w0 + w) * nG * nG;
-          e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG, nullptr, Bp + 2 * w * set, s);
+          e = launch_mod_pack_rows(G, nG, nG, nG, z.Kp, false, sB + (size_t)2 * w * nG,
+                                   nB + (size_t)2 * w * nG, Bp + 2 * w * set, s);
           if (e == cudaSuccess)
-            e = launch_mod_pack_cols(G, nG, nG, z.Kp, true, sB + (size_t)(2 * w + 1) * nG, nullptr, Bp + (2 * w + 1) * set,
-                                          b + z.off_ws, s);
+            e = launch_mod_pack_cols(G, nG, nG, z.Kp, true, sB + (size_t)(2 * w + 1) * nG, nB + (size_t)(2 * w + 1) * nG,
+                                     Bp + (2 * w + 1) * set, b + z.off_ws, s);
           if (e != cudaSuccess) return e;
         }
-      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::NPL, mod::NPL, 2 * nw * mod::NPL, mod::NPL, nullptr};
+      ModGemm g{Ap, Bp, R, K, 0, K, nG, z.ldR, z.Kp, 2 * nw * mod::CPL, mod::CPL, 2 * nw * mod::CPL, mod::CPL, nullptr};
       e = launch_mod_gemm(p, g, s);
+      if (e == cudaSuccess) e = launch_mod_check(R, K, nG, z.ldR, 0, nA, 0, nB, nG, flags, 0, 2 * nw, s);
       if (e != cudaSuccess) return e;
       k_bwd_mod<C><<<dim3(ntile, (K + BM_PAIRS - 1) / BM_PAIRS), 256, 0, s>>>(R, K, z.ldR, sA, sB, M + p0 * nG, nG, p0, n_c, E_v, E_col,
                                                               w_col, p->d_omega, w0, nw, p->delta, gM + p0 * nG, part,
                                                               ntile);
     }
+    dense_direct<C>(p, nG, M + p0 * nG, p0, K, n_c, E_v, E_col, w_col, gamma, gM + p0 * nG, part, flags, s);
     k_rowsum<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(part, K, ntile, gdE);
     const int64_t rows = (p0 + K - 1) / n_c - p0 / n_c + 1;
     k_reduce_rows<<<(unsigned)rows, 128, 0, s>>>(gdE, p0, K, n_c, gEv);

@@ -673,6 +673,13 @@ cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+cudaError_t launch_mod_check(const int16_t* R, int rows, int cols, int ldR, int row0, const float* nA, size_t stepA,
+                             const float* nB, size_t stepB, int* flags, size_t flag_step, int products, cudaStream_t s) {
+  k_mod_check<<<dim3((cols + 63) / 64, (rows + 63) / 64, products), 128, 0, s>>>(R, rows, cols, ldR, row0, nA, stepA, nB,
+                                                                               stepB, flags, flag_step);
+  return cudaGetLastError();
+}
+
 // Workspace of the contraction: pairs and frequencies held at a time, rows of chi0 per product
 ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
   constexpr int64_t kPlanes = (int64_t)4 << 30, kRes = (int64_t)4 << 30;   // operand planes, residues
@@ -779,8 +786,9 @@ cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_
       ModGemm g{Ap, Bp, R, nG, r0, rows, nG, z.ldR, Kp, CPL * nw, CPL * nw, CPL, CPL, nullptr};
       e = launch_mod_gemm(p, g, s);
       if (e != cudaSuccess) return e;
-      k_mod_check<<<dim3(nt, (rows + 63) / 64, nw), 128, 0, s>>>(R, rows, nG, z.ldR, r0, norm + (size_t)(1 + w0) * nG, nG,
-                                                                 norm, 0, flags + (size_t)w0 * nt * nt, (size_t)nt * nt);
+      e = launch_mod_check(R, rows, nG, z.ldR, r0, norm + (size_t)(1 + w0) * nG, nG, norm, 0,
+                           flags + (size_t)w0 * nt * nt, (size_t)nt * nt, nw, s);
+      if (e != cudaSuccess) return e;
       k_mod_add<<<dim3((z.ldR / 8 + 3) / 4, (rows + 15) / 16, nw), 128, 0, s>>>(R, rows, r0, nG, z.ldR, scale, w0, flags,
                                                                                chi);
     }
