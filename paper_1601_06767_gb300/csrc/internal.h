@@ -204,16 +204,16 @@ struct ModGemm {
 };
 cudaError_t launch_mod_gemm(chi0_plan_s* p, const ModGemm& g, cudaStream_t s);
 // scales [rows] and residue planes [26][rows][Kp] of X [rows][n] (row stride ld), operand A or B; norm not
-// NULL: scaled norms [rows] and a 27th plane of magnitudes.
+// NULL: scaled norms [rows] and a 27th plane of magnitudes; rest: eight planes of remainders.
 // todo (here, below and in ModGemm): not NULL = the kernels do nothing where it points at 0
 cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
+                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr, bool rest = false);
 cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale,
-                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr);
+                                 float* norm, uint16_t* planes, cudaStream_t s, const int* todo = nullptr, bool rest = false);
 // the same of the transpose (conj: conjugate transpose) of X [n][rows] (operand B; ws: mod_cols_ws_bytes)
 size_t mod_cols_ws_bytes(int n, int rows);
 cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, float* norm,
-                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo = nullptr);
+                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo = nullptr, bool rest = false);
 // flags[z flag_step + tile] = 1 for the 64 x 64 tiles of the products z that want FP64 multiply-adds (modgemm.cuh)
 cudaError_t launch_mod_check(const int16_t* R, int rows, int cols, int ldR, int row0, const float* nA, size_t stepA,
                              const float* nB, size_t stepB, int* flags, size_t flag_step, int products, cudaStream_t s);

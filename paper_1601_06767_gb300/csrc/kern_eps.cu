@@ -750,7 +750,11 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 // with both products exact modular ones on the tensor cores (modgemm.cuh).  A step
 // with |R| <= 2^-26.5 in the Frobenius norm is a matrix's last: the error left, X R^2,
 // is at most 2^-53 of X.  (A bound on the largest element alone leaves up to N^2
-// times its square.)  A matrix that has no such step within STEPS (ill conditioned
+// times its square.)  From the second step on, the first one that may be the last, A X
+// includes the first order of what its integers leave out (store_remainders): equal
+// small elements of a row are all rounded one way, and a nearly singular A would
+// amplify their sum (I - (1 - e) / N 11^T, N 1000, cond 40: 3.0e-14, 9.0e-16 by the
+// elimination).  A matrix that has no such step within STEPS (ill conditioned
 // beyond FP32, out of its range, singular, not finite) is inverted by the FP64
 // elimination from A, whose kernels skip the others.
 //
@@ -803,8 +807,8 @@ __global__ void k_ref_init(int* __restrict__ todo, int nf) {
 }
 
 // values of the residue planes of one N x N product.  ADD = false: R = I - value and the sum of
-// |R|^2 over the block's elements; true: X += value.  A warp takes 16 rows x 8 columns (as k_mod_add).
-template <bool ADD>
+// |R|^2 over the block's elements; true: X += value.  REST: with the remainders' planes.  A warp takes 16 rows x 8 columns (as k_mod_add).
+template <bool ADD, bool REST = false>
 __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P, int N, int ldR,
                                                    const int* __restrict__ sA, const int* __restrict__ sB,
                                                    double2* __restrict__ out, float* __restrict__ part,
@@ -823,6 +827,19 @@ __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P
     mod::Frac re[4] = {}, im[4] = {};
     mod::gather_fractions(P + mod::res_index(N, ldR, 0, i, j0), mod::res_plane(N, ldR), lane & 1 ? mod::ODD : mod::EVEN, re, im);
     const int sa = sA[i];
+    int lr[4] = {}, li[4] = {};                    // remainders, in units of 2^(BETA_B - CHECK_BITS)
+    if (REST) {
+      const int16_t* r = P + mod::res_index(N, ldR, mod::NPL, i, j0);
+      const int sh = (lane & 1) * 16;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint4 u = *reinterpret_cast<const uint4*>(r + k * mod::res_plane(N, ldR));
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+        const int f = (k < 4 ? 1 : mod::BETA_A == mod::BETA_B + 1 ? 2 : 0) * (k == 1 || k == 5 ? -1 : 1);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ((k & 2) ? li : lr)[c] += f * (int16_t)(w[c] >> sh);
+      }
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const int j = j0 + 2 * c + (lane & 1);
@@ -830,7 +847,12 @@ __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P
       const int sb = sB[j];
       const bool bad = sa == mod::NO_SCALE || sb == mod::NO_SCALE;
       const double x = bad ? nan("") : mod::frac_value(re[c], -sa - sb), y = bad ? nan("") : mod::frac_value(im[c], -sa - sb);
-      const double2 r = ADD ? make_double2(v[c].x + x, v[c].y + y) : make_double2((i == j ? 1.0 : 0.0) - x, -y);
+      double2 r = ADD ? make_double2(v[c].x + x, v[c].y + y) : make_double2((i == j ? 1.0 : 0.0) - x, -y);
+      if (REST && !bad) {
+        const int k = mod::BETA_B - mod::CHECK_BITS - sa - sb;
+        r.x -= scalbn((double)lr[c], k);
+        r.y -= scalbn((double)li[c], k);
+      }
       if (!ADD) sq = fmaf((float)r.x, (float)r.x, fmaf((float)r.y, (float)r.y, sq));
       o[2 * c] = r;
     }
@@ -887,14 +909,14 @@ RefSizes ref_sizes(int N, int nf) {
   RefSizes z;
   z.Kp = (N + 63) / 64 * 64;
   z.ldR = (N + 7) / 8 * 8;
-  const size_t planes = al((size_t)mod::NPL * 2 * N * z.Kp), mat = al((size_t)N * N * sizeof(double2)), sc = al((size_t)N * sizeof(int));
+  const size_t planes = al((size_t)mod::RPL * 2 * N * z.Kp), mat = al((size_t)N * N * sizeof(double2)), sc = al((size_t)N * sizeof(int));
   z.x = al((size_t)nf * N * N * sizeof(float2));
   z.r = z.x + mat;
   z.pa = z.r + mat;
   z.px = z.pa + planes;
   z.pt = z.px + planes;
   z.res = z.pt + planes;
-  z.sa = z.res + al((size_t)mod::NPL * 2 * mod::res_plane(N, z.ldR));
+  z.sa = z.res + al((size_t)mod::RPL * 2 * mod::res_plane(N, z.ldR));
   z.sx = z.sa + sc;
   z.st = z.sx + sc;
   z.cols = z.st + sc;
@@ -932,18 +954,20 @@ cudaError_t refined_inverse(chi0_plan_s* p, double2* eps, int N, int nf, void* Z
     ProfScope ps(p, CHI0_K_INV_UPDATE, s, 4 + STEPS * 15);
     const double2* A = eps + w * n2;
     k_from_c64<<<4 * 152, 256, 0, s>>>(a32 + w * n2, n2, X);
-    e = launch_mod_pack_rows(A, N, N, N, z.Kp, true, sA, nullptr, PA, s);
+    e = launch_mod_pack_rows(A, N, N, N, z.Kp, true, sA, nullptr, PA, s, nullptr, true);
     for (int it = 0; it < STEPS && e == cudaSuccess; ++it) {
-      e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, nullptr, PT, b + z.cols, s, todo + w);
+      e = launch_mod_pack_cols(X, N, N, z.Kp, false, sT, nullptr, PT, b + z.cols, s, todo + w, it > 0);
+      const int np = it ? mod::RPL : mod::NPL;
       if (e == cudaSuccess)
-        e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
-      k_ref_value<false><<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, part, todo + w);
+        e = launch_mod_gemm(p, ModGemm{PA, PT, res, N, 0, N, N, z.ldR, z.Kp, np, mod::RPL, np, np, todo + w}, s);
+      auto* value = it ? k_ref_value<false, true> : k_ref_value<false, false>;
+      value<<<gv, 128, 0, s>>>(res, N, z.ldR, sA, sT, R, part, todo + w);
       if (e == cudaSuccess) e = launch_mod_pack_rows(X, N, N, N, z.Kp, true, sX, nullptr, PX, s, todo + w);
       if (e == cudaSuccess) e = launch_mod_pack_cols(R, N, N, z.Kp, false, sT, nullptr, PT, b + z.cols, s, todo + w);
       if (e == cudaSuccess)
         e = launch_mod_gemm(p, ModGemm{PX, PT, res, N, 0, N, N, z.ldR, z.Kp, mod::NPL, mod::NPL, mod::NPL, mod::NPL, todo + w}, s);
       k_ref_value<true><<<gv, 128, 0, s>>>(res, N, z.ldR, sX, sT, X, nullptr, todo + w);
-      k_ref_decide<<<1, 256, 0, s>>>(part, (int)(gv.x * gv.y), todo + w);
+      if (it) k_ref_decide<<<1, 256, 0, s>>>(part, (int)(gv.x * gv.y), todo + w);
     }
     k_ref_store<<<4 * 152, 256, 0, s>>>(X, N, cmax + (size_t)w * N, eps + w * n2, todo + w, 0);
     if (e == cudaSuccess) e = cudaGetLastError();

@@ -175,9 +175,9 @@ constexpr int PK_G = 16, PK_K = 64;   // tile: 16 sphere points x 64 pairs, tran
 
 // Planes [26][nG][Kp] (FP16) of conj(M) (of M: conj = false) into Bp (when not NULL) and of W_w = f(w) M,
 // w = w0 .. w0 + nw, into Ap (26 planes per frequency; CHECK: 27, with the
-// magnitudes).  A warp holds one sphere point, a lane two neighbouring pairs:
+// magnitudes; REST: 34, with the remainders).  A warp holds one sphere point, a lane two neighbouring pairs:
 // 128-byte stores per plane.
-template <bool CHECK>
+template <mod::Extra X>
 __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M, int nG, int64_t K, int Kp,
                                                   const double2* __restrict__ f, int w0, int nw,
                                                   const int* __restrict__ scale, bool conj, uint32_t* __restrict__ Bp,
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
     }
     __syncthreads();
     const int* sc = scale + (size_t)(slot < 0 ? 0 : 1 + w0 + slot) * nG;
-    uint32_t* dst = slot < 0 ? Bp : Ap + (size_t)slot * (CHECK ? CPL : NPL) * plane;
+    uint32_t* dst = slot < 0 ? Bp : Ap + (size_t)slot * (X == mod::CHECK ? CPL : NPL) * plane;
     for (int g = warp; g < PK_G; g += 8) {
       const int G = G0 + g;
       if (G >= nG) break;
@@ -213,11 +213,14 @@ __global__ void __launch_bounds__(256) k_mod_pack(const double2* __restrict__ M,
         a = cmul(fs[2 * lane], a);
         b = cmul(fs[2 * lane + 1], b);
       }
-      const mod::Limbs x = mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s));
-      const mod::Limbs y = mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s));
+      const int64_t ax = mod::quantise(a.x, s), bx = mod::quantise(b.x, s), ay = mod::quantise(a.y, s), by = mod::quantise(b.y, s);
+      const mod::Limbs x = mod::limbs(ax, bx), y = mod::limbs(ay, by);
       uint32_t* o = dst + (size_t)G * (Kp / 2) + p0 / 2 + lane;
       mod::store_residues(x, y, slot < 0 && conj, o, plane);
-      if (CHECK) mod::store_magnitudes(x, y, slot < 0 ? mod::BETA_B : mod::BETA_A, o, plane);
+      if (X == mod::CHECK) mod::store_magnitudes(x, y, slot < 0 ? mod::BETA_B : mod::BETA_A, o, plane);
+      if (X == mod::REST)
+        mod::store_remainders(x, y, mod::pack2(mod::rest_of(a.x, s, ax), mod::rest_of(b.x, s, bx)),
+                              mod::pack2(mod::rest_of(a.y, s, ay), mod::rest_of(b.y, s, by)), mod::BETA_B, o, plane);
     }
   }
 }
@@ -265,8 +268,9 @@ __global__ void __launch_bounds__(128) k_mod_row_scales(const C* __restrict__ X,
   }
 }
 
-// planes [26][rows][Kp] of X (beta not 0: 27, with the magnitudes); a warp takes 64 elements of a row
-template <typename C>
+// planes [26][rows][Kp] of X (CHECK: 27, with the magnitudes, REST: 34, with the remainders); a warp takes 64
+// elements of a row
+template <typename C, mod::Extra E>
 __global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, int rows, int n, size_t ld, int Kp,
                                                        const int* __restrict__ scale, int beta,
                                                        uint32_t* __restrict__ dst, const int* __restrict__ todo) {
@@ -279,18 +283,21 @@ __global__ void __launch_bounds__(256) k_mod_pack_rows(const C* __restrict__ X, 
   const int s = scale[r];
   const double2 a = k < n ? ld_wide(x, k) : make_double2(0.0, 0.0);
   const double2 b = k + 1 < n ? ld_wide(x, k + 1) : make_double2(0.0, 0.0);
-  const mod::Limbs u = mod::limbs(mod::quantise(a.x, s), mod::quantise(b.x, s));
-  const mod::Limbs v = mod::limbs(mod::quantise(a.y, s), mod::quantise(b.y, s));
+  const int64_t ax = mod::quantise(a.x, s), bx = mod::quantise(b.x, s), ay = mod::quantise(a.y, s), by = mod::quantise(b.y, s);
+  const mod::Limbs u = mod::limbs(ax, bx), v = mod::limbs(ay, by);
   uint32_t* o = dst + (size_t)r * (Kp / 2) + k / 2;
   mod::store_residues(u, v, false, o, (size_t)rows * (Kp / 2));
-  if (beta) mod::store_magnitudes(u, v, beta, o, (size_t)rows * (Kp / 2));
+  if (E == mod::CHECK) mod::store_magnitudes(u, v, beta, o, (size_t)rows * (Kp / 2));
+  if (E == mod::REST)
+    mod::store_remainders(u, v, mod::pack2(mod::rest_of(a.x, s, ax), mod::rest_of(b.x, s, bx)),
+                          mod::pack2(mod::rest_of(a.y, s, ay), mod::rest_of(b.y, s, by)), beta, o, (size_t)rows * (Kp / 2));
 }
 
 // ---------------------------------------------------------------------------
 // modular products
 // ---------------------------------------------------------------------------
-// R[b][i][j] = sum_k A[b][i][k] B[b][j][k] (mod m of plane b), |R| <= 257; of the magnitudes' plane
-// the sum itself, rounded.
+// R[b][i][j] = sum_k A[b][i][k] B[b][j][k] (mod m of plane b), |R| <= 255; of the planes after the
+// residues the sum itself, rounded.
 // A CTA pair computes a 256 x 256 tile with tcgen05.mma.cta_group::2 (each CTA
 // holds 128 rows of A and 128 of B: 32 KB per 512 MMA cycles, half the operand
 // traffic per flop of two single-CTA 128 x 128 tiles).  Warp 0 issues the TMA
@@ -319,7 +326,7 @@ struct GemmArgs {
   int row0;                    // first row of A
   int tiles_m, tiles_n, n_b;   // tiles and planes
   int a_planes, b_planes;      // planes of A and B (a plane index is taken modulo these)
-  int set;                     // planes of a product: NPL, or CPL with the magnitudes
+  int set;                     // planes of a product: NPL, CPL with the magnitudes, RPL with the remainders
   int nK;                      // stages of GK
   const int* todo;             // not NULL: nothing is done where it points at 0
 };
@@ -349,9 +356,9 @@ __device__ __forceinline__ void gemm_item(const GemmArgs& P, int item, int& b, i
   tn = within / rows;
 }
 
-// the moduli; for the magnitudes' plane one that their sums (below 2^14) never reach
-__constant__ float c_mod[NM + 1] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f,
-                                    433.f, 421.f, 409.f, 401.f, 397.f, 389.f, 1048576.f};
+// the moduli; for the planes after the residues one that their sums (below 2^15) never reach
+__constant__ float c_mod[mod::RPL / 2] = {509.f, 505.f, 493.f, 481.f, 461.f, 457.f, 449.f, 433.f, 421.f,
+                                          409.f, 401.f, 397.f, 389.f, 0x1p20f, 0x1p20f, 0x1p20f, 0x1p20f};
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 k_mod_gemm(const __grid_constant__ GemmArgs P, int* __restrict__ status) {
@@ -712,26 +719,26 @@ ModSizes mod_sizes(const chi0_plan_s* p, int nG) {
 
 template <typename C>
 static cudaError_t pack_rows(const C* X, int rows, int n, size_t ld, int Kp, int beta, int* scale, float* norm,
-                             uint16_t* planes, const int* todo, cudaStream_t s) {
+                             bool rest, uint16_t* planes, const int* todo, cudaStream_t s) {
   k_mod_row_scales<C><<<rows, 128, 0, s>>>(X, n, ld, beta, scale, norm, todo);
   const int64_t units = (int64_t)rows * (Kp / 64);
-  k_mod_pack_rows<C><<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, norm ? beta : 0,
-                                                                      (uint32_t*)planes, todo);
+  auto* pack = rest ? k_mod_pack_rows<C, mod::REST> : norm ? k_mod_pack_rows<C, mod::CHECK> : k_mod_pack_rows<C, mod::PLAIN>;
+  pack<<<(unsigned)((units + 7) / 8), 256, 0, s>>>(X, rows, n, ld, Kp, scale, beta, (uint32_t*)planes, todo);
   return cudaGetLastError();
 }
 cudaError_t launch_mod_pack_rows(const double2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale, float* norm,
-                                 uint16_t* planes, cudaStream_t s, const int* todo) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, planes, todo, s);
+                                 uint16_t* planes, cudaStream_t s, const int* todo, bool rest) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, rest, planes, todo, s);
 }
 cudaError_t launch_mod_pack_rows(const float2* X, int rows, int n, size_t ld, int Kp, bool a, int* scale, float* norm,
-                                 uint16_t* planes, cudaStream_t s, const int* todo) {
-  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, planes, todo, s);
+                                 uint16_t* planes, cudaStream_t s, const int* todo, bool rest) {
+  return pack_rows(X, rows, n, ld, Kp, a ? mod::BETA_A : mod::BETA_B, scale, norm, rest, planes, todo, s);
 }
 size_t mod_cols_ws_bytes(int n, int rows) {
   return al256(sizeof(uint32_t) * rows) + sizeof(double) * ((n + ST_ROWS - 1) / ST_ROWS) * (size_t)rows;
 }
 cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool conj, int* scale, float* norm,
-                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo) {
+                                 uint16_t* planes, void* ws, cudaStream_t s, const int* todo, bool rest) {
   uint32_t* eg = reinterpret_cast<uint32_t*>(ws);
   double* part = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(ws) + al256(sizeof(uint32_t) * rows));
   cudaError_t e = cudaMemsetAsync(eg, 0, sizeof(uint32_t) * rows, s);
@@ -741,7 +748,7 @@ cudaError_t launch_mod_pack_cols(const double2* X, int n, int rows, int Kp, bool
   k_mod_rowmax<<<gst, 256, 0, s>>>(X, rows, n, eg, todo);
   k_mod_col_norms<<<gst, 256, 0, s>>>(X, rows, n, eg, part, todo);
   k_mod_scales<<<dim3((rows + 255) / 256, 1), 256, 0, s>>>(part, n_part, rows, 0, eg, nullptr, scale, norm);
-  auto* pack = norm ? k_mod_pack<true> : k_mod_pack<false>;
+  auto* pack = rest ? k_mod_pack<mod::REST> : norm ? k_mod_pack<mod::CHECK> : k_mod_pack<mod::PLAIN>;
   pack<<<dim3((rows + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(X, rows, n, Kp, nullptr, 0, 0, scale, conj,
                                                                (uint32_t*)planes, nullptr, todo);
   return cudaGetLastError();
@@ -779,7 +786,7 @@ cudaError_t launch_contract_mod(chi0_plan_s* p, int nG, const double2* M, int64_
   k_mod_scales<<<dim3((nG + 255) / 256, nf + 1), 256, 0, s>>>(part, n_part, nG, nf, eg, ef, scale, norm);
   for (int w0 = 0; w0 < nf; w0 += z.nw) {
     const int nw = std::min(z.nw, nf - w0);
-    k_mod_pack<true><<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(
+    k_mod_pack<mod::CHECK><<<dim3((nG + PK_G - 1) / PK_G, Kp / PK_K), 256, 0, s>>>(
         M, nG, K, Kp, f, w0, nw, scale, true, w0 == 0 ? (uint32_t*)Bp : nullptr, (uint32_t*)Ap, nullptr);
     for (int r0 = 0; r0 < nG; r0 += z.rows) {
       const int rows = std::min(z.rows, nG - r0);

@@ -36,6 +36,8 @@ constexpr int NPL = 2 * NM;          // residue planes (u and v of every modulus
 constexpr int CHECK_PLANE = NPL;     // magnitudes, norm below 2^CHECK_BITS
 constexpr int CPL = NPL + 1;         // planes of a checked product
 constexpr int CHECK_BITS = 7;
+constexpr int RPL = NPL + 8;         // planes of a product with the remainders (store_remainders)
+enum Extra { PLAIN, CHECK, REST };   // what follows the residues
 constexpr float CHECK_MIN = 1.0f / 32;
 constexpr int BETA_A = 57, BETA_B = 56;   // bits of the rows' norms after scaling
 constexpr int NO_SCALE = -(1 << 28);      // scale exponent of a row holding an infinity or a NaN
@@ -254,6 +256,32 @@ __device__ __forceinline__ void store_magnitudes(const Limbs& x, const Limbs& y,
   dst[CHECK_PLANE * plane] = r;
 }
 
+// The first order of what the rounding to integers leaves out of A B: with A = Ah + Al and B = Bh + Bl (integers
+// and remainders below 1/2), Al Bh + Ah Bl as eight real products in planes NPL .. RPL, to some 2^-7 of it.
+// Remainders as they are, integers scaled to norms of at most 2^CHECK_BITS; the order of the parts gives
+//   Re: + (0) - (1) + (4) - (5),   Im: + (2) + (3) + (6) + (7).
+// The sums stay below 2^15: the remainders' norm is at most 2^7.5 for 2^16 elements.
+__device__ __forceinline__ float rest_of(double x, int s, int64_t q) {
+  return (float)(x * pow2d(s / 2) * pow2d(s - s / 2) - (double)q);      // exact: both are multiples of x's last bit
+}
+__device__ __forceinline__ void store_remainders(const Limbs& x, const Limbs& y, uint64_t rx, uint64_t ry, int beta,
+                                                 uint32_t* __restrict__ dst, size_t plane) {
+  const uint64_t s = both(__int_as_float((127 + 36 + CHECK_BITS - beta) << 23));
+  const uint64_t v[4] = {rx, ry, mul2(s, fma2(x.l[4], both(4096.f), x.l[3])), mul2(s, fma2(y.l[4], both(4096.f), y.l[3]))};
+  uint32_t h[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float a, b;
+    unpack2(v[i], a, b);
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h[i]) : "f"(b), "f"(a));
+  }
+  const bool A = beta == BETA_A;
+  const uint32_t lr = h[0], li = h[1], hr = h[2], hi = h[3];
+  const uint32_t o[8] = {A ? lr : hr, A ? li : hi, A ? lr : hi, A ? li : hr, A ? hr : lr, A ? hi : li, A ? hr : li, A ? hi : lr};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) dst[(NPL + i) * plane] = o[i];
+}
+
 // ---------------------------------------------------------------------------
 // reconstruction
 // ---------------------------------------------------------------------------
@@ -326,7 +354,7 @@ __device__ __forceinline__ size_t res_index(int rows, int ldR, int b, int row, i
 
 // Fractions of the real and imaginary parts of four elements: r points at eight columns of one row,
 // the lane takes the even ones (sh = EVEN: sign-extended low halves) or the odd ones (sh = ODD)
-constexpr uint32_t EVEN = 0x9910, ODD = 0xbb32;   // byte selectors, the sign byte replicated
+constexpr uint32_t EVEN = 0x1110, ODD = 0x3332;   // byte selectors, the high byte replicated: residues are below 256
 template <int I0, int I, int N>
 __device__ __forceinline__ void add_words(const uint4 (&w)[2 * N], uint32_t sh, Frac (&re)[4], Frac (&im)[4]) {
   const uint4 u = w[2 * (I - I0)], v = w[2 * (I - I0) + 1];
