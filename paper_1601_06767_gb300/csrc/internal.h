@@ -104,10 +104,10 @@ struct chi0_plan_s {
   void* wfn_ws = nullptr;    // scratch of the three-pass wavefunction transform (FP32 plans on 96^3)
   size_t wfn_ws_bytes = 0;
   // workspaces that calls on different streams use apart: contraction of FP64 plans, dense adjoint,
-  // fixed-point pair stage, fixed-point wavefunctions, COH, dielectric inverse
-  LazyWs ws_mod, ws_bwd, ws_fx, ws_wfn, ws_coh, ws_inv;
+  // fixed-point pair stage, COH, dielectric inverse
+  LazyWs ws_mod, ws_bwd, ws_fx, ws_coh, ws_inv;
+  cudaMemPool_t wfn_pool = nullptr;    // scratch of the fixed-point wavefunctions, per call and stream
   std::vector<void*> ws_kept;          // outgrown workspaces that a caller's captured graph still names
-  cudaEvent_t wfn_ev = nullptr;        // last use of ws_wfn
   // pipelined chi0_build (split plans): the pair stage and packing of block k+1 run on a
   // low-priority stream beside the contraction of block k on a high-priority one, with a
   // second M / factor / split-plane set (allocated on first use)
@@ -170,8 +170,7 @@ cudaError_t fx_setup(const chi0_plan_s* p, SphereQ* s);
 // the same for the wavefunctions (w->fx_tw stays NULL where they do not fit)
 cudaError_t fx_setup_wfn(const chi0_plan_s* p, WfnSphere* w);
 size_t fx_wfn_ws_bytes(const chi0_plan_s* p, int64_t bands);
-cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, int64_t bands,
-                          cudaStream_t s);
+cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, cudaStream_t s);
 size_t fx_ws_bytes(const chi0_plan_s* p, int64_t pairs);
 cudaError_t launch_fx_planes(const chi0_plan_s* p, int iq, const double2* psi_v, const int32_t* v_idx, int v0, int nv,
                              const double2* psi_c, const int32_t* c_idx, int c0, int nc, void* D, void* ex,

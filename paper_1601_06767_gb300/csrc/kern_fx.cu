@@ -54,36 +54,6 @@ __device__ __forceinline__ int64_t fx_int(double x, int emax) {
   return b < 0 ? -q : q;
 }
 
-// mx[b] = largest magnitude word of band b (cleared by the caller)
-__global__ void __launch_bounds__(256) k_fx_max(const double2* __restrict__ c, int b0, int64_t n,
-                                                uint32_t* __restrict__ mx) {
-  const double2* x = c + (int64_t)(b0 + blockIdx.y) * n;
-  uint32_t m = 0;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = x[e];
-    m = max(m, max(mod::mag_word(v.x), mod::mag_word(v.y)));
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(mx + blockIdx.y, m);
-}
-
-__device__ __forceinline__ int fx_scale(uint32_t w) {
-  return w >= 0x7ff00000u ? mod::NO_SCALE : (w < 0x00100000u ? 0 : WBITS - 1 - mod::word_exp(w));
-}
-
-// q[b][r] = (re1, re0, im1, im0): limbs of the coefficients 2^scale
-__global__ void __launch_bounds__(256) k_fx_quant(const double2* __restrict__ c, int b0, int64_t n,
-                                                  const uint32_t* __restrict__ mx, int4* __restrict__ q) {
-  const double2* x = c + (int64_t)(b0 + blockIdx.y) * n;
-  const int s = fx_scale(mx[blockIdx.y]);
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const double2 v = x[e];
-    const int64_t a = mod::quantise(v.x, s), b = mod::quantise(v.y, s);
-    const int a0 = ((int)a << (32 - WL)) >> (32 - WL), b0l = ((int)b << (32 - WL)) >> (32 - WL);
-    q[blockIdx.y * n + e] = make_int4((int)((a - a0) >> WL), a0, (int)((b - b0l) >> WL), b0l);
-  }
-}
-
 // ---- line transforms ----
 // x 2^-s, rounded to nearest (s may be negative)
 __device__ __forceinline__ int64_t shift_round(int64_t x, int s) {
@@ -371,10 +341,11 @@ __global__ void __launch_bounds__(256) k_fx_gather(const longlong2* __restrict__
 //   X(i + h) = (Ee - Eo) + i (Oe - Oo),  X(h - i) = (Ee - Eo) - i (Oe - Oo),  h = n / 2,
 // E = sum P cos, O = sum M sin, for i = 0 .. n / 4 (odd n: i = 0 .. (n - 1) / 2, the
 // first row only).  The line is kept as slots G + g, folded in place (P at +g, M at -g).
-__device__ __forceinline__ void fold_synth(longlong2* __restrict__ r, int G, int g, int s) {
+// sp, sm: shifts of the slots at +g and -g.
+__device__ __forceinline__ void fold_synth(longlong2* __restrict__ r, int G, int g, int sp, int sm) {
   int4* w = reinterpret_cast<int4*>(r);
-  const longlong2 p = r[G + g], m = r[G - g];
-  const int64_t px = shift_round(p.x, s), py = shift_round(p.y, s), mx = shift_round(m.x, s), my = shift_round(m.y, s);
+  const longlong2 p = line_int(r[G + g], sp), m = line_int(r[G - g], sm);
+  const int64_t px = p.x, py = p.y, mx = m.x, my = m.y;
   if (g == 0) {
     w[G] = limbs_w(px, py);
     return;
@@ -419,11 +390,38 @@ __device__ __forceinline__ void synth_unit(const int4* __restrict__ w, const FxA
   }
 }
 
+// q[band][k] = limbs of the coefficients in column order, each column in the unit of its own largest one:
+// col_unit[band][column] (BAD_UNIT: an infinity or a NaN).  Eight lanes per column.
+constexpr int BAD_UNIT = 1 << 20;
+__global__ void __launch_bounds__(256) k_fx_cols(const double2* __restrict__ coeff, int npw, int ncols,
+                                                 const int* __restrict__ col_start, const int* __restrict__ col_pw,
+                                                 int4* __restrict__ q, int* __restrict__ col_unit) {
+  const int c = blockIdx.x * 32 + (threadIdx.x >> 3), l = threadIdx.x & 7;
+  const int64_t b = blockIdx.y;
+  const double2* cb = coeff + b * npw;
+  const int k0 = c < ncols ? col_start[c] : 0, k1 = c < ncols ? col_start[c + 1] : 0;
+  uint32_t big = 0;
+  for (int k = k0 + l; k < k1; k += 8) {
+    const double2 v = cb[col_pw[k]];
+    big = max(big, max(mod::mag_word(v.x), mod::mag_word(v.y)));
+  }
+  for (int o = 4; o; o >>= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, o));
+  const int emax = fx_exp(big);
+  for (int k = k0 + l; k < k1; k += 8) {
+    const double2 v = cb[col_pw[k]];
+    q[b * npw + k] = limbs_w(fx_int(v.x, emax), fx_int(v.y, emax));
+  }
+  if (l == 0 && c < ncols) col_unit[b * ncols + c] = big >= 0x7ff00000u ? BAD_UNIT : fx_unit(emax);
+}
+
 // psi[band][i1] for one plane and band: along g1 for every (g2, g3) column of the sphere (direct sums
-// over its few coefficients), along g2 for every g3, along g3 for every i2.
-__global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict__ mx, int npw, int n1, int n2, int n3,
+// over its few coefficients), along g2 for every g3, along g3 for every i2.  The columns' sums join at the
+// plane's exponent.
+constexpr int TOP0 = 4096;                                 // exponents are compared as positive words, 0: none
+constexpr int NO_UNIT = -(1 << 20);                        // of zeros: they stay zeros in any other unit
+__global__ void k_fx_wfn(const int4* __restrict__ q, const int* __restrict__ col_unit, int npw, int n1, int n2, int n3,
                          int nw1, int w2min, int w3min, int nw2, int nw3, const int* __restrict__ col_start,
-                         const int* __restrict__ col_pw, const int* __restrict__ col_g1, int w1min,
+                         const int* __restrict__ col_g1, int w1min,
                          const int4* __restrict__ tw1, const __grid_constant__ FxAxis a2, const __grid_constant__ FxAxis a3,
                          double2* __restrict__ psi) {
   extern __shared__ __align__(16) unsigned char smem_fx[];
@@ -432,41 +430,53 @@ __global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict_
   const int G2 = a2.items, G3 = a3.items, lda = 2 * G2 + 1, ldb = 2 * G3 + 1;   // odd
   longlong2* A = reinterpret_cast<longlong2*>(smem_fx);    // [2 G3 + 1][lda]: slot of g3, slot of g2
   longlong2* B = A + (size_t)(2 * G3 + 1) * lda;           // [n2][ldb]
+  int* U = reinterpret_cast<int*>(B);                      // [2 G3 + 1][lda] units of A's values, before B is needed
   const int i1 = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const int64_t b = blockIdx.y;
   double2* out = psi + (b * n1 + i1) * (int64_t)n2 * n3;
-  const int s = fx_scale(mx[b]);
-  if (s == mod::NO_SCALE) {                                // an infinity or a NaN among the coefficients
-    for (int e = tid; e < n2 * n3; e += nt) out[e] = make_double2(nan(""), nan(""));
-    return;
-  }
   if (tid < 2) slot[tid] = 0;
   for (int g = tid; g < nw1; g += nt) {
     int k = (int)((int64_t)(w1min + g) * i1 % n1);
     tws[g] = tw1[k < 0 ? k + n1 : k];
   }
-  for (int e = tid; e < (2 * G3 + 1) * lda; e += nt) A[e] = make_longlong2(0, 0);
+  for (int e = tid; e < (2 * G3 + 1) * lda; e += nt) {
+    A[e] = make_longlong2(0, 0);
+    U[e] = NO_UNIT;
+  }
   __syncthreads();
   const int4* qb = q + b * npw;
+  const int* ub = col_unit + b * (nw2 * nw3);
   uint32_t m = 0;
   for (int c = tid; c < nw2 * nw3; c += nt) {
-    const int r = c / nw3, g3 = w3min + c - r * nw3, g2 = w2min + r, k1 = col_start[c + 1];
+    const int r = c / nw3, g3 = w3min + c - r * nw3, g2 = w2min + r;
+    const int k0 = col_start[c], k1 = col_start[c + 1];
+    const int unit = ub[c];
     Acc re, im;
-    for (int k = col_start[c]; k < k1; ++k) {
-      const int4 x = qb[col_pw[k]], t = tws[col_g1[k]];    // t = (cos, sin) in two limbs each
+    for (int k = k0; k < k1; ++k) {
+      const int4 x = qb[k], t = tws[col_g1[k]];            // t = (cos, sin) in two limbs each
       re.add(x.x, x.y, t.x, t.y);
       re.add(-x.z, -x.w, t.z, t.w);
       im.add(x.z, x.w, t.x, t.y);
       im.add(x.x, x.y, t.z, t.w);
     }
     const longlong2 v = make_longlong2(re.value(), im.value());
-    A[(G3 + g3) * lda + G2 + g2] = v;
-    m = max(m, max(abs_word(v.x), abs_word(v.y)));
+    if (unit == BAD_UNIT) m = 0xffffffffu;
+    const int at = (G3 + g3) * lda + G2 + g2;
+    if (unit != BAD_UNIT && (v.x | v.y)) {
+      A[at] = v;
+      U[at] = unit;
+      m = max(m, (uint32_t)(TOP0 + unit + word_bits(max(abs_word(v.x), abs_word(v.y)))));
+    }
   }
-  const int sa = word_bits(block_max(m, slot)) - WBITS;
+  m = block_max(m, slot);
+  if (m == 0xffffffffu) {
+    for (int e = tid; e < n2 * n3; e += nt) out[e] = make_double2(nan(""), nan(""));
+    return;
+  }
+  const int base = (int)m - TOP0 - WBITS;
   for (int e = tid; e < (2 * G3 + 1) * (G2 + 1); e += nt) {
-    const int c = e % (2 * G3 + 1), g = e / (2 * G3 + 1);
-    fold_synth(A + c * lda, G2, g, sa);
+    const int c = e % (2 * G3 + 1), g = e / (2 * G3 + 1), *u = U + c * lda + G2;
+    fold_synth(A + c * lda, G2, g, base - u[g], base - u[-g]);
   }
   __syncthreads();
   m = 0;
@@ -480,10 +490,10 @@ __global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict_
   const int sb = word_bits(block_max(m, slot + 1)) - WBITS;
   for (int e = tid; e < n2 * (G3 + 1); e += nt) {
     const int i2 = e % n2, g = e / n2;
-    fold_synth(B + i2 * ldb, G3, g, sb);
+    fold_synth(B + i2 * ldb, G3, g, sb, sb);
   }
   __syncthreads();
-  const int unit = -s + sa + sb;
+  const int unit = base + sb;
   for (int e = tid; e < n2 * a3.units; e += nt) {              // along g3
     const int i = e % a3.units, i2 = e / a3.units;
     synth_unit(reinterpret_cast<const int4*>(B + i2 * ldb), a3, i, [&](int i3, longlong2 v) {
@@ -493,14 +503,14 @@ __global__ void k_fx_wfn(const int4* __restrict__ q, const uint32_t* __restrict_
 }
 
 size_t wfn_smem(const chi0_plan_s* p, const WfnSphere& w) {
-  return ((size_t)(2 * w.fx[1].items + 1) * (2 * w.fx[0].items + 1) + (size_t)p->n2 * (2 * w.fx[1].items + 1)) * 16;
+  const size_t a = (size_t)(2 * w.fx[1].items + 1) * (2 * w.fx[0].items + 1), b = (size_t)p->n2 * (2 * w.fx[1].items + 1);
+  return a * 16 + std::max(b * 16, a * 4);
 }
 
 size_t planes_smem(const chi0_plan_s* p, const SphereQ& s) {
   return ((size_t)p->n2 * (p->n3 | 1) + (size_t)s.nk3 * (p->n2 | 1)) * 16;
 }
 constexpr size_t SMEM_CAP = 220 * 1024;
-size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
 // (cos, sin) of 2 pi m / n, m < n, in two limbs each; evaluated on the first octant only (long double
 // is software on the Arm hosts)
@@ -611,30 +621,23 @@ cudaError_t fx_setup_wfn(const chi0_plan_s* p, WfnSphere* w) {
   return e;
 }
 
+// scratch per band: limbs of its coefficients and units of its columns
 size_t fx_wfn_ws_bytes(const chi0_plan_s* p, int64_t bands) {
-  return al256((size_t)bands * p->w.npw * 16) + al256((size_t)bands * 4);
+  return (size_t)bands * ((size_t)p->w.npw * sizeof(int4) + (size_t)p->w.nw2 * p->w.nw3 * sizeof(int));
 }
 
-cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, int64_t bands,
-                          cudaStream_t s) {
+// nb bands (at most 65535: grid y)
+cudaError_t launch_fx_wfn(const chi0_plan_s* p, const double2* coeff, int nb, double2* psi, void* ws, cudaStream_t s) {
   const WfnSphere& w = p->w;
-  int4* q = reinterpret_cast<int4*>(ws);
-  uint32_t* mx = reinterpret_cast<uint32_t*>((unsigned char*)ws + al256((size_t)bands * w.npw * 16));
   const size_t sm = wfn_smem(p, w);
   cudaError_t e = cudaFuncSetAttribute(k_fx_wfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  for (int b0 = 0; b0 < nb; b0 += (int)bands) {
-    const int n = (int)std::min<int64_t>(bands, nb - b0);
-    e = cudaMemsetAsync(mx, 0, (size_t)n * 4, s);
-    if (e != cudaSuccess) return e;
-    const int gx = (int)std::min<int64_t>((w.npw + 1023) / 1024, std::max(1, 4096 / n));
-    k_fx_max<<<dim3(gx, n), 256, 0, s>>>(coeff, b0, w.npw, mx);
-    k_fx_quant<<<dim3(gx, n), 256, 0, s>>>(coeff, b0, w.npw, mx, q);
-    const int nt = sm <= 32 * 1024 ? 128 : (sm <= 72 * 1024 ? 256 : 512);
-    k_fx_wfn<<<dim3(p->n1, n), nt, sm, s>>>(q, mx, w.npw, p->n1, p->n2, p->n3, w.nw1, w.w2min, w.w3min, w.nw2, w.nw3,
-                                            w.col_start, w.col_pw, w.col_g1, w.w1min, w.fx_tw, w.fx[0], w.fx[1],
-                                            psi + (int64_t)b0 * p->nr);
-  }
+  const int nt = sm <= 32 * 1024 ? 128 : (sm <= 72 * 1024 ? 256 : 512), ncols = w.nw2 * w.nw3;
+  int4* q = reinterpret_cast<int4*>(ws);
+  int* unit = reinterpret_cast<int*>(q + (size_t)nb * w.npw);
+  k_fx_cols<<<dim3((ncols + 31) / 32, nb), 256, 0, s>>>(coeff, w.npw, ncols, w.col_start, w.col_pw, q, unit);
+  k_fx_wfn<<<dim3(p->n1, nb), nt, sm, s>>>(q, unit, w.npw, p->n1, p->n2, p->n3, w.nw1, w.w2min, w.w3min, w.nw2, w.nw3,
+                                           w.col_start, w.col_g1, w.w1min, w.fx_tw, w.fx[0], w.fx[1], psi);
   return cudaGetLastError();
 }
 

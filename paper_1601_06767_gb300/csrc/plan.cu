@@ -105,15 +105,15 @@ void free_plan(chi0_plan_s* p) {
   for (auto& a : w.fx) cudaFree((void*)a.coef);
   cudaFree(p->d_omega); cudaFree(p->d_D); cudaFree(p->d_M); cudaFree(p->d_f);
   cudaFree(p->d_pack); cudaFree(p->d_status); cudaFree(p->d_bwd); cudaFree(p->wfn_ws);
-  cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p); cudaFree(p->ws_wfn.p);
+  cudaFree(p->ws_mod.p); cudaFree(p->ws_bwd.p); cudaFree(p->ws_fx.p);
   cudaFree(p->ws_coh.p); cudaFree(p->ws_inv.p);
   for (void* w : p->ws_kept) cudaFree(w);
-  if (p->wfn_ev) cudaEventDestroy(p->wfn_ev);
   for (size_t i = 1; i < p->bq_M.size(); ++i) {
     cudaFree(p->bq_M[i]);
     cudaFree(p->bq_f[i]);
     cudaFree(p->bq_pack[i]);
   }
+  if (p->wfn_pool) cudaMemPoolDestroy(p->wfn_pool);
   if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
   if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
   cudaFree(p->pipe_M); cudaFree(p->pipe_f); cudaFree(p->pipe_pack);
@@ -224,6 +224,19 @@ bool env_fault(const char* what) {
 bool ws_fault(size_t need) {
   const char* e = getenv("CHI0_FAULT");
   return e && strncmp(e, "ws:", 3) == 0 && need >= strtoull(e + 3, nullptr, 10);
+}
+
+// A pool that keeps what it has until the plan is destroyed: at most 1 GiB per stream in use at a time
+bool wfn_pool_setup(chi0_plan_s* p) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = p->device;
+  uint64_t keep = UINT64_MAX;
+  if (cudaMemPoolCreate(&p->wfn_pool, &props) != cudaSuccess) p->wfn_pool = nullptr;
+  else if (cudaMemPoolSetAttribute(p->wfn_pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess) return true;
+  cudaGetLastError();
+  return false;
 }
 
 chi0_status check_plan(chi0_plan_s* p) {
@@ -371,7 +384,13 @@ const char* chi0_last_error(chi0_plan plan) {
   return plan ? plan->err.c_str() : g_create_err.c_str();
 }
 
-size_t chi0_workspace_bytes(chi0_plan plan) { return plan ? plan->ws_bytes : 0; }
+size_t chi0_workspace_bytes(chi0_plan plan) {
+  if (!plan) return 0;
+  uint64_t pool = 0;
+  if (plan->wfn_pool && cudaMemPoolGetAttribute(plan->wfn_pool, cudaMemPoolAttrReservedMemCurrent, &pool) != cudaSuccess)
+    cudaGetLastError();
+  return plan->ws_bytes + (size_t)pool;
+}
 
 chi0_status chi0_plan_create(chi0_plan* out, const chi0_plan_desc* d) {
   if (!out) return fail(nullptr, CHI0_ERR_INVALID, "out is NULL");
@@ -452,6 +471,7 @@ chi0_status chi0_plan_create(chi0_plan* out, const chi0_plan_desc* d) {
   if (!chi0::is_split(p)) {
     cudaError_t fe = chi0::fx_setup_wfn(p, &p->w);
     if (fe != cudaSuccess) { p->err = cudaGetErrorString(fe); return bail(fe == cudaErrorMemoryAllocation ? CHI0_ERR_OOM : CHI0_ERR_CUDA); }
+    if (p->w.fx_tw && !wfn_pool_setup(p)) { p->err = "memory pool"; return bail(CHI0_ERR_CUDA); }
   }
   if (!chi0::is_split(p))
     for (auto& sq : p->q)
@@ -778,32 +798,29 @@ chi0_status chi0_wfn_to_grid(chi0_plan p, const void* coeff, int nb, void* psi, 
   if (p->w.npw <= 0) return fail(p, CHI0_ERR_INVALID, "the plan has no wavefunction sphere");
   if (nb < 0 || (nb > 0 && (!coeff || !psi))) return fail(p, CHI0_ERR_INVALID, "bad band count or NULL buffer");
   if (nb == 0) return CHI0_OK;
-  if (p->w.fx_tw) {
-    // coefficients in fixed point for up to 1 GiB (and 65535) bands at a time
-    const int64_t bands = std::min<int64_t>({nb, 65535, std::max<int64_t>(1, ((int64_t)1 << 30) / (16 * (int64_t)p->w.npw))});
-    // Calls on several streams share the workspace one after the other.  A captured call could run beside
-    // any of them when its graph is launched: it keeps the direct sums, which need none.
-    cudaStream_t s = (cudaStream_t)stream;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CK(p, cudaStreamIsCapturing(s, &cap));
-    if (cap == cudaStreamCaptureStatusNone && ws_ready(p, p->ws_wfn, chi0::fx_wfn_ws_bytes(p, bands), s)) {
-      if (!p->wfn_ev)
-        CK(p, cudaEventCreateWithFlags(&p->wfn_ev, cudaEventDisableTiming));
-      else
-        CK(p, cudaStreamWaitEvent(s, p->wfn_ev, 0));
-      cudaError_t e;
-      {
-        chi0::ProfScope ps(p, CHI0_K_WFN, s, 3 * (int)((nb + bands - 1) / bands));
-        e = chi0::launch_fx_wfn(p, (const double2*)coeff, nb, (double2*)psi, p->ws_wfn.p, bands, s);
-      }
-      const cudaError_t er = cudaEventRecord(p->wfn_ev, s);
-      CK(p, e);
-      CK(p, er);
-      return CHI0_OK;
-    }
+  cudaStream_t s = (cudaStream_t)stream;
+  // Fixed point: scratch for up to 1 GiB of coefficients and 65535 bands at a time, in stream order (calls on
+  // several streams have their own, a captured call's belongs to its graph); direct sums where it cannot be had.
+  const int64_t bands = std::min<int64_t>({nb, 65535, std::max<int64_t>(1, ((int64_t)1 << 30) / (16 * std::max<int64_t>(1, p->w.npw)))});
+  const size_t need = p->w.fx_tw ? chi0::fx_wfn_ws_bytes(p, bands) : 0;
+  void* ws = nullptr;
+  if (need && !ws_fault(need) && cudaMallocFromPoolAsync(&ws, need, p->wfn_pool, s) != cudaSuccess) {
+    cudaGetLastError();
+    ws = nullptr;
   }
-  chi0::ProfScope ps(p, CHI0_K_WFN, (cudaStream_t)stream, 1);
-  CK(p, chi0::launch_wfn_to_grid(p, (const double2*)coeff, nb, psi, (cudaStream_t)stream));
+  if (ws) {
+    chi0::ProfScope ps(p, CHI0_K_WFN, s, 2 * (int)((nb + bands - 1) / bands));
+    cudaError_t e = cudaSuccess;
+    for (int64_t b0 = 0; b0 < nb && e == cudaSuccess; b0 += bands)
+      e = chi0::launch_fx_wfn(p, (const double2*)coeff + b0 * p->w.npw, (int)std::min<int64_t>(bands, nb - b0),
+                              (double2*)psi + b0 * p->nr, ws, s);
+    const cudaError_t ef = cudaFreeAsync(ws, s);
+    CK(p, e);
+    CK(p, ef);
+    return CHI0_OK;
+  }
+  chi0::ProfScope ps(p, CHI0_K_WFN, s, 1);
+  CK(p, chi0::launch_wfn_to_grid(p, (const double2*)coeff, nb, psi, s));
   return CHI0_OK;
 }
 
