@@ -101,66 +101,93 @@ __global__ void __launch_bounds__(128) k_bwd_factors(int64_t p0, int64_t K, int 
   fac[blockIdx.y * K + k] = make_double2(2.0 * f.x, fp.x);
 }
 
-// A CTA per BD_PAIRS pairs of the block p0..p0+K, g [n_freq][nG] real, read once for
+// A CTA per P pairs of the block p0..p0+K, g [n_freq][nG] real, read once for
 // them:  gM = sum_w 2 Re f_w g_w M,  gdE = sum_w Re f'_w sum_G g_w |M|^2.
 // ONE: a single frequency, its factors out of the loop: two FP64 operations per
 // element in FP32 plans.  Bound by the FP64 pipe and the integer squares: 1.01 ms
 // for 128,000 pairs, N_G 1200 (2.4 TB/s); 3.97 ms with the square, both products,
 // the conversions and every CTA's own factors on the FP64 pipe, and 2.2 ms more for
 // the row sums by one thread per row.
-constexpr int BD_PAIRS = 4, BD_THREADS = 128;
-template <typename C, bool ONE>
-__global__ void __launch_bounds__(BD_THREADS)
-k_bwd_diag(const C* __restrict__ M, int nG, int64_t K, const double2* __restrict__ fac, int n_freq,
-           const double* __restrict__ g, C* __restrict__ gM, double* __restrict__ gdE) {
-  __shared__ double s_fr2[BD_PAIRS][kMaxFreqBwd];   // 2 Re f
-  __shared__ double s_fpr[BD_PAIRS][kMaxFreqBwd];   // Re f'
-  __shared__ double s_red[BD_THREADS / 32][BD_PAIRS];
-  const int64_t k0 = (int64_t)blockIdx.x * BD_PAIRS;
-  const int np = (int)min((int64_t)BD_PAIRS, K - k0);
-  for (int e = threadIdx.x; e < np * n_freq; e += BD_THREADS) {
+//
+// P = 4 pairs by 128 threads.  Up to BD_FEW pairs that leaves most of the GPU idle
+// (64 pairs, N_G 2000, nine frequencies: 146 us a call): P = 1 by 256 threads, with
+// several frequencies 512, which take the pair's factors themselves (60 us; 75 by the
+// kernel before the grouping).  The line, six CTAs per SM: 1216 pairs, N_G 1200, one
+// frequency 68 us by fours and 75 one by one, at 532 67 and 62; with nine they meet there.
+constexpr int64_t BD_FEW = 912;
+template <typename C, bool ONE, int P, int NT>
+__global__ void __launch_bounds__(NT)
+k_bwd_diag(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
+           const double* __restrict__ E_col, const double* __restrict__ w_col, const double2* __restrict__ omega,
+           double delta, const double2* __restrict__ fac, int n_freq, const double* __restrict__ g, C* __restrict__ gM,
+           double* __restrict__ gdE) {
+  __shared__ double s_fr2[P][kMaxFreqBwd];   // 2 Re f
+  __shared__ double s_fpr[P][kMaxFreqBwd];   // Re f'
+  __shared__ double s_red[NT / 32][P];
+  const int64_t k0 = (int64_t)blockIdx.x * P;
+  const int np = (int)min((int64_t)P, K - k0);
+  for (int e = threadIdx.x; e < np * n_freq; e += NT) {
     const int j = e / n_freq, iw = e - j * n_freq;
-    const double2 f = fac[iw * K + k0 + j];
+    double2 f;
+    if (P == 1) {
+      const int64_t p = p0 + k0, iv = p / n_c, ic = p - iv * n_c;
+      double2 d;
+      factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, omega[iw], delta, &f, &d);
+      f = make_double2(2.0 * f.x, d.x);
+    } else {
+      f = fac[iw * K + k0 + j];
+    }
     s_fr2[j][iw] = f.x;
     s_fpr[j][iw] = f.y;
   }
   __syncthreads();
-  double t[BD_PAIRS] = {}, c[BD_PAIRS];
-  Split cs[BD_PAIRS];
+  double t[P] = {}, c[P];
+  Split cs[P];
   if (ONE)
 #pragma unroll
-    for (int j = 0; j < BD_PAIRS; ++j) {
+    for (int j = 0; j < P; ++j) {
       c[j] = j < np ? s_fr2[j][0] : 0.0;
       cs[j] = split_of(c[j]);
     }
-  for (int G = threadIdx.x; G < nG; G += BD_THREADS) {
-    C m[BD_PAIRS];
+  for (int G = threadIdx.x; G < nG; G += NT) {
+    C m[P];
 #pragma unroll
-    for (int j = 0; j < BD_PAIRS; ++j)
+    for (int j = 0; j < P; ++j)
       if (j < np) m[j] = M[(k0 + j) * nG + G];
-    if (ONE) {
+    if constexpr (ONE) {
       const double gw = g[G];
       const Split gs = split_of(gw);
 #pragma unroll
-      for (int j = 0; j < BD_PAIRS; ++j)
+      for (int j = 0; j < P; ++j)
         if (j < np) {
           gM[(k0 + j) * nG + G] = scaled(c[j], cs[j], gw, gs, m[j]);
           t[j] = fma(gw, square(m[j].x), t[j]);
           t[j] = fma(gw, square(m[j].y), t[j]);
         }
+    } else if constexpr (P == 1) {
+      const double2 d = make_double2((double)m[0].x, (double)m[0].y);
+      const double m2 = d.x * d.x + d.y * d.y;
+      double s = 0.0, s2 = 0.0;
+      for (int iw = 0; iw < n_freq; ++iw) {
+        const double gw = g[(int64_t)iw * nG + G];
+        s = fma(s_fr2[0][iw], gw, s);
+        s2 = fma(s_fpr[0][iw], gw, s2);
+      }
+      t[0] = fma(s2, m2, t[0]);
+      st_c(gM, k0 * nG + G, make_double2(s * d.x, s * d.y));
     } else {
-      double s[BD_PAIRS] = {}, s2[BD_PAIRS] = {};
+      double s[P] = {}, s2[P] = {};
       for (int iw = 0; iw < n_freq; ++iw) {
         const double gw = g[(int64_t)iw * nG + G];
 #pragma unroll
-        for (int j = 0; j < BD_PAIRS; ++j)
+        for (int j = 0; j < P; ++j)
           if (j < np) {
             s[j] = fma(s_fr2[j][iw], gw, s[j]);
             s2[j] = fma(s_fpr[j][iw], gw, s2[j]);
           }
       }
 #pragma unroll
-      for (int j = 0; j < BD_PAIRS; ++j)
+      for (int j = 0; j < P; ++j)
         if (j < np) {
           st_c(gM, (k0 + j) * nG + G, make_double2(s[j] * (double)m[j].x, s[j] * (double)m[j].y));
           t[j] = fma(s2[j], square(m[j].x), t[j]);
@@ -168,19 +195,24 @@ k_bwd_diag(const C* __restrict__ M, int nG, int64_t K, const double2* __restrict
         }
     }
   }
-  // four sums over the warp in six additions: lanes keep two, then one of them
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  static_assert(BD_PAIRS == 4, "reduction of four sums");
-  const bool hi = lane & 16, hi2 = lane & 8;
-  const double a0 = hi ? t[2] : t[0], a1 = hi ? t[3] : t[1], b0 = hi ? t[0] : t[2], b1 = hi ? t[1] : t[3];
-  const double u0 = a0 + __shfl_xor_sync(0xffffffffu, b0, 16), u1 = a1 + __shfl_xor_sync(0xffffffffu, b1, 16);
-  double r = (hi2 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 8);
-  for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  if ((lane & 7) == 0) s_red[warp][(hi ? 2 : 0) + (hi2 ? 1 : 0)] = r;
+  if constexpr (P == 4) {
+    // four sums over the warp in six additions: lanes keep two, then one of them
+    const bool hi = lane & 16, hi2 = lane & 8;
+    const double a0 = hi ? t[2] : t[0], a1 = hi ? t[3] : t[1], b0 = hi ? t[0] : t[2], b1 = hi ? t[1] : t[3];
+    const double u0 = a0 + __shfl_xor_sync(0xffffffffu, b0, 16), u1 = a1 + __shfl_xor_sync(0xffffffffu, b1, 16);
+    double r = (hi2 ? u1 : u0) + __shfl_xor_sync(0xffffffffu, hi2 ? u0 : u1, 8);
+    for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    if ((lane & 7) == 0) s_red[warp][(hi ? 2 : 0) + (hi2 ? 1 : 0)] = r;
+  } else {
+    static_assert(P == 1, "reduction of one or four sums");
+    for (int o = 16; o; o >>= 1) t[0] += __shfl_xor_sync(0xffffffffu, t[0], o);
+    if (lane == 0) s_red[warp][0] = t[0];
+  }
   __syncthreads();
   if (threadIdx.x < np) {
     double sum = 0.0;
-    for (int w = 0; w < BD_THREADS / 32; ++w) sum += s_red[w][threadIdx.x];
+    for (int w = 0; w < NT / 32; ++w) sum += s_red[w][threadIdx.x];
     gdE[k0 + threadIdx.x] = ONE ? s_fpr[threadIdx.x][0] * sum : sum;
   }
 }
@@ -495,13 +527,14 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
   double* gdE = work;
   if (diag) {
     double2* fac = reinterpret_cast<double2*>(work + (K + 1) / 2 * 2);
-    k_bwd_factors<<<dim3((unsigned)((K + 127) / 128), p->n_freq), 128, 0, s>>>(p0, K, n_c, E_v, E_col, w_col, p->d_omega,
-                                                                              p->delta, fac);
-    const unsigned grid = (unsigned)((K + BD_PAIRS - 1) / BD_PAIRS);
-    if (p->n_freq == 1)
-      k_bwd_diag<C, true><<<grid, BD_THREADS, 0, s>>>(M, nG, K, fac, p->n_freq, diag, gM, gdE);
-    else
-      k_bwd_diag<C, false><<<grid, BD_THREADS, 0, s>>>(M, nG, K, fac, p->n_freq, diag, gM, gdE);
+    const bool one = p->n_freq == 1, few = K <= BD_FEW;
+    if (!few)
+      k_bwd_factors<<<dim3((unsigned)((K + 127) / 128), p->n_freq), 128, 0, s>>>(p0, K, n_c, E_v, E_col, w_col, p->d_omega,
+                                                                                p->delta, fac);
+    auto* kern = few ? (one ? k_bwd_diag<C, true, 1, 256> : k_bwd_diag<C, false, 1, 512>)
+                     : (one ? k_bwd_diag<C, true, 4, 128> : k_bwd_diag<C, false, 4, 128>);
+    kern<<<(unsigned)(few ? K : (K + 3) / 4), few ? (one ? 256 : 512) : 128, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, p->d_omega,
+                                                                      p->delta, fac, p->n_freq, diag, gM, gdE);
   } else {
     const int ntile = (nG + 63) / 64;
     double* part = work + K;
