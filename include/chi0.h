@@ -50,8 +50,9 @@ typedef enum {
 } chi0_status;
 
 typedef enum {
-  CHI0_FP64 = 0,        /* FP64 accuracy end to end (contraction by exact modular products on the tensor
-                           cores, or FP64 multiply-adds where that is faster) */
+  CHI0_FP64 = 0,        /* FP64 accuracy end to end.  The contraction runs as exact modular products on the
+                           tensor cores where every element keeps an error of a few 2^-53 of its own
+                           sum_p |f_p M_p(G) M_p(G')|, else (and where that is faster) as FP64 multiply-adds */
   CHI0_SPLIT_BF16 = 1,  /* FP32 pair stage; contraction on tcgen05 with hi+lo BF16 operands */
   CHI0_SPLIT_FP16 = 2   /* FP32 pair stage; contraction on tcgen05 with hi+lo FP16 operands */
 } chi0_precision;
@@ -118,7 +119,9 @@ chi0_status chi0_plan_hermitian(chi0_plan plan, int* on);
 const char* chi0_last_error(chi0_plan plan);
 
 /* Bytes of device workspace held by the plan.  It grows on the first use of some calls (the
- * contraction of FP64 plans, the pipelined build, the dielectric inverse). */
+ * wavefunctions, pairs and contraction of FP64 plans, the pipelined build, the dielectric inverse).
+ * What a captured call uses is held until the plan is destroyed.  A workspace that cannot be had is
+ * asked for again by a later call. */
 size_t chi0_workspace_bytes(chi0_plan plan);
 
 /* Synchronise `stream` and report device-side failures recorded since the
@@ -129,7 +132,9 @@ chi0_status chi0_sync_status(chi0_plan plan, void* stream);
 /* Wavefunctions on the grid (plane-wave expansion used by M after Eq. 1):
  *   psi[b][r] = sum_{g in wavefunction sphere} coeff[b][g] exp(2 pi i g.r).
  * coeff: (device) [nb][npw] complex128 in the order of desc.gw.
- * psi:   (device) [nb][n1*n2*n3] complex (complex64 for split plans). */
+ * psi:   (device) [nb][n1*n2*n3] complex (complex64 for split plans).
+ * FP64 plans take scratch (at most 1 GiB) from a pool of the plan in stream order; a captured call's
+ * belongs to its graph. */
 chi0_status chi0_wfn_to_grid(chi0_plan plan, const void* coeff, int nb, void* psi, void* stream);
 
 /* Pair matrix elements (definition following Eq. 1), pruned to sphere iq:
@@ -376,11 +381,13 @@ chi0_status chi0_epsilon(chi0_plan plan, int iq, const void* chi0, const double*
  * complex128, row-major) by blocked Gauss-Jordan elimination with partial
  * pivoting (largest |re| + |im| in the column).  FP64 plans compute to FP64 accuracy:
  * an FP32 elimination refined by Newton steps in FP64, or, for matrices those do not
- * bring to FP64 accuracy and small ones, the elimination in FP64;
+ * bring to FP64 accuracy and small ones, the elimination in FP64 (in both, scaling a
+ * column by a power of two changes no digit);
  * split plans compute in FP32 on a complex64 copy and write the result back
  * as complex128 (forward error about cond(eps) x 1e-7).  Workspace (the
  * complex64 copy for split plans, panel buffers) is allocated at the first
- * call for a sphere this large and kept by the plan.  A zero pivot (singular
+ * call for a sphere this large and kept by the plan (a captured call needs one
+ * before it).  A zero pivot (singular
  * matrix) leaves non-finite values and makes the next chi0_sync_status return
  * CHI0_ERR_SINGULAR. */
 chi0_status chi0_epsilon_inverse(chi0_plan plan, int iq, void* eps, void* stream);

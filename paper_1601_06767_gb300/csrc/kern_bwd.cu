@@ -333,7 +333,7 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
 // neighbouring lanes share a pair and take its even and odd points.  Bound by the integer pipe
 // (reconstruction of two values from 52 residues), the FP64 pipe a third of it: 356 us for 4096
 // pairs, N_G 1200, one frequency (530 us with one CTA per SM, before its registers were bounded).
-// The whole adjoint of that size: 77.0 -> 1.02 ms.
+// The whole adjoint of that size: 77.0 -> 1.02 ms (0.98 without the check of the products' S).
 constexpr int BM_PAIRS = 16;
 template <typename C>
 __global__ void __launch_bounds__(256, 2)
@@ -533,8 +533,8 @@ static cudaError_t bwd_impl(chi0_plan_s* p, int nG, const C* M, int64_t p0, int6
                                                                                 p->delta, fac);
     auto* kern = few ? (one ? k_bwd_diag<C, true, 1, 256> : k_bwd_diag<C, false, 1, 512>)
                      : (one ? k_bwd_diag<C, true, 4, 128> : k_bwd_diag<C, false, 4, 128>);
-    kern<<<(unsigned)(few ? K : (K + 3) / 4), few ? (one ? 256 : 512) : 128, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, p->d_omega,
-                                                                      p->delta, fac, p->n_freq, diag, gM, gdE);
+    kern<<<(unsigned)(few ? K : (K + 3) / 4), few ? (one ? 256 : 512) : 128, 0, s>>>(
+        M, nG, p0, K, n_c, E_v, E_col, w_col, p->d_omega, p->delta, fac, p->n_freq, diag, gM, gdE);
   } else {
     const int ntile = (nG + 63) / 64;
     double* part = work + K;

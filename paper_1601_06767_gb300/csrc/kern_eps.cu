@@ -763,9 +763,10 @@ cudaError_t launch_epsilon(chi0_plan_s* p, int nG, const double2* chi, const dou
 // |row of A| |column of X|, where a graded A would lose the ratio of its columns (an
 // elimination does not: it gives the same digits for any column scaling).
 //
-// 1200^2: 42.6 -> 7.9 ms (FP32 inverse 6.2, one matrix's latency; two steps 0.8,
-// skipped kernels 0.7); 9 x 2500^2: 1047 ms at first, 72 ms.  Against quad precision
-// 1.8e-16 (relative Frobenius, eps-like matrices), 3.3e-16 by the elimination.
+// 1200^2: 42.6 -> 7.6 ms (FP32 inverse 6.2, one matrix's latency; two steps 0.8,
+// skipped kernels 0.6); 9 x 2500^2: 1047 -> 75 ms.  Against quad precision 5e-17
+// (relative Frobenius, eps-like matrices; 1.8e-16 before the remainders, at 71 ms),
+// 3.3e-16 by the elimination.
 namespace {
 constexpr int STEPS = 3;
 constexpr double LAST_STEP = 1.1102230246251565e-16;            // |R|^2 = 2^-53
@@ -807,7 +808,8 @@ __global__ void k_ref_init(int* __restrict__ todo, int nf) {
 }
 
 // values of the residue planes of one N x N product.  ADD = false: R = I - value and the sum of
-// |R|^2 over the block's elements; true: X += value.  REST: with the remainders' planes.  A warp takes 16 rows x 8 columns (as k_mod_add).
+// |R|^2 over the block's elements; true: X += value.  REST: with the remainders' planes.  A warp takes 16 rows
+// x 8 columns (as k_mod_add).
 template <bool ADD, bool REST = false>
 __global__ void __launch_bounds__(128) k_ref_value(const int16_t* __restrict__ P, int N, int ldR,
                                                    const int* __restrict__ sA, const int* __restrict__ sB,

@@ -49,74 +49,78 @@ constexpr int kK = 16;   // pairs per shared-memory step
 // one CTA per (64x64 tile of G', 64x64 tile of G, frequency); 16x16 threads, 4x4 outputs each.
 // FLAGS: only the tiles whose flag [n_freq][tiles][tiles] is not 0, and the sums of kK pairs are added up
 // apart: such tiles stand beside modular products (kern_mod.cu), and a sum of K terms of one sign in a
-// single chain carries 0.2 sqrt(K) 2^-53 of them, in chains of kK a quarter of that.
+// single chain carries 0.2 sqrt(K) 2^-53 of them, in chains of kK a quarter of that.  A CTA then steps
+// through the frequencies by the grid's depth (mostly there is nothing to do: 14,400 CTAs, one per tile and
+// frequency at N_G 2500 and nine of them, took 57 us to find that out).
 template <bool FLAGS>
 __global__ void __launch_bounds__(256)
-k_contract_f64(int nG, const double2* __restrict__ M, int64_t K, const double2* __restrict__ f,
+k_contract_f64(int nG, const double2* __restrict__ M, int64_t K, const double2* __restrict__ f, int n_freq,
                double2* __restrict__ chi, const int* __restrict__ flags) {
-  if (FLAGS && flags[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] == 0) return;
   __shared__ double2 As[kK][kT];
   __shared__ double2 Bs[kK][kT];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int H0 = blockIdx.x * kT, G0 = blockIdx.y * kT, iw = blockIdx.z;
-  const double2* fw = f + (int64_t)iw * K;
-  double2 acc[4][4], sum[4][4];
+  const int H0 = blockIdx.x * kT, G0 = blockIdx.y * kT;
+  for (int iw = blockIdx.z; iw < n_freq; iw += gridDim.z) {
+    if (FLAGS && flags[((size_t)iw * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] == 0) continue;
+    const double2* fw = f + (int64_t)iw * K;
+    double2 acc[4][4], sum[4][4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = sum[r][c] = make_double2(0.0, 0.0);
-  for (int64_t k0 = 0; k0 < K; k0 += kK) {
-    for (int e = threadIdx.x; e < kK * kT; e += blockDim.x) {
-      const int kk = e / kT, g = e - kk * kT;
-      const int64_t p = k0 + kk;
-      double2 a = make_double2(0.0, 0.0), b = make_double2(0.0, 0.0);
-      if (p < K) {
-        if (G0 + g < nG) a = cmul(fw[p], M[p * nG + G0 + g]);
-        if (H0 + g < nG) {
-          b = M[p * nG + H0 + g];
-          b.y = -b.y;
+      for (int c = 0; c < 4; ++c) acc[r][c] = sum[r][c] = make_double2(0.0, 0.0);
+    for (int64_t k0 = 0; k0 < K; k0 += kK) {
+      for (int e = threadIdx.x; e < kK * kT; e += blockDim.x) {
+        const int kk = e / kT, g = e - kk * kT;
+        const int64_t p = k0 + kk;
+        double2 a = make_double2(0.0, 0.0), b = make_double2(0.0, 0.0);
+        if (p < K) {
+          if (G0 + g < nG) a = cmul(fw[p], M[p * nG + G0 + g]);
+          if (H0 + g < nG) {
+            b = M[p * nG + H0 + g];
+            b.y = -b.y;
+          }
         }
+        As[kk][g] = a;
+        Bs[kk][g] = b;
       }
-      As[kk][g] = a;
-      Bs[kk][g] = b;
-    }
-    __syncthreads();
+      __syncthreads();
 #pragma unroll 4
-    for (int kk = 0; kk < kK; ++kk) {
-      double2 a[4], b[4];
+      for (int kk = 0; kk < kK; ++kk) {
+        double2 a[4], b[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+        for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
+        for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) cfma(acc[r][c], a[r], b[c]);
+          for (int c = 0; c < 4; ++c) cfma(acc[r][c], a[r], b[c]);
+      }
+      if (FLAGS)
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            sum[r][c].x += acc[r][c].x;
+            sum[r][c].y += acc[r][c].y;
+            acc[r][c] = make_double2(0.0, 0.0);
+          }
+      __syncthreads();
     }
-    if (FLAGS)
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < 4; ++r) {
+      const int G = G0 + ty + 16 * r;
+      if (G >= nG) continue;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          sum[r][c].x += acc[r][c].x;
-          sum[r][c].y += acc[r][c].y;
-          acc[r][c] = make_double2(0.0, 0.0);
-        }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int G = G0 + ty + 16 * r;
-    if (G >= nG) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int H = H0 + tx + 16 * c;
-      if (H >= nG) continue;
-      double2* o = chi + ((int64_t)iw * nG + G) * nG + H;
-      double2 v = *o;
-      v.x += FLAGS ? sum[r][c].x : acc[r][c].x;
-      v.y += FLAGS ? sum[r][c].y : acc[r][c].y;
-      *o = v;
+      for (int c = 0; c < 4; ++c) {
+        const int H = H0 + tx + 16 * c;
+        if (H >= nG) continue;
+        double2* o = chi + ((int64_t)iw * nG + G) * nG + H;
+        double2 v = *o;
+        v.x += FLAGS ? sum[r][c].x : acc[r][c].x;
+        v.y += FLAGS ? sum[r][c].y : acc[r][c].y;
+        *o = v;
+      }
     }
   }
 }
@@ -136,9 +140,12 @@ cudaError_t launch_contract_f64(const chi0_plan_s* p, int nG, const double2* M, 
                                 double2* chi, cudaStream_t s, const int* flags) {
   if (K <= 0) return cudaSuccess;
   const int t = (nG + kT - 1) / kT;
-  dim3 grid(t, t, p->n_freq);
-  if (flags) k_contract_f64<true><<<grid, 256, 0, s>>>(nG, M, K, f, chi, flags);
-  else k_contract_f64<false><<<grid, 256, 0, s>>>(nG, M, K, f, chi, nullptr);
+  if (flags) {
+    const int64_t deep = std::max<int64_t>(1, std::min<int64_t>(p->n_freq, 2048 / ((int64_t)t * t)));
+    k_contract_f64<true><<<dim3(t, t, (unsigned)deep), 256, 0, s>>>(nG, M, K, f, p->n_freq, chi, flags);
+  } else {
+    k_contract_f64<false><<<dim3(t, t, p->n_freq), 256, 0, s>>>(nG, M, K, f, p->n_freq, chi, nullptr);
+  }
   return cudaGetLastError();
 }
 
@@ -276,7 +283,7 @@ extern "C" chi0_status chi0_accumulate_fp64_noalloc(int n_G, const void* M, int 
     k_weights_noalloc<<<(unsigned)((K + 255) / 256), 256, 0, s>>>(p0, K, n_c, E_v, E_col, w_col, fl, n_freq, delta,
                                                                  scratch);
     k_contract_f64<false><<<dim3(t, t, n_freq), 256, 0, s>>>(n_G, (const double2*)M + p0 * n_G, K, scratch,
-                                                     (double2*)chi0, nullptr);
+                                                            n_freq, (double2*)chi0, nullptr);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
       set_global_error(std::string("chi0_accumulate_fp64_noalloc: launch: ") + cudaGetErrorString(e));

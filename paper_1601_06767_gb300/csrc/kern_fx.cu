@@ -14,7 +14,9 @@
 //
 // The unit follows the products and not the bands, so bands that overlap little lose
 // nothing: what a plane holds is rounded to 2^-56 of its own largest product, against
-// 2^-53 of every partial sum in FP64.
+// 2^-53 of every partial sum in FP64.  Against quad precision (relative Frobenius,
+// grids of 21 to 48 points): pairs 1.0-1.2e-16, FP64 sums 4.7-6.6e-16; wavefunctions
+// 0.9e-16, FP64 sums 5.8-7.0e-16.
 //
 // A line of n points is transformed at the wanted frequencies only, with the
 // symmetries of the twiddles folded out first: with h = n / 2 and a_i = x_i +

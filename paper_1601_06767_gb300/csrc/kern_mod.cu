@@ -4,14 +4,16 @@
 //
 // Steps of a block of K pairs: row norms and scales (k_mod_fmax, k_mod_rowmax,
 // k_mod_norms, k_mod_scales), residue planes of conj(M) and of W_w = f(w) M
-// (k_mod_pack), 26 products per frequency with their sums reduced modulo m
-// (k_mod_gemm), reconstruction and addition into chi0 (k_mod_add).
+// (k_mod_pack), 26 products per frequency with their sums reduced modulo m and one
+// of the magnitudes (k_mod_gemm), tiles that want FP64 sums (k_mod_check),
+// reconstruction and addition into chi0 (k_mod_add), those tiles (k_contract_f64).
 //
 // The CUDA-core contraction ran at the FP64 pipe's rate (two multiply-adds per clock
 // and SM): 790 ms for 2048 pairs, N_G 2500, nine frequencies.  This form takes
-// 6.4 ms: 4.0 ms of products (the 16-bit tensor pipe 67 % busy at 1.9 GHz, 1.6
-// PFLOP/s executed), 1.3 ms reconstruction, 0.75 ms planes, 0.2 ms norms.  The
-// static 8-atom contraction (3840 pairs, N_G 350): 15.97 ms -> 0.20 ms.
+// 6.4 ms: 4.05 ms of products (the 16-bit tensor pipe 67 % busy at 1.9 GHz, 1.6
+// PFLOP/s executed), 1.15 ms reconstruction, 0.71 ms planes, 0.19 ms norms; the check
+// of S (k_mod_check, its plane in all the steps) is 0.25 ms of it.  The static 8-atom
+// contraction (3840 pairs, N_G 350): 15.97 ms -> 0.20 ms.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 

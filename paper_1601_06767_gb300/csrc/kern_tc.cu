@@ -1220,7 +1220,8 @@ k_contract_tc2(const __grid_constant__ TcBatch P, int* __restrict__ status) {
 // 254 us).  The sums over pairs cannot be shared out (their FP32 order is
 // fixed), but the components and columns can: a stage has half the MMAs, of half the
 // columns.  It takes 1.0 us of 2.1 (six products; about 1.5 with 128 columns, whose ring has two
-// stages): loads of 512-byte rows, one load per operand and four accumulators did
+// stages), where its 24 MMAs alone would take some 0.4 us.  What else sets the pace is not
+// known: loads of 512-byte rows, one load per operand and four accumulators did
 // not shorten it.  Same bits; whole accumulate calls with 64 columns, N_G 350,
 // one frequency: 3840 pairs BF16 286 -> 160 us, 4096 pairs FP16 201 -> 131 us, 256
 // pairs 62 -> 46 us; 500 points and two frequencies (128 items): 311 -> 173 us.
