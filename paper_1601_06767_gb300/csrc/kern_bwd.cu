@@ -217,16 +217,17 @@ k_bwd_diag(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, cons
   }
 }
 
-// dense upstream, one frequency: tile of 32 pairs x 64 sphere points, K loop over H
+// dense upstream, one frequency after the other: tile of 32 pairs x 64 sphere points, K loop over H
 //   Y[p][G] = sum_H M[p][H] Gam[G][H],  Z[p][G] = sum_H M[p][H] conj(Gam[H][G])
 //   gM[p][G] += conj(f_p) Y + f_p Z;  part[p][gt] += Re( f'_p conj(sum_{G in tile} conj(M[p][G]) Y[p][G]) )
-// flags (or NULL): [pairs / 64][ntile], only the tiles that are not 0.  first: = in place of +=
+// (= at the first frequency).  flags (or NULL): [pairs / 64][ntile], only the tiles that are not 0 (mostly none, so one
+// launch and not one per frequency to find that out).
 template <typename C>
 __global__ void __launch_bounds__(256)
 k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, const double* __restrict__ E_v,
-            const double* __restrict__ E_col, const double* __restrict__ w_col, double2 om, double delta,
-            const double2* __restrict__ Gam, C* __restrict__ gM, double* __restrict__ part, int ntile,
-            const int* __restrict__ flags, bool first) {
+            const double* __restrict__ E_col, const double* __restrict__ w_col, const double2* __restrict__ omega,
+            int n_freq, double delta, const double2* __restrict__ Gam, C* __restrict__ gM, double* __restrict__ part,
+            int ntile, const int* __restrict__ flags) {
   if (flags && flags[(blockIdx.y >> 1) * ntile + blockIdx.x] == 0) return;
   constexpr int TP = 32, TG = 64, TH = 16;
   __shared__ double2 Ms[TP][TH + 1];
@@ -237,90 +238,93 @@ k_bwd_dense(const C* __restrict__ M, int nG, int64_t p0, int64_t K, int n_c, con
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // 16 x 16 threads: 2 pairs x 4 points each
   const int64_t kp0 = (int64_t)blockIdx.y * TP;
   const int G0 = blockIdx.x * TG;
-  if (threadIdx.x < TP) {
-    const int64_t k = kp0 + threadIdx.x;
-    double2 f = make_double2(0, 0), fp = make_double2(0, 0);
-    if (k < K) {
-      const int64_t p = p0 + k, iv = p / n_c, ic = p - iv * n_c;
-      factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, om, delta, &f, &fp);
+  for (int iw = 0; iw < n_freq; ++iw, Gam += (int64_t)nG * nG) {
+    __syncthreads();                       // the previous frequency's readers are done
+    if (threadIdx.x < TP) {
+      const int64_t k = kp0 + threadIdx.x;
+      double2 f = make_double2(0, 0), fp = make_double2(0, 0);
+      if (k < K) {
+        const int64_t p = p0 + k, iv = p / n_c, ic = p - iv * n_c;
+        factors(E_v[iv] - E_col[ic], w_col ? w_col[ic] : 1.0, omega[iw], delta, &f, &fp);
+      }
+      sf[threadIdx.x] = f;
+      sfp[threadIdx.x] = fp;
     }
-    sf[threadIdx.x] = f;
-    sfp[threadIdx.x] = fp;
-  }
-  double2 y[2][4], z[2][4];
+    double2 y[2][4], z[2][4];
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+    for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) y[r][c] = z[r][c] = make_double2(0, 0);
-  for (int H0 = 0; H0 < nG; H0 += TH) {
-    for (int e = threadIdx.x; e < TP * TH; e += blockDim.x) {
-      const int r = e / TH, h = e - r * TH;
-      const int64_t k = kp0 + r;
-      Ms[r][h] = (k < K && H0 + h < nG) ? ld_d(M, k * nG + H0 + h) : make_double2(0, 0);
-    }
-    for (int e = threadIdx.x; e < TG * TH; e += blockDim.x) {
-      const int gg = e / TH, h = e - gg * TH;
-      const int G = G0 + gg, H = H0 + h;
-      Gs[gg][h] = (G < nG && H < nG) ? Gam[(int64_t)G * nG + H] : make_double2(0, 0);
-      const int hh = e / TG, g2 = e - hh * TG;
-      const int Gb = G0 + g2, Hb = H0 + hh;
-      double2 v = (Gb < nG && Hb < nG) ? Gam[(int64_t)Hb * nG + Gb] : make_double2(0, 0);
-      v.y = -v.y;
-      Gt[hh][g2] = v;
-    }
-    __syncthreads();
+      for (int c = 0; c < 4; ++c) y[r][c] = z[r][c] = make_double2(0, 0);
+    for (int H0 = 0; H0 < nG; H0 += TH) {
+      for (int e = threadIdx.x; e < TP * TH; e += blockDim.x) {
+        const int r = e / TH, h = e - r * TH;
+        const int64_t k = kp0 + r;
+        Ms[r][h] = (k < K && H0 + h < nG) ? ld_d(M, k * nG + H0 + h) : make_double2(0, 0);
+      }
+      for (int e = threadIdx.x; e < TG * TH; e += blockDim.x) {
+        const int gg = e / TH, h = e - gg * TH;
+        const int G = G0 + gg, H = H0 + h;
+        Gs[gg][h] = (G < nG && H < nG) ? Gam[(int64_t)G * nG + H] : make_double2(0, 0);
+        const int hh = e / TG, g2 = e - hh * TG;
+        const int Gb = G0 + g2, Hb = H0 + hh;
+        double2 v = (Gb < nG && Hb < nG) ? Gam[(int64_t)Hb * nG + Gb] : make_double2(0, 0);
+        v.y = -v.y;
+        Gt[hh][g2] = v;
+      }
+      __syncthreads();
 #pragma unroll 4
-    for (int h = 0; h < TH; ++h) {
-      double2 m[2];
+      for (int h = 0; h < TH; ++h) {
+        double2 m[2];
 #pragma unroll
-      for (int r = 0; r < 2; ++r) m[r] = Ms[ty + 16 * r][h];
+        for (int r = 0; r < 2; ++r) m[r] = Ms[ty + 16 * r][h];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const double2 a = Gs[tx + 16 * c][h], b = Gt[h][tx + 16 * c];
+        for (int c = 0; c < 4; ++c) {
+          const double2 a = Gs[tx + 16 * c][h], b = Gt[h][tx + 16 * c];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          cfma(y[r][c], m[r], a);
-          cfma(z[r][c], m[r], b);
+          for (int r = 0; r < 2; ++r) {
+            cfma(y[r][c], m[r], a);
+            cfma(z[r][c], m[r], b);
+          }
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
-  }
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    const int rr = ty + 16 * r;
-    const int64_t k = kp0 + rr;
-    double2 qs = make_double2(0, 0);
-    if (k < K) {
-      const double2 f = sf[rr];
-      const double2 fc = make_double2(f.x, -f.y);
+    for (int r = 0; r < 2; ++r) {
+      const int rr = ty + 16 * r;
+      const int64_t k = kp0 + rr;
+      double2 qs = make_double2(0, 0);
+      if (k < K) {
+        const double2 f = sf[rr];
+        const double2 fc = make_double2(f.x, -f.y);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int G = G0 + tx + 16 * c;
-        if (G >= nG) continue;
-        double2 gv = first ? make_double2(0, 0) : ld_d(gM, k * nG + G);
-        const double2 t1 = cmul(fc, y[r][c]), t2 = cmul(f, z[r][c]);
-        gv.x += t1.x + t2.x;
-        gv.y += t1.y + t2.y;
-        st_c(gM, k * nG + G, gv);
-        const double2 m = ld_d(M, k * nG + G);
-        cfma(qs, make_double2(m.x, -m.y), y[r][c]);
+        for (int c = 0; c < 4; ++c) {
+          const int G = G0 + tx + 16 * c;
+          if (G >= nG) continue;
+          double2 gv = iw == 0 ? make_double2(0, 0) : ld_d(gM, k * nG + G);
+          const double2 t1 = cmul(fc, y[r][c]), t2 = cmul(f, z[r][c]);
+          gv.x += t1.x + t2.x;
+          gv.y += t1.y + t2.y;
+          st_c(gM, k * nG + G, gv);
+          const double2 m = ld_d(M, k * nG + G);
+          cfma(qs, make_double2(m.x, -m.y), y[r][c]);
+        }
+      }
+      sq[rr][tx] = 0.0;
+      if (k < K) {
+        const double2 fp = sfp[rr];
+        sq[rr][tx] = fp.x * qs.x + fp.y * qs.y;     // Re(f' conj(q))
       }
     }
-    sq[rr][tx] = 0.0;
-    if (k < K) {
-      const double2 fp = sfp[rr];
-      sq[rr][tx] = fp.x * qs.x + fp.y * qs.y;     // Re(f' conj(q))
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < TP) {
-    const int64_t k = kp0 + threadIdx.x;
-    if (k < K) {
-      double sum = 0.0;
-      for (int t = 0; t < 16; ++t) sum += sq[threadIdx.x][t];
-      double* o = part + k * ntile + blockIdx.x;
-      *o = first ? sum : *o + sum;
+    __syncthreads();
+    if (threadIdx.x < TP) {
+      const int64_t k = kp0 + threadIdx.x;
+      if (k < K) {
+        double sum = 0.0;
+        for (int t = 0; t < 16; ++t) sum += sq[threadIdx.x][t];
+        double* o = part + k * ntile + blockIdx.x;
+        *o = iw == 0 ? sum : *o + sum;
+      }
     }
   }
 }
@@ -512,12 +516,8 @@ static void dense_direct(chi0_plan_s* p, int nG, const C* M, int64_t p0, int64_t
                          const double* E_col, const double* w_col, const double2* gamma, C* gM, double* part,
                          const int* flags, cudaStream_t s) {
   const int ntile = (nG + 63) / 64;
-  const dim3 grid(ntile, (unsigned)((K + 31) / 32));
-  for (int iw = 0; iw < p->n_freq; ++iw) {
-    const double2 om = make_double2(p->om_re[iw], p->om_im[iw]);
-    k_bwd_dense<C><<<grid, 256, 0, s>>>(M, nG, p0, K, n_c, E_v, E_col, w_col, om, p->delta,
-                                        gamma + (size_t)iw * nG * nG, gM, part, ntile, flags, iw == 0);
-  }
+  k_bwd_dense<C><<<dim3(ntile, (unsigned)((K + 31) / 32)), 256, 0, s>>>(
+      M, nG, p0, K, n_c, E_v, E_col, w_col, p->d_omega, p->n_freq, p->delta, gamma, gM, part, ntile, flags);
 }
 
 template <typename C>
